@@ -32,16 +32,17 @@ extern "C" mirror_status mirror_create(mirror_ctx** out, const mirror_model_desc
     int count = 0;
     if (cudaGetDeviceCount(&count) != cudaSuccess || device < 0 || device >= count) return MIRROR_ERR_CUDA;
     MIRROR_CUDA_OK(cudaSetDevice(device));
-    cudaDeviceProp prop;
-    MIRROR_CUDA_OK(cudaGetDeviceProperties(&prop, device));
-    if (prop.major != 10) return MIRROR_ERR_UNSUPPORTED;   // the kernels are sm_100a only: no fallback path
+    int major = 0, num_sms = 0;                            // (two attributes: the whole property struct takes milliseconds)
+    MIRROR_CUDA_OK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device));
+    MIRROR_CUDA_OK(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device));
+    if (major != 10) return MIRROR_ERR_UNSUPPORTED;        // the kernels are sm_100a only: no fallback path
 
     mirror_ctx* ctx = new (std::nothrow) mirror_ctx();
     if (!ctx) return MIRROR_ERR_ARG;
     ctx->desc = *desc;
     mirror_tuning_from_env(&ctx->tune);
     ctx->device = device;
-    ctx->num_sms = prop.multiProcessorCount;
+    ctx->num_sms = num_sms;
     ctx->scale = desc->softmax_scale > 0.f ? desc->softmax_scale : 1.0f / sqrtf((float)desc->head_dim);
     ctx->temperature = desc->temperature > 0.f ? desc->temperature : 1.0f;
     void* fn = nullptr;
@@ -67,7 +68,6 @@ void mirror_tuning_from_env(MirrorTuning* t) {
     geti("MIRROR_ATTN_GROUPS", &t->attn_groups, 1, 1 << 20);
     geti("MIRROR_ATTN_WHOLE_UNITS", &t->attn_whole_units, 0, 1);
     geti("MIRROR_ATTN_SNAP", &t->attn_snap, 0, 1 << 20);
-    geti("MIRROR_ATTN_RING", &t->attn_ring, 44, 66);
     geti("MIRROR_LM_PAIR2_MAX_ROWS", &t->lm_pair2_max_rows, 0, 128);
     geti("MIRROR_LM_CTAS_PER_SM", &t->lm_ctas_per_sm, 1, 2);
     geti("MIRROR_LM_STAGES", &t->lm_stages, 2, 64);
@@ -201,8 +201,8 @@ void mirror_ws_layout(const mirror_ctx* ctx, size_t M, MirrorWsLayout* out, size
     L.zeroed = at;
     at += kWsZeroedBytes;
     L.attn_partial = at;
-    // two partial slots per CTA (a CTA's range of KV tiles cuts at most two units), 128 rows each
-    L.attn_partial_bytes = align_up((size_t)ctx->num_sms * 2 * 128 * (size_t)(ctx->desc.head_dim + 4) * sizeof(float), 256);
+    // two record slots per CTA (a CTA's range of KV tiles cuts at most two units) for each of its two streams of 128 rows
+    L.attn_partial_bytes = align_up((size_t)ctx->num_sms * 4 * 128 * (size_t)(ctx->desc.head_dim + 4) * sizeof(float), 256);
     at += L.attn_partial_bytes;
     L.end_attn = at;
     L.lm_partial = at;
@@ -223,11 +223,13 @@ void mirror_ws_layout(const mirror_ctx* ctx, size_t M, MirrorWsLayout* out, size
     L.accept_scratch = at;
     at += align_up(B * 2 * (size_t)ctx->desc.vocab * sizeof(double), 256);
     L.end_accept = at;
-    // the candidate lists of the fused Top-kappa share the front of the logits region (a call either spills or selects)
-    L.lm_topk = L.logits;
-    // (four lists per CTA and row, two CTAs per SM; only up to 256 rows, one row chunk: beyond, Top-kappa selects from spilled logits)
+    // The candidate lists of the fused Top-kappa (four per CTA and row, two CTAs per SM; only up to 256 rows, one row chunk:
+    // beyond, Top-kappa selects from spilled logits) share the attention's records, which no LM-head call needs, or where
+    // those are too small the front of the logits region (a call either spills or selects).
     L.lm_topk_bytes = M <= 256 ? align_up((size_t)8 * ctx->num_sms * M * (size_t)MIRROR_MAX_TOPK * 8, 256) : 0;
-    L.end_topk = L.lm_topk + L.lm_topk_bytes;
+    const bool in_attn = L.lm_topk_bytes <= L.attn_partial_bytes;
+    L.lm_topk = in_attn ? L.attn_partial : L.logits;
+    L.end_topk = in_attn ? L.end_lmhead : L.lm_topk + L.lm_topk_bytes;
     *out = L;
 }
 

@@ -28,7 +28,6 @@ struct MirrorTuning {
     int attn_groups = 0;             // MIRROR_ATTN_GROUPS: upper limit of CTA groups (0: all)
     int attn_whole_units = 1;        // MIRROR_ATTN_WHOLE_UNITS: 0 = never trade CTA groups for whole units
     int attn_snap = 4;               // MIRROR_ATTN_SNAP: boundary snapping distance in tiles
-    int attn_ring = 0;               // MIRROR_ATTN_RING: K/V ring depths as two digits, e.g. 64 (0: deepest that fits)
     int lm_pair2_max_rows = 128;     // MIRROR_LM_PAIR2_MAX_ROWS: two CTAs per SM up to this many rows
     int lm_ctas_per_sm = 0;          // MIRROR_LM_CTAS_PER_SM: 1 or 2 (0: by rows)
     int lm_stages = 0;               // MIRROR_LM_STAGES: fewer pipeline stages than fit (0: all)
@@ -120,9 +119,13 @@ struct MirrorAttnFp8 {
 // serialization.
 mirror_status mirror_kv_quantize_launch(mirror_ctx* ctx, const void* x, int n_layers, int64_t layer_stride, int64_t layer_elems,
                                        int inner, const float* scale, void* out_fp8, cudaStream_t stream);
+// keep_rounding: the call has to give the same bits as earlier ones on the same inputs and sizes (mirror_target_forward).
 mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
-                                 float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8 = nullptr);
+                                 float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8 = nullptr, bool keep_rounding = false);
+mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
+                                        const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
+                                        float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8);
 
 // bf16 tensor map with 128-byte swizzle.  dims/box are innermost-first; strides_bytes[i] is the byte
 // stride of dimension i+1 (rank-1 entries).
