@@ -31,6 +31,24 @@ EXPORTS = [
 ]
 
 
+# Argument types of the exports, one letter each: p pointer, i int, u unsigned, f float, z size_t, l int64.  (Declared, so that
+# plain Python integers can be passed for pointers: wrapping every argument costs more than the call.)
+_SIGNATURES = {
+    "mirror_create": "ppi", "mirror_destroy": "p", "mirror_workspace_bytes": "pppup", "mirror_set_workspace": "ppz",
+    "mirror_attn_verify": "p" * 9, "mirror_attn_verify_fp8": "ppppppppfppp", "mirror_kv_scales_fp8": "ppillipp",
+    "mirror_kv_quantize_fp8": "ppillippp", "mirror_lmhead_reduce": "ppipippi" + "p" * 8, "mirror_quantize_rows_fp8": "ppiippp",
+    "mirror_lmhead_reduce_fp8": "pppi" + "p" * 7, "mirror_lmhead_reduce_noalloc": "ipipiif" + "p" * 4,
+    "mirror_lmhead_noalloc_status": "ipp", "mirror_accept_select": "ppppp", "mirror_early_exit_tap": "ppipippp",
+    "mirror_overlap_mass": "ppppiipp", "mirror_kv_commit": "p" * 9, "mirror_kv_commit_fp8": "p" * 9, "mirror_trie_build": "piiipppp",
+    "mirror_verify_step": "p" * 13, "mirror_linear_scratch_bytes": "piiip", "mirror_linear": "ppipiipppzp",
+    "mirror_embed_rows": "pppipp", "mirror_rmsnorm": "pppiifpp", "mirror_target_scratch_bytes": "pppp",
+    "mirror_target_forward": "p" * 12 + "zp", "mirror_target_forward_fp8": "p" * 17 + "zp",
+    "mirror_verify_step_fp8": "p" * 8 + "f" + "p" * 7, "mirror_verify_step_host": "p" * 17, "mirror_set_stage_events": "pp",
+    "mirror_device_status": "ppp", "mirror_launch_count": "pp",
+}
+_CTYPES = {"p": C.c_void_p, "i": C.c_int, "u": C.c_uint, "f": C.c_float, "z": C.c_size_t, "l": C.c_int64}
+
+
 class MirrorError(RuntimeError):
     def __init__(self, code: int, where: str, text: str):
         super().__init__(f"{where}: mirror_status {code} ({text})")
@@ -94,7 +112,9 @@ def load_library():
         lib.mirror_status_str.argtypes = [C.c_int]
         for name in EXPORTS:
             if name != "mirror_status_str":
-                getattr(lib, name).restype = C.c_int
+                fn = getattr(lib, name)
+                fn.restype = C.c_int
+                fn.argtypes = [_CTYPES[c] for c in _SIGNATURES[name]]
         _lib = lib
     return _lib
 
@@ -105,20 +125,21 @@ def _check(code: int, where: str):
 
 
 def _ptr(t: Optional[torch.Tensor], dtype=None, name: str = "tensor"):
+    """Device address of a tensor, as an integer (None for None)."""
     if t is None:
         return None
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if dtype is not None and t.dtype != dtype:
+    if dtype is not None and t.dtype is not dtype:
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> C.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+def _stream(stream) -> int:
+    # (the raw handle: building a torch.cuda.Stream object costs 2 us a call)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
 
 
 def mirror_trie_build(branch_tokens, root_token: int):
@@ -180,8 +201,16 @@ class AcceptResult:
         self.decide_row = torch.empty(batch, **i32)
         self.reuse_slot = torch.empty(batch, **i32)
 
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        object.__setattr__(self, "_struct", None)          # (another tensor: the addresses are looked up again)
+
     def struct(self) -> AcceptOut:
-        return AcceptOut(*[C.c_void_p(getattr(self, f).data_ptr()) for f, _ in AcceptOut._fields_])
+        s = self._struct
+        if s is None:
+            s = AcceptOut(*[getattr(self, f).data_ptr() for f, _ in AcceptOut._fields_])
+            object.__setattr__(self, "_struct", s)
+        return s
 
     def cpu(self) -> dict:
         return {f: getattr(self, f).cpu().numpy() for f, _ in AcceptOut._fields_}
@@ -198,6 +227,7 @@ class Mirror:
         self._ctx = C.c_void_p()
         _check(self.lib.mirror_create(C.byref(self._ctx), C.byref(self.desc), device), "mirror_create")
         self._ws = None
+        self._need = {}              # workspace bytes by (what, batch, nodes): they depend on nothing else
         self._keep = []
 
     def close(self):
@@ -236,14 +266,19 @@ class Mirror:
     def workspace_bytes(self, tree: Tree, kv: Optional[KV], what: int) -> int:
         out = C.c_size_t()
         _check(self.lib.mirror_workspace_bytes(self._ctx, C.byref(tree), C.byref(kv) if kv is not None else None,
-                                               C.c_uint(what), C.byref(out)), "mirror_workspace_bytes")
+                                               what, C.byref(out)), "mirror_workspace_bytes")
         return out.value
 
     def ensure_workspace(self, tree: Tree, kv: Optional[KV], what: int):
-        need = self.workspace_bytes(tree, kv, what)
+        key = (what, tree.batch, tree.n_nodes)
+        need = self._need.get(key)
+        if need is None:
+            need = self.workspace_bytes(tree, kv, what)
+            if len(self._need) < 4096:
+                self._need[key] = need
         if self._ws is None or self._ws.numel() < need:
             self._ws = torch.empty(need, dtype=torch.uint8, device=self.device)
-            _check(self.lib.mirror_set_workspace(self._ctx, C.c_void_p(self._ws.data_ptr()), C.c_size_t(need)),
+            _check(self.lib.mirror_set_workspace(self._ctx, C.c_void_p(self._ws.data_ptr()), need),
                    "mirror_set_workspace")
 
     # ---- entry points -----------------------------------------------------------------------
@@ -277,7 +312,7 @@ class Mirror:
         """x bf16 [L, ..., Hkv, <inner elements>] -> fp32 scales [L, Hkv] (max|x| / 448 per layer and KV head)."""
         L, stride, layer_elems, inner = self._kv_fp8_dims(x, inner)
         scale = torch.empty((L, self.desc.n_kv_heads), dtype=torch.float32, device=x.device)
-        _check(self.lib.mirror_kv_scales_fp8(self._ctx, _ptr(x, torch.bfloat16, "x"), L, C.c_int64(stride), C.c_int64(layer_elems),
+        _check(self.lib.mirror_kv_scales_fp8(self._ctx, _ptr(x, torch.bfloat16, "x"), L, stride, layer_elems,
                                              inner, _ptr(scale, torch.float32, "scale"), _stream(stream)), "mirror_kv_scales_fp8")
         return scale
 
@@ -285,7 +320,7 @@ class Mirror:
         """x bf16 -> e4m3 codes (uint8, same shape) under the given [L, Hkv] scales."""
         L, stride, layer_elems, inner = self._kv_fp8_dims(x, inner)
         out = torch.empty(x.shape, dtype=torch.uint8, device=x.device)
-        _check(self.lib.mirror_kv_quantize_fp8(self._ctx, _ptr(x, torch.bfloat16, "x"), L, C.c_int64(stride), C.c_int64(layer_elems),
+        _check(self.lib.mirror_kv_quantize_fp8(self._ctx, _ptr(x, torch.bfloat16, "x"), L, stride, layer_elems,
                                                inner, _ptr(scale, torch.float32, "scale"), _ptr(out, torch.uint8, "out"),
                                                _stream(stream)), "mirror_kv_quantize_fp8")
         return out
@@ -408,7 +443,7 @@ class Mirror:
         refs = [norm_final]
         for i, w in enumerate(layers):
             for f, _ in LayerWeights._fields_:
-                setattr(arr[i], f, _ptr(w[f], torch.bfloat16, f).value)
+                setattr(arr[i], f, _ptr(w[f], torch.bfloat16, f))
                 refs.append(w[f])
         t = Target(len(layers), intermediate, rope_theta, rms_eps, arr, _ptr(norm_final, torch.bfloat16, "norm_final"))
         t._refs = (arr, refs)
@@ -426,7 +461,7 @@ class Mirror:
         out = torch.empty((M, N), dtype=torch.bfloat16, device=self.device)
         _check(self.lib.mirror_linear(self._ctx, _ptr(x, torch.bfloat16, "x"), M, _ptr(W, torch.bfloat16, "W"), N, K,
                                       _ptr(residual, torch.bfloat16, "residual"), _ptr(out), _ptr(scratch),
-                                      C.c_size_t(scratch.numel()), _stream(stream)), "mirror_linear")
+                                      scratch.numel(), _stream(stream)), "mirror_linear")
         return out
 
     def mirror_embed_rows(self, table: torch.Tensor, tokens: torch.Tensor, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
@@ -466,7 +501,7 @@ class Mirror:
         self.ensure_workspace(tree, kv, WS_ATTN)
         _check(self.lib.mirror_target_forward(self._ctx, C.byref(target), C.byref(kv), C.byref(tree), _ptr(x, torch.bfloat16, "x"),
                                               _ptr(out["q"]), _ptr(out["k_new"]), _ptr(out["v_new"]), _ptr(out["attn_out"]),
-                                              _ptr(out["x_out"]), _ptr(out["hidden"]), _ptr(scratch), C.c_size_t(scratch.numel()),
+                                              _ptr(out["x_out"]), _ptr(out["hidden"]), _ptr(scratch), scratch.numel(),
                                               _stream(stream)), "mirror_target_forward")
         out["_scratch"] = scratch
         return out
@@ -489,7 +524,7 @@ class Mirror:
                                                   _ptr(k_scale, torch.float32, "k_scale"), _ptr(v_scale, torch.float32, "v_scale"), qs,
                                                   _ptr(out["q"]), _ptr(out["k_new"]), _ptr(out["v_new"]), _ptr(out["k_new8"]),
                                                   _ptr(out["v_new8"]), _ptr(out["attn_out"]), _ptr(out["x_out"]), _ptr(out["hidden"]),
-                                                  _ptr(scratch), C.c_size_t(scratch.numel()), _stream(stream)),
+                                                  _ptr(scratch), scratch.numel(), _stream(stream)),
                "mirror_target_forward_fp8")
         out["_scratch"] = scratch
         return out
