@@ -74,7 +74,8 @@ struct AttnParams {
     int n_rt;                             // row tiles of one KV head
     int n_groups;                         // CTA groups (grid = n_groups * n_cta)
     int snap_cap;                         // boundaries move to a unit boundary that is at most this many tiles away
-    int whole_units;                      // 1: prefer a group count that divides equal-length units (no cuts)
+    int units;                            // layers x requests x heads (or pairs of heads)
+    int whole_groups;                     // group count that divides the units evenly (attn::whole_unit_groups), 0: none
     int never_cut;                        // 1: units are so short that they are dealt out whole whatever their lengths
     int max_pages, num_pages, layer_pages;
     int tree_slots;
@@ -103,20 +104,20 @@ __device__ __forceinline__ void dev_check(const AttnParams& p, int detail) {
 struct UnitPos {
     int layer, b, g;
     int tile_in_unit, tiles_in_unit;
-    long long unit_first_tile;
+    int unit_first_tile;
 };
-__device__ __noinline__ UnitPos locate(long long x, const AttnParams& p, const int* cumT, long long tiles_per_layer) {
+__device__ __noinline__ UnitPos locate(int x, const AttnParams& p, const int* cumT, int tiles_per_layer) {
     UnitPos u;
     const int hu = p.Hkv / p.heads_per_unit;
     u.layer = (int)((uint32_t)x / (uint32_t)tiles_per_layer);         // (the tile count fits 31 bits: checked in the prologue)
-    const long long rem = x - (long long)u.layer * tiles_per_layer;
+    const int rem = x - u.layer * tiles_per_layer;
     int b = 0;
-    while (b + 1 < p.B && (long long)hu * cumT[b + 1] <= rem) ++b;
+    while (b + 1 < p.B && hu * cumT[b + 1] <= rem) ++b;
     const int Tb = cumT[b + 1] - cumT[b];
-    const long long r2 = rem - (long long)hu * cumT[b];
+    const int r2 = rem - hu * cumT[b];
     u.b = b;
     u.g = (int)((uint32_t)r2 / (uint32_t)Tb);
-    u.tile_in_unit = (int)(r2 - (long long)u.g * Tb);
+    u.tile_in_unit = r2 - u.g * Tb;
     u.tiles_in_unit = Tb;
     u.unit_first_tile = x - u.tile_in_unit;
     return u;
@@ -140,12 +141,12 @@ __device__ __forceinline__ void fill_segment(Segment& s, int left, const AttnPar
     s.tiles = tiles_of(s.len, p.tree_slots);
     s.t_last = min(s.tiles, s.t_first + left);
 }
-__device__ __noinline__ Segment first_segment(long long x, long long x_end, const AttnParams& p, const int* cumT, const int* s_len,
-                                              long long tiles_per_layer) {
+__device__ __noinline__ Segment first_segment(int x, int x_end, const AttnParams& p, const int* cumT, const int* s_len,
+                                              int tiles_per_layer) {
     const UnitPos u = locate(x, p, cumT, tiles_per_layer);
     Segment s;
     s.layer = u.layer; s.b = u.b; s.g = u.g; s.t_first = u.tile_in_unit;
-    fill_segment(s, (int)(x_end - x), p, s_len);
+    fill_segment(s, x_end - x, p, s_len);
     return s;
 }
 // the unit behind s (a segment that is followed by another one ends with its unit)
@@ -202,68 +203,76 @@ __device__ __forceinline__ bool elect_one() {            // one lane of a conver
     return r != 0;
 }
 
-// How the tile sequence is cut into one range per CTA group.
+// How the tile sequence is cut into one range per CTA group.  (This runs in front of every launch's first copy, by one
+// warp and from a cold instruction cache: few divisions, and those of 32 bits.)
 struct Partition {
-    long long tiles_per_layer, total_tiles, snap_tol;
-    int n_groups;
+    int tiles_per_layer, total_tiles;     // (total_tiles -1: the sequence does not fit 31 bits)
+    int n_groups, snap_tol;
+    int share, rest;                      // total_tiles = n_groups * share + rest
 };
 __device__ __forceinline__ Partition make_partition(const AttnParams& p, const int* cumT) {
     Partition q;
-    const int hu = p.Hkv / p.heads_per_unit;
-    q.tiles_per_layer = (long long)hu * cumT[p.B];
-    q.total_tiles = q.tiles_per_layer * p.L;
-    const long long units = (long long)p.L * p.B * hu;
+    const long long per = (long long)(p.Hkv / p.heads_per_unit) * cumT[p.B], total = per * p.L;
+    q.tiles_per_layer = (int)per;
+    q.total_tiles = total < (1ll << 31) ? (int)total : -1;
     // Units of equal length (every request has the same number of tiles): a group count that divides the units, if one
     // exists within 15% of the CTA groups there are, gives every group the same number of WHOLE units: no unit is cut,
     // nothing is left to merge and all groups end together, which is worth more than the few SMs left idle.
     bool equal_units = true;
     for (int b = 1; b < p.B; ++b) equal_units &= (cumT[b + 1] - cumT[b]) == cumT[1];
-    const int g = (p.whole_units && equal_units && units >= p.n_groups) ? attn::whole_unit_groups(p.n_groups, units) : 0;
     // Else every group gets at least one tile, or two where its streams take alternate tiles (one alone would leave a stream
     // without work and the merge with twice the records).
-    q.n_groups = p.never_cut ? (int)min((long long)p.n_groups, units)
-               : g > 0       ? g
-                             : (int)min((long long)p.n_groups, max(1ll, q.total_tiles / (p.mode == kSplit ? 2 : 1)));
+    q.n_groups = p.never_cut                        ? min(p.n_groups, p.units)
+               : p.whole_groups > 0 && equal_units ? p.whole_groups
+                                                   : min(p.n_groups, max(1, p.mode == kSplit ? q.total_tiles >> 1 : q.total_tiles));
+    q.share = (int)((uint32_t)q.total_tiles / (uint32_t)q.n_groups);
+    q.rest = q.total_tiles - q.share * q.n_groups;
     // A boundary that falls within snap_tol tiles of a unit boundary moves there (a cut costs about as much as a tile).
     // snap_tol is at most a quarter of the smallest even share, so boundaries stay strictly increasing.
-    q.snap_tol = q.n_groups > 0 ? min((long long)p.snap_cap, (q.total_tiles / q.n_groups) / 4) : 0;
+    q.snap_tol = min(p.snap_cap, q.share >> 2);
     return q;
 }
-__device__ __noinline__ long long group_begin(const Partition& q, int g, const AttnParams& p, const int* cumT) {
+__device__ __noinline__ int group_begin(const Partition& q, int g, const AttnParams& p, const int* cumT) {
     if (g <= 0) return 0;
     if (g >= q.n_groups) return q.total_tiles;
     if (p.never_cut) {                                                // first tile of unit number units * g / n_groups
-        const int hu = p.Hkv / p.heads_per_unit;
-        const long long unit = (long long)p.L * p.B * hu * g / q.n_groups;
-        const int layer = (int)(unit / (p.B * hu)), r = (int)(unit - (long long)layer * p.B * hu), b = r / hu;
-        return layer * q.tiles_per_layer + (long long)hu * cumT[b] + (long long)(r - b * hu) * (cumT[b + 1] - cumT[b]);
+        const int hu = p.Hkv / p.heads_per_unit, per = p.B * hu;
+        const int us = p.units / q.n_groups, unit = us * g + (p.units - us * q.n_groups) * g / q.n_groups;
+        const int layer = unit / per, r = unit - layer * per, b = r / hu;
+        return layer * q.tiles_per_layer + hu * cumT[b] + (r - b * hu) * (cumT[b + 1] - cumT[b]);
     }
-    const long long e = q.total_tiles * g / q.n_groups;
+    const int e = q.share * g + (int)((uint32_t)(q.rest * g) / (uint32_t)q.n_groups);       // total_tiles * g / n_groups
     if (q.snap_tol == 0) return e;
     const UnitPos u = locate(e, p, cumT, q.tiles_per_layer);
-    const long long lo = u.unit_first_tile, hi = lo + u.tiles_in_unit;
-    const long long best = (e - lo <= hi - e) ? lo : hi;
-    const long long dist = best > e ? best - e : e - best;
+    const int lo = u.unit_first_tile, hi = lo + u.tiles_in_unit;
+    const int best = (e - lo <= hi - e) ? lo : hi;
+    const int dist = best > e ? best - e : e - best;
     return dist <= q.snap_tol ? best : e;
 }
 
-// Prefix lengths (clamped to the page table) and the tile counts they give; all threads of the block.
+// Prefix lengths (clamped to the page table) and the tile counts they give, by one warp.
 __device__ __forceinline__ void load_lengths(const AttnParams& p, int* cumT, int* s_len, bool report) {
-    for (int b = threadIdx.x; b < p.B; b += blockDim.x) {
-        int len = p.prefix_len[b];
+    const int lane = threadIdx.x & 31;
+    int acc = 0;
+    if (lane == 0) cumT[0] = 0;
+#pragma unroll 1
+    for (int b0 = 0; b0 < p.B; b0 += 32) {
+        const int b = b0 + lane;
+        int len = b < p.B ? p.prefix_len[b] : 0;
         if (len < 0 || len > p.max_pages * kSlotTok) {
             if (report) dev_check(p, 300 + b);
             len = len < 0 ? 0 : p.max_pages * kSlotTok;
         }
-        s_len[b] = len;
+        int sum = b < p.B ? tiles_of(len, p.tree_slots) : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += v;
+        }
+        if (b < p.B) { s_len[b] = len; cumT[b + 1] = acc + sum; }
+        acc += __shfl_sync(0xffffffffu, sum, 31);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        cumT[0] = 0;
-        for (int b = 0; b < p.B; ++b) cumT[b + 1] = (acc += tiles_of(s_len[b], p.tree_slots));
-    }
-    __syncthreads();
+    __syncwarp();
 }
 
 // Which (head of the unit, row tile) stream `grp` of CTA `rb` of a group is, and whether both streams share K/V tiles.
@@ -387,23 +396,24 @@ __device__ __noinline__ void mask_tile(uint32_t s_addr, int slot0, const Segment
     }
     tmem_st_wait();
 }
-// Row maximum over chunks of 16 scores (a unit's first tile, and what is redone).
+// Row maximum over chunks of 32 scores (a unit's first tile, and what is redone).
 __device__ __noinline__ float tile_max(uint32_t s_addr, int chunks) {
     float m = -INFINITY;
 #pragma unroll 1
     for (int c = 0; c < chunks; ++c) {
-        uint32_t r[16];
-        ptx::tmem_ld_32x32b_x16(s_addr + (uint32_t)(c * 16), r);
-        tmem_ld_wait16(r);
+        uint32_t r[32];
+        ptx::tmem_ld_32x32b_x32(s_addr + (uint32_t)(c * 32), r);
+        tmem_ld_wait32(r);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) m = fmaxf(m, __uint_as_float(r[j]));
+        for (int j = 0; j < 32; j += 2)          // (three operands: one instruction for two scores)
+            asm("max.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(__uint_as_float(r[j])), "f"(__uint_as_float(r[j + 1])));
     }
     return m;
 }
 // A new offset for the rows whose sum over the 64 scores at s_addr outgrew the limit (`grow`): the maximum of those scores.
 // The row's accumulator (o_cols columns, 0: none yet) is rescaled to it.  Returns (offset, factor).
 __device__ __noinline__ float2 move_offset(uint32_t s_addr, uint32_t o_addr, int o_cols, bool grow, float off, float sc) {
-    const float mx = tile_max(s_addr, 4);
+    const float mx = tile_max(s_addr, 2);
     const float next = grow ? mx * sc : off, alpha = grow ? exp2f(off - next) : 1.f;
 #pragma unroll 1
     for (int c = 0; c < o_cols; c += 16) {
@@ -470,18 +480,21 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
     ptx::tc_fence_after();
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();                 // the kernel behind may be scheduled as soon as SMs free up
-    load_lengths(p, cumT, s_len, true);
-    const uint32_t tmem_base = ctrl->tmem_base;
-    if (tid == 0) {
+    if (warp == 0) {
+        load_lengths(p, cumT, s_len, true);
         const Partition part = make_partition(p, cumT);
-        const bool fits = part.total_tiles < (1ll << 31) && (ptx::smem_u32(smem) & 1023) == 0;
-        if (!fits) dev_check(p, 600);
-        const bool works = fits && group < part.n_groups;
-        const long long x0 = works ? group_begin(part, group, p, cumT) : 0, x1 = works ? group_begin(part, group + 1, p, cumT) : 0;
-        ctrl->n_tiles = (int)(x1 - x0);
-        if (x0 < x1) ctrl->first = first_segment(x0, x1, p, cumT, s_len, part.tiles_per_layer);
+        const bool fits = part.total_tiles >= 0 && (ptx::smem_u32(smem) & 1023) == 0;
+        if (!fits && lane == 0) dev_check(p, 600);
+        int x = 0;
+        if (fits && group < part.n_groups && lane < 2) x = group_begin(part, group + lane, p, cumT);
+        const int x1 = __shfl_sync(0xffffffffu, x, 1);
+        if (lane == 0) {
+            ctrl->n_tiles = x1 - x;
+            if (x < x1) ctrl->first = first_segment(x, x1, p, cumT, s_len, part.tiles_per_layer);
+        }
     }
     __syncthreads();
+    const uint32_t tmem_base = ctrl->tmem_base;
     const int n_tiles = ctrl->n_tiles;               // tiles of this CTA's range
 
     if (warp < 4) {
@@ -489,8 +502,9 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             // ======================================================================= K and V producers
             // Ring order (first use by the issuing warps): K of step 0, then per step V, next K -- of stream 0 and, when the
             // streams have K/V tiles of their own, of stream 1.  Both warps walk that order; each fills its own stages.
-            auto produce = [&](auto v_tag) {
-                constexpr bool V = decltype(v_tag)::value;
+            // (one copy of the code for both)
+            {
+                const bool V = warp == 3;
                 const CUtensorMap* const map = V ? &tm.v : &tm.k;
                 Segment sg = ctrl->first;                          // of the step that is filled next
                 int t = sg.t_first, left = n_tiles;                // its tile; tiles from it to the end of the range
@@ -650,9 +664,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     // let copies already in flight land before the CTA's shared memory goes away (every stage's last fill)
                     for (int s = 0; s < n_stages; ++s) ptx::mbar_wait(&ctrl->full[s], (s < (int)st ? ph : ph ^ 1) ^ 1, 20000000ll);
                 }
-            };
-            if (warp == 3) produce(std::true_type{});
-            else produce(std::false_type{});
+            }
         } else if (n_tiles > 0) {
             // ======================================================================= tensor-core issuers
             // One warp per stream: what a warp executes between two chains (waits, ring bookkeeping, ~800 cycles) is more than the
@@ -810,7 +822,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     if ((t + 1) * kTileSlots > sg.pages_full) mask_tile(s_addr, t * kTileSlots, sg, anc0, anc1);
                     // The offset is set by the first tile in which the row sees anything (before that every P was 0).
                     if (__any_sync(0xffffffffu, off == -INFINITY)) {
-                        const float mx = tile_max(s_addr, 8);
+                        const float mx = tile_max(s_addr, 4);
                         if (off == -INFINITY) off = mx * sc;       // (-inf when nothing is visible yet)
                     }
                     // Two halves of 64 scores, one copy of the code.  P of a half goes over S columns that have been read.
@@ -904,41 +916,33 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             ptx::tc_fence_after();
             if (warp_has_rows) {
                 const float inv = 1.f / Lsum;
-                // split: this warp combines its half of the columns of both accumulators; otherwise all columns of its own
-                const int c_lo = split ? grp * (D / 64) : 0, c_hi = split ? c_lo + D / 64 : D / 32;
+                // split: this warp combines its half of the columns of both accumulators; otherwise all columns of its own.
+                // (16 columns at a time: this runs once per unit, and what it costs is mostly the instruction fetch)
+                const int c_lo = split ? grp * (D / 2) : 0, c_hi = split ? c_lo + D / 2 : D;
+                const uint32_t o_first = split ? lane_base + kTmemO : o_addr;
+                if (!split) w0 = M != -INFINITY ? 1.f : 0.f;
+                if (whole) { w0 *= inv; w1 *= inv; }
 #pragma unroll 1
-                for (int c4 = c_lo; c4 < c_hi; ++c4) {
-                    uint32_t r[32];
-                    float acc[32];
-                    ptx::tmem_ld_32x32b_x32((split ? lane_base + kTmemO : o_addr) + (uint32_t)(c4 * 32), r);
-                    tmem_ld_wait32(r);
-                    if (!split) {
+                for (int c = c_lo; c < c_hi; c += 16) {
+                    uint32_t r[16];
+                    float acc[16];
+                    ptx::tmem_ld_32x32b_x16(o_first + (uint32_t)c, r);
+                    tmem_ld_wait16(r);
+                    // (an accumulator that no P V wrote may hold anything: a weight of 0 does not read it)
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) acc[j] = M != -INFINITY ? __uint_as_float(r[j]) : 0.f;
-                    } else {
-                        // (an accumulator that no P V wrote may hold anything: a weight of 0 does not read it)
+                    for (int j = 0; j < 16; ++j) acc[j] = w0 != 0.f ? w0 * __uint_as_float(r[j]) : 0.f;
+                    if (split) {
+                        ptx::tmem_ld_32x32b_x16(o_first + (uint32_t)(D + c), r);
+                        tmem_ld_wait16(r);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) acc[j] = w0 != 0.f ? w0 * __uint_as_float(r[j]) : 0.f;
-                        ptx::tmem_ld_32x32b_x32(lane_base + kTmemO + (uint32_t)(D + c4 * 32), r);
-                        tmem_ld_wait32(r);
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) acc[j] = w1 != 0.f ? fmaf(w1, __uint_as_float(r[j]), acc[j]) : acc[j];
+                        for (int j = 0; j < 16; ++j) acc[j] = w1 != 0.f ? fmaf(w1, __uint_as_float(r[j]), acc[j]) : acc[j];
                     }
-                    if (whole) {
-                        if (row_ok) {
+                    if (!whole) {
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                uint4 v;
-                                v.x = pack_bf16(acc[j * 8 + 0] * inv, acc[j * 8 + 1] * inv);
-                                v.y = pack_bf16(acc[j * 8 + 2] * inv, acc[j * 8 + 3] * inv);
-                                v.z = pack_bf16(acc[j * 8 + 4] * inv, acc[j * 8 + 5] * inv);
-                                v.w = pack_bf16(acc[j * 8 + 6] * inv, acc[j * 8 + 7] * inv);
-                                *reinterpret_cast<uint4*>(orow + c4 * 32 + j * 8) = v;
-                            }
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) rec[(size_t)(c4 * 32 + j) * kRows] = acc[j];
+                        for (int j = 0; j < 16; ++j) rec[(size_t)(c + j) * kRows] = acc[j];
+                    } else if (row_ok) {
+                        *reinterpret_cast<uint4*>(orow + c) = make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
+                        *reinterpret_cast<uint4*>(orow + c + 8) = make_uint4(pack_bf16(acc[8], acc[9]), pack_bf16(acc[10], acc[11]), pack_bf16(acc[12], acc[13]), pack_bf16(acc[14], acc[15]));
                     }
                 }
                 if (!split || grp == 0) {
@@ -977,10 +981,11 @@ template <int D>
 __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_constant__ AttnParams p) {
     __shared__ int cumT[kAttnMaxBatch + 1];
     __shared__ int s_len[kAttnMaxBatch];
-    __shared__ long long s_begin[kMergeMaxGroups];
+    __shared__ int s_begin[kMergeMaxGroups];
     const int tid = threadIdx.x;
     // (the prefix lengths were complete before the attention kernel began)
-    load_lengths(p, cumT, s_len, false);
+    if (tid < 32) load_lengths(p, cumT, s_len, false);
+    __syncthreads();
     const Partition part = make_partition(p, cumT);
     const int g = blockIdx.x + 1;
     const int n_str = p.mode == kSplit ? 1 : 2;
@@ -989,8 +994,8 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_
     // A block with nothing to merge must still wait for the attention kernel: the kernel behind this one in the stream
     // only waits for THIS grid to complete, so a grid whose blocks all left early would let it read attention outputs
     // that are still being written.
-    if (g >= part.n_groups || part.total_tiles >= (1ll << 31) || !id.exists) { ptx::grid_dep_wait(); return; }
-    const long long x = group_begin(part, g, p, cumT);
+    if (g >= part.n_groups || part.total_tiles < 0 || !id.exists) { ptx::grid_dep_wait(); return; }
+    const int x = group_begin(part, g, p, cumT);
     const UnitPos u = locate(x, p, cumT, part.tiles_per_layer);
     if (u.tile_in_unit == 0) { ptx::grid_dep_wait(); return; }                  // the boundary is a unit boundary (block-uniform)
     // every group's first tile, computed side by side (a unit shared by many groups is looked up from here instead of
@@ -1000,12 +1005,12 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_
         for (int t = tid; t < part.n_groups; t += kMergeThreads) s_begin[t] = group_begin(part, t, p, cumT);
         __syncthreads();
     }
-    auto begin_of = [&](int t) -> long long { return tabled ? s_begin[t] : group_begin(part, t, p, cumT); };
+    auto begin_of = [&](int t) -> int { return tabled ? s_begin[t] : group_begin(part, t, p, cumT); };
     // the groups ga..gb hold this unit's parts; the blocks of the boundaries ga+1..gb share the merge by columns
     int ga = g - 1;
     while (ga > 0 && begin_of(ga) > u.unit_first_tile) --ga;
     int gb = g;
-    const long long unit_last = u.unit_first_tile + u.tiles_in_unit - 1;
+    const int unit_last = u.unit_first_tile + u.tiles_in_unit - 1;
     while (gb + 1 < part.n_groups && begin_of(gb + 1) <= unit_last) ++gb;
     const int parts = gb - ga + 1;
     const int n_blocks = parts - 1, j_blk = g - (ga + 1);
@@ -1118,10 +1123,14 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     if (ctx->tune.attn_groups >= 1 && ctx->tune.attn_groups <= p.n_groups) p.n_groups = ctx->tune.attn_groups;
     if (p.n_groups < 1) return MIRROR_ERR_SHAPE;
     p.snap_cap = (ctx->tune.attn_snap + 1) / 2;              // (given in tiles of 64 tokens)
-    p.whole_units = ctx->tune.attn_whole_units;
     // Units of at most six tiles (the page table says how long a prefix can be) take a CTA less time whole than the merge
     // kernel behind a cut would: a launch and a pass over the records, ~6 us.
-    p.never_cut = p.whole_units && (kv->max_pages_per_req + (p.n + kSlotTok - 1) / kSlotTok + kTileSlots - 1) / kTileSlots <= 6;
+    const bool whole = ctx->tune.attn_whole_units != 0;
+    const int64_t units = (int64_t)p.L * p.B * (Hkv / p.heads_per_unit);
+    if (units >= (1 << 24)) return MIRROR_ERR_SHAPE;
+    p.units = (int)units;
+    p.whole_groups = whole && units >= p.n_groups ? attn::whole_unit_groups(p.n_groups, units) : 0;
+    p.never_cut = whole && (kv->max_pages_per_req + (p.n + kSlotTok - 1) / kSlotTok + kTileSlots - 1) / kTileSlots <= 6;
     p.wait_limit = ctx->tune.wait_limit_cycles;
     p.stall_after = (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_attn_left-- > 0) ? ctx->tune.test_stall_after : -1;
     p.max_pages = kv->max_pages_per_req; p.num_pages = kv->num_pages;
@@ -1175,8 +1184,7 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         MIRROR_CUDA_OK(cudaGetLastError());
         // One request: all units have the same length whatever it is, so the host can tell when the partition gives every
         // group whole units (each unit holds at least one tile): nothing is cut and the merge kernel has nothing to do.
-        const long long units = (long long)p.L * p.B * (Hkv / p.heads_per_unit);
-        const bool no_cuts = p.never_cut || (p.whole_units && p.B == 1 && units >= p.n_groups && attn::whole_unit_groups(p.n_groups, units) > 0);
+        const bool no_cuts = p.never_cut || (p.B == 1 && p.whole_groups > 0);
         if (p.n_groups > 1 && !no_cuts) {
             // which units the partition cut is only known on the device (it depends on the prefix lengths)
             const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)(p.n_cta * (p.mode == kSplit ? 1 : 2)));
