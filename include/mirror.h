@@ -418,10 +418,11 @@ mirror_status mirror_verify_step_fp8(mirror_ctx* ctx, const mirror_kv* kv, const
  *   d_q, d_k_new, d_v_new: DEVICE staging buffers of the same shapes, and tree->tokens (device, written here);
  *                   they must not be in use by work on other streams
  *   h_out           HOST copies of the decision (any member may be NULL); valid once `stream` has been synchronised
- * Copies run on an internal stream (created on first use) and begin after all work already queued on `stream`.  The
- * layers' attention problems are independent and the LM head reads only the last layer's output, so the last layer is
- * copied and attended to first, the LM head and the acceptance follow, and the other layers arrive in up to eleven pieces
- * while the LM head runs; each is attended to once it has landed, after the decision has been sent back.
+ * Copies run on internal streams (created on first use) and begin after all work already queued on `stream`.  The
+ * layers' attention problems are independent and the LM head reads only the last layer's output (not even that with
+ * explicit hidden rows), so the LM head and the acceptance come first, behind the last layer's attention where they need
+ * it; the other layers arrive while the LM head runs, and are attended to after the decision has been sent back: what has
+ * arrived by then in one launch, the rest piece by piece.
  * Everything else as in mirror_verify_step (attn_out holds all layers when `stream` has drained).  Does not synchronise. */
 typedef struct {
     int32_t* n_accepted;   /* [B] */

@@ -84,6 +84,7 @@ extern "C" mirror_status mirror_destroy(mirror_ctx* ctx) {
     if (ctx->d_status) cudaFree(ctx->d_status);
     if (ctx->copy_stream) {
         cudaStreamDestroy(ctx->copy_stream);
+        if (ctx->back_stream) cudaStreamDestroy(ctx->back_stream);
         for (cudaEvent_t e : ctx->copy_ev)
             if (e) cudaEventDestroy(e);
     }

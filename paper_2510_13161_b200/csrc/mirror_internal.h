@@ -41,10 +41,8 @@ struct MirrorTuning {
 };
 void mirror_tuning_from_env(MirrorTuning* t);
 
-// mirror_verify_step_host copies and attends to a step's layers in this many pieces (the last layer first, alone).  The
-// pieces' copies are what bounds the host-buffer step on a large model (1.7 GB of Q per step on the 66B-class workload),
-// and the last piece's attention is what is left exposed behind them, so the pieces are kept small.
-constexpr int kMirrorHostChunks = 12;
+// mirror_verify_step_host copies and attends to a step's layers in at most this many pieces (see verify_step.cu).
+constexpr int kMirrorHostChunks = 32;
 struct mirror_ctx {
     mirror_model_desc desc;
     MirrorTuning tune;
@@ -61,7 +59,8 @@ struct mirror_ctx {
     cudaEvent_t stage_ev[4] = {nullptr, nullptr, nullptr, nullptr};
     bool stage_ev_on = false;
     cudaStream_t copy_stream = nullptr;                     // mirror_verify_step_host: created on first use
-    cudaEvent_t copy_ev[kMirrorHostChunks + 1] = {};
+    cudaStream_t back_stream = nullptr;                     // ... and the decision's way back
+    cudaEvent_t copy_ev[kMirrorHostChunks + 4] = {};        // the pieces, then: tokens, call begins, decision made, decision sent
     PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
 };
 

@@ -67,12 +67,42 @@ struct HostIO {                       // host-buffer variant: pinned host inputs
 };
 
 constexpr int kHostChunks = kMirrorHostChunks;
+enum { kEvTokens = kHostChunks, kEvBegin, kEvDecided, kEvSent };       // events behind the pieces' own
 
 mirror_status ensure_copy_stream(mirror_ctx* ctx) {
     if (ctx->copy_stream) return MIRROR_OK;
     MIRROR_CUDA_OK(cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
-    for (int i = 0; i < kHostChunks + 1; ++i) MIRROR_CUDA_OK(cudaEventCreateWithFlags(&ctx->copy_ev[i], cudaEventDisableTiming));
+    MIRROR_CUDA_OK(cudaStreamCreateWithFlags(&ctx->back_stream, cudaStreamNonBlocking));
+    for (cudaEvent_t& e : ctx->copy_ev) MIRROR_CUDA_OK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     return MIRROR_OK;
+}
+
+// Pieces of a host-buffer step: layers [l0[c], l1[c]) are copied together and attended to in one launch, in this order.
+//   - Without explicit hidden rows the LM head needs the last layer's output: that layer is a piece of its own, the first.
+//   - What arrives while the LM head streams its weights (its time from the bytes and operations it moves; copies at 50 GB/s,
+//     PCIe as measured) is one piece: it is attended to after the decision anyway, and one launch over 47 layers takes 94 us
+//     where eleven launches took 300.
+//   - The rest is attended to as it arrives, in pieces of at least 3 MB (60 us of copying: a launch costs ~27 us however few
+//     layers it has), and small enough that the last one's attention, which nothing hides, stays short.
+struct HostPieces {
+    int n = 0, l0[kHostChunks], l1[kHostChunks];
+    void add(int a, int b) { if (b > a) { l0[n] = a; l1[n] = b; ++n; } }
+};
+HostPieces plan_pieces(int layers, bool last_first, double layer_bytes, double lm_bytes, double lm_flops) {
+    constexpr double kCopyRate = 50e9, kPiece = 3e6;
+    const double lm_s = lm_bytes / 6.4e12 > lm_flops / 1.2e15 ? lm_bytes / 6.4e12 : lm_flops / 1.2e15;
+    HostPieces h;
+    const int rest = last_first ? layers - 1 : layers;
+    if (last_first) h.add(layers - 1, layers);
+    int bulk = (int)(lm_s * kCopyRate / layer_bytes);
+    if (bulk > rest || (rest - bulk) * layer_bytes < kPiece) bulk = rest;
+    h.add(0, bulk);
+    const int left = rest - bulk;
+    int k = (int)(left * layer_bytes / kPiece);
+    if (k > kHostChunks - 2) k = kHostChunks - 2;
+    if (k > left) k = left;
+    for (int c = 0; c < k; ++c) h.add(bulk + (int)((long long)left * c / k), bulk + (int)((long long)left * (c + 1) / k));
+    return h;
 }
 
 mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const void* q, const void* k_new,
@@ -102,12 +132,12 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     cudaStream_t s = (cudaStream_t)stream;
 
     // (host-buffer variant) pieces of layers, copied on the second stream and attended to in that order
-    int n_pieces = 0, piece_l0[kHostChunks] = {}, piece_l1[kHostChunks] = {};
+    HostPieces pieces;
     const size_t q_layer = M * (size_t)ctx->desc.n_q_heads * ctx->desc.head_dim * 2;        // bytes per layer
     const size_t kv_layer = M * (size_t)ctx->desc.n_kv_heads * ctx->desc.head_dim * 2;
     auto attend_piece = [&](int c) -> mirror_status {
         MIRROR_CUDA_OK(cudaStreamWaitEvent(s, ctx->copy_ev[c], 0));
-        const int l0 = piece_l0[c], l1 = piece_l1[c];
+        const int l0 = pieces.l0[c], l1 = pieces.l1[c];
         mirror_kv kv_c = *kv;
         kv_c.k_pool = (const __nv_bfloat16*)kv->k_pool + (size_t)l0 * kv->layer_stride;
         kv_c.v_pool = (const __nv_bfloat16*)kv->v_pool + (size_t)l0 * kv->layer_stride;
@@ -122,26 +152,21 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
         st = mirror_attn_launch(ctx, kv, tree, ti, q, k_new, v_new, attn_out, nullptr, (float*)(ws + L.attn_partial), s, f8);
         if (st != MIRROR_OK) return st;
     } else {
-        // Host inputs.  The layers' attention problems are independent of one another and the LM head reads only the
-        // last layer's output, so the last layer is copied and attended to first, the LM head and the acceptance follow
-        // at once, and the other layers are copied in pieces on a second stream while the LM head streams its weights;
-        // each piece is attended to as soon as it has landed (after the decision has gone back to the host).  The
-        // copies start only after everything already queued on `stream` (the previous step may still read the staging
-        // buffers).
+        // Host inputs.  The layers' attention problems are independent of one another and the LM head reads only the last
+        // layer's output (or rows of its own), so the decision comes first and the layers it does not need are copied on a
+        // second stream meanwhile.  The copies start only after everything already queued on `stream` (the previous step may
+        // still read the staging buffers).
         st = ensure_copy_stream(ctx);
         if (st != MIRROR_OK) return st;
         cudaStream_t cs = ctx->copy_stream;
-        MIRROR_CUDA_OK(cudaEventRecord(ctx->copy_ev[kHostChunks], s));
-        MIRROR_CUDA_OK(cudaStreamWaitEvent(cs, ctx->copy_ev[kHostChunks], 0));
+        MIRROR_CUDA_OK(cudaEventRecord(ctx->copy_ev[kEvBegin], s));
+        MIRROR_CUDA_OK(cudaStreamWaitEvent(cs, ctx->copy_ev[kEvBegin], 0));
         MIRROR_CUDA_OK(cudaMemcpyAsync((void*)tree->tokens, io->h_tokens, M * sizeof(int32_t), cudaMemcpyHostToDevice, cs));
-        const int Lyr = kv->num_layers;
-        n_pieces = 1 + (Lyr - 1 < kHostChunks - 1 ? Lyr - 1 : kHostChunks - 1);
-        for (int c = 0; c < n_pieces; ++c) {
-            // piece 0: the last layer; pieces 1..: the layers before it, in order
-            const int l0 = c == 0 ? Lyr - 1 : (int)((long long)(Lyr - 1) * (c - 1) / (n_pieces - 1));
-            const int l1 = c == 0 ? Lyr : (int)((long long)(Lyr - 1) * c / (n_pieces - 1));
-            piece_l0[c] = l0; piece_l1[c] = l1;
-            const size_t nl = (size_t)(l1 - l0);
+        MIRROR_CUDA_OK(cudaEventRecord(ctx->copy_ev[kEvTokens], cs));
+        pieces = plan_pieces(kv->num_layers, hidden == nullptr, (double)(q_layer + 2 * kv_layer), 2.0 * ctx->desc.vocab * ctx->desc.hidden,
+                             2.0 * M * ctx->desc.vocab * ctx->desc.hidden);
+        for (int c = 0; c < pieces.n; ++c) {
+            const size_t l0 = (size_t)pieces.l0[c], nl = (size_t)(pieces.l1[c] - pieces.l0[c]);
             MIRROR_CUDA_OK(cudaMemcpyAsync((uint8_t*)q + l0 * q_layer, (const uint8_t*)io->h_q + l0 * q_layer, nl * q_layer,
                                            cudaMemcpyHostToDevice, cs));
             MIRROR_CUDA_OK(cudaMemcpyAsync((uint8_t*)k_new + l0 * kv_layer, (const uint8_t*)io->h_k_new + l0 * kv_layer, nl * kv_layer,
@@ -150,8 +175,10 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
                                            cudaMemcpyHostToDevice, cs));
             MIRROR_CUDA_OK(cudaEventRecord(ctx->copy_ev[c], cs));
         }
-        st = attend_piece(0);
-        if (st != MIRROR_OK) return st;
+        if (!hidden) {
+            st = attend_piece(0);
+            if (st != MIRROR_OK) return st;
+        }
     }
     if (ev) MIRROR_CUDA_OK(cudaEventRecord(ctx->stage_ev[1], s));
 
@@ -169,6 +196,7 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
                               ev ? ctx->stage_ev[2] : nullptr);
     if (st != MIRROR_OK) return st;
 
+    if (io) MIRROR_CUDA_OK(cudaStreamWaitEvent(s, ctx->copy_ev[kEvTokens], 0));
     mirror_accept_in in = *acc;
     in.target_argmax = d_argmax;
     in.logits = d_logits;
@@ -178,18 +206,24 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     st = mirror_accept_launch(ctx, tree, ti, &in, out, s, tree_scratch);
     if (st != MIRROR_OK) return st;
     if (ev) MIRROR_CUDA_OK(cudaEventRecord(ctx->stage_ev[3], s));
-    if (io && io->h_out) {
-        const mirror_accept_host_out* h = io->h_out;
+    const mirror_accept_host_out* h = io ? io->h_out : nullptr;
+    if (h) {
+        // the decision goes back on a stream of its own: four short copies would hold the attention up by ~10 us
         const size_t B = (size_t)tree->batch;
-        if (h->n_accepted) MIRROR_CUDA_OK(cudaMemcpyAsync(h->n_accepted, out->n_accepted, B * 4, cudaMemcpyDeviceToHost, s));
-        if (h->best_branch) MIRROR_CUDA_OK(cudaMemcpyAsync(h->best_branch, out->best_branch, B * 4, cudaMemcpyDeviceToHost, s));
-        if (h->n_emitted) MIRROR_CUDA_OK(cudaMemcpyAsync(h->n_emitted, out->n_emitted, B * 4, cudaMemcpyDeviceToHost, s));
-        if (h->emitted) MIRROR_CUDA_OK(cudaMemcpyAsync(h->emitted, out->emitted, B * (size_t)(tree->gamma + 1) * 4, cudaMemcpyDeviceToHost, s));
+        cudaStream_t bs = ctx->back_stream;
+        MIRROR_CUDA_OK(cudaEventRecord(ctx->copy_ev[kEvDecided], s));
+        MIRROR_CUDA_OK(cudaStreamWaitEvent(bs, ctx->copy_ev[kEvDecided], 0));
+        if (h->n_accepted) MIRROR_CUDA_OK(cudaMemcpyAsync(h->n_accepted, out->n_accepted, B * 4, cudaMemcpyDeviceToHost, bs));
+        if (h->best_branch) MIRROR_CUDA_OK(cudaMemcpyAsync(h->best_branch, out->best_branch, B * 4, cudaMemcpyDeviceToHost, bs));
+        if (h->n_emitted) MIRROR_CUDA_OK(cudaMemcpyAsync(h->n_emitted, out->n_emitted, B * 4, cudaMemcpyDeviceToHost, bs));
+        if (h->emitted) MIRROR_CUDA_OK(cudaMemcpyAsync(h->emitted, out->emitted, B * (size_t)(tree->gamma + 1) * 4, cudaMemcpyDeviceToHost, bs));
+        MIRROR_CUDA_OK(cudaEventRecord(ctx->copy_ev[kEvSent], bs));
     }
-    for (int c = 1; c < n_pieces; ++c) {
+    for (int c = hidden ? 0 : 1; c < pieces.n; ++c) {
         st = attend_piece(c);
         if (st != MIRROR_OK) return st;
     }
+    if (h) MIRROR_CUDA_OK(cudaStreamWaitEvent(s, ctx->copy_ev[kEvSent], 0));
     return MIRROR_OK;
 }
 
