@@ -24,7 +24,7 @@
  *   - All compute calls only enqueue work on `stream` (a cudaStream_t passed as void*) and return without
  *     synchronising.  Host-side argument errors are returned immediately; device-side problems (a bounded
  *     wait that ran out, an index outside its table) set a status word read by mirror_device_status().
- *   - The library allocates device memory only inside mirror_create() (one status word).  Scratch memory
+ *   - The library allocates device memory only inside mirror_create() (a status word and 256 KB for Top-kappa).  Scratch memory
  *     is a caller-provided workspace, sized by mirror_workspace_bytes() and attached with
  *     mirror_set_workspace(); its contents need not survive between calls but two calls that use the
  *     same ctx must not overlap on the GPU.
@@ -138,7 +138,7 @@ typedef struct {
 #define MIRROR_WS_STEP_TREE 31u     /* mirror_verify_step, MIRROR_ACCEPT_SPEC_TREE */
 
 /* Create a context for one model shape on CUDA device `device` (made current for the call).
- * Allocates one device status word.  Fails with MIRROR_ERR_UNSUPPORTED on a device that is not sm_100. */
+ * Allocates the device status word and 256 KB of Top-kappa state.  Fails with MIRROR_ERR_UNSUPPORTED on a device that is not sm_100. */
 mirror_status mirror_create(mirror_ctx** out, const mirror_model_desc* desc, int device);
 mirror_status mirror_destroy(mirror_ctx* ctx);
 
@@ -197,8 +197,8 @@ mirror_status mirror_kv_quantize_fp8(mirror_ctx* ctx, const void* x, int n_layer
  *   gather_row/gather_tok int32 [n_gather] -> gather_logit fp32 [n_gather] = logits[row][tok]  (nullable)
  *   logits_out fp32 [M, V], nullable: the full logits (needed by speculative sampling)
  * Needs a workspace sized for MIRROR_WS_LMHEAD; with topk > 0 one sized for MIRROR_WS_LMHEAD_TOPK: with up to 256 rows the
- * Top-kappa is then selected inside the GEMM's epilogue (sorted lists per epilogue warp and row that live as long as the
- * CTA, merged afterwards) and the logits never reach memory; with more rows the selection runs over spilled fp32 logits. */
+ * Top-kappa is then selected inside the GEMM's epilogue (sorted candidate lists, merged afterwards) and the logits never
+ * reach memory; with more rows the selection runs over spilled fp32 logits. */
 mirror_status mirror_lmhead_reduce(mirror_ctx* ctx, const void* hidden, int M, const void* W, int topk,
                                    const int32_t* gather_row, const int32_t* gather_tok, int n_gather,
                                    int32_t* argmax, float* maxlogit, float* lse,

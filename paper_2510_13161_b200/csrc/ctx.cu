@@ -53,10 +53,13 @@ extern "C" mirror_status mirror_create(mirror_ctx** out, const mirror_model_desc
         return MIRROR_ERR_CUDA;
     }
     ctx->encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
-    if (cudaMalloc(&ctx->d_status, 2 * sizeof(int)) != cudaSuccess || cudaMemset(ctx->d_status, 0, 2 * sizeof(int)) != cudaSuccess) {
+    // the status words, and the bars of the fused Top-kappa (zero between calls, so not in the caller's workspace)
+    constexpr size_t kBarAt = 256, kBytes = kBarAt + (size_t)MIRROR_MAX_TOPK * 256 * 32;
+    if (cudaMalloc(&ctx->d_status, kBytes) != cudaSuccess || cudaMemset(ctx->d_status, 0, kBytes) != cudaSuccess) {
         delete ctx;
         return MIRROR_ERR_CUDA;
     }
+    ctx->d_topk_bar = (uint32_t*)((uint8_t*)ctx->d_status + kBarAt);
     *out = ctx;
     return MIRROR_OK;
 }

@@ -31,12 +31,12 @@ constexpr int kThreads = 192;
 constexpr int kBK = 64;
 constexpr int kTileV = 128;                 // vocabulary rows per CTA and unit
 constexpr int kPairV = 2 * kTileV;          // per pair
-constexpr int kATileBytes = kTileV * kBK * 2;
 constexpr int kMaxStages = 8;
 constexpr int kAcc = 2;
 constexpr int kMaxChunkRows = 256;
 constexpr int kSmemBudget = 232448;
 constexpr int kCtrlBytes = 1024 + 4 * kMaxChunkRows * 12;
+constexpr int kTopkBytes = 5 * kMaxChunkRows * 4;      // Top-kappa: each epilogue warp's row maxima of one unit, and the rows' bars
 
 struct PairParams {
     int M, V, H;
@@ -54,10 +54,10 @@ struct PairParams {
     int* part_idx;
     float* part_sum;
     int* status;
-    int topk;                               // > 0: the epilogue keeps each row's topk best (logit, id) pairs per CTA or unit
-    int topk_bytes;                         // shared memory of those lists
-    float* part_topv;                       // [partials][M][topk]
+    int topk;                               // > 0: the epilogue collects candidates for each row's topk best (logit, id) pairs
+    float* part_topv;                       // [4 * CTA + warp][M][topk]: sorted lists
     int* part_topi;
+    uint32_t* topk_bar;                     // largest logit seen in each of topk shares of the vocabulary (bar_word; order_key, 0: none)
     int fp8;                                // 1: W and the hidden rows are e4m3 bytes (K counted in 128-byte blocks all the same)
     const float* w_scale;                   // fp8: [V] scale of each weight row
     const float* h_scale;                   // fp8: [M] scale of each hidden row
@@ -164,16 +164,66 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
                  : "memory");
 }
 
-// Fused Top-kappa (Eq. 6).  Every epilogue warp keeps, for every hidden row, its own sorted list of K (logit, id) pairs in
-// shared memory (order: logit descending, id ascending); lane j owns the lists of the rows in column j of each 32-column
-// group, so 32 rows are updated side by side and nothing is locked.  A list lives as long as the CTA (one row chunk: the CTA
-// meets the same rows in every unit), so after the first tiles only a few logits pass its last entry.
+// Fused Top-kappa (Eq. 6).  Every epilogue warp has, for every hidden row, a sorted list of K (logit, id) pairs in global
+// memory (order: logit descending, id ascending); lmhead_topk_merge_kernel merges the lists of a row.  A list alone would
+// be a poor filter (a warp meets only ~150 of a row's logits), so the CTAs share a bar: the vocabulary falls into K shares
+// by the CTA that meets it, the largest logit met so far in each share is kept in global memory (atomicMax, one per CTA
+// and row and only when it grows: one per warp and unit on neighbouring words queued for 50 us), and the smallest of those
+// K maxima is at most the row's K-th best logit, since K different ids attain it.  A row whose maximum in a unit -- which
+// the reduction has anyway -- is below the bar is done with one comparison; after the first unit that is nearly every
+// row.  (What a list holds depends on timing, which candidates are best does not.)
+__device__ __forceinline__ uint32_t order_key(float x) {        // unsigned order = order of the floats; never 0
+    const uint32_t u = __float_as_uint(x);
+    return (u & 0x80000000u) ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ size_t bar_word(int share, int row) { return ((size_t)share * kMaxChunkRows + row) * 8; }    // (a sector each)
+// Insertion by a whole warp: lane i has the list's i-th pair.
 __device__ __forceinline__ void topk_list_insert(float* lv, int* li, int K, float x, int xi) {
-    int i = K - 1;
-    if (!(x > lv[i] || (x == lv[i] && xi < li[i]))) return;
-    while (i > 0 && (x > lv[i - 1] || (x == lv[i - 1] && xi < li[i - 1]))) { lv[i] = lv[i - 1]; li[i] = li[i - 1]; --i; }
-    lv[i] = x;
-    li[i] = xi;
+    const int lane = threadIdx.x & 31;
+    const float v = lane < K ? __ldcg(lv + lane) : INFINITY;
+    const int i = lane < K ? __ldcg(li + lane) : -1;
+    const unsigned behind = __ballot_sync(0xffffffffu, lane < K && (x > v || (x == v && xi < i)));   // pairs that x goes in front of
+    const float pv = __shfl_up_sync(0xffffffffu, v, 1);
+    const int pi = __shfl_up_sync(0xffffffffu, i, 1);
+    if ((behind >> lane) & 1u) {
+        const bool first = lane == __ffs(behind) - 1;
+        __stcg(lv + lane, first ? x : pv);
+        __stcg(li + lane, first ? xi : pi);
+    }
+    __syncwarp();
+}
+
+// The 32 pairs of a warp, one per lane, best first (bitonic network; `merge`: the input is bitonic already).
+__device__ __forceinline__ void warp_sort_pairs(float& v, int& i, bool merge = false) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1) {
+        if (merge && k < 32) continue;
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, v, j);
+            const int oi = __shfl_xor_sync(0xffffffffu, i, j);
+            const bool mine_better = v > ov || (v == ov && i < oi);
+            const bool keep_better = ((lane & j) == 0) == ((lane & k) == 0);
+            if (mine_better != keep_better) { v = ov; i = oi; }
+        }
+    }
+}
+// A list and up to 32 candidates (lane: x, xi; -inf for none) at once: what the first units bring, before there is a bar.
+// empty: the list holds nothing yet.
+__device__ __noinline__ void topk_list_merge(float* lv, int* li, int K, float x, int xi, bool empty) {
+    const int lane = threadIdx.x & 31;
+    warp_sort_pairs(x, xi);
+    if (!empty) {
+        const float rv = __shfl_sync(0xffffffffu, x, 31 - lane);
+        const int ri = __shfl_sync(0xffffffffu, xi, 31 - lane);
+        x = lane < K ? __ldcg(lv + lane) : -INFINITY;
+        xi = lane < K ? __ldcg(li + lane) : 0x7fffffff;
+        if (rv > x || (rv == x && ri < xi)) { x = rv; xi = ri; }          // best 32 of both, as a bitonic sequence
+        warp_sort_pairs(x, xi, true);
+    }
+    if (lane < K) { __stcg(lv + lane, x); __stcg(li + lane, xi); }
+    __syncwarp();
 }
 
 // kReduce: LM head (row reductions in the epilogue, optional spill).  !kReduce: plain GEMM C = W h^T for the layer
@@ -190,8 +240,6 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
     float* st_max = (float*)((uint8_t*)ctrl + 1024);          // [4][kMaxChunkRows]
     int* st_idx = (int*)(st_max + 4 * kMaxChunkRows);
     float* st_sum = (float*)(st_idx + 4 * kMaxChunkRows);
-    float* tk_val = (float*)((uint8_t*)ctrl + kCtrlBytes);    // [4 warps][chunk_rows][topk]  (only when p.topk > 0)
-    int* tk_idx = (int*)(tk_val + (size_t)4 * p.chunk_rows * p.topk);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_rank();
@@ -301,6 +349,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
         float* my_max = st_max + q * kMaxChunkRows;
         int* my_idx = st_idx + q * kMaxChunkRows;
         float* my_sum = st_sum + q * kMaxChunkRows;
+        float* const unit_max = kTopk ? (float*)((uint8_t*)ctrl + kCtrlBytes) + q * kMaxChunkRows : nullptr;    // this unit's maxima
         const int n_cg = (p.chunk_rows + 31) / 32;
         // the four warps hold disjoint vocabulary rows: one partial per hidden row out of their four states
         auto flush = [&](size_t pbase, int rbase) {
@@ -324,18 +373,11 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                 p.part_max[pbase + row] = m;
                 p.part_idx[pbase + row] = idx;
                 p.part_sum[pbase + row] = s;
-                // each warp's list is a partial list of its own: [4 * CTA + warp][row][topk]
-                for (int w = 0; w < 4 && kTopk; ++w)
-                    for (int i = 0; i < p.topk; ++i) {
-                        const size_t at = (((size_t)blockIdx.x * 4 + w) * p.M + row) * p.topk + i;
-                        p.part_topv[at] = tk_val[((size_t)w * p.chunk_rows + c) * p.topk + i];
-                        p.part_topi[at] = tk_idx[((size_t)w * p.chunk_rows + c) * p.topk + i];
-                    }
             }
         };
-        // this warp's Top-kappa lists start empty: (-inf, no id)
-        float* const my_tv = tk_val + (size_t)q * p.chunk_rows * p.topk;
-        int* const my_ti = tk_idx + (size_t)q * p.chunk_rows * p.topk;
+        // this warp's Top-kappa lists: [M][topk] (one row chunk, so the CTA meets all rows in every unit)
+        float* const my_tv = kTopk ? p.part_topv + ((size_t)blockIdx.x * 4 + q) * p.M * p.topk : nullptr;
+        int* const my_ti = kTopk ? p.part_topi + ((size_t)blockIdx.x * 4 + q) * p.M * p.topk : nullptr;
         int ab = 0;
         uint32_t aph = 0;
         bool ok = true;
@@ -347,7 +389,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
             __syncwarp();
         }
         if constexpr (kReduce && kTopk) {
-            for (int i = lane; i < p.chunk_rows * p.topk; i += 32) { my_tv[i] = -INFINITY; my_ti[i] = 0x7fffffff; }
+            for (int i = lane; i < p.M * p.topk; i += 32) { __stcg(my_tv + i, -INFINITY); __stcg(my_ti + i, 0x7fffffff); }      // empty
             __syncwarp();
         }
         for (int u = pair; u < p.n_units; u += n_pairs) {
@@ -390,35 +432,6 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                             for (int j = 0; j < 32; ++j)
                                 if (j < ncol) dst[(size_t)j * p.V] = v[j];
                         }
-                        if constexpr (kReduce && kTopk) {
-                            // lane j owns column j's list.  Its last entry is the bar: which lanes hold a logit of column j that
-                            // passes it?  (Nothing to do but for a few tiles.)
-                            const int K = p.topk;
-                            float* const lv = my_tv + (size_t)(cg * 32 + lane) * K;
-                            int* const li = my_ti + (size_t)(cg * 32 + lane) * K;
-                            const float bar_mine = lane < ncol ? lv[K - 1] : INFINITY;
-                            unsigned myhit = 0;
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) {
-                                const float bar_j = __shfl_sync(0xffffffffu, bar_mine, j);
-                                const unsigned hit = __ballot_sync(0xffffffffu, v[j] >= bar_j && v[j] > -INFINITY);
-                                if (lane == j) myhit = hit;
-                            }
-                            // rounds: every owner takes the next lane of its mask; one shuffle per column fetches that logit
-                            while (__any_sync(0xffffffffu, myhit != 0)) {
-                                const int src = myhit ? __ffs(myhit) - 1 : 0;
-                                const bool have = myhit != 0;
-                                myhit &= myhit - 1;
-                                float x = -INFINITY;
-#pragma unroll
-                                for (int j = 0; j < 32; ++j) {
-                                    const float t = __shfl_sync(0xffffffffu, v[j], src);
-                                    if (lane == j) x = t;
-                                }
-                                if (have) topk_list_insert(lv, li, K, x, vid - lane + src);
-                            }
-                            __syncwarp();
-                        }
                         if (kReduce) {
 #pragma unroll
                         for (int o = 16; o > 0; o >>= 1) {
@@ -442,6 +455,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                         }
                     }
                     const int c = cg * 32 + lane;          // lane j holds column cg*32+j of this unit
+                    if constexpr (kTopk) unit_max[c] = upd_m;
                     if (!kReduce) {
                     } else if (!running) {
                         my_max[c] = upd_m; my_idx[c] = upd_i; my_sum[c] = upd_s;
@@ -456,6 +470,60 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                         }
                     }
                 }
+            }
+            if constexpr (kReduce && kTopk) {
+                // (all four warps meet here whatever happened to one of them)
+                const int K = p.topk, n_rows = min(p.chunk_rows, p.M - rbase);
+                float* const all_max = (float*)((uint8_t*)ctrl + kCtrlBytes);
+                uint32_t* const bars = (uint32_t*)(all_max + 4 * kMaxChunkRows);
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                for (int c = (warp - 2) * 32 + lane; c < n_rows; c += 128) {
+                    const int share = (int)(blockIdx.x % (uint32_t)K);
+                    uint32_t key = 0, bar = 0xffffffffu;
+                    if (ok)
+                        for (int w = 0; w < 4; ++w) {
+                            const float m = all_max[w * kMaxChunkRows + c];
+                            if (m > -INFINITY) key = max(key, order_key(m));
+                        }
+#pragma unroll 4
+                    for (int k = 0; k < K; ++k) {
+                        const uint32_t word = __ldcg(p.topk_bar + bar_word(k, c));
+                        if (k == share && key > word) atomicMax(p.topk_bar + bar_word(k, c), key);
+                        bar = min(bar, k == share ? max(word, key) : word);
+                    }
+                    bars[c] = bar;
+                }
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                const int vid = vt * p.rows_cta + q * 32 + lane;
+                const bool valid = q * 32 + lane < p.rows_cta && vid < p.V;
+                for (int cg = 0; ok && cg < n_cg; ++cg) {
+                    const int c = cg * 32 + lane;
+                    unsigned cols = __ballot_sync(0xffffffffu, c < n_rows && unit_max[c] > -INFINITY && order_key(unit_max[c]) >= bars[c]);
+                    while (cols) {
+                        const int j = __ffs(cols) - 1;
+                        cols &= cols - 1;
+                        uint32_t w;
+                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(w)
+                                     : "r"(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * p.acc_stride + cg * 32 + j)) : "memory");
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(w) :: "memory");
+                        const float x = valid ? __uint_as_float(w) : -INFINITY;
+                        unsigned hit = __ballot_sync(0xffffffffu, x > -INFINITY && order_key(x) >= bars[cg * 32 + j]);
+                        float* const lv = my_tv + (size_t)(cg * 32 + j) * K;
+                        int* const li = my_ti + (size_t)(cg * 32 + j) * K;
+                        if (__popc(hit) > 2) {
+                            const bool in = (hit >> lane) & 1u;
+                            topk_list_merge(lv, li, K, in ? x : -INFINITY, in ? vid : 0x7fffffff, u == pair);
+                            continue;
+                        }
+                        while (hit) {
+                            const int src = __ffs(hit) - 1;
+                            hit &= hit - 1;
+                            topk_list_insert(lv, li, K, __shfl_sync(0xffffffffu, x, src), vid - lane + src);
+                        }
+                    }
+                }
+            }
+            if (ok) {
                 ptx::tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(map_to_rank(&ctrl->acc_empty[ab], 0));
@@ -529,10 +597,8 @@ mirror_status pair_shape(const MirrorTuning& tune, int M, int V, int H, PairPara
     // eight, deal the units to twice as many pairs, and let the CTAs of the next kernel move in one by one.
     p->ctas_per_sm = ctas_per_sm_for(tune, M);
     p->topk = topk;
-    p->topk_bytes = topk > 0 ? (int)align_up((size_t)4 * p->chunk_rows * (size_t)topk * 8, 256) : 0;
-    p->part_topv = nullptr; p->part_topi = nullptr;
-    if (p->topk_bytes > (32 << 10)) p->ctas_per_sm = 1;
-    p->stages = (kSmemBudget / p->ctas_per_sm - kCtrlBytes - 2048 - p->topk_bytes) / p->stage_bytes;
+    p->part_topv = nullptr; p->part_topi = nullptr; p->topk_bar = nullptr;
+    p->stages = (kSmemBudget / p->ctas_per_sm - kCtrlBytes - 2048 - (topk > 0 ? kTopkBytes : 0)) / p->stage_bytes;
     if (p->stages > kMaxStages) p->stages = kMaxStages;
     if (tune.lm_stages >= 2 && tune.lm_stages < p->stages) p->stages = tune.lm_stages;
     p->wait_limit = tune.wait_limit_cycles;
@@ -560,7 +626,7 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
         st = mirror_make_tmap(ctx, &tm_h, x, 2, hdims, strides, box_h);
         if (st != MIRROR_OK) return st;
     }
-    const size_t smem = (size_t)p.stages * p.stage_bytes + kCtrlBytes + p.topk_bytes + 1024;
+    const size_t smem = (size_t)p.stages * p.stage_bytes + kCtrlBytes + (p.topk > 0 ? kTopkBytes : 0) + 1024;
     if (!ctx->lm_pair_attr_set) {
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
@@ -595,9 +661,7 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
 int mirror_lmhead_pair_partials(int V) { return 2 * ((V + kPairV - 1) / kPairV); }
 
 bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk) {
-    if (topk <= 0 || M > kMaxChunkRows || M < ctx->tune.lm_pair_min_rows) return false;
-    const size_t bytes = (size_t)4 * align_up((size_t)M, 16) * (size_t)topk * 8;
-    return bytes <= ((size_t)96 << 10);           // (beyond 32 KB the kernel runs one CTA per SM)
+    return topk > 0 && M <= kMaxChunkRows && M >= ctx->tune.lm_pair_min_rows;
 }
 
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,
@@ -641,11 +705,11 @@ mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int
     p.part_sum = (float*)(p.part_idx + P * M);
     p.status = ctx->d_status;
     if (topk > 0) {
-        // the lists live as long as the CTA: one row chunk only (and four lists per CTA and row have to fit beside the stages)
-        if (p.n_chunks != 1 || p.stages < 3) return MIRROR_ERR_UNSUPPORTED;
+        if (p.n_chunks != 1 || !ctx->d_topk_bar) return MIRROR_ERR_UNSUPPORTED;      // (one row chunk: a list lives as long as its CTA)
         if (!topk_ws || topk_ws_bytes < 4 * P * M * (size_t)topk * 8) return MIRROR_ERR_WORKSPACE;
         p.part_topv = (float*)topk_ws;
         p.part_topi = (int*)(p.part_topv + 4 * P * M * (size_t)topk);
+        p.topk_bar = ctx->d_topk_bar;
     }
     p.fp8 = fp8 ? 1 : 0;
     p.w_scale = w_scale;

@@ -51,6 +51,7 @@ struct mirror_ctx {
     float scale = 0.f;
     float temperature = 1.f;
     int* d_status = nullptr;        // [2]: {code, detail}
+    uint32_t* d_topk_bar = nullptr; // [MIRROR_MAX_TOPK][256 rows] sectors behind the status: zero between calls (lmhead_pair.cu)
     void* ws = nullptr;
     size_t ws_bytes = 0;
     long long launches = 0;
@@ -95,8 +96,7 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
 // LM-head GEMM + per-unit row partials on CTA pairs (many hidden rows); *n_partials partials of [M] rows are left in
 // partial_ws for lmhead_merge_kernel.  mirror_lmhead_pair_partials(V) is that count.
 int mirror_lmhead_pair_partials(int V);
-// Can the Top-kappa of M rows be selected inside the GEMM's epilogue?  (One row chunk, and four lists per CTA and row in
-// shared memory beside a pipeline that is still deep enough.)
+// Can the Top-kappa of M rows be selected inside the GEMM's epilogue?  (One row chunk.)
 bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk);
 // w_scale / h_scale non-null: W and hidden are e4m3 bytes with one scale per row (the GEMM runs on kind::f8f6f4).
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,
