@@ -55,6 +55,7 @@ constexpr int kTileTok = kSlotTok * kTileSlots;     // 64
 constexpr int kRows = 128;                          // UMMA M: rows per row block
 constexpr int kMaxBatch = kAttnMaxBatch;
 constexpr int kMaxStages = 8;                       // ring depths are template parameters (even: tiles are staged in pairs)
+constexpr int kCtrlBytes = 640;
 constexpr int kSBufs = 4;                           // S buffers in TMEM (power of two)
 // A row's offset puts the maximum of the tile that set it at 2^bias and moves when a tile's sum of P passes the limit
 // (no single P is beyond the limit then).  bf16 P: 2^0 and 2^14.  e4m3 P: 2^2 and 448, the largest e4m3 value (a tile
@@ -72,7 +73,7 @@ struct AttnParams {
     int rows, n_rb, rows_per_rb;          // rows per unit, row blocks, rows per block
     int n_groups;                         // CTA groups (grid = n_groups * n_rb)
     int snap_cap;                         // boundaries move to a unit boundary that is at most this many tiles away
-    int whole_units;                      // 1: prefer a group count that divides equal-length units (no cuts)
+    int whole_groups;                     // group count that divides the units evenly (attn::whole_unit_groups), 0: none
     int max_pages, num_pages, layer_pages;
     int q_half_bytes;                     // one 64-column half of a Q buffer: rows rounded up to 8, 128 B each
     int tree_slots;
@@ -87,6 +88,7 @@ struct AttnParams {
     __nv_bfloat16* out;
     float* lse_out;
     float* partial;                       // [grid][2][D+4][128]
+    attn::GroupBegin* begins;             // [n_groups]
     int* status;
     // e4m3 cache: pools, k_new and v_new hold e4m3 codes (one byte per element); a code times its (layer, KV head)
     // scale is the value.  Q stays bf16 in memory; its operand is e4m3(q / q_scale), rounded when it is staged.
@@ -97,63 +99,26 @@ struct AttnParams {
     int stall_after;                      // test aid: the K producer stops after this many stages (-1: never)
 };
 
-struct UnitPos {                          // where a global tile index falls
+struct UnitPos {                          // where a global tile index falls (indexes fit 31 bits: checked in the prologue)
     int layer, b, g;
     int tile_in_unit, tiles_in_unit;
-    long long unit_first_tile;            // global index of the unit's first tile
-};
-
-struct Ctrl {
-    uint64_t k_full[kMaxStages], k_empty[kMaxStages];   // K ring: refilled as soon as Q K^T has read a stage
-    uint64_t v_full[kMaxStages], v_empty[kMaxStages];   // V ring: refilled once P V has read a stage
-    uint64_t s_full[kSBufs], s_free[kSBufs];
-    uint64_t p_full[kSBufs], pv_done[2];
-    uint64_t q_full[2];
-    uint64_t pair[4];                                   // softmax warp pairs' exchange
-    uint64_t o_free;                                    // accumulators read out at the end of a unit's part
-    uint32_t tmem_base;
-    volatile int abort;
+    int unit_first_tile;                  // global index of the unit's first tile
 };
 
 __device__ __forceinline__ void dev_check(const AttnParams& p, int detail) {
     if (atomicCAS(p.status, 0, MIRROR_DEV_CHECK) == 0) atomicExch(p.status + 1, detail);
 }
-__device__ __forceinline__ void timeout(const AttnParams& p, Ctrl* c, int where) {
-    c->abort = 1;
-    if (atomicCAS(p.status, 0, MIRROR_DEV_TIMEOUT) == 0) atomicExch(p.status + 1, where);
-}
-
-// A bounded wait that looks at the CTA's abort flag only when the barrier is not complete yet (the common case is one
-// try_wait), and between parks while it waits.
-__device__ __forceinline__ bool wait_bar(Ctrl* c, uint64_t* bar, uint32_t parity, long long limit_cycles) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    for (;;) {
-        if (c->abort) return false;
-        if (ptx::mbar_try_wait_park(bar, parity, MIRROR_PARK_NS)) return true;
-        if (clock64() - t0 > limit_cycles) return false;
-    }
-}
-
-// Two barriers at once: both polls are issued before either result is looked at.
-__device__ __forceinline__ bool wait_bar2(Ctrl* c, uint64_t* bar_a, uint32_t par_a, uint64_t* bar_b, uint32_t par_b, long long limit_cycles) {
-    const bool a = ptx::mbar_try_wait(bar_a, par_a), b = ptx::mbar_try_wait(bar_b, par_b);
-    if (a && b) return true;
-    return (a || wait_bar(c, bar_a, par_a, limit_cycles)) && (b || wait_bar(c, bar_b, par_b, limit_cycles));
-}
-
-__device__ __noinline__ UnitPos locate(long long x, const AttnParams& p, const int* cumT, long long tiles_per_layer) {
+__device__ __noinline__ UnitPos locate(int x, const AttnParams& p, const int* cumT, int tiles_per_layer) {
     UnitPos u;
-    // (the tile count fits 31 bits: checked in the prologue; 32-bit divisions are several times cheaper)
     u.layer = (int)((uint32_t)x / (uint32_t)tiles_per_layer);
-    const long long rem = x - (long long)u.layer * tiles_per_layer;
+    const int rem = x - u.layer * tiles_per_layer;
     int b = 0;
-    while (b + 1 < p.B && (long long)p.Hkv * cumT[b + 1] <= rem) ++b;
+    while (b + 1 < p.B && p.Hkv * cumT[b + 1] <= rem) ++b;
     const int Tb = cumT[b + 1] - cumT[b];
-    const long long r2 = rem - (long long)p.Hkv * cumT[b];
+    const int r2 = rem - p.Hkv * cumT[b];
     u.b = b;
     u.g = (int)((uint32_t)r2 / (uint32_t)Tb);
-    u.tile_in_unit = (int)(r2 - (long long)u.g * Tb);
+    u.tile_in_unit = r2 - u.g * Tb;
     u.tiles_in_unit = Tb;
     u.unit_first_tile = x - u.tile_in_unit;
     return u;
@@ -260,7 +225,7 @@ struct Cfg {
     static constexpr int kSlotBytes = kHalves * kSlotTok * 128;    // one slot of K or V (see kv_slot_off) = one TMA box
     static constexpr int kGroupStride = kHalves * 1024;            // between the 8-token groups of one half
     static constexpr int kStageBytes = kStageSlots * kSlotBytes;   // one K (or V) stage: 4 slots; stages are contiguous
-    static constexpr size_t kSmemFixed = 512 /*ctrl*/ + 2 * 2 * kRows * 4 /*pair exchange*/ + (2 * kMaxBatch + 2) * 4 + 1024 /*align*/;
+    static constexpr size_t kSmemFixed = kCtrlBytes + 2 * 2 * kRows * 4 /*pair exchange*/ + (2 * kMaxBatch + 2) * 4 + 1024 /*align*/;
     // Shared memory: two Q buffers sized by the rows a CTA really has (the UMMA reads 128 rows per half and
     // runs on into whatever follows; those rows only reach TMEM lanes nobody reads), then the K and V rings.
     // What the rings can hold in flight bounds the bandwidth one SM can pull at HBM latency, so they get
@@ -283,12 +248,12 @@ struct Segment {
     int t_first, t_last;                  // tiles [t_first, t_last) of the unit
     int len, pages_full, pages_all, slots_all;
 };
-__device__ __noinline__ Segment make_segment(long long x, long long x_end, const AttnParams& p, const int* cumT,
-                                                const int* s_len, long long tiles_per_layer) {
+__device__ __noinline__ Segment make_segment(int x, int x_end, const AttnParams& p, const int* cumT,
+                                                const int* s_len, int tiles_per_layer) {
     Segment s;
     s.u = locate(x, p, cumT, tiles_per_layer);
     s.t_first = s.u.tile_in_unit;
-    s.t_last = (int)min((long long)s.u.tiles_in_unit, (long long)s.t_first + (x_end - x));
+    s.t_last = min(s.u.tiles_in_unit, s.t_first + (x_end - x));
     s.len = s_len[s.u.b];
     s.pages_full = s.len / kSlotTok;
     s.pages_all = (s.len + kSlotTok - 1) / kSlotTok;
@@ -296,43 +261,83 @@ __device__ __noinline__ Segment make_segment(long long x, long long x_end, const
     return s;
 }
 
+struct Ctrl {
+    uint64_t k_full[kMaxStages], k_empty[kMaxStages];   // K ring: refilled as soon as Q K^T has read a stage
+    uint64_t v_full[kMaxStages], v_empty[kMaxStages];   // V ring: refilled once P V has read a stage
+    uint64_t s_full[kSBufs], s_free[kSBufs];
+    uint64_t p_full[kSBufs], pv_done[2];
+    uint64_t q_full[2];
+    uint64_t pair[4];                                   // softmax warp pairs' exchange
+    uint64_t o_free;                                    // accumulators read out at the end of a unit's part
+    Segment first;                                      // where this CTA's range begins
+    int x_begin, x_end, tiles_per_layer;
+    uint32_t tmem_base;
+    volatile int abort;
+};
+static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block");
+
+__device__ __forceinline__ void timeout(const AttnParams& p, Ctrl* c, int where) {
+    c->abort = 1;
+    if (atomicCAS(p.status, 0, MIRROR_DEV_TIMEOUT) == 0) atomicExch(p.status + 1, where);
+}
+
+// A bounded wait that looks at the CTA's abort flag only when the barrier is not complete yet (the common case is one
+// try_wait), and between parks while it waits.
+__device__ __forceinline__ bool wait_bar(Ctrl* c, uint64_t* bar, uint32_t parity, long long limit_cycles) {
+    if (ptx::mbar_try_wait(bar, parity)) return true;
+    const long long t0 = clock64();
+    for (;;) {
+        if (c->abort) return false;
+        if (ptx::mbar_try_wait_park(bar, parity, MIRROR_PARK_NS)) return true;
+        if (clock64() - t0 > limit_cycles) return false;
+    }
+}
+
+// Two barriers at once: both polls are issued before either result is looked at.
+__device__ __forceinline__ bool wait_bar2(Ctrl* c, uint64_t* bar_a, uint32_t par_a, uint64_t* bar_b, uint32_t par_b, long long limit_cycles) {
+    const bool a = ptx::mbar_try_wait(bar_a, par_a), b = ptx::mbar_try_wait(bar_b, par_b);
+    if (a && b) return true;
+    return (a || wait_bar(c, bar_a, par_a, limit_cycles)) && (b || wait_bar(c, bar_b, par_b, limit_cycles));
+}
+
 // How the tile sequence is cut into one range per CTA group.
 struct Partition {
-    long long tiles_per_layer, total_tiles, total_pairs, snap_tol;
-    int n_groups;
+    int tiles_per_layer, total_tiles;     // (total_tiles -1: the sequence does not fit 31 bits)
+    int n_groups, snap_tol;
+    int share, rest;                      // pairs of tiles = n_groups * share + rest
 };
 __device__ __forceinline__ Partition make_partition(const AttnParams& p, const int* cumT) {
     Partition q;
-    q.tiles_per_layer = (long long)p.Hkv * cumT[p.B];
-    q.total_tiles = q.tiles_per_layer * p.L;
+    const long long per = (long long)p.Hkv * cumT[p.B], total = per * p.L;
+    q.tiles_per_layer = (int)per;
+    q.total_tiles = total < (1ll << 31) ? (int)total : -1;
     // CTA groups own whole pairs of tiles; never more groups than pairs, so that every group's range is non-empty
-    q.total_pairs = q.total_tiles / 2;
-    q.n_groups = (int)min((long long)p.n_groups, q.total_pairs);
+    const int pairs = q.total_tiles >> 1;
+    q.n_groups = min(p.n_groups, max(1, pairs));
     // Units of equal length (every request has the same number of tiles): a group count that divides the units, if one
     // exists within 15% of the CTA groups there are, gives every group the same number of WHOLE units: no unit is cut,
     // nothing is left to merge and all groups end together, which is worth more than the few SMs left idle
     // (384 units on 148 SMs: 128 groups of 3 units, attention 111 -> 105 us).
     bool equal_units = true;
     for (int b = 1; b < p.B; ++b) equal_units &= (cumT[b + 1] - cumT[b]) == cumT[1];
-    if (p.whole_units && equal_units && q.n_groups == p.n_groups) {
-        const int g = attn::whole_unit_groups(p.n_groups, (long long)p.L * p.B * p.Hkv);
-        if (g > 0) q.n_groups = g;
-    }
+    if (p.whole_groups > 0 && equal_units && q.n_groups == p.n_groups) q.n_groups = p.whole_groups;
+    q.share = (int)((uint32_t)pairs / (uint32_t)q.n_groups);
+    q.rest = pairs - q.share * q.n_groups;
     // A boundary that falls within snap_tol tiles (a cut costs about as much as a few tiles) of a unit boundary
     // moves there: both neighbours then hold whole units and no partial has to be left and merged.  snap_tol is
     // at most a quarter of the smallest even share, so boundaries stay strictly increasing.
-    q.snap_tol = q.n_groups > 0 ? min((long long)p.snap_cap, (2 * (q.total_pairs / q.n_groups)) / 4) : 0;
+    q.snap_tol = min(p.snap_cap, q.share >> 1);
     return q;
 }
-__device__ __noinline__ long long group_begin(const Partition& q, int g, const AttnParams& p, const int* cumT) {
+__device__ __noinline__ int group_begin(const Partition& q, int g, const AttnParams& p, const int* cumT) {
     if (g <= 0) return 0;
     if (g >= q.n_groups) return q.total_tiles;
-    const long long e = 2 * (q.total_pairs * g / q.n_groups);
+    const int e = 2 * (q.share * g + (int)((uint32_t)(q.rest * g) / (uint32_t)q.n_groups));     // 2 * (pairs * g / n_groups)
     if (q.snap_tol == 0) return e;
     const UnitPos u = locate(e, p, cumT, q.tiles_per_layer);
-    const long long lo = u.unit_first_tile, hi = lo + u.tiles_in_unit;
-    const long long best = (e - lo <= hi - e) ? lo : hi;
-    const long long dist = best > e ? best - e : e - best;
+    const int lo = u.unit_first_tile, hi = lo + u.tiles_in_unit;
+    const int best = (e - lo <= hi - e) ? lo : hi;
+    const int dist = best > e ? best - e : e - best;
     return dist <= q.snap_tol ? best : e;
 }
 
@@ -350,8 +355,8 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     uint8_t* sK = sQ + 2 * q_buf_bytes;                             // [KS]  [slot][half][16 tokens][128 B]
     uint8_t* sV = sK + KS * C::kStageBytes;                         // [VS]  [slot][half][16 tokens][128 B]
     Ctrl* ctrl = (Ctrl*)(sV + VS * C::kStageBytes);
-    float* xch = (float*)((uint8_t*)ctrl + 512);                    // [2 tiles][2 halves][128 rows] pair exchange
-    int* cumT = (int*)((uint8_t*)ctrl + 512 + 2 * 2 * kRows * 4);   // [B+1] tiles per request, prefix-summed
+    float* xch = (float*)((uint8_t*)ctrl + kCtrlBytes);                    // [2 tiles][2 halves][128 rows] pair exchange
+    int* cumT = (int*)((uint8_t*)ctrl + kCtrlBytes + 2 * 2 * kRows * 4);   // [B+1] tiles per request, prefix-summed
     int* s_len = cumT + (kMaxBatch + 1);                            // [B] clamped prefix lengths
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -386,30 +391,44 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     ptx::tc_fence_after();
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();                 // the merge kernel behind may be scheduled as soon as SMs free up
-    for (int b = tid; b < p.B; b += kThreads) {
-        int len = p.prefix_len[b];
-        if (len < 0 || len > p.max_pages * kSlotTok) { dev_check(p, 300 + b); len = len < 0 ? 0 : p.max_pages * kSlotTok; }
-        s_len[b] = len;
-    }
-    __syncthreads();
-    if (tid == 0) {
+    // one warp finds this CTA's range of tiles and the part of a unit that it begins with
+    if (warp == 0) {
         int acc = 0;
-        cumT[0] = 0;
-        for (int b = 0; b < p.B; ++b) {
-            const int slots = (s_len[b] + kSlotTok - 1) / kSlotTok + p.tree_slots;
-            acc += 2 * ((slots + 2 * kStageSlots - 1) / (2 * kStageSlots));      // whole pairs of tiles
-            cumT[b + 1] = acc;
+        if (lane == 0) cumT[0] = 0;
+#pragma unroll 1
+        for (int b0 = 0; b0 < p.B; b0 += 32) {
+            const int b = b0 + lane;
+            int len = b < p.B ? p.prefix_len[b] : 0;
+            if (len < 0 || len > p.max_pages * kSlotTok) { dev_check(p, 300 + b); len = len < 0 ? 0 : p.max_pages * kSlotTok; }
+            const int slots = (len + kSlotTok - 1) / kSlotTok + p.tree_slots;
+            int sum = b < p.B ? 2 * ((slots + 2 * kStageSlots - 1) / (2 * kStageSlots)) : 0;     // whole pairs of tiles
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, sum, o);
+                if (lane >= o) sum += v;
+            }
+            if (b < p.B) { s_len[b] = len; cumT[b + 1] = acc + sum; }
+            acc += __shfl_sync(0xffffffffu, sum, 31);
+        }
+        __syncwarp();
+        const Partition part = make_partition(p, cumT);
+        if (part.total_tiles < 0 && lane == 0) dev_check(p, 600);
+        int x = 0;
+        if (part.total_tiles >= 0 && group < part.n_groups && lane < 2) x = group_begin(part, group + lane, p, cumT);
+        const int x1 = __shfl_sync(0xffffffffu, x, 1);
+        if (lane == 0) {
+            ctrl->x_begin = x;
+            ctrl->x_end = x1;
+            ctrl->tiles_per_layer = part.tiles_per_layer;
+            if (x < x1) ctrl->first = make_segment(x, x1, p, cumT, s_len, part.tiles_per_layer);
+            const Segment& s = ctrl->first;
+            if (rb == 0) p.begins[group] = {x < x1 && s.t_first > 0 ? 1 : 0, s.u.layer, s.u.b, s.u.g};
         }
     }
     __syncthreads();
     const uint32_t tmem_base = ctrl->tmem_base;
-    const Partition part = make_partition(p, cumT);
-    const long long tiles_per_layer = part.tiles_per_layer, total_tiles = part.total_tiles;
-    const int n_groups = part.n_groups;
-    const bool fits = total_tiles < (1ll << 31);
-    if (!fits && tid == 0) dev_check(p, 600);
-    const long long x_begin = (fits && group < n_groups) ? group_begin(part, group, p, cumT) : 0;
-    const long long x_end = (fits && group < n_groups) ? group_begin(part, group + 1, p, cumT) : 0;
+    const int x_begin = ctrl->x_begin, x_end = ctrl->x_end, tiles_per_layer = ctrl->tiles_per_layer;
+    auto segment_at = [&](int x) -> Segment { return x == x_begin ? ctrl->first : make_segment(x, x_end, p, cumT, s_len, tiles_per_layer); };
     if (warp == 0 || warp == kVProducerWarp) {
         // =========================================================================== producers
         // warp 0 stages K, the last warp stages V: a warp issues its TMA boxes one after the other, so two
@@ -419,12 +438,12 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
         uint64_t* const empty = vrole ? ctrl->v_empty : ctrl->k_empty;
         uint32_t it = 0;                   // tiles issued by this CTA so far (ring index and parity source)
         bool ok = true;
-        long long x = x_begin;
+        int x = x_begin;
         // one TMA box (a whole page of this tensor) per lane
         const bool has_box = lane < kStageSlots;
         const int my_slot = lane;
         while (x < x_end && ok) {
-            const Segment sg = make_segment(x, x_end, p, cumT, s_len, tiles_per_layer);
+            const Segment sg = segment_at(x);
             const UnitPos& u = sg.u;
             const int32_t* pt = p.page_table + (size_t)u.b * p.max_pages;
             // the page id a lane needs is fetched one tile ahead, so its latency hides behind the ring wait
@@ -540,9 +559,9 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
             uint32_t sb = 0, s_par = 1;            // S buffer of the next tile and the parity that says it is free
             bool ready = false;                    // both barriers of the next tile were seen complete already
             bool ok = true;
-            long long x = x_begin;
+            int x = x_begin;
             while (x < x_end && ok) {
-                const Segment sg = make_segment(x, x_end, p, cumT, s_len, tiles_per_layer);
+                const Segment sg = segment_at(x);
                 if (!wait_bar(ctrl, &ctrl->q_full[seg & 1], (seg >> 1) & 1, p.wait_limit)) { timeout(p, ctrl, 20); ok = false; break; }
                 const uint32_t q_seg = q_lo + (uint32_t)(((seg & 1) * q_buf_bytes) >> 4);
                 ++seg;
@@ -593,10 +612,10 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
             int st = 0, sb = 0;                     // V ring stage and S / P buffer of the next tile, with their parities
             uint32_t v_par = 0, p_par = 0;
             bool ok = true;
-            long long x = x_begin;
+            int x = x_begin;
             uint32_t seg = 0;
             while (x < x_end && ok) {
-                const Segment sg = make_segment(x, x_end, p, cumT, s_len, tiles_per_layer);
+                const Segment sg = segment_at(x);
                 // the accumulators of the previous part must have been read out by every softmax warp
                 if (seg > 0 && (!wait_bar(ctrl, &ctrl->o_free, (seg - 1) & 1, p.wait_limit))) { timeout(p, ctrl, 24); ok = false; break; }
                 ++seg;
@@ -696,7 +715,7 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
 
         uint32_t it = 0;
         bool ok = true;
-        long long x = x_begin;
+        int x = x_begin;
         Segment sg;
         // P of one tile from the row's 64 scores v[]: p = exp2(s*c - offset) as bf16 pairs, and the row sum in fp32
         float sc = p.scale_log2e;                                  // scores -> log2 units (e4m3: times the unit's Q and K scales)
@@ -731,7 +750,7 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
 
         uint32_t seg = 0;                                          // parts walked so far: Q buffer = seg & 1
         if (x < x_end) {
-            sg = make_segment(x, x_end, p, cumT, s_len, tiles_per_layer);
+            sg = segment_at(x);
             stage_q(sg.u, 0);
             q_ready(0);
         }
@@ -746,10 +765,10 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
             // the part after this one: its Q goes into the other Q buffer now (every Q K^T that read that buffer
             // belongs to the part before this one and has completed), so the issuer can run on into the next unit
             Segment sg_next;
-            const long long x_next = x + (sg.t_last - sg.t_first);
+            const int x_next = x + (sg.t_last - sg.t_first);
             const bool has_next = x_next < x_end;
             if (has_next) {
-                sg_next = make_segment(x_next, x_end, p, cumT, s_len, tiles_per_layer);
+                sg_next = segment_at(x_next);
                 stage_q(sg_next.u, (seg + 1) & 1);
             }
             bool q_pending = has_next;
@@ -949,140 +968,19 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     }
 }
 
-// Merge of the units that the partition cut across CTA groups.  One block per (inner boundary, row block).  A unit
-// cut by k boundaries left k + 1 (max, sum, accumulator) records, like split-KV partials; the k blocks of those
-// boundaries share its merge by output columns (8-column chunks dealt round-robin), each combining all parts of its
-// columns in group order, so a unit that many CTAs shared (few units per launch, long contexts) is not merged by one
-// block alone.  Blocks whose boundary coincides with a unit boundary have nothing to do.
-constexpr int kMergeThreads = 512;        // 128 rows x 4 column quarters
-constexpr int kMergeMaxGroups = 512;      // groups whose first tiles fit the lookup table (more: computed on demand)
+// Merge of the units that the partition cut: one block per (inner boundary, row block).
 template <int D>
-__global__ void __launch_bounds__(kMergeThreads) attn_tile64_merge_kernel(const AttnParams p) {
-    __shared__ int cumT[kMaxBatch + 1];
-    __shared__ int s_len[kMaxBatch];
-    const int tid = threadIdx.x;
-    for (int b = tid; b < p.B; b += kMergeThreads) {
-        const int len = p.prefix_len[b];
-        s_len[b] = len < 0 ? 0 : (len > p.max_pages * kSlotTok ? p.max_pages * kSlotTok : len);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int acc = 0;
-        cumT[0] = 0;
-        for (int b = 0; b < p.B; ++b) {
-            const int slots = (s_len[b] + kSlotTok - 1) / kSlotTok + p.tree_slots;
-            acc += 2 * ((slots + 2 * kStageSlots - 1) / (2 * kStageSlots));
-            cumT[b + 1] = acc;
-        }
-    }
-    __syncthreads();
-    const Partition part = make_partition(p, cumT);
-    const int g = blockIdx.x + 1, rb = blockIdx.y;
-    // A block with nothing to merge must still wait for the attention kernel: the kernel behind this one in the stream
-    // only waits for THIS grid to complete, so a grid whose blocks all left early would let it read attention outputs
-    // that are still being written.
-    if (g >= part.n_groups || part.total_tiles >= (1ll << 31)) { ptx::grid_dep_wait(); return; }
-    const long long x = group_begin(part, g, p, cumT);
-    const UnitPos u = locate(x, p, cumT, part.tiles_per_layer);
-    if (u.tile_in_unit == 0) { ptx::grid_dep_wait(); return; }                  // the boundary is a unit boundary (block-uniform)
-    // every group's first tile, computed side by side (a unit shared by many groups is looked up from here instead of
-    // by a chain of dependent calls)
-    __shared__ long long s_begin[kMergeMaxGroups];
-    const bool tabled = part.n_groups <= kMergeMaxGroups;
-    if (tabled) {
-        for (int t = tid; t < part.n_groups; t += kMergeThreads) s_begin[t] = group_begin(part, t, p, cumT);
-        __syncthreads();
-    }
-    auto begin_of = [&](int t) -> long long { return tabled ? s_begin[t] : group_begin(part, t, p, cumT); };
-    // the groups ga..gb hold this unit's parts; the blocks of the boundaries ga+1..gb share the merge by columns
-    int ga = g - 1;
-    while (ga > 0 && begin_of(ga) > u.unit_first_tile) --ga;
-    int gb = g;
-    const long long unit_last = u.unit_first_tile + u.tiles_in_unit - 1;
-    while (gb + 1 < part.n_groups && begin_of(gb + 1) <= unit_last) ++gb;
-    const int parts = gb - ga + 1;
-    const int n_blocks = parts - 1, j_blk = g - (ga + 1);
-    // launched with programmatic stream serialization: everything above overlaps the attention kernel's tail;
-    // its records (and the outputs this block overwrites) are only touched after it has completed
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
-
-    constexpr int kRowW = D + 4;
-    constexpr int kChunks = D / 8;                                              // 8 output columns = one 16-byte store
-    constexpr int kPer = (kChunks + 3) / 4;                                     // chunks per thread when one block has them all
-    const int row = tid & (kRows - 1), cq = tid >> 7;
-    const int rb_row0 = rb * p.rows_per_rb;
-    const int rb_rows = min(p.rows_per_rb, p.rows - rb_row0);
-    if (row >= rb_rows) return;
-    const int r_abs = rb_row0 + row, node = r_abs / p.G, hl = r_abs % p.G;
-    // chunk c belongs to block c mod n_blocks; inside the block its chunks go round the four thread quarters
-    int chunk[kPer];
-    bool any = false;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-        chunk[i] = j_blk + (cq + 4 * i) * n_blocks;
-        any |= chunk[i] < kChunks;
-    }
-    const bool writes_lse = p.lse_out && j_blk == 0 && cq == 0;
-    if (!any && !writes_lse) return;
-    // group ga holds the unit's first tile (its record is in slot 1), the later groups began inside the unit (slot 0)
-    auto part_of = [&](int k) -> const float* {
-        return p.partial + ((size_t)((ga + k) * p.n_rb + rb) * 2 + (k == 0 ? 1 : 0)) * kRowW * kRows + row;
-    };
-    float Mm = -INFINITY;
-#pragma unroll 4
-    for (int k = 0; k < parts; ++k) Mm = fmaxf(Mm, __ldcg(part_of(k) + (size_t)D * kRows));
-    float Lm = 0.f;
-    float acc[kPer][8];
-#pragma unroll
-    for (int i = 0; i < kPer; ++i)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[i][c] = 0.f;
-    if (n_blocks >= 4) {
-        // many parts, at most one chunk per thread: six parts' loads in flight at a time (same order of additions)
-        if (chunk[0] < kChunks || writes_lse) {
-            const bool has = chunk[0] < kChunks;
-            const int c0 = has ? chunk[0] * 8 : 0;
-#pragma unroll 6
-            for (int k = 0; k < parts; ++k) {
-                const float* src = part_of(k);
-                const float pm = __ldcg(src + (size_t)D * kRows);
-                const float wgt = (pm == -INFINITY) ? 0.f : exp2f(pm - Mm);
-                Lm = fmaf(wgt, __ldcg(src + (size_t)(D + 1) * kRows), Lm);
-                if (has) {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) acc[0][c] = fmaf(wgt, __ldcg(src + (size_t)(c0 + c) * kRows), acc[0][c]);
-                }
-            }
-        }
-    } else
-#pragma unroll 2
-    for (int k = 0; k < parts; ++k) {
-        const float* src = part_of(k);
-        const float pm = __ldcg(src + (size_t)D * kRows);
-        const float wgt = (pm == -INFINITY) ? 0.f : exp2f(pm - Mm);
-        Lm = fmaf(wgt, __ldcg(src + (size_t)(D + 1) * kRows), Lm);
-#pragma unroll
-        for (int i = 0; i < kPer; ++i)
-            if (chunk[i] < kChunks) {
-#pragma unroll
-                for (int c = 0; c < 8; ++c) acc[i][c] = fmaf(wgt, __ldcg(src + (size_t)(chunk[i] * 8 + c) * kRows), acc[i][c]);
-            }
-    }
-    const float inv = 1.f / Lm;
-    __nv_bfloat16* orow = p.out + ((((size_t)u.layer * p.B + u.b) * p.n + node) * (size_t)p.Hq + u.g * p.G + hl) * D;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i)
-        if (chunk[i] < kChunks) {
-            uint4 v;
-            v.x = pack_bf16(acc[i][0] * inv, acc[i][1] * inv);
-            v.y = pack_bf16(acc[i][2] * inv, acc[i][3] * inv);
-            v.z = pack_bf16(acc[i][4] * inv, acc[i][5] * inv);
-            v.w = pack_bf16(acc[i][6] * inv, acc[i][7] * inv);
-            *reinterpret_cast<uint4*>(orow + chunk[i] * 8) = v;
-        }
-    if (writes_lse)
-        p.lse_out[(((size_t)u.layer * p.B + u.b) * p.Hq + u.g * p.G + hl) * p.n + node] = Mm * kLn2 + logf(Lm);
+__global__ void __launch_bounds__(attn::kMergeThreads) attn_tile64_merge_kernel(const __grid_constant__ AttnParams p) {
+    const int rb = blockIdx.y;
+    attn::merge_boundary<D>(
+        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out,
+        [&](int row, const attn::GroupBegin& u, int& node, int& head) {
+            const int r_abs = rb * p.rows_per_rb + row;
+            node = r_abs / p.G;
+            head = u.g * p.G + r_abs % p.G;
+            return row < p.rows_per_rb && r_abs < p.rows;
+        },
+        [&](int group, int slot) { return p.partial + ((size_t)(group * p.n_rb + rb) * 2 + slot) * (D + 4) * kRows; });
 }
 
 }  // namespace
@@ -1098,9 +996,9 @@ mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, co
     p.rows_per_rb = (p.rows + p.n_rb - 1) / p.n_rb;
     p.n_groups = ctx->num_sms / p.n_rb;
     if (ctx->tune.attn_groups >= 1 && ctx->tune.attn_groups <= p.n_groups) p.n_groups = ctx->tune.attn_groups;
-    if (p.n_groups < 1) return MIRROR_ERR_SHAPE;
+    if (p.n_groups < 1 || p.n_groups * sizeof(attn::GroupBegin) > kWsNotesBytes) return MIRROR_ERR_SHAPE;
     p.snap_cap = ctx->tune.attn_snap;
-    p.whole_units = ctx->tune.attn_whole_units;
+    p.whole_groups = ctx->tune.attn_whole_units ? attn::whole_unit_groups(p.n_groups, (long long)kv->num_layers * tree->batch * ctx->desc.n_kv_heads) : 0;
     p.wait_limit = ctx->tune.wait_limit_cycles;
     p.stall_after = (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_attn_left-- > 0) ? ctx->tune.test_stall_after : -1;
     p.max_pages = kv->max_pages_per_req; p.num_pages = kv->num_pages;
@@ -1120,7 +1018,7 @@ mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, co
     p.k_pool = (const __nv_bfloat16*)kv->k_pool; p.v_pool = (const __nv_bfloat16*)kv->v_pool;
     p.k_new = (const __nv_bfloat16*)k_new; p.v_new = (const __nv_bfloat16*)v_new;
     p.out = (__nv_bfloat16*)out; p.lse_out = lse_out;
-    p.partial = partial_ws; p.status = ctx->d_status;
+    p.partial = partial_ws; p.begins = (attn::GroupBegin*)((uint8_t*)partial_ws - kWsNotesBytes); p.status = ctx->d_status;
     if (p.B > kMaxBatch) return MIRROR_ERR_SHAPE;
 
     AttnTree at;
@@ -1174,13 +1072,13 @@ mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, co
     // One request: all units have the same length whatever it is, so the host can tell when the partition gives every
     // group whole units (each unit holds at least one pair of tiles, so there are at least L * Hkv pairs): nothing is cut
     // and the merge kernel has nothing to do.
-    const bool no_cuts = p.whole_units && p.B == 1 && (long long)p.L * p.Hkv >= p.n_groups &&
-                         attn::whole_unit_groups(p.n_groups, (long long)p.L * p.B * p.Hkv) > 0;
+    const bool no_cuts = p.B == 1 && (long long)p.L * p.Hkv >= p.n_groups && p.whole_groups > 0;
     if (p.n_groups > 1 && !no_cuts) {
         // which units the partition cut is only known on the device (it depends on the prefix lengths)
-        const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)p.n_rb);
-        if (D == 128) MIRROR_CUDA_OK(mirror_launch_pdl(attn_tile64_merge_kernel<128>, mgrid, dim3(kMergeThreads), 0, stream, p));
-        else MIRROR_CUDA_OK(mirror_launch_pdl(attn_tile64_merge_kernel<64>, mgrid, dim3(kMergeThreads), 0, stream, p));
+        // (a unit is cut by one boundary or a few where there are many: more blocks per boundary then)
+        const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)p.n_rb, (int64_t)p.L * p.B * Hkv >= p.n_groups / 2 ? 4 : 1);
+        if (D == 128) MIRROR_CUDA_OK(mirror_launch_pdl(attn_tile64_merge_kernel<128>, mgrid, dim3(attn::kMergeThreads), 0, stream, p));
+        else MIRROR_CUDA_OK(mirror_launch_pdl(attn_tile64_merge_kernel<64>, mgrid, dim3(attn::kMergeThreads), 0, stream, p));
         ctx->launches += 1;
         MIRROR_CUDA_OK(cudaGetLastError());
     }

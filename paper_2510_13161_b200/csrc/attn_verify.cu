@@ -86,6 +86,7 @@ struct AttnParams {
     __nv_bfloat16* out;
     float* lse_out;
     float* partial;                       // [grid][2 slots][2 streams][D + 4][128]
+    attn::GroupBegin* begins;             // [n_groups]
     int* status;
     long long wait_limit;                 // SM cycles after which a wait gives up
     int stall_after;                      // test aid: the K producer stops after this many stages (-1: never)
@@ -491,6 +492,8 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         if (lane == 0) {
             ctrl->n_tiles = x1 - x;
             if (x < x1) ctrl->first = first_segment(x, x1, p, cumT, s_len, part.tiles_per_layer);
+            const Segment& s = ctrl->first;
+            if (rb == 0) p.begins[group] = {x < x1 && s.t_first > 0 ? 1 : 0, s.layer, s.b, s.g};
         }
     }
     __syncthreads();
@@ -970,128 +973,21 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
     }
 }
 
-// Merge of the units that the partition cut across CTA groups.  One block per (inner boundary, row tile of the group).
-// A unit cut by k boundaries left k + 1 (max, sum, accumulator) records, like split-KV partials; the k blocks of those
-// boundaries share its merge by output columns (8-column chunks dealt round-robin), each combining all parts of its
-// columns in group order, so a unit that many CTAs shared (few units per launch, long contexts) is not merged by one
-// block alone.  Blocks whose boundary coincides with a unit boundary have nothing to do.
-constexpr int kMergeThreads = 512;        // 128 rows x 4 column quarters
-constexpr int kMergeMaxGroups = 512;      // groups whose first tiles fit the lookup table (more: computed on demand)
+// Merge of the units that the partition cut: one block per (inner boundary, row tile of the group).
 template <int D>
-__global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_constant__ AttnParams p) {
-    __shared__ int cumT[kAttnMaxBatch + 1];
-    __shared__ int s_len[kAttnMaxBatch];
-    __shared__ int s_begin[kMergeMaxGroups];
-    const int tid = threadIdx.x;
-    // (the prefix lengths were complete before the attention kernel began)
-    if (tid < 32) load_lengths(p, cumT, s_len, false);
-    __syncthreads();
-    const Partition part = make_partition(p, cumT);
-    const int g = blockIdx.x + 1;
+__global__ void __launch_bounds__(attn::kMergeThreads) attn_merge_kernel(const __grid_constant__ AttnParams p) {
     const int n_str = p.mode == kSplit ? 1 : 2;
     const int rb = blockIdx.y / n_str, grp = blockIdx.y % n_str;
     const StreamId id = stream_of(p, rb, grp);
-    // A block with nothing to merge must still wait for the attention kernel: the kernel behind this one in the stream
-    // only waits for THIS grid to complete, so a grid whose blocks all left early would let it read attention outputs
-    // that are still being written.
-    if (g >= part.n_groups || part.total_tiles < 0 || !id.exists) { ptx::grid_dep_wait(); return; }
-    const int x = group_begin(part, g, p, cumT);
-    const UnitPos u = locate(x, p, cumT, part.tiles_per_layer);
-    if (u.tile_in_unit == 0) { ptx::grid_dep_wait(); return; }                  // the boundary is a unit boundary (block-uniform)
-    // every group's first tile, computed side by side (a unit shared by many groups is looked up from here instead of
-    // by a chain of dependent calls)
-    const bool tabled = part.n_groups <= kMergeMaxGroups;
-    if (tabled) {
-        for (int t = tid; t < part.n_groups; t += kMergeThreads) s_begin[t] = group_begin(part, t, p, cumT);
-        __syncthreads();
-    }
-    auto begin_of = [&](int t) -> int { return tabled ? s_begin[t] : group_begin(part, t, p, cumT); };
-    // the groups ga..gb hold this unit's parts; the blocks of the boundaries ga+1..gb share the merge by columns
-    int ga = g - 1;
-    while (ga > 0 && begin_of(ga) > u.unit_first_tile) --ga;
-    int gb = g;
-    const int unit_last = u.unit_first_tile + u.tiles_in_unit - 1;
-    while (gb + 1 < part.n_groups && begin_of(gb + 1) <= unit_last) ++gb;
-    const int parts = gb - ga + 1;
-    const int n_blocks = parts - 1, j_blk = g - (ga + 1);
-    // launched with programmatic stream serialization: everything above overlaps the attention kernel's tail;
-    // its records (and the outputs this block overwrites) are only touched after it has completed
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
-
-    constexpr int kRowW = D + 4;
-    constexpr int kChunks = D / 8;                                              // 8 output columns = one 16-byte store
-    constexpr int kPer = (kChunks + 3) / 4;                                     // chunks per thread when one block has them all
-    const int row = tid & (kRows - 1), cq = tid >> 7;
-    const int hl = (id.rt / p.node_tiles) * p.gs + row % p.gs, node = (id.rt % p.node_tiles) * p.nodes_tile + row / p.gs;
-    if (row >= p.gs * p.nodes_tile || hl >= p.G || node >= p.n) return;
-    const int head = (u.g * p.heads_per_unit + id.head_off) * p.G + hl;
-    // chunk c belongs to block c mod n_blocks; inside the block its chunks go round the four thread quarters
-    int chunk[kPer];
-    bool any = false;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-        chunk[i] = j_blk + (cq + 4 * i) * n_blocks;
-        any |= chunk[i] < kChunks;
-    }
-    const bool writes_lse = p.lse_out && j_blk == 0 && cq == 0;
-    if (!any && !writes_lse) return;
-    // group ga holds the unit's first tile (its record is in slot 1), the later groups began inside the unit (slot 0)
-    auto part_of = [&](int k) -> const float* {
-        return p.partial + (((size_t)((ga + k) * p.n_cta + rb) * 2 + (k == 0 ? 1 : 0)) * 2 + grp) * kRowW * kRows + row;
-    };
-    float Mm = -INFINITY;
-#pragma unroll 4
-    for (int k = 0; k < parts; ++k) Mm = fmaxf(Mm, __ldcg(part_of(k) + (size_t)D * kRows));
-    float Lm = 0.f;
-    float acc[kPer][8];
-#pragma unroll
-    for (int i = 0; i < kPer; ++i)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[i][c] = 0.f;
-    if (n_blocks >= 4) {
-        // many parts, at most one chunk per thread: six parts' loads in flight at a time (same order of additions)
-        const bool has = chunk[0] < kChunks;
-        const int c0 = has ? chunk[0] * 8 : 0;
-#pragma unroll 6
-        for (int k = 0; k < parts; ++k) {
-            const float* src = part_of(k);
-            const float pm = __ldcg(src + (size_t)D * kRows);
-            const float wgt = (pm == -INFINITY) ? 0.f : exp2f(pm - Mm);
-            Lm = fmaf(wgt, __ldcg(src + (size_t)(D + 1) * kRows), Lm);
-            if (has) {
-#pragma unroll
-                for (int c = 0; c < 8; ++c) acc[0][c] = fmaf(wgt, __ldcg(src + (size_t)(c0 + c) * kRows), acc[0][c]);
-            }
-        }
-    } else
-#pragma unroll 2
-    for (int k = 0; k < parts; ++k) {
-        const float* src = part_of(k);
-        const float pm = __ldcg(src + (size_t)D * kRows);
-        const float wgt = (pm == -INFINITY) ? 0.f : exp2f(pm - Mm);
-        Lm = fmaf(wgt, __ldcg(src + (size_t)(D + 1) * kRows), Lm);
-#pragma unroll
-        for (int i = 0; i < kPer; ++i)
-            if (chunk[i] < kChunks) {
-#pragma unroll
-                for (int c = 0; c < 8; ++c) acc[i][c] = fmaf(wgt, __ldcg(src + (size_t)(chunk[i] * 8 + c) * kRows), acc[i][c]);
-            }
-    }
-    const float inv = 1.f / Lm;
-    const size_t lb = (size_t)u.layer * p.B + u.b;
-    __nv_bfloat16* orow = p.out + ((lb * p.n + node) * (size_t)p.Hq + head) * D;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i)
-        if (chunk[i] < kChunks) {
-            uint4 v;
-            v.x = pack_bf16(acc[i][0] * inv, acc[i][1] * inv);
-            v.y = pack_bf16(acc[i][2] * inv, acc[i][3] * inv);
-            v.z = pack_bf16(acc[i][4] * inv, acc[i][5] * inv);
-            v.w = pack_bf16(acc[i][6] * inv, acc[i][7] * inv);
-            *reinterpret_cast<uint4*>(orow + chunk[i] * 8) = v;
-        }
-    if (writes_lse) p.lse_out[(lb * p.Hq + head) * p.n + node] = Mm * kAttnLn2 + logf(Lm);
+    attn::merge_boundary<D>(
+        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out,
+        [&](int row, const attn::GroupBegin& u, int& node, int& head) {
+            const int hl = (id.rt / p.node_tiles) * p.gs + row % p.gs;
+            node = (id.rt % p.node_tiles) * p.nodes_tile + row / p.gs;
+            head = (u.g * p.heads_per_unit + id.head_off) * p.G + hl;
+            return id.exists && row < p.gs * p.nodes_tile && hl < p.G && node < p.n;
+        },
+        [&](int group, int slot) { return p.partial + (((size_t)(group * p.n_cta + rb) * 2 + slot) * 2 + grp) * (D + 4) * kRows; });
 }
 
 }  // namespace
@@ -1121,7 +1017,7 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     p.n_cta = p.heads_per_unit == 2 ? p.n_rt : (p.n_rt + 1) / 2;
     p.n_groups = ctx->num_sms / p.n_cta;
     if (ctx->tune.attn_groups >= 1 && ctx->tune.attn_groups <= p.n_groups) p.n_groups = ctx->tune.attn_groups;
-    if (p.n_groups < 1) return MIRROR_ERR_SHAPE;
+    if (p.n_groups < 1 || p.n_groups * sizeof(attn::GroupBegin) > kWsNotesBytes) return MIRROR_ERR_SHAPE;
     p.snap_cap = (ctx->tune.attn_snap + 1) / 2;              // (given in tiles of 64 tokens)
     // Units of at most six tiles (the page table says how long a prefix can be) take a CTA less time whole than the merge
     // kernel behind a cut would: a launch and a pass over the records, ~6 us.
@@ -1142,7 +1038,7 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     p.page_table = kv->page_table; p.prefix_len = kv->prefix_len;
     p.v_pool = (const __nv_bfloat16*)kv->v_pool;
     p.out = (__nv_bfloat16*)out; p.lse_out = lse_out;
-    p.partial = partial_ws; p.status = ctx->d_status;
+    p.partial = partial_ws; p.begins = (attn::GroupBegin*)((uint8_t*)partial_ws - kWsNotesBytes); p.status = ctx->d_status;
 
     AttnTree at;
     memcpy(at.anc, ti.anc, sizeof at.anc);
@@ -1187,8 +1083,9 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         const bool no_cuts = p.never_cut || (p.B == 1 && p.whole_groups > 0);
         if (p.n_groups > 1 && !no_cuts) {
             // which units the partition cut is only known on the device (it depends on the prefix lengths)
-            const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)(p.n_cta * (p.mode == kSplit ? 1 : 2)));
-            MIRROR_CUDA_OK(mirror_launch_pdl(merge, mgrid, dim3(kMergeThreads), 0, stream, p));
+            // (a unit is cut by one boundary or a few where there are many: more blocks per boundary then)
+            const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)(p.n_cta * (p.mode == kSplit ? 1 : 2)), (int64_t)p.L * p.B * Hkv >= p.n_groups / 2 ? 4 : 1);
+            MIRROR_CUDA_OK(mirror_launch_pdl(merge, mgrid, dim3(attn::kMergeThreads), 0, stream, p));
             ctx->launches += 1;
             MIRROR_CUDA_OK(cudaGetLastError());
         }

@@ -104,7 +104,6 @@ extern "C" mirror_status mirror_device_status(mirror_ctx* ctx, int* code, int* d
     if (detail) *detail = h[1];
     if (h[0] != 0) {
         MIRROR_CUDA_OK(cudaMemset(ctx->d_status, 0, sizeof h));
-        if (ctx->ws) MIRROR_CUDA_OK(cudaMemset(ctx->ws, 0, ctx->ws_bytes < kWsZeroedBytes ? ctx->ws_bytes : kWsZeroedBytes));
     }
     return MIRROR_OK;
 }
@@ -202,8 +201,8 @@ extern "C" mirror_status mirror_trie_build(const int32_t* branch_tokens, int kap
 void mirror_ws_layout(const mirror_ctx* ctx, size_t M, MirrorWsLayout* out, size_t B) {
     MirrorWsLayout L;
     size_t at = 0;
-    L.zeroed = at;
-    at += kWsZeroedBytes;
+    L.notes = at;
+    at += kWsNotesBytes;
     L.attn_partial = at;
     // two record slots per CTA (a CTA's range of KV tiles cuts at most two units) for each of its two streams of 128 rows
     L.attn_partial_bytes = align_up((size_t)ctx->num_sms * 4 * 128 * (size_t)(ctx->desc.head_dim + 4) * sizeof(float), 256);
@@ -262,10 +261,6 @@ extern "C" mirror_status mirror_set_workspace(mirror_ctx* ctx, void* dev_ptr, si
     if (dev_ptr && ((uintptr_t)dev_ptr & 255)) return MIRROR_ERR_ARG;
     ctx->ws = dev_ptr;
     ctx->ws_bytes = dev_ptr ? bytes : 0;
-    if (dev_ptr) {
-        MIRROR_CUDA_OK(cudaSetDevice(ctx->device));
-        MIRROR_CUDA_OK(cudaMemset(dev_ptr, 0, bytes < kWsZeroedBytes ? bytes : kWsZeroedBytes));
-    }
     return MIRROR_OK;
 }
 

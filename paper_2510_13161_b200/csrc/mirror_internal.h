@@ -68,11 +68,11 @@ struct mirror_ctx {
 mirror_status mirror_build_tree(const mirror_tree* tree, MirrorTreeInfo* info);
 
 // Workspace carving.  The layout depends only on the model shape and the row count M, so every entry
-// point finds the same regions: [zeroed words | attention split records | LM-head partials | lse, argmax
-// scratch | fp32 logits | fp64 acceptance scratch].  Offsets are 256-byte aligned; the first region is zeroed when the workspace is attached.
-constexpr size_t kWsZeroedBytes = 4096;     // words at the front of the workspace that are zero between launches (none in use now)
+// point finds the same regions: [attention notes | attention split records | LM-head partials | lse, argmax
+// scratch | fp32 logits | fp64 acceptance scratch].  Offsets are 256-byte aligned.
+constexpr size_t kWsNotesBytes = 8192;      // what the attention kernel's CTA groups leave for the merge kernel, in front of their records
 struct MirrorWsLayout {
-    size_t zeroed = 0;                                   // kWsZeroedBytes of zeroed words
+    size_t notes = 0;                                    // kWsNotesBytes in front of the attention's records
     size_t attn_partial = 0, attn_partial_bytes = 0;     // split-KV partial accumulators
     size_t lm_partial = 0, lm_partial_bytes = 0;         // per-CTA (or per-unit) row partials
     size_t lse = 0, argmax = 0;                          // [M] scratch each
