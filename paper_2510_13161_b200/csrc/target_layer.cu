@@ -46,69 +46,95 @@ __global__ void rope_table_kernel(const int32_t* prefix_len, const TreeDepths td
     cs[idx] = make_float2((float)c, (float)s);
 }
 
+__device__ __forceinline__ float4 sum_slices4(const float* partial, int slices, size_t slice_elems, size_t idx) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int s = 0; s < slices; ++s) {                                                 // fixed order
+        const float4 v = *reinterpret_cast<const float4*>(partial + (size_t)s * slice_elems + idx);
+        a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+    }
+    return a;
+}
+__device__ __forceinline__ void store4(__nv_bfloat16* dst, float a, float b, float c, float d) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
+    *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+}
+
 // Q/K/V projection finish: split-K sum, rotary embedding on the query and key heads, bf16 stores into the step's
-// [M, Hq, d] / [M, Hkv, d] tensors.  One block per (row, head), one thread per rotation pair (f, f + d/2); all
-// slices of a thread's two columns are loaded before they are added (the loads are independent, the order of the sum
-// is fixed).
-__global__ void finish_qkv_kernel(const float* partial, int slices, int M, int Hq, int Hkv, int d, const float2* cs,
-                                  __nv_bfloat16* q_out, __nv_bfloat16* k_out, __nv_bfloat16* v_out) {
+// [M, Hq, d] / [M, Hkv, d] tensors.  A thread does four rotation pairs (f, f + d/2) of one head; all slices of its columns
+// are loaded before they are added (the loads are independent, the order of the sum is fixed).  Few and small blocks: the
+// next kernel's blocks have to find room beside them (952 blocks of 64 threads took 4.7 us at 17 rows, these 2.5).
+constexpr int kQkvThreads = 128;
+__global__ void __launch_bounds__(kQkvThreads)
+finish_qkv_kernel(const float* partial, int slices, int M, int Hq, int Hkv, int d, const float2* cs,
+                  __nv_bfloat16* q_out, __nv_bfloat16* k_out, __nv_bfloat16* v_out) {
+    const int row = blockIdx.x, half = d >> 1, per = half >> 2;
+    const int t = blockIdx.y * kQkvThreads + threadIdx.x, head = t / per, f = (t - head * per) * 4;
+    const bool in = head < Hq + 2 * Hkv;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    const int row = blockIdx.x, head = blockIdx.y, half = d >> 1, f = threadIdx.x;
-    if (f >= half) return;
+    if (!in) return;
     const int N = (Hq + 2 * Hkv) * d;
-    const size_t MN = (size_t)M * N;
-    const float* p0 = partial + (size_t)row * N + (size_t)head * d + f;
-    float a = 0.f, b = 0.f;
-#pragma unroll 8
-    for (int s = 0; s < slices; ++s) {
-        a += p0[(size_t)s * MN];
-        b += p0[(size_t)s * MN + half];
-    }
+    const size_t MN = (size_t)M * N, at = (size_t)row * N + (size_t)head * d + f;
+    const float4 a = sum_slices4(partial, slices, MN, at), b = sum_slices4(partial, slices, MN, at + half);
+    __nv_bfloat16* dst = head < Hq         ? q_out + ((size_t)row * Hq + head) * d
+                         : head < Hq + Hkv ? k_out + ((size_t)row * Hkv + (head - Hq)) * d
+                                           : v_out + ((size_t)row * Hkv + (head - Hq - Hkv)) * d;
     if (head < Hq + Hkv) {
-        const float2 t = cs[(size_t)row * half + f];
-        const float ra = a * t.x - b * t.y, rb = b * t.x + a * t.y;
-        __nv_bfloat16* dst = head < Hq ? q_out + ((size_t)row * Hq + head) * d : k_out + ((size_t)row * Hkv + (head - Hq)) * d;
-        dst[f] = __float2bfloat16_rn(ra);
-        dst[f + half] = __float2bfloat16_rn(rb);
+        const float4 t0 = *reinterpret_cast<const float4*>(cs + (size_t)row * half + f);          // (cos, sin) of f and f + 1
+        const float4 t1 = *reinterpret_cast<const float4*>(cs + (size_t)row * half + f + 2);
+        store4(dst + f, a.x * t0.x - b.x * t0.y, a.y * t0.z - b.y * t0.w, a.z * t1.x - b.z * t1.y, a.w * t1.z - b.w * t1.w);
+        store4(dst + f + half, b.x * t0.x + a.x * t0.y, b.y * t0.z + a.y * t0.w, b.z * t1.x + a.z * t1.y, b.w * t1.z + a.w * t1.w);
     } else {
-        __nv_bfloat16* dst = v_out + ((size_t)row * Hkv + (head - Hq - Hkv)) * d;
-        dst[f] = __float2bfloat16_rn(a);
-        dst[f + half] = __float2bfloat16_rn(b);
+        store4(dst + f, a.x, a.y, a.z, a.w);
+        store4(dst + f + half, b.x, b.y, b.z, b.w);
     }
 }
 
 // Residual add + RMSNorm: r = residual + split-K sum, x_out = bf16(r); normed = bf16(x_out / sqrt(mean(x_out^2) + eps)
-// * gamma) (from the ROUNDED x_out: what a later reader of x_out would compute).  One block of 1024 threads per row;
-// a thread keeps its columns (every 1024th) in registers between the two passes and issues the loads of all slices
-// of all its columns before adding them (in slice order).  partial == nullptr: plain RMSNorm of `residual`;
+// * gamma) (from the ROUNDED x_out: what a later reader of x_out would compute).  A cluster of four CTAs of 256 threads
+// per row: with few rows one block per row leaves the chip empty and pulls a row's partial sums through one SM (17 rows x
+// 7 slices: 5.8 us).  A thread keeps its columns (every 1024th) in registers between the two passes and issues the loads
+// of all slices of all its columns before adding them (in slice order); the 32 warps' sums of squares meet in every
+// CTA's shared memory and are added in warp order.  partial == nullptr: plain RMSNorm of `residual`;
 // gamma == nullptr: no norm.
-constexpr int kNormThreads = 1024;
+constexpr int kNormThreads = 1024;            // per row, four CTAs together
+constexpr int kNormCluster = 4;
 constexpr int kNormMaxCols = 16;              // columns per thread: rows of up to 16384 elements
 template <int kNormCols, int kUnroll>         // kNormCols * 1024 >= H; kUnroll slices' loads in flight at a time
-__global__ void __launch_bounds__(kNormThreads)
+__global__ void __launch_bounds__(kNormThreads / kNormCluster)
 finish_residual_norm_kernel(const float* partial, int slices, int M, int H, const __nv_bfloat16* residual,
                             const __nv_bfloat16* gamma, float eps, __nv_bfloat16* x_out, __nv_bfloat16* normed) {
     __shared__ float s_red[kNormThreads / 32];
+    const int row = blockIdx.x / kNormCluster, rank = blockIdx.x % kNormCluster;
+    const int t = rank * (kNormThreads / kNormCluster) + threadIdx.x;
+    const size_t MN = (size_t)M * H, base = (size_t)row * H;
+    // (a CTA may be written to once it has started: arrive now, wait in front of the exchange)
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    float r[kNormCols], gm[kNormCols];
+    auto load_early = [&]() {
+#pragma unroll
+        for (int c = 0; c < kNormCols; ++c) {
+            const int col = t + c * kNormThreads;
+            r[c] = col < H ? __bfloat162float(residual[base + col]) : 0.f;
+            gm[c] = col < H && gamma ? __bfloat162float(gamma[col]) : 0.f;
+        }
+    };
+    // behind a projection, the residual stream and the weight are older than the kernel ahead: no need to wait for it
+    if (partial) load_early();
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    const int row = blockIdx.x;
-    const size_t MN = (size_t)M * H, base = (size_t)row * H;
-    float r[kNormCols];
-#pragma unroll
-    for (int c = 0; c < kNormCols; ++c) {
-        const int col = threadIdx.x + c * kNormThreads;
-        r[c] = col < H ? __bfloat162float(residual[base + col]) : 0.f;
-    }
+    if (!partial) load_early();
     if (partial) {
         // several slices' loads in flight at a time; the additions stay in slice order
+#pragma unroll 1
         for (int s0 = 0; s0 < slices; s0 += kUnroll) {
             float v[kUnroll][kNormCols];
 #pragma unroll
             for (int k = 0; k < kUnroll; ++k)
 #pragma unroll
                 for (int c = 0; c < kNormCols; ++c) {
-                    const int col = threadIdx.x + c * kNormThreads;
+                    const int col = t + c * kNormThreads;
                     v[k][c] = (col < H && s0 + k < slices) ? partial[(size_t)(s0 + k) * MN + base + col] : 0.f;
                 }
 #pragma unroll
@@ -120,7 +146,7 @@ finish_residual_norm_kernel(const float* partial, int slices, int M, int H, cons
     float ss = 0.f;
 #pragma unroll
     for (int c = 0; c < kNormCols; ++c) {
-        const int col = threadIdx.x + c * kNormThreads;
+        const int col = t + c * kNormThreads;
         if (col < H) {
             const __nv_bfloat16 xb = __float2bfloat16_rn(r[c]);
             if (x_out) x_out[base + col] = xb;
@@ -128,32 +154,40 @@ finish_residual_norm_kernel(const float* partial, int slices, int M, int H, cons
             ss = fmaf(r[c], r[c], ss);
         }
     }
-    if (!gamma || !normed) return;
+    const bool norm = gamma && normed;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = ss;
-    __syncthreads();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if ((threadIdx.x & 31) < kNormCluster) {                                   // lane j: this warp's sum to CTA j
+        uint32_t dst;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(ptx::smem_u32(&s_red[t >> 5])), "r"(threadIdx.x & 31));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(ss) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (!norm) return;
     float tot = 0.f;
 #pragma unroll
     for (int w = 0; w < kNormThreads / 32; ++w) tot += s_red[w];               // same order in every thread
     const float rinv = 1.0f / sqrtf(tot / (float)H + eps);
 #pragma unroll
     for (int c = 0; c < kNormCols; ++c) {
-        const int col = threadIdx.x + c * kNormThreads;
-        if (col < H) normed[base + col] = __float2bfloat16_rn(r[c] * rinv * __bfloat162float(gamma[col]));
+        const int col = t + c * kNormThreads;
+        if (col < H) normed[base + col] = __float2bfloat16_rn(r[c] * rinv * gm[c]);
     }
 }
 
-// Gated MLP finish: act[row, j] = bf16(silu(gate) * up), gate = sum of column j, up = sum of column I + j.
+// Gated MLP finish: act[row, j] = bf16(silu(gate) * up), gate = sum of column j, up = sum of column I + j; four columns a thread.
 __global__ void __launch_bounds__(kFinThreads)
 finish_swiglu_kernel(const float* partial, int slices, int M, int I, __nv_bfloat16* act) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
     const size_t MN = (size_t)M * 2 * I, total = (size_t)M * I;
-    for (size_t idx = (size_t)blockIdx.x * kFinThreads + threadIdx.x; idx < total; idx += (size_t)gridDim.x * kFinThreads) {
+    for (size_t idx = ((size_t)blockIdx.x * kFinThreads + threadIdx.x) * 4; idx < total; idx += (size_t)gridDim.x * kFinThreads * 4) {
         const size_t row = idx / I, j = idx - row * I;
-        const float g = sum_slices(partial, slices, MN, row * 2 * I + j), u = sum_slices(partial, slices, MN, row * 2 * I + I + j);
-        act[idx] = __float2bfloat16_rn(g / (1.0f + expf(-g)) * u);
+        const float4 g = sum_slices4(partial, slices, MN, row * 2 * I + j), u = sum_slices4(partial, slices, MN, row * 2 * I + I + j);
+        store4(act + idx, g.x / (1.0f + expf(-g.x)) * u.x, g.y / (1.0f + expf(-g.y)) * u.y, g.z / (1.0f + expf(-g.z)) * u.z,
+               g.w / (1.0f + expf(-g.w)) * u.w);
     }
 }
 
@@ -171,14 +205,20 @@ finish_store_kernel(const float* partial, int slices, size_t MN, const __nv_bflo
 
 cudaError_t launch_residual_norm(cudaStream_t s, const float* partial, int slices, int M, int H, const __nv_bfloat16* residual,
                                  const __nv_bfloat16* gamma, float eps, __nv_bfloat16* x_out, __nv_bfloat16* normed) {
-    if (H <= 4 * kNormThreads)
-        return mirror_launch_pdl(finish_residual_norm_kernel<4, 6>, dim3(M), dim3(kNormThreads), 0, s, partial, slices, M, H, residual, gamma,
-                                 eps, x_out, normed);
-    if (H <= 8 * kNormThreads)
-        return mirror_launch_pdl(finish_residual_norm_kernel<8, 4>, dim3(M), dim3(kNormThreads), 0, s, partial, slices, M, H, residual, gamma,
-                                 eps, x_out, normed);
-    return mirror_launch_pdl(finish_residual_norm_kernel<16, 2>, dim3(M), dim3(kNormThreads), 0, s, partial, slices, M, H, residual, gamma,
-                             eps, x_out, normed);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)M * kNormCluster);
+    cfg.blockDim = dim3(kNormThreads / kNormCluster);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = kNormCluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    auto kern = H <= 4 * kNormThreads ? finish_residual_norm_kernel<4, 8> : H <= 8 * kNormThreads ? finish_residual_norm_kernel<8, 7> : finish_residual_norm_kernel<16, 3>;
+    return cudaLaunchKernelEx(&cfg, kern, partial, slices, M, H, residual, gamma, eps, x_out, normed);
 }
 
 // Rows of the embedding table for the step's tokens: out[r] = table[tokens[r]] (16-byte copies; a token outside the
@@ -307,7 +347,7 @@ mirror_status target_forward_impl(mirror_ctx* ctx, const mirror_target* t, const
     if (!t->layers || !t->norm_final || t->n_layers <= 0 || t->n_layers > kv->num_layers) return MIRROR_ERR_ARG;
     const int H = ctx->desc.hidden, Hq = ctx->desc.n_q_heads, Hkv = ctx->desc.n_kv_heads, d = ctx->desc.head_dim, I = t->intermediate;
     if (I <= 0 || I % 64 != 0 || H % 64 != 0 || (Hq * d) % 64 != 0 || (d & 1)) return MIRROR_ERR_SHAPE;
-    if (H > kNormThreads * kNormMaxCols || d / 2 > 1024) return MIRROR_ERR_SHAPE;
+    if (H > kNormThreads * kNormMaxCols ) return MIRROR_ERR_SHAPE;
     if (!kv->k_pool || !kv->v_pool || !kv->page_table || !kv->prefix_len) return MIRROR_ERR_ARG;
     if (((uintptr_t)x & 15) || ((uintptr_t)scratch & 255)) return MIRROR_ERR_ARG;
     for (int l = 0; l < t->n_layers; ++l) {
@@ -358,7 +398,7 @@ mirror_status target_forward_impl(mirror_ctx* ctx, const mirror_target* t, const
         // Q/K/V projection + rotary embedding
         st = mirror_linear_partial_launch(ctx, h, M, w.w_qkv, Nqkv, H, partial, sc.partial_bytes, s, &slices);
         if (st != MIRROR_OK) return st;
-        MIRROR_CUDA_OK(mirror_launch_pdl(finish_qkv_kernel, dim3(M, Hq + 2 * Hkv), dim3(half), 0, s, (const float*)partial, slices, M, Hq, Hkv, d,
+        MIRROR_CUDA_OK(mirror_launch_pdl(finish_qkv_kernel, dim3(M, (Nqkv / 8 + kQkvThreads - 1) / kQkvThreads), dim3(kQkvThreads), 0, s, (const float*)partial, slices, M, Hq, Hkv, d,
                                          (const float2*)cs, q_l, k_l, v_l));
         ctx->launches += 1;
         // attention of this layer over its slab of the cache
@@ -390,7 +430,7 @@ mirror_status target_forward_impl(mirror_ctx* ctx, const mirror_target* t, const
         // gate / up projection + SiLU gate
         st = mirror_linear_partial_launch(ctx, h, M, w.w_gate_up, 2 * I, H, partial, sc.partial_bytes, s, &slices);
         if (st != MIRROR_OK) return st;
-        MIRROR_CUDA_OK(mirror_launch_pdl(finish_swiglu_kernel, dim3(grid_for((size_t)M * I, ctx->num_sms)), dim3(kFinThreads), 0, s,
+        MIRROR_CUDA_OK(mirror_launch_pdl(finish_swiglu_kernel, dim3(grid_for((size_t)M * I / 4, ctx->num_sms)), dim3(kFinThreads), 0, s,
                                          (const float*)partial, slices, M, I, act));
         ctx->launches += 1;
         // down projection + residual + the next layer's (or the final) norm
