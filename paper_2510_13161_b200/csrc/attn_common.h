@@ -51,25 +51,30 @@ struct GroupBegin {
     int part, layer, b, g;
 };
 constexpr int kMergeThreads = 512;        // 128 rows x 4 column quarters
-constexpr int kMergeBatch = 32;           // parts whose (max, sum) are in shared memory at a time
+constexpr int kMergeSlots = 32;           // (part, 8-column chunk) pairs in shared memory at a time
+constexpr int kMergeSmem = kMergeSlots * 10 * 128 * 4;      // their columns, then the parts' (max, sum)
 
-// A block per (inner boundary, row tile) and blockIdx.z.  A unit cut by k boundaries left k + 1 (max, sum, accumulator)
-// records, like split-KV partials; the blocks of those boundaries share its merge by output columns (8-column chunks
-// dealt round-robin), each combining all parts of its columns in group order, so a unit that many CTAs shared (few units
-// per launch, long contexts) is not merged by one block alone.  Which unit a boundary cuts is read from the groups' own
-// notes (finding it again from the lengths cost more than the merge).  What bounds it is the chain of loads and the
-// fetch of code that runs once, so the code is small: the parts' (max, sum) come side by side into shared memory and
-// become weights there, and the loop over the parts is two loads and three multiply-adds.
+// A block per (inner boundary, row tile).  A unit cut by k boundaries left k + 1 (max, sum, accumulator) records, like
+// split-KV partials; the k blocks of those boundaries share its merge by output columns (8-column chunks dealt
+// round-robin), each combining all parts of its columns in group order, so a unit that many CTAs shared (few units per
+// launch, long contexts) is not merged by one block alone.  Which unit a boundary cuts is read from the groups' own notes
+// (finding it again from the lengths cost more than the merge).  What bounds it is the chain of loads and the fetch of
+// code that runs once: a chunk of a record is 4 KB in one piece, so bulk copies bring everything a block needs at once,
+// and the arithmetic runs out of shared memory (17 parts of 85 rows: 15 us with loads in the loop over the parts, 8 with
+// eight parts' loads in flight).
 // map(row, GroupBegin) -> false, or the row's node and query head; record(group, slot) -> its record in slot 0 (of the unit
 // that began before the group's range) or 1, [column][128 rows], D accumulator columns, then (max, sum).
 template <int D, class Map, class Record>
 __device__ __forceinline__ void merge_boundary(const GroupBegin* table, int n_groups, int n, int Hq, int B, __nv_bfloat16* out, float* lse_out,
-                                               Map map, Record record) {
+                                               int* status, Map map, Record record) {
+    extern __shared__ __align__(128) float s_cols[];                            // [slot][8 columns][128 rows]
+    float(*const s_ml)[2][128] = (float(*)[2][128])(s_cols + kMergeSlots * 8 * 128);     // [part][max, then weight | sum][128 rows]
     __shared__ GroupBegin s_begin[512];
-    __shared__ float s_w[kMergeBatch][128], s_l[kMergeBatch][128];              // max, then weight; sum
-    const int tid = threadIdx.x, g = blockIdx.x + 1;
+    __shared__ uint64_t s_bar;
+    const int tid = threadIdx.x, warp = tid >> 5, g = blockIdx.x + 1;
+    ptx::grid_dep_launch();                       // (the kernel behind only sets itself up before this one has completed)
+    if (tid == 0) { ptx::mbar_init(&s_bar, 1); ptx::fence_mbar_init(); }
     ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
     for (int i = tid; i < n_groups; i += kMergeThreads) s_begin[i] = table[i];
     __syncthreads();
     const GroupBegin u = s_begin[g];
@@ -80,69 +85,88 @@ __device__ __forceinline__ void merge_boundary(const GroupBegin* table, int n_gr
     while (ga > 0 && same(ga)) --ga;
     while (gb + 1 < n_groups && same(gb + 1)) ++gb;
     const int parts = gb - ga + 1;
-    const int n_blocks = (parts - 1) * gridDim.z, j_blk = (g - (ga + 1)) * gridDim.z + blockIdx.z;
-
+    const int n_blocks = parts - 1, j_blk = g - (ga + 1);
     constexpr int kChunks = D / 8;                                              // 8 output columns, 2 of them a thread quarter's
     const int row = tid & 127, cq = tid >> 7;
     int node = 0, head = 0;
     const bool has_row = map(row, u, node, head);
     const size_t lb = (size_t)u.layer * B + u.b;
     // group ga holds the unit's first tile (its record is in slot 1), the later groups began inside the unit (slot 0)
-    const float* const first = record(ga, 1) + row;
-    const float* const second = record(ga + 1, 0) + row;
+    const float* const first = record(ga, 1);
+    const float* const second = record(ga + 1, 0);
     const size_t stride = record(1, 0) - record(0, 0);
-    auto part_of = [&](int k) -> const float* { return k == 0 ? first : second + (size_t)(k - 1) * stride; };
-    auto load_batch = [&](int k0) {                                             // (max, sum) of the parts from k0 on
-        const int nk = has_row ? min(kMergeBatch, parts - k0) : 0;
-#pragma unroll 4
-        for (int k = cq; k < nk; k += 4) {
-            const float* src = part_of(k0 + k) + (size_t)D * 128;
-            s_w[k][row] = __ldcg(src);
-            s_l[k][row] = __ldcg(src + 128);
+    uint32_t phase = 0;
+    // One load: n_ch chunks (c0, c0 + n_blocks, ...) of the parts [k0, k0 + nk), with the parts' (max, sum) unless n_ch < 0 (then
+    // only those).  false: the copies did not arrive (reported).
+    auto fetch = [&](int k0, int nk, int c0, int n_ch, bool ml) -> bool {
+        __syncthreads();
+        if (tid == 0) ptx::mbar_arrive_expect_tx(&s_bar, (uint32_t)(nk * (n_ch * 4096 + (ml ? 1024 : 0))));
+        __syncthreads();
+        for (int i = warp; i < nk * (n_ch + 1); i += kMergeThreads / 32) {
+            const int c = i / nk, k = i - c * nk;
+            const float* src = k0 + k == 0 ? first : second + (size_t)(k0 + k - 1) * stride;
+            if (c == n_ch && !ml) continue;
+            src += c == n_ch ? (size_t)D * 128 : (size_t)(c0 + c * n_blocks) * 8 * 128;
+            float* const dst = c == n_ch ? &s_ml[k][0][0] : s_cols + (size_t)i * 8 * 128;
+            if ((tid & 31) == 0)
+                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                             ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(c == n_ch ? 1024u : 4096u), "r"(ptx::smem_u32(&s_bar)) : "memory");
         }
-        __syncthreads();
-        return nk;
+        const bool ok = ptx::mbar_wait(&s_bar, phase);
+        phase ^= 1;
+        if (!ok && atomicCAS(status, 0, MIRROR_DEV_TIMEOUT) == 0) atomicExch(status + 1, 38);
+        return __syncthreads_and(ok);
     };
-    auto weigh = [&](int nk, float M) {
-        __syncthreads();                                                        // (all maxima of the batch have been read)
-        for (int k = cq; k < nk; k += 4) s_w[k][row] = s_w[k][row] == -INFINITY ? 0.f : exp2f(s_w[k][row] - M);
+    auto weigh = [&](int nk, float M) {                                         // maxima -> weights
+        __syncthreads();
+        for (int k = cq; k < nk; k += 4) s_ml[k][0][row] = s_ml[k][0][row] == -INFINITY ? 0.f : exp2f(s_ml[k][0][row] - M);
         __syncthreads();
     };
+    const bool one_batch = parts <= kMergeSlots;
+    const int n_ch = max(1, kMergeSlots / parts);                               // chunks side by side when the parts are few
     float Mm = -INFINITY;
-    int nk = 0;
+    if (!one_batch)
+        for (int k0 = 0; k0 < parts; k0 += kMergeSlots) {
+            const int nk = min(kMergeSlots, parts - k0);
+            if (!fetch(k0, nk, 0, 0, true)) return;
+            for (int k = 0; k < nk; ++k) Mm = fmaxf(Mm, s_ml[k][0][row]);
+        }
 #pragma unroll 1
-    for (int k0 = 0; k0 < parts; k0 += kMergeBatch) {
-        if (k0 > 0) __syncthreads();
-        nk = load_batch(k0);
-        for (int k = 0; k < nk; ++k) Mm = fmaxf(Mm, s_w[k][row]);
-    }
-    const bool one_batch = parts <= kMergeBatch;
-    if (one_batch) weigh(nk, Mm);
-    const bool writes_lse = lse_out && j_blk == 0;
-#pragma unroll 1
-    for (int chunk = j_blk; chunk < kChunks; chunk += n_blocks) {
+    for (int c0 = j_blk; c0 < kChunks; c0 += n_ch * n_blocks) {
+        const int nc = min(n_ch, (kChunks - c0 + n_blocks - 1) / n_blocks);
         float Lm = 0.f, a0 = 0.f, a1 = 0.f;
-        const size_t col = (size_t)(chunk * 8 + cq * 2) * 128;
-#pragma unroll 1
-        for (int k0 = 0; k0 < parts; k0 += kMergeBatch) {
-            if (!one_batch) {
-                __syncthreads();
-                nk = load_batch(k0);
-                weigh(nk, Mm);
-            }
-#pragma unroll 8
-            for (int k = 0; k < nk; ++k) {
-                const float* src = part_of(k0 + k) + col;
-                const float wgt = s_w[k][row];
-                Lm = fmaf(wgt, s_l[k][row], Lm);
-                a0 = fmaf(wgt, __ldcg(src), a0);
-                a1 = fmaf(wgt, __ldcg(src + 128), a1);
+        if (one_batch) {
+            if (!fetch(0, parts, c0, nc, c0 == j_blk)) return;
+            if (c0 == j_blk) {
+                for (int k = 0; k < parts; ++k) Mm = fmaxf(Mm, s_ml[k][0][row]);
+                weigh(parts, Mm);
             }
         }
-        if (!has_row) continue;
-        const float inv = 1.f / Lm;
-        *reinterpret_cast<uint32_t*>(out + ((lb * n + node) * (size_t)Hq + head) * D + chunk * 8 + cq * 2) = pack_bf16(a0 * inv, a1 * inv);
-        if (writes_lse && chunk == 0 && cq == 0) lse_out[(lb * Hq + head) * n + node] = Mm * kAttnLn2 + logf(Lm);
+#pragma unroll 1
+        for (int c = 0; c < nc; ++c) {
+            Lm = a0 = a1 = 0.f;
+#pragma unroll 1
+            for (int k0 = 0; k0 < parts; k0 += kMergeSlots) {
+                const int nk = min(kMergeSlots, parts - k0);
+                if (!one_batch) {
+                    if (!fetch(k0, nk, c0, 1, true)) return;
+                    weigh(nk, Mm);
+                }
+                const float* col = s_cols + (size_t)(c * nk * 8 + cq * 2) * 128 + row;
+#pragma unroll 4
+                for (int k = 0; k < nk; ++k) {
+                    const float wgt = s_ml[k][0][row];
+                    Lm = fmaf(wgt, s_ml[k][1][row], Lm);
+                    a0 = fmaf(wgt, col[k * 1024], a0);
+                    a1 = fmaf(wgt, col[k * 1024 + 128], a1);
+                }
+            }
+            const int chunk = c0 + c * n_blocks;
+            if (!has_row) continue;
+            const float inv = 1.f / Lm;
+            *reinterpret_cast<uint32_t*>(out + ((lb * n + node) * (size_t)Hq + head) * D + chunk * 8 + cq * 2) = pack_bf16(a0 * inv, a1 * inv);
+            if (lse_out && chunk == 0 && cq == 0) lse_out[(lb * Hq + head) * n + node] = Mm * kAttnLn2 + logf(Lm);
+        }
     }
 }
 

@@ -973,7 +973,7 @@ template <int D>
 __global__ void __launch_bounds__(attn::kMergeThreads) attn_tile64_merge_kernel(const __grid_constant__ AttnParams p) {
     const int rb = blockIdx.y;
     attn::merge_boundary<D>(
-        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out,
+        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out, p.status,
         [&](int row, const attn::GroupBegin& u, int& node, int& head) {
             const int r_abs = rb * p.rows_per_rb + row;
             node = r_abs / p.G;
@@ -1075,10 +1075,10 @@ mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, co
     const bool no_cuts = p.B == 1 && (long long)p.L * p.Hkv >= p.n_groups && p.whole_groups > 0;
     if (p.n_groups > 1 && !no_cuts) {
         // which units the partition cut is only known on the device (it depends on the prefix lengths)
-        // (a unit is cut by one boundary or a few where there are many: more blocks per boundary then)
-        const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)p.n_rb, (int64_t)p.L * p.B * Hkv >= p.n_groups / 2 ? 4 : 1);
-        if (D == 128) MIRROR_CUDA_OK(mirror_launch_pdl(attn_tile64_merge_kernel<128>, mgrid, dim3(attn::kMergeThreads), 0, stream, p));
-        else MIRROR_CUDA_OK(mirror_launch_pdl(attn_tile64_merge_kernel<64>, mgrid, dim3(attn::kMergeThreads), 0, stream, p));
+        const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)p.n_rb);
+        auto merge = D == 128 ? attn_tile64_merge_kernel<128> : attn_tile64_merge_kernel<64>;
+        MIRROR_CUDA_OK(cudaFuncSetAttribute(merge, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::kMergeSmem));
+        MIRROR_CUDA_OK(mirror_launch_pdl(merge, mgrid, dim3(attn::kMergeThreads), attn::kMergeSmem, stream, p));
         ctx->launches += 1;
         MIRROR_CUDA_OK(cudaGetLastError());
     }

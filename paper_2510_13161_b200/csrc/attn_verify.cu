@@ -980,7 +980,7 @@ __global__ void __launch_bounds__(attn::kMergeThreads) attn_merge_kernel(const _
     const int rb = blockIdx.y / n_str, grp = blockIdx.y % n_str;
     const StreamId id = stream_of(p, rb, grp);
     attn::merge_boundary<D>(
-        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out,
+        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out, p.status,
         [&](int row, const attn::GroupBegin& u, int& node, int& head) {
             const int hl = (id.rt / p.node_tiles) * p.gs + row % p.gs;
             node = (id.rt % p.node_tiles) * p.nodes_tile + row / p.gs;
@@ -1083,9 +1083,9 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         const bool no_cuts = p.never_cut || (p.B == 1 && p.whole_groups > 0);
         if (p.n_groups > 1 && !no_cuts) {
             // which units the partition cut is only known on the device (it depends on the prefix lengths)
-            // (a unit is cut by one boundary or a few where there are many: more blocks per boundary then)
-            const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)(p.n_cta * (p.mode == kSplit ? 1 : 2)), (int64_t)p.L * p.B * Hkv >= p.n_groups / 2 ? 4 : 1);
-            MIRROR_CUDA_OK(mirror_launch_pdl(merge, mgrid, dim3(attn::kMergeThreads), 0, stream, p));
+            const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)(p.n_cta * (p.mode == kSplit ? 1 : 2)));
+            MIRROR_CUDA_OK(cudaFuncSetAttribute(merge, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::kMergeSmem));
+            MIRROR_CUDA_OK(mirror_launch_pdl(merge, mgrid, dim3(attn::kMergeThreads), attn::kMergeSmem, stream, p));
             ctx->launches += 1;
             MIRROR_CUDA_OK(cudaGetLastError());
         }

@@ -63,6 +63,7 @@ struct PairParams {
     const float* h_scale;                   // fp8: [M] scale of each hidden row
     long long wait_limit;                   // SM cycles after which a wait gives up
     int stall_after;                        // test aid: the producers stop after this many stages (-1: never)
+    int w_early;                            // 1: W is older than the kernel ahead: the first stages' weights are requested before the wait
 };
 
 struct Ctrl {
@@ -273,6 +274,19 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
     cluster_sync_all();                 // the other CTA's barriers exist before anything arrives on them
     ptx::tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
+    // The weights of the first stages, while the kernel ahead is still at work (their rows of x follow behind the wait).
+    int n_early = 0;
+    if (p.w_early && warp == 0 && lane == 0 && pair < p.n_units) {
+        int tile, slice, chunk;
+        decode(pair, tile, slice, chunk);
+        const int kb0 = slice * p.kb_per_slice;
+        n_early = min(p.stages, min(n_kb, kb0 + p.kb_per_slice) - kb0);
+        const uint64_t pol_w = p.w_keep ? ptx::policy_evict_normal() : ptx::policy_evict_first();
+        for (int s = 0; s < n_early; ++s) {
+            if (rank == 0) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
+            tma_load_2d_pair(stage_base + s * p.stage_bytes, &tm_w, map_to_rank(&ctrl->full[s], 0), (kb0 + s) * kBK, (tile * 2 + (int)rank) * p.rows_cta, pol_w);
+        }
+    }
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
 
@@ -293,10 +307,11 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                 for (int kb = slice * p.kb_per_slice; kb < kb_end; ++kb) {
                     if (p.stall_after >= 0 && n_issued >= p.stall_after) { ok = false; break; }       // (test aid: neither arms nor copies)
                     if (ctrl->abort || !ptx::mbar_wait(&ctrl->empty[s], ph ^ 1, p.wait_limit)) { fail(p, ctrl, 11); ok = false; break; }
-                    if (rank == 0) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
+                    const bool early = n_issued < n_early;
+                    if (rank == 0 && !early) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
                     const uint32_t bar = map_to_rank(&ctrl->full[s], 0);
                     uint8_t* dst = stage_base + s * p.stage_bytes;
-                    tma_load_2d_pair(dst, &tm_w, bar, kb * kBK, w_row, pol_w);
+                    if (!early) tma_load_2d_pair(dst, &tm_w, bar, kb * kBK, w_row, pol_w);
                     tma_load_2d_pair(dst + p.a_bytes, &tm_h, bar, kb * kBK, h_row, pol_h);
                     ++n_issued;
                     if (++s == p.stages) { s = 0; ph ^= 1; }
@@ -603,6 +618,7 @@ mirror_status pair_shape(const MirrorTuning& tune, int M, int V, int H, PairPara
     if (tune.lm_stages >= 2 && tune.lm_stages < p->stages) p->stages = tune.lm_stages;
     p->wait_limit = tune.wait_limit_cycles;
     p->stall_after = -1;
+    p->w_early = 0;
     if (p->stages < 2) return MIRROR_ERR_SHAPE;
     p->k_slices = 1;
     p->kb_per_slice = H / kBK;
@@ -741,7 +757,7 @@ int mirror_linear_slices(const mirror_ctx* ctx, int M, int N, int K) {
 
 // partial[s][M][N] (fp32) = sum over K slice s of x[M, K] * W[N, K]^T; the caller sums the slices in order.
 mirror_status mirror_linear_partial_launch(mirror_ctx* ctx, const void* x, int M, const void* W, int N, int K, float* partial,
-                                           size_t partial_bytes, cudaStream_t stream, int* k_slices) {
+                                           size_t partial_bytes, cudaStream_t stream, int* k_slices, bool w_early) {
     PairParams p;
     mirror_status st = pair_shape(ctx->tune, M, N, K, &p);
     if (st != MIRROR_OK) return st;
@@ -755,6 +771,7 @@ mirror_status mirror_linear_partial_launch(mirror_ctx* ctx, const void* x, int M
     if (n_pairs > p.n_units) n_pairs = p.n_units;
     if (n_pairs < 1) return MIRROR_ERR_UNSUPPORTED;
     p.w_keep = p.n_chunks > 1;
+    p.w_early = w_early;
     p.logits_out = partial;
     p.status = ctx->d_status;
     st = pair_launch(ctx, false, x, W, p, n_pairs, stream);

@@ -104,10 +104,11 @@ mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int
                                         const float* w_scale = nullptr, const float* h_scale = nullptr,
                                         int topk = 0, void* topk_ws = nullptr, size_t topk_ws_bytes = 0);
 // Plain GEMM on CTA pairs: partial[s][M][N] (fp32) = x[M, K-slice s] * W[N, K-slice s]^T for the *k_slices slices that
-// mirror_linear_slices() picks (1 when the output tiles alone fill the GPU); the caller adds the slices in order.
+// mirror_linear_slices() picks (1 when the output tiles alone fill the GPU); the caller adds the slices in order.  w_early:
+// no kernel that may still be running when the one ahead of this launch begins writes W (see target_layer.cu).
 int mirror_linear_slices(const mirror_ctx* ctx, int M, int N, int K);
 mirror_status mirror_linear_partial_launch(mirror_ctx* ctx, const void* x, int M, const void* W, int N, int K, float* partial,
-                                           size_t partial_bytes, cudaStream_t stream, int* k_slices);
+                                           size_t partial_bytes, cudaStream_t stream, int* k_slices, bool w_early = false);
 // e4m3 cache for mirror_attn_launch: pools, k_new and v_new hold codes; device scales per (layer, KV head), host Q scale.
 struct MirrorAttnFp8 {
     const float* k_scale;

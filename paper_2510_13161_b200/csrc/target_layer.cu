@@ -9,7 +9,9 @@
 // extra trip through HBM: rotary embedding and the split into Q / K / V, residual add + the next RMSNorm, or the
 // SiLU gate.  Activations are stored in bf16 (one rounding per stored tensor), sums are fp32.
 // Every kernel is launched with programmatic stream serialization and waits for the kernel ahead before it touches
-// global memory.
+// what that kernel writes.  The finishing kernels (and the attention's merge) let the kernel behind them be launched at once,
+// so that its set-up and its first weights overlap theirs; the GEMMs and the attention do so only once they have waited
+// themselves: whatever runs behind one of those may rely on everything ahead of it being complete.
 #include <math.h>
 
 #include "mirror_internal.h"
@@ -71,8 +73,8 @@ finish_qkv_kernel(const float* partial, int slices, int M, int Hq, int Hkv, int 
     const int row = blockIdx.x, half = d >> 1, per = half >> 2;
     const int t = blockIdx.y * kQkvThreads + threadIdx.x, head = t / per, f = (t - head * per) * 4;
     const bool in = head < Hq + 2 * Hkv;
-    ptx::grid_dep_wait();
     ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     if (!in) return;
     const int N = (Hq + 2 * Hkv) * d;
     const size_t MN = (size_t)M * N, at = (size_t)row * N + (size_t)head * d + f;
@@ -122,8 +124,8 @@ finish_residual_norm_kernel(const float* partial, int slices, int M, int H, cons
     };
     // behind a projection, the residual stream and the weight are older than the kernel ahead: no need to wait for it
     if (partial) load_early();
-    ptx::grid_dep_wait();
     ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     if (!partial) load_early();
     if (partial) {
         // several slices' loads in flight at a time; the additions stay in slice order
@@ -180,8 +182,8 @@ finish_residual_norm_kernel(const float* partial, int slices, int M, int H, cons
 // Gated MLP finish: act[row, j] = bf16(silu(gate) * up), gate = sum of column j, up = sum of column I + j; four columns a thread.
 __global__ void __launch_bounds__(kFinThreads)
 finish_swiglu_kernel(const float* partial, int slices, int M, int I, __nv_bfloat16* act) {
-    ptx::grid_dep_wait();
     ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const size_t MN = (size_t)M * 2 * I, total = (size_t)M * I;
     for (size_t idx = ((size_t)blockIdx.x * kFinThreads + threadIdx.x) * 4; idx < total; idx += (size_t)gridDim.x * kFinThreads * 4) {
         const size_t row = idx / I, j = idx - row * I;
@@ -396,7 +398,7 @@ mirror_status target_forward_impl(mirror_ctx* ctx, const mirror_target* t, const
         __nv_bfloat16* a_l = (__nv_bfloat16*)attn_out + (size_t)l * q_elems;
         int slices = 0;
         // Q/K/V projection + rotary embedding
-        st = mirror_linear_partial_launch(ctx, h, M, w.w_qkv, Nqkv, H, partial, sc.partial_bytes, s, &slices);
+        st = mirror_linear_partial_launch(ctx, h, M, w.w_qkv, Nqkv, H, partial, sc.partial_bytes, s, &slices, true);
         if (st != MIRROR_OK) return st;
         MIRROR_CUDA_OK(mirror_launch_pdl(finish_qkv_kernel, dim3(M, (Nqkv / 8 + kQkvThreads - 1) / kQkvThreads), dim3(kQkvThreads), 0, s, (const float*)partial, slices, M, Hq, Hkv, d,
                                          (const float2*)cs, q_l, k_l, v_l));
@@ -423,18 +425,18 @@ mirror_status target_forward_impl(mirror_ctx* ctx, const mirror_target* t, const
         }
         if (st != MIRROR_OK) return st;
         // output projection + residual + the MLP's norm
-        st = mirror_linear_partial_launch(ctx, a_l, M, w.w_o, H, Hq * d, partial, sc.partial_bytes, s, &slices);
+        st = mirror_linear_partial_launch(ctx, a_l, M, w.w_o, H, Hq * d, partial, sc.partial_bytes, s, &slices, true);
         if (st != MIRROR_OK) return st;
         MIRROR_CUDA_OK(launch_residual_norm(s, partial, slices, M, H, x_cur, (const __nv_bfloat16*)w.norm_mlp, t->rms_eps, xa, h));
         ctx->launches += 1;
         // gate / up projection + SiLU gate
-        st = mirror_linear_partial_launch(ctx, h, M, w.w_gate_up, 2 * I, H, partial, sc.partial_bytes, s, &slices);
+        st = mirror_linear_partial_launch(ctx, h, M, w.w_gate_up, 2 * I, H, partial, sc.partial_bytes, s, &slices, true);
         if (st != MIRROR_OK) return st;
         MIRROR_CUDA_OK(mirror_launch_pdl(finish_swiglu_kernel, dim3(grid_for((size_t)M * I / 4, ctx->num_sms)), dim3(kFinThreads), 0, s,
                                          (const float*)partial, slices, M, I, act));
         ctx->launches += 1;
         // down projection + residual + the next layer's (or the final) norm
-        st = mirror_linear_partial_launch(ctx, act, M, w.w_down, H, I, partial, sc.partial_bytes, s, &slices);
+        st = mirror_linear_partial_launch(ctx, act, M, w.w_down, H, I, partial, sc.partial_bytes, s, &slices, true);
         if (st != MIRROR_OK) return st;
         const void* g_next = last ? t->norm_final : t->layers[l + 1].norm_attn;
         __nv_bfloat16* x_new = last ? (__nv_bfloat16*)x_out : xb;
