@@ -1,17 +1,28 @@
 // Acceptance, branch selection, emitted tokens and reuse lookup (Sec. 3.1; Eq. 3 / Eq. 10).
 //
-// One thread block per request.  Warps take branches round-robin; lane j of a warp tests the node at
-// depth j+1 of its branch, a ballot gives the number of leading passes (the acceptance operator of
-// Eq. 3 applied to that branch).  Thread 0 then picks the longest branch (lowest index on ties) and the
-// deciding row R.  Greedy mode emits argmax[R]; speculative-sampling mode draws the extra token by an
-// inverse-CDF search over the vocabulary that the whole block cooperates on, all in fp64.
-#include <cooperative_groups.h>
+// Greedy: one thread block per request.  Warps take branches round-robin; lane j of a warp tests the node at depth j+1 of
+// its branch, a ballot gives the number of leading passes (the acceptance operator of Eq. 3 applied to that branch).
+// Thread 0 then picks the longest branch (lowest index on ties) and the deciding row R, and emits argmax[R].
+//
+// Speculative sampling and the rule over the tree draw a token by inverse CDF over the vocabulary, in fp64.  What bounds
+// them is the fp64 exponentials (150 k per pass: 30 us on one SM), so a CLUSTER of 8 or 16 CTAs per request shares the
+// vocabulary: 512-thread CTAs, each warp one contiguous chunk that it reads coalesced.  The chunks' sums go to every CTA
+// through distributed shared memory; all of them scan the same numbers and take the same decisions, one cluster barrier
+// per pass, nothing spins.  The chunk that holds the crossing is then summed again in 16 parts and the part searched, so
+// the search is three short steps.  (One block per request with a contiguous segment per thread: 97-117 us for 8 and 16
+// requests x 128-152 k ids.)
+#include <string.h>
 
 #include "mirror_internal.h"
 
 namespace {
 
-constexpr int kThreads = 1024;
+constexpr int kGreedyThreads = 256;
+constexpr int kThreads = 512;                         // of a CTA of the clusters
+constexpr int kWarps = kThreads / 32;
+constexpr int kMaxCluster = 16;                       // CTAs per request (above 8: opt-in)
+constexpr int kMaxChunks = kMaxCluster * kWarps;
+constexpr int kAhead = 8;                             // ids a thread loads before it works on the first
 
 struct AcceptTreeParams {
     int n, n_branches, gamma;
@@ -46,147 +57,42 @@ __device__ __forceinline__ double warp_excl_scan(double v, int lane, double* tot
     *total = __shfl_sync(0xffffffffu, inc, 31);
     return inc - v;
 }
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
 
-__global__ void __launch_bounds__(kThreads, 1)
-accept_select_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs a) {
-    __shared__ int s_len[MIRROR_MAX_BRANCHES];
-    __shared__ int s_A, s_best, s_R, s_rej_node, s_extra, s_last_pos, s_seg;
-    __shared__ double s_seg_p[kThreads], s_seg_r[kThreads];
-    __shared__ double s_thr, s_excl;
-    __shared__ int s_use_res;
+// What a branch test says about node c (token x, parent row r): the target's probability and the draft's, its uniform.
+struct NodeTest {
+    double p, q, u;
+};
+__device__ __forceinline__ NodeTest node_test(const AcceptTreeParams& tp, const AcceptArgs& a, int b, int c, bool& ok) {
+    NodeTest t = {0.0, 0.0, 0.0};
+    const int x = a.tokens[(size_t)b * tp.n + c];
+    ok = x >= 0 && x < a.V;
+    if (!ok) {
+        if (atomicCAS(a.status, 0, MIRROR_DEV_CHECK) == 0) atomicExch(a.status + 1, 100 + c);   // first error wins
+        return t;
+    }
+    const size_t row = (size_t)b * tp.n + tp.parent[c];
+    t.u = (double)a.u_accept[(size_t)b * tp.n + c];
+    t.q = (double)a.q_probs[((size_t)b * (tp.n - 1) + (c - 1)) * a.V + x];
+    t.p = exp((double)a.logits[row * a.V + x] * a.inv_T - (double)a.lse[row]);
+    return t;
+}
 
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = tp.n, V = a.V;
+// The decision's outputs, by the first threads of one block.
+__device__ __forceinline__ void write_out(const AcceptTreeParams& tp, const AcceptArgs& a, int b, int A, int best, int R, bool have_extra, int extra,
+                                          const unsigned char* path) {
+    const int tid = threadIdx.x, gamma = tp.gamma, n = tp.n;
     const int32_t* tok = a.tokens + (size_t)b * n;
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
-
-    for (int br = warp; br < tp.n_branches; br += kThreads / 32) {
-        const int len = tp.path_len[br];
-        bool pass = true;
-        if (lane < len) {
-            const int c = tp.path[br][lane];
-            const int r = tp.parent[c];
-            const int x = tok[c];
-            if (a.mode == MIRROR_ACCEPT_GREEDY) {
-                pass = (x == a.target_argmax[(size_t)b * n + r]);
-            } else if (x < 0 || x >= V) {
-                pass = false;
-                if (atomicCAS(a.status, 0, MIRROR_DEV_CHECK) == 0) atomicExch(a.status + 1, 100 + c);   // first error wins
-            } else {
-                const size_t row = (size_t)b * n + r;
-                const double p = exp((double)a.logits[row * V + x] * a.inv_T - (double)a.lse[row]);
-                const double lhs = (double)a.u_accept[(size_t)b * n + c] *
-                                   (double)a.q_probs[((size_t)b * (n - 1) + (c - 1)) * V + x];
-                pass = (lhs <= p);
-            }
-        }
-        const unsigned fail = __ballot_sync(0xffffffffu, lane < len && !pass);
-        if (lane == 0) s_len[br] = fail ? (__ffs(fail) - 1) : len;
-    }
-    __syncthreads();
-
-    if (tid == 0) {
-        int A = 0, best = 0;
-        for (int i = 0; i < tp.n_branches; ++i)
-            if (s_len[i] > A) { A = s_len[i]; best = i; }
-        const int R = (A == 0) ? 0 : tp.path[best][A - 1];
-        const bool rejected = tp.n_branches > 0 && A < tp.path_len[best];
-        s_A = A; s_best = best; s_R = R;
-        s_rej_node = rejected ? tp.path[best][A] : -1;
-        s_extra = -1; s_last_pos = -1; s_seg = -1;
-    }
-    __syncthreads();
-    const int A = s_A, best = s_best, R = s_R, rej_node = s_rej_node;
-    const bool have_extra = (rej_node >= 0) || tp.n_branches == 0 || a.emit_bonus != 0;
-
-    if (have_extra) {
-        if (a.mode == MIRROR_ACCEPT_GREEDY) {
-            if (tid == 0) s_extra = a.target_argmax[(size_t)b * n + R];
-        } else {
-            // inverse-CDF draw over the vocabulary from max(0, p - q') (rejection) or p (bonus), fp64
-            const size_t rowR = (size_t)b * n + R;
-            const float* lr = a.logits + rowR * V;
-            const double lseR = (double)a.lse[rowR];
-            const float* qc = (rej_node >= 0) ? a.q_probs + ((size_t)b * (n - 1) + (rej_node - 1)) * V : nullptr;
-            const int S = (V + kThreads - 1) / kThreads;
-            const int v0 = min(tid * S, V), v1 = min(v0 + S, V);
-            double sp = 0.0, sr = 0.0;
-            for (int v = v0; v < v1; ++v) {
-                const double p = exp((double)lr[v] * a.inv_T - lseR);
-                sp += p;
-                if (qc) {
-                    const double res = p - (double)qc[v];
-                    sr += (res > 0.0) ? res : 0.0;
-                }
-            }
-            s_seg_p[tid] = sp;
-            s_seg_r[tid] = sr;
-            __syncthreads();
-            if (warp == 0) {
-                // totals in segment order, then the first segment whose inclusive prefix passes the threshold
-                double lp = 0.0, lres = 0.0;
-                for (int k = 0; k < 32; ++k) { lp += s_seg_p[lane * 32 + k]; lres += s_seg_r[lane * 32 + k]; }
-                double tot_p, tot_r;
-                const double ex_p = warp_excl_scan(lp, lane, &tot_p);
-                const double ex_r = warp_excl_scan(lres, lane, &tot_r);
-                const int use_res = (qc != nullptr) && (tot_r > 0.0);
-                const double thr = (double)a.u_resample[(size_t)b * n + R] * (use_res ? tot_r : tot_p);
-                double run = use_res ? ex_r : ex_p;
-                int found = -1;
-                double found_excl = 0.0;
-                for (int k = 0; k < 32; ++k) {
-                    const double seg = use_res ? s_seg_r[lane * 32 + k] : s_seg_p[lane * 32 + k];
-                    if (found < 0 && run + seg > thr) { found = lane * 32 + k; found_excl = run; }
-                    run += seg;
-                }
-                const unsigned m = __ballot_sync(0xffffffffu, found >= 0);
-                if (m) {
-                    const int src = __ffs(m) - 1;
-                    if (lane == src) { s_seg = found; s_excl = found_excl; }
-                }
-                if (lane == 0) { s_thr = thr; s_use_res = use_res; }
-            }
-            __syncthreads();
-            const int use_res = s_use_res;
-            if (s_seg >= 0) {
-                if (tid == s_seg) {
-                    const double thr = s_thr, excl = s_excl;
-                    double loc = 0.0;
-                    int pick = v1 - 1;
-                    for (int v = v0; v < v1; ++v) {
-                        const double p = exp((double)lr[v] * a.inv_T - lseR);
-                        double mass = p;
-                        if (use_res) { const double res = p - (double)qc[v]; mass = (res > 0.0) ? res : 0.0; }
-                        loc += mass;
-                        if (excl + loc > thr) { pick = v; break; }
-                    }
-                    s_extra = pick;
-                }
-            } else {
-                // rounding left no crossing: take the last id with positive mass
-                int last = -1;
-                for (int v = v0; v < v1; ++v) {
-                    const double p = exp((double)lr[v] * a.inv_T - lseR);
-                    double mass = p;
-                    if (use_res) { const double res = p - (double)qc[v]; mass = (res > 0.0) ? res : 0.0; }
-                    if (mass > 0.0) last = v;
-                }
-                if (last >= 0) atomicMax(&s_last_pos, last);
-                __syncthreads();
-                if (tid == 0) s_extra = s_last_pos;
-            }
-        }
-    }
-    __syncthreads();
-
-    const int gamma = tp.gamma;
     if (tid <= gamma) {
         int e = -1;
-        if (tid < A) e = tok[tp.path[best][tid]];
-        else if (tid == A && have_extra) e = s_extra;
+        if (tid < A) e = tok[path[tid]];
+        else if (tid == A && have_extra) e = extra;
         a.out.emitted[(size_t)b * (gamma + 1) + tid] = e;
-        if (tid < gamma) a.out.accepted_nodes[(size_t)b * gamma + tid] = (tid < A) ? (int)tp.path[best][tid] : -1;
+        if (tid < gamma) a.out.accepted_nodes[(size_t)b * gamma + tid] = (tid < A) ? (int)path[tid] : -1;
     }
     if (tid == 0) {
         a.out.n_accepted[b] = A;
@@ -196,143 +102,318 @@ accept_select_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptAr
         int slot = -1;
         if (have_extra && a.cand_ids)
             for (int k = 0; k < a.n_cand; ++k)
-                if (a.cand_ids[((size_t)b * n + R) * a.n_cand + k] == s_extra) { slot = k; break; }
+                if (a.cand_ids[((size_t)b * n + R) * a.n_cand + k] == extra) { slot = k; break; }
         a.out.reuse_slot[b] = slot;
     }
 }
 
+// Longest branch out of the branches' leading accepts (lowest index on ties), by one thread.
+struct Choice {
+    int A, best, R, rej_node;
+};
+__device__ __forceinline__ Choice choose(const AcceptTreeParams& tp, const int* len) {
+    Choice c = {0, 0, 0, -1};
+    for (int i = 0; i < tp.n_branches; ++i)
+        if (len[i] > c.A) { c.A = len[i]; c.best = i; }
+    if (c.A > 0) c.R = tp.path[c.best][c.A - 1];
+    if (tp.n_branches > 0 && c.A < tp.path_len[c.best]) c.rej_node = tp.path[c.best][c.A];
+    return c;
+}
+
+__global__ void __launch_bounds__(kGreedyThreads)
+accept_greedy_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs a) {
+    __shared__ int s_len[MIRROR_MAX_BRANCHES];
+    __shared__ Choice s_choice;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = tp.n;
+    const int32_t* tok = a.tokens + (size_t)b * n;
+    const int32_t* am = a.target_argmax + (size_t)b * n;
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    for (int br = warp; br < tp.n_branches; br += kGreedyThreads / 32) {
+        const int len = tp.path_len[br];
+        bool pass = true;
+        if (lane < len) {
+            const int c = tp.path[br][lane];
+            pass = tok[c] == am[tp.parent[c]];
+        }
+        const unsigned fail = __ballot_sync(0xffffffffu, lane < len && !pass);
+        if (lane == 0) s_len[br] = fail ? (__ffs(fail) - 1) : len;
+    }
+    __syncthreads();
+    if (tid == 0) s_choice = choose(tp, s_len);
+    __syncthreads();
+    const Choice c = s_choice;
+    const bool have_extra = (c.rej_node >= 0) || tp.n_branches == 0 || a.emit_bonus != 0;
+    write_out(tp, a, b, c.A, c.best, c.R, have_extra, have_extra ? am[c.R] : -1, tp.path[c.best]);
+}
+
+// ---- the cluster's view of the vocabulary --------------------------------------------------------------------------
+__device__ __forceinline__ void cluster_barrier() {       // release / acquire: also of what the CTAs wrote to global memory
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t remote(const void* smem, uint32_t rank) {      // the same object in CTA `rank`
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(ptx::smem_u32(smem)), "r"(rank));
+    return r;
+}
+
+struct DrawShared {
+    double sum[2][2][kMaxChunks];                         // [pass parity][which sum][chunk]: the same in every CTA after a pass
+    double sub[kWarps];
+    int token;                                            // CTA 0's: the drawn token (-1: none yet)
+    int last;                                             // CTA 0's: last id with positive mass
+};
+struct Draw {
+    DrawShared& s;
+    int V, rank, n_cta, chunk_len, lo, hi;                // [lo, hi): this warp's chunk
+    uint32_t pass = 0;
+    __device__ Draw(DrawShared& sh, int vocab) : s(sh), V(vocab) {
+        uint32_t r, n;
+        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+        asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+        rank = (int)r;
+        n_cta = (int)n;
+        const int chunks = n_cta * kWarps;
+        chunk_len = ((V + chunks - 1) / chunks + 31) & ~31;
+        lo = min((rank * kWarps + (int)(threadIdx.x >> 5)) * chunk_len, V);
+        hi = min(lo + chunk_len, V);
+        cluster_barrier();                                // (every CTA of the cluster has started: its shared memory may be written to)
+    }
+    // One pass over the vocabulary: load(v) fetches what id v's masses need, add(v, loaded, x0, x1) adds them to x0 and x1;
+    // eight loads are in flight per thread.  Returns this warp's chunk sums to all CTAs.
+    template <class L, class F>
+    __device__ __forceinline__ void sums(L load, F add) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        double x = 0.0, y = 0.0;
+#pragma unroll 1
+        for (int v0 = lo + lane; v0 < hi; v0 += 32 * kAhead) {
+            decltype(load(0)) in[kAhead];
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k)
+                if (v0 + 32 * k < hi) in[k] = load(v0 + 32 * k);
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k)
+                if (v0 + 32 * k < hi) add(v0 + 32 * k, in[k], x, y);
+        }
+        const double sx = warp_sum(x), sy = warp_sum(y);
+        const uint32_t par = pass & 1;
+        if (lane < n_cta) {
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote(&s.sum[par][0][rank * kWarps + warp], lane)), "d"(sx) : "memory");
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote(&s.sum[par][1][rank * kWarps + warp], lane)), "d"(sy) : "memory");
+        }
+        cluster_barrier();        // (the words of this parity are written again two passes later, behind another barrier)
+        ++pass;
+    }
+    // After sums(): total of one of the two, the same number in every thread of every CTA; *excl: of the chunks before this lane's.
+    __device__ __forceinline__ double total(int which, double* excl = nullptr) const {
+        const int lane = threadIdx.x & 31, per = n_cta * kWarps / 32;
+        const double* c = s.sum[(pass - 1) & 1][which] + lane * per;
+        double mine = 0.0, tot;
+        for (int k = 0; k < per; ++k) mine += c[k];
+        const double e = warp_excl_scan(mine, lane, &tot);
+        if (excl) *excl = e;
+        return tot;
+    }
+    // After sums(): min{v : sum_{w <= v} mass(w) > u * total}, searched in the chunk that holds the crossing; the last id with
+    // positive mass if rounding leaves none.  Collective; the token is valid in CTA 0.
+    template <class F>
+    __device__ __forceinline__ int pick(int which, double u, F mass) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, per = n_cta * kWarps / 32;
+        double excl;
+        const double thr = u * total(which, &excl);
+        const double* c = s.sum[(pass - 1) & 1][which] + lane * per;
+        int found = -1;
+        double found_excl = 0.0;
+        for (int k = 0; k < per; ++k) {
+            if (found < 0 && excl + c[k] > thr) { found = lane * per + k; found_excl = excl; }
+            excl += c[k];
+        }
+        const unsigned any = __ballot_sync(0xffffffffu, found >= 0);
+        if (threadIdx.x == 0 && rank == 0) s.token = s.last = -1;
+        if (any) {
+            const int src = __ffs(any) - 1;
+            found = __shfl_sync(0xffffffffu, found, src);
+            found_excl = __shfl_sync(0xffffffffu, found_excl, src);
+        }
+        cluster_barrier();
+        if (any && found / kWarps == rank) {
+            // the chunk in as many parts as the CTA has warps, then the part with the crossing id by id
+            const int c_lo = min(found * chunk_len, V), c_hi = min(c_lo + chunk_len, V);
+            const int part = (((chunk_len >> 5) + kWarps - 1) / kWarps) << 5;
+            auto part_lo = [&](int w) { return min(c_lo + w * part, c_hi); };
+            double x = 0.0;
+            for (int v = part_lo(warp) + lane; v < part_lo(warp + 1); v += 32) x += mass(v);
+            x = warp_sum(x);
+            if (lane == 0) s.sub[warp] = x;
+            __syncthreads();
+            double tot;
+            const double mine = lane < kWarps ? s.sub[lane] : 0.0;
+            const double before = found_excl + warp_excl_scan(mine, lane, &tot);
+            const unsigned over = __ballot_sync(0xffffffffu, lane < kWarps && before + mine > thr);
+            const unsigned some = __ballot_sync(0xffffffffu, mine > 0.0);
+            // (the parts' sums may round below the chunk's: then the last part with any mass)
+            const int w = over ? __ffs(over) - 1 : some ? 31 - __clz(some) : 0;
+            if (warp == w) {
+                double run = __shfl_sync(0xffffffffu, before, w);
+                int tok = -1, last = part_lo(w);
+                for (int v0 = part_lo(w); v0 < part_lo(w + 1) && tok < 0; v0 += 32) {
+                    const int v = v0 + lane;
+                    const double m = v < part_lo(w + 1) ? mass(v) : 0.0;
+                    double step;
+                    const double e = run + warp_excl_scan(m, lane, &step);
+                    const unsigned hit = __ballot_sync(0xffffffffu, m > 0.0 && e + m > thr);
+                    const unsigned pos = __ballot_sync(0xffffffffu, m > 0.0);
+                    if (hit) tok = v0 + __ffs(hit) - 1;
+                    if (pos) last = v0 + 31 - __clz(pos);
+                    run += step;
+                }
+                if (lane == 0) asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(remote(&s.token, 0)), "r"(tok >= 0 ? tok : last) : "memory");
+            }
+        } else if (!any) {
+            // rounding left the threshold above every cumulative sum (the same in every CTA): the last id with positive mass
+            int last = -1;
+            for (int v = lo + lane; v < hi; v += 32)
+                if (mass(v) > 0.0) last = v;
+            if (last >= 0) asm volatile("red.shared::cluster.max.s32 [%0], %1;" ::"r"(remote(&s.last, 0)), "r"(last) : "memory");
+        }
+        cluster_barrier();
+        return s.token >= 0 ? s.token : s.last;
+    }
+};
+
+__global__ void __launch_bounds__(kThreads, 1)
+accept_spec_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs a) {
+    __shared__ DrawShared s_draw;
+    __shared__ int s_len[MIRROR_MAX_BRANCHES];
+    __shared__ unsigned char s_pass[MIRROR_MAX_NODES];
+    __shared__ Choice s_choice;
+    Draw draw(s_draw, a.V);
+    const int b = blockIdx.x / draw.n_cta, tid = threadIdx.x, n = tp.n, V = a.V;
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    // every CTA evaluates the tests itself, from numbers that are identical in all of them
+    if (tid > 0 && tid < n) {
+        bool ok;
+        const NodeTest t = node_test(tp, a, b, tid, ok);
+        s_pass[tid] = ok && t.u * t.q <= t.p;
+    }
+    __syncthreads();
+    for (int br = tid; br < tp.n_branches; br += kThreads) {
+        int k = 0;
+        while (k < tp.path_len[br] && s_pass[tp.path[br][k]]) ++k;
+        s_len[br] = k;
+    }
+    __syncthreads();
+    if (tid == 0) s_choice = choose(tp, s_len);
+    __syncthreads();
+    const Choice c = s_choice;
+    const bool have_extra = (c.rej_node >= 0) || tp.n_branches == 0 || a.emit_bonus != 0;
+    int extra = -1;
+    if (have_extra) {
+        // inverse-CDF draw from max(0, p - q') (rejection) or p (bonus, or a residual without mass)
+        const size_t row = (size_t)b * n + c.R;
+        const float* lr = a.logits + row * V;
+        const double lse = (double)a.lse[row];
+        const float* qc = c.rej_node >= 0 ? a.q_probs + ((size_t)b * (n - 1) + (c.rej_node - 1)) * V : nullptr;
+        draw.sums([&](int v) { return make_float2(lr[v], qc ? qc[v] : 0.f); },
+                  [&](int, float2 in, double& sp, double& sr) {
+                      const double p = exp((double)in.x * a.inv_T - lse);
+                      sp += p;
+                      sr += fmax(p - (double)in.y, 0.0);        // (without q: not looked at)
+                  });
+        const bool use_res = qc && draw.total(1) > 0.0;
+        extra = draw.pick(use_res ? 1 : 0, (double)a.u_resample[row], [&](int v) {
+            const double p = exp((double)lr[v] * a.inv_T - lse);
+            return use_res ? fmax(p - (double)qc[v], 0.0) : p;
+        });
+    }
+    if (draw.rank == 0) write_out(tp, a, b, c.A, c.best, c.R, have_extra, extra, tp.path[c.best]);
+    cluster_barrier();                                    // no CTA may leave while a peer can still write to its shared memory
+}
+
 // ---------------------------------------------------------------------------------------------------
 // Lossless acceptance over a token tree: sequential multi-round rejection over the siblings of each accepted
-// row (the speculative-sampling rule of Sec. 3.1 applied to sibling sets, for tree drafts).  A cluster of
-// kTreeCluster CTAs per request walks down from the root, every CTA holding one contiguous slice of the vocabulary.
-// At row r the current distribution m starts as the target's p_r; the children of r are tested in node order
+// row (the speculative-sampling rule of Sec. 3.1 applied to sibling sets, for tree drafts).  The walk goes down from the
+// root: at row r the current distribution m starts as the target's p_r; the children of r are tested in node order
 // against m: child c (token x, draft distribution q_c) passes iff u_accept[c] * q_c[x] <= m[x] and the walk moves to
 // c; a child that fails turns m into the normalised residual max(0, m - q_c).  m[v] is either re-evaluated from the
 // logits, the rejected siblings' q rows and their normalisers Z_i, or -- when the caller's workspace has room --
 // kept in fp64 scratch memory (two buffers, so that a residual without mass can be dropped); both follow the
-// definition's operation order per element.  A rejection costs one pass over the vocabulary for Z, the final draw
-// one more; the CTAs exchange their slice sums through distributed shared memory and add them in rank order, so
-// all of them see identical numbers, take identical decisions and stay in step (one hardware cluster barrier per
-// pass, nothing spins).
+// definition's operation order per element.  A rejection costs one pass over the vocabulary for Z, the final draw one
+// more.  What the tests read of p and q themselves is fetched for all nodes at once in front of the walk.
 // ---------------------------------------------------------------------------------------------------
 constexpr int kMaxRejected = MIRROR_MAX_BRANCHES;     // siblings rejected at one row
-constexpr int kTreeCluster = 8;                       // CTAs per request
+struct Loaded {
+    double m;
+    float q;
+};
 
 __global__ void __launch_bounds__(kThreads, 1)
 accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs a) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    __shared__ double s_seg[kThreads];
+    __shared__ DrawShared s_draw;
+    __shared__ NodeTest s_test[MIRROR_MAX_NODES];
+    __shared__ bool s_ok[MIRROR_MAX_NODES];
     __shared__ double s_Z[kMaxRejected];
     __shared__ int s_rej[kMaxRejected];
-    __shared__ int s_path[MIRROR_MAX_DEPTH];
-    __shared__ double s_slice[2];                     // this CTA's slice sum of the current pass (by pass parity): read by peers
-    __shared__ double s_excl;
-    __shared__ int s_pass, s_found, s_extra, s_last;
-
-    const int rank = (int)cluster.block_rank();
-    const int b = blockIdx.x / kTreeCluster, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = tp.n, V = a.V;
+    __shared__ unsigned char s_path[MIRROR_MAX_DEPTH];
+    Draw draw(s_draw, a.V);
+    const int b = blockIdx.x / draw.n_cta, tid = threadIdx.x, n = tp.n, V = a.V;
     const int32_t* tok = a.tokens + (size_t)b * n;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    // this CTA's slice of the vocabulary and this thread's contiguous segment of it
-    const int Vs = (V + kTreeCluster - 1) / kTreeCluster;
-    const int s0 = min(rank * Vs, V), s1 = min(s0 + Vs, V);
-    const int S = (Vs + kThreads - 1) / kThreads;
-    const int v0 = min(s0 + tid * S, s1), v1 = min(v0 + S, s1);
+    if (tid > 0 && tid < n) s_test[tid] = node_test(tp, a, b, tid, s_ok[tid]);
+    __syncthreads();
 
     int r = 0, A = 0, n_rej = 0, n_children = 0;
-    uint32_t pass_no = 0;                          // vocabulary passes so far (identical in every CTA)
     double* const buf0 = a.tree_scratch ? a.tree_scratch + (size_t)b * 2 * V : nullptr;
     double* const buf1 = buf0 ? buf0 + V : nullptr;
     int cur = 0;                                   // buffer that holds the current residual (when n_rej > 0)
     double inv_Z = 1.0;                            // 1 / Z of the last effective rejection
-    // m[v] at row r after the rejections recorded so far
-    auto mass = [&](const float* lr, double lse_r, int v) -> double {
-        if (buf0 && n_rej > 0) return (cur ? buf1 : buf0)[v] * inv_Z;       // (times 1/Z: one rounding away from the quotient)
-        double m = exp((double)lr[v] * a.inv_T - lse_r);
+    // m[v] at row r after the rejections recorded so far, from the logit or (kept) the unnormalised residual
+    auto source = [&](const float* lr, int v) -> double { return buf0 && n_rej > 0 ? (cur ? buf1 : buf0)[v] : (double)lr[v]; };
+    auto raw = [&](double src, double lse_r, int v) -> double {             // before the division by the last Z
+        if (buf0 && n_rej > 0) return src;
+        double m = exp(src * a.inv_T - lse_r);
         for (int i = 0; i < n_rej; ++i) {
-            const double res = m - (double)a.q_probs[((size_t)b * (n - 1) + (s_rej[i] - 1)) * V + v];
-            m = ((res > 0.0) ? res : 0.0) / s_Z[i];
+            if (i > 0) m /= s_Z[i - 1];
+            m = fmax(m - (double)a.q_probs[((size_t)b * (n - 1) + (s_rej[i] - 1)) * V + v], 0.0);
         }
         return m;
     };
-    // Sum of f over the whole vocabulary in a fixed order: per-thread partial sums over this CTA's slice (contiguous
-    // segments, whose sums the inverse-CDF search reuses, or ids interleaved over the threads, which keeps a warp's
-    // loads in one line), warp 0 adds them in order, then every CTA adds the eight slice sums in rank order.
-    // excl_out: sum of the slices before this CTA's.
-    auto cluster_total = [&](auto f, bool contiguous, double* excl_out) -> double {
-        double part = 0.0;
-        if (contiguous) {
-            for (int v = v0; v < v1; ++v) part += f(v);
-        } else {
-            double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
-            int v = s0 + tid;
-            for (; v + 3 * kThreads < s1; v += 4 * kThreads) {
-                p0 += f(v); p1 += f(v + kThreads); p2 += f(v + 2 * kThreads); p3 += f(v + 3 * kThreads);
-            }
-            for (; v < s1; v += kThreads) p0 += f(v);
-            part = (p0 + p1) + (p2 + p3);
-        }
-        s_seg[tid] = part;
-        __syncthreads();
-        const int par = pass_no & 1;
-        if (warp == 0) {
-            double lp = 0.0;
-            for (int k = 0; k < 32; ++k) lp += s_seg[lane * 32 + k];
-            double tot;
-            warp_excl_scan(lp, lane, &tot);
-            if (lane == 0) s_slice[par] = tot;
-        }
-        // (release / acquire at cluster scope: the slice sums and, with scratch memory, the residuals the peers wrote
-        // to global memory in this pass are visible after the barrier.  A buffer of this parity is written again two
-        // passes later, after every peer has passed the barrier in between and so finished reading it.)
-        cluster.sync();
-        double tot = 0.0, excl = 0.0;
-        for (int c = 0; c < kTreeCluster; ++c) {
-            if (c == rank) excl = tot;
-            tot += *cluster.map_shared_rank(&s_slice[par], c);
-        }
-        ++pass_no;
-        if (excl_out) *excl_out = excl;
-        return tot;
+    auto mass = [&](double src, double lse_r, int v) -> double {            // (times 1/Z: one rounding away from the quotient)
+        const double m = raw(src, lse_r, v);
+        return n_rej == 0 ? m : buf0 ? m * inv_Z : m / s_Z[n_rej - 1];
     };
-
+    bool summed = false;                           // the last pass's sums are those of the current m, times Z
+    // (the whole walk is the same in every thread of every CTA)
     for (;;) {
         const size_t row = (size_t)b * n + r;
         const float* lr = a.logits + row * V;
         const double lse_r = (double)a.lse[row];
         n_rej = 0;
         n_children = 0;
+        summed = false;
         int next = -1;
         for (int c = r + 1; c < n; ++c) {
             if (tp.parent[c] != r) continue;
             ++n_children;
-            const float* qc = a.q_probs + ((size_t)b * (n - 1) + (c - 1)) * V;
-            if (tid == 0) {
-                // (every CTA evaluates the test itself, from numbers that are identical in all of them)
-                const int x = tok[c];
-                int pass = 0;
-                if (x < 0 || x >= V) {
-                    if (atomicCAS(a.status, 0, MIRROR_DEV_CHECK) == 0) atomicExch(a.status + 1, 100 + c);   // first error wins
-                } else {
-                    const double lhs = (double)a.u_accept[(size_t)b * n + c] * (double)qc[x];
-                    pass = (lhs <= mass(lr, lse_r, x)) ? 1 : 0;
-                }
-                s_pass = pass;
+            if (s_ok[c]) {
+                const NodeTest t = s_test[c];
+                if (t.u * t.q <= (n_rej == 0 ? t.p : mass(source(lr, tok[c]), lse_r, tok[c]))) { next = c; break; }
             }
-            __syncthreads();
-            if (s_pass) { next = c; break; }
             // rejected: normaliser of the residual (a residual without mass leaves m as it is)
+            const float* qc = a.q_probs + ((size_t)b * (n - 1) + (c - 1)) * V;
             double* const nxt = !buf0 ? nullptr : ((n_rej > 0 && cur == 0) ? buf1 : buf0);      // the buffer not in use
-            const double Z = cluster_total([&](int v) {
-                double res = mass(lr, lse_r, v) - (double)qc[v];
-                res = (res > 0.0) ? res : 0.0;
-                if (nxt) nxt[v] = res;
-                return res;
-            }, false, nullptr);
-            if (Z > 0.0 && n_rej < kMaxRejected) {
+            draw.sums([&](int v) { return Loaded{source(lr, v), qc[v]}; },
+                      [&](int v, const Loaded& in, double& x, double&) {
+                          const double res = fmax(mass(in.m, lse_r, v) - (double)in.q, 0.0);
+                          if (nxt) nxt[v] = res;
+                          x += res;
+                      });
+            const double Z = draw.total(0);
+            summed = Z > 0.0 && n_rej < kMaxRejected;
+            if (summed) {
                 if (tid == 0) { s_rej[n_rej] = c; s_Z[n_rej] = Z; }
                 if (nxt) cur = (nxt == buf1) ? 1 : 0;
                 inv_Z = 1.0 / Z;
@@ -340,105 +421,42 @@ accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
             }
             __syncthreads();
         }
-        if (next >= 0) {
-            if (tid == 0 && A < MIRROR_MAX_DEPTH) s_path[A] = next;
-            ++A;
-            r = next;
-            __syncthreads();
-            if (A >= MIRROR_MAX_DEPTH) { n_children = 0; n_rej = 0; break; }      // (cannot happen: depth <= gamma <= 32)
-            continue;
-        }
-        break;
+        if (next < 0) break;
+        if (tid == 0 && A < MIRROR_MAX_DEPTH) s_path[A] = (unsigned char)next;
+        ++A;
+        r = next;
+        __syncthreads();
+        if (A >= MIRROR_MAX_DEPTH) { n_children = 0; n_rej = 0; summed = false; break; }      // (cannot happen: depth <= gamma <= 32)
     }
     const bool have_extra = (n_children > 0) || a.emit_bonus != 0;
-    if (tid == 0) { s_extra = -1; s_last = -1; s_found = -1; }
-    __syncthreads();
+    int extra = -1;
     if (have_extra) {
-        // inverse-CDF draw from m at row r: the CTA whose slice holds the crossing searches it
         const size_t row = (size_t)b * n + r;
         const float* lr = a.logits + row * V;
         const double lse_r = (double)a.lse[row];
-        double excl_cta = 0.0;
-        const double tot = cluster_total([&](int v) { return mass(lr, lse_r, v); }, true, &excl_cta);
-        const double thr = (double)a.u_resample[row] * tot;
-        if (warp == 0) {
-            double lp = 0.0;
-            for (int k = 0; k < 32; ++k) lp += s_seg[lane * 32 + k];
-            double dummy;
-            double run = excl_cta + warp_excl_scan(lp, lane, &dummy);
-            int found = -1;
-            double found_excl = 0.0;
-            for (int k = 0; k < 32; ++k) {
-                const double seg = s_seg[lane * 32 + k];
-                if (found < 0 && run + seg > thr) { found = lane * 32 + k; found_excl = run; }
-                run += seg;
-            }
-            // only the first CTA whose cumulative sum passes the threshold holds the crossing
-            if (!(excl_cta <= thr)) found = -1;
-            const unsigned mk = __ballot_sync(0xffffffffu, found >= 0);
-            if (mk) {
-                const int src = __ffs(mk) - 1;
-                if (lane == src) { s_found = found; s_excl = found_excl; }
-            }
-        }
-        __syncthreads();
-        if (s_found >= 0 && tid == s_found) {
-            const double excl = s_excl;
-            double loc = 0.0;
-            int pick = v1 - 1;
-            for (int v = v0; v < v1; ++v) {
-                loc += mass(lr, lse_r, v);
-                if (excl + loc > thr) { pick = v; break; }
-            }
-            *cluster.map_shared_rank(&s_extra, 0) = pick;              // hand the token to the CTA that writes the outputs
-        }
-        cluster.sync();
-        if (*cluster.map_shared_rank(&s_extra, 0) < 0) {
-            // rounding left the threshold above every cumulative sum (the same in every CTA): the last id with positive mass
-            int last = -1;
-            for (int v = v0; v < v1; ++v)
-                if (mass(lr, lse_r, v) > 0.0) last = v;
-            if (last >= 0) atomicMax(&s_last, last);
-            cluster.sync();
-            if (rank == 0 && tid == 0) {
-                int best_last = -1;
-                for (int c = 0; c < kTreeCluster; ++c) best_last = max(best_last, *cluster.map_shared_rank(&s_last, c));
-                s_extra = best_last;
-            }
-        }
+        // (a rejection has just added the same masses up: the draw needs them only up to a factor)
+        if (!summed) draw.sums([&](int v) { return source(lr, v); }, [&](int v, double in, double& x, double&) { x += raw(in, lse_r, v); });
+        extra = draw.pick(0, (double)a.u_resample[row], [&](int v) { return raw(source(lr, v), lse_r, v); });
     }
-    __syncthreads();
+    if (draw.rank == 0) {
+        // the lowest-index branch that contains the accepted path
+        int best = 0;
+        for (int i = 0; i < tp.n_branches; ++i) {
+            bool same = tp.path_len[i] >= A;
+            for (int k = 0; k < A && same; ++k) same = (tp.path[i][k] == s_path[k]);
+            if (same) { best = i; break; }
+        }
+        write_out(tp, a, b, A, best, r, have_extra, extra, s_path);
+    }
+    cluster_barrier();                                    // no CTA may leave while a peer can still write to its shared memory
+}
 
-    const int gamma = tp.gamma;
-    if (rank == 0) {
-        if (tid <= gamma) {
-            int e = -1;
-            if (tid < A) e = tok[s_path[tid]];
-            else if (tid == A && have_extra) e = s_extra;
-            a.out.emitted[(size_t)b * (gamma + 1) + tid] = e;
-            if (tid < gamma) a.out.accepted_nodes[(size_t)b * gamma + tid] = (tid < A) ? s_path[tid] : -1;
-        }
-        if (tid == 0) {
-            // the lowest-index branch that contains the accepted path
-            int best = 0;
-            for (int i = 0; i < tp.n_branches; ++i) {
-                bool ok = tp.path_len[i] >= A;
-                for (int k = 0; k < A && ok; ++k) ok = (tp.path[i][k] == s_path[k]);
-                if (ok) { best = i; break; }
-            }
-            a.out.n_accepted[b] = A;
-            a.out.best_branch[b] = best;
-            a.out.decide_row[b] = r;
-            a.out.n_emitted[b] = A + (have_extra ? 1 : 0);
-            int slot = -1;
-            if (have_extra && a.cand_ids)
-                for (int k = 0; k < a.n_cand; ++k)
-                    if (a.cand_ids[((size_t)b * n + r) * a.n_cand + k] == s_extra) { slot = k; break; }
-            a.out.reuse_slot[b] = slot;
-        }
-    }
-    // no CTA may leave while a peer can still read its shared memory
-    cluster.sync();
+// CTAs per request: enough that a warp's chunk is a few steps, no more (a pass ends with a barrier of the cluster); 16 only
+// for few requests: a cluster lives in one GPC, and eight of 16 CTAs do not all fit at once (B = 8: 20.7 us against 16.9 with 8 CTAs).
+int cluster_size(const mirror_ctx* ctx, int batch) {
+    const int V = ctx->desc.vocab;
+    if (V > 65536 && batch * 32 <= ctx->num_sms) return 16;
+    return V > 32768 ? 8 : V > 8192 ? 4 : 2;
 }
 
 }  // namespace
@@ -470,9 +488,13 @@ mirror_status mirror_accept_launch(mirror_ctx* ctx, const mirror_tree* tree, con
     a.out = *out;
     a.tree_scratch = tree_scratch;
     a.status = ctx->d_status;
-    if (in->mode == MIRROR_ACCEPT_SPEC_TREE) {
+    if (in->mode == MIRROR_ACCEPT_GREEDY) {
+        MIRROR_CUDA_OK(mirror_launch_pdl(accept_greedy_kernel, dim3(tree->batch), dim3(kGreedyThreads), 0, stream, tp, a));
+    } else {
+        auto kern = in->mode == MIRROR_ACCEPT_SPEC_TREE ? accept_tree_kernel : accept_spec_kernel;
+        const unsigned n_cta = (unsigned)cluster_size(ctx, tree->batch);
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)tree->batch * kTreeCluster);
+        cfg.gridDim = dim3((unsigned)tree->batch * n_cta);
         cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = 0;
         cfg.stream = stream;
@@ -480,13 +502,14 @@ mirror_status mirror_accept_launch(mirror_ctx* ctx, const mirror_tree* tree, con
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = kTreeCluster;
+        attr[1].val.clusterDim.x = n_cta;
         attr[1].val.clusterDim.y = 1;
         attr[1].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        MIRROR_CUDA_OK(cudaLaunchKernelEx(&cfg, accept_tree_kernel, tp, a));
-    } else MIRROR_CUDA_OK(mirror_launch_pdl(accept_select_kernel, dim3(tree->batch), dim3(kThreads), 0, stream, tp, a));
+        if (n_cta > 8) MIRROR_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        MIRROR_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, tp, a));
+    }
     ctx->launches += 1;
     MIRROR_CUDA_OK(cudaGetLastError());
     return MIRROR_OK;
