@@ -1,5 +1,5 @@
-// Branch-tree attention on 64-token key tiles: the kernel of the 8-bit (e4m3) cache and of mirror_target_forward's layers
-// (attn_verify.cu has the faster kernel of every other bf16 call, and the problem's definition).
+// Branch-tree attention on 64-token key tiles: the kernel of mirror_target_forward's layers, over a bf16 or an 8-bit (e4m3)
+// cache (attn_verify.cu has the faster kernel of every other call, and the problem's definition).
 //
 // Why the layer stack stays here: a stack of layers amplifies any difference in rounding (an attention output that differs
 // by 0.2%, or a projection whose fp32 sums are added in another order, differs by 3.5% after 48 random layers), so
@@ -45,6 +45,7 @@
 namespace {
 
 using attn::pack_bf16;
+using attn::pack_e4m3x4;
 
 constexpr int kSoftmaxWarps = 8;
 constexpr int kThreads = 32 * (4 + kSoftmaxWarps);   // K producer, Q K^T issuer, P V issuer, softmax pairs, V producer
@@ -139,30 +140,12 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
     return m;
 }
-// Four fp32 values as e4m3 codes in one word (element 0 in the lowest byte, as the tensor core reads an 8-bit operand);
-// values beyond +-448 saturate.
-__device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float d) {
-    uint32_t r;
-    asm("{\n\t.reg .b16 lo, hi;\n\t"
-        "cvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n\t"
-        "cvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n\t"
-        "mov.b32 %0, {lo, hi};\n\t}"
-        : "=r"(r) : "f"(a), "f"(b), "f"(c), "f"(d));
-    return r;
-}
 // tcgen05.mma with both operands in shared memory (descriptor halves) or A in tensor memory; F8 selects e4m3 inputs.
 template <bool F8>
 __device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                         uint32_t idesc, uint32_t accumulate) {
     if constexpr (F8) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-            "mov.b64 da, {%1, %2};\n\t"
-            "mov.b64 db, {%3, %4};\n\t"
-            "setp.ne.b32 p, %6, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], da, db, %5, p;\n\t}"
-            ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
-            : "memory");
+        attn::umma_e4m3_lohi(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, accumulate);
     } else {
         ptx::umma_f16_lohi(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, accumulate);
     }
@@ -182,11 +165,6 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32
         ptx::umma_f16_tmem_a(d_tmem, a_tmem, b_lo, b_hi, idesc, accumulate);
     }
 }
-// Instruction descriptor: e4m3 x e4m3 -> fp32 (format codes 0), tile M x N.
-__device__ __forceinline__ uint32_t umma_idesc_e4m3(int M, int N) {
-    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
 // Shared-memory operand tiles are [64-column half][row][128 B] with the 128-byte swizzle: the 16-byte chunk
 // index is XORed with (row % 8).  A half of Q or P holds 128 rows (16 KB), a half of a K/V stage 64 tokens (8 KB).
 constexpr int kStageSlots = 4;                      // slots per ring stage
@@ -553,7 +531,7 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
             // one instruction per ~100 cycles and holds it up meanwhile), so what it does between two chains is kept
             // short: ring stage, buffer and their parities are running counters, and the descriptor of a full tile is
             // made once.
-            const uint32_t idesc_full = F8 ? umma_idesc_e4m3(kRows, kTileTok) : ptx::umma_idesc_bf16(kRows, kTileTok);
+            const uint32_t idesc_full = F8 ? attn::umma_idesc_plain(kRows, kTileTok) : ptx::umma_idesc_bf16(kRows, kTileTok);
             uint32_t seg = 0;
             uint32_t st = 0, k_par = 0;            // K ring stage of the next tile and the parity its data completes
             uint32_t sb = 0, s_par = 1;            // S buffer of the next tile and the parity that says it is free
@@ -580,7 +558,7 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
                     const bool s_next = ptx::mbar_try_wait(&ctrl->s_free[sb_n], s_par_n);
                     if (rem_t > 0) {                                                   // (a pair's second tile may be empty)
                         const uint32_t idesc = rem_t >= kStageSlots ? idesc_full
-                                             : (F8 ? umma_idesc_e4m3(kRows, rem_t * kSlotTok) : ptx::umma_idesc_bf16(kRows, rem_t * kSlotTok));
+                                             : (F8 ? attn::umma_idesc_plain(kRows, rem_t * kSlotTok) : ptx::umma_idesc_bf16(kRows, rem_t * kSlotTok));
                         const uint32_t kb = k_lo + st * (uint32_t)(C::kStageBytes >> 4);
                         const uint32_t d = tmem_base + sb * (uint32_t)kTileTok;
 #pragma unroll
@@ -607,7 +585,7 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
         if (lane == 0) {
             const uint32_t hi_v = ptx::umma_desc_hi_sw128(C::kGroupStride);                // the two 8-token groups of a slot
             const uint32_t v_lo = ptx::umma_desc_lo(ptx::smem_u32(sV), 1024);             // MN-major: LBO = next 64-column atom
-            const uint32_t idesc_pv = (F8 ? umma_idesc_e4m3(kRows, D) : ptx::umma_idesc_bf16(kRows, D)) | (1u << 16);   // B operand MN-major
+            const uint32_t idesc_pv = (F8 ? attn::umma_idesc_plain(kRows, D) : ptx::umma_idesc_bf16(kRows, D)) | (1u << 16);   // B operand MN-major
             uint32_t it = 0;
             int st = 0, sb = 0;                     // V ring stage and S / P buffer of the next tile, with their parities
             uint32_t v_par = 0, p_par = 0;

@@ -1,4 +1,4 @@
-// Branch-tree attention of the verify step over a bf16 cache: every tree node (kappa x gamma draft tokens + the root)
+// Branch-tree attention of the verify step: every tree node (kappa x gamma draft tokens + the root)
 // attends to the paged KV cache of the verified prefix and to the tree's own K/V under the branch-causal mask (node i
 // sees tree token j iff j is i or an ancestor of i), for all layers.
 //
@@ -26,6 +26,10 @@
 //               over the first half of S's columns as bf16.  The row's offset is the maximum of the first tile in which
 //               it sees anything; it moves only when a half tile's sum of P passes 2^80 (that half is then redone from
 //               S, which is still there), and is carried exactly through the sum and the division.
+// e4m3 cache (d = 128; F8): Q K^T multiplies codes (kind::f8f6f4, Q divided by its scale and rounded when it is staged), but P V
+// does not: four more warps (12..15) widen each V tile to f16, exactly, and P is f16.  In an 8-bit P V, P as e4m3 costs 2.6% of
+// the output (root mean square) and its own conversions; the tensor cores have the time, the softmax sets the pace.  K and
+// V then have rings of their own, and the widening warps stage the next unit's Q in passing, eight rows per V tile.
 // TMEM: S0 | S1 (128 columns each) | O0 | O1 (d columns each) = 512 columns at d = 128.
 // Every mbarrier wait is bounded; on expiry the kernel records MIRROR_DEV_TIMEOUT and unwinds.
 //
@@ -37,7 +41,8 @@
 // line on purpose; unrolled, the same step took 4900 cycles, most of them in instruction fetch.  Tried and neutral: a
 // third of the exponentials as polynomials on the FMA pipe, and turns between the softmax warps of a scheduler.
 // Measured (bf16, d = 128, tiles of 16-token pages): 80 layers x 16 requests x 520 rows 25.0 -> 20.5 ms at the same
-// power; 64 layers x 32768 tokens x 264 rows 4.0 -> 3.4 ms.
+// power; 64 layers x 32768 tokens x 264 rows 4.0 -> 3.4 ms; e4m3 cache, 64 layers x 4 x 4096..16384 tokens x 136 rows (64-token
+// tiles with e4m3 P before): 2.25 -> 1.85 ms.
 #include <math.h>
 #include <string.h>
 
@@ -51,12 +56,16 @@ using attn::pack_bf16;
 using attn::slot_mask;
 
 constexpr int kThreads = 384;
+constexpr int kConvWarps = 4;                       // (e4m3 cache) warps 12..15
+constexpr int kWideStages = 2;                      // (e4m3 cache) V tiles widened to f16
 constexpr int kSlotTok = kAttnSlotTok;
 constexpr int kTileSlots = 8;
 constexpr int kTileTok = kSlotTok * kTileSlots;     // 128
 constexpr int kRows = 128;                          // UMMA M: rows of a stream
 constexpr int kMaxStages = 10;
-constexpr float kSumLimit = 1.2089258196146292e24f; // 2^80: no P of such a half tile overflows bf16, no sum of them fp32
+// A half tile whose sum of P stays below this is as it should be: no P of it overflows its 16-bit format (bf16: 2^80, so that
+// no sum of them overflows fp32 either; f16, of the e4m3 cache: 2^14).
+template <bool F8> constexpr float kSumLimit = F8 ? 16384.f : 1.2089258196146292e24f;
 constexpr int kTmemCols = 512;
 constexpr int kTmemO = 2 * kTileTok;
 constexpr int kCtrlBytes = 512;
@@ -83,6 +92,12 @@ struct AttnParams {
     const int32_t* page_table;
     const int32_t* prefix_len;
     const __nv_bfloat16* v_pool;
+    // e4m3 cache: pools, k_new and v_new hold e4m3 codes; a code times its (layer, KV head) scale is the value.  Q stays bf16
+    // in memory; its operand is e4m3(q / q_scale), rounded when it is staged.
+    const __nv_bfloat16* q;
+    const float* k_scale;                 // [L, Hkv]
+    const float* v_scale;                 // [L, Hkv]
+    float q_scale;
     __nv_bfloat16* out;
     float* lse_out;
     float* partial;                       // [grid][2 slots][2 streams][D + 4][128]
@@ -164,8 +179,9 @@ __device__ __noinline__ Segment next_segment(const Segment& s, int left, const A
 
 // ---- barriers ------------------------------------------------------------------------------------------------
 struct Ctrl {
-    uint64_t full[kMaxStages], empty[kMaxStages];       // K/V ring
-    uint64_t q_full[2], q_empty[2];
+    uint64_t full[kMaxStages], empty[kMaxStages];       // K/V ring (e4m3: the first half K, the second V, rings of their own)
+    uint64_t wide_full[kWideStages], wide_empty[kWideStages];       // e4m3: V tiles widened to f16
+    uint64_t q_full[4], q_empty[4];                     // (as many as Q buffers)
     uint64_t s_full[2], p_full[2][2], o_full[2];        // per stream (P: per half of the tile)
     uint64_t pv_half[2];                                // P V of a tile's first half is through
     uint64_t turn[2];                                   // the issuing warps take turns
@@ -354,8 +370,9 @@ __device__ __forceinline__ void tmem_ld_wait16(uint32_t (&r)[16]) {
                  :: "memory");
 }
 
-// 32 scores of a row -> 16 words of bf16 P = exp2(s * c - offset); the fp32 values are added to four running sums (two
-// packed pairs).
+// 32 scores of a row -> 16 words of bf16 (F8: f16) P = exp2(s * c - offset); the fp32 values are added to four running sums
+// (two packed pairs).
+template <bool F8>
 __device__ __forceinline__ void exp_chunk(const uint32_t (&r)[32], uint64_t sc2, uint64_t neg_off2, uint32_t* pk, uint64_t& s0, uint64_t& s1) {
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
@@ -365,19 +382,26 @@ __device__ __forceinline__ void exp_chunk(const uint32_t (&r)[32], uint64_t sc2,
         b = ptx::ex2_approx(b);
         if (j & 1) s1 = add2(s1, pack2(a, b));
         else s0 = add2(s0, pack2(a, b));
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(b), "f"(a));
+        if (F8) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(b), "f"(a));
+        else asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(b), "f"(a));
     }
 }
 
-template <int D>
+template <int D, bool F8>
 struct Cfg {
-    static constexpr int kRowBytes = D * 2;                        // one token's K (or V) row of one head
+    static_assert(!F8 || D == 128, "an e4m3 row must fill a 128-byte swizzle row");
+    static constexpr int kThreads = ::kThreads + (F8 ? 32 * kConvWarps : 0);
+    static constexpr int kRowBytes = D * (F8 ? 1 : 2);             // one token's K (or V) row of one head
     static constexpr int kHalves = kRowBytes / 128;
     static constexpr int kSlotBytes = kHalves * kSlotTok * 128;    // one slot of K or V = one TMA box
     static constexpr int kGroupStride = kHalves * 1024;            // between the 8-token groups of one half
     static constexpr int kStageBytes = kTileSlots * kSlotBytes;    // one K or V tile
     static constexpr int kQHalfBytes = kRows * 128;                // one 64-column half of a Q buffer
     static constexpr int kQBytes = kHalves * kQHalfBytes;
+    static constexpr int kVHalves = D * 2 / 128;                   // V as P V reads it: 16 bits per element
+    static constexpr int kVSlotBytes = kVHalves * kSlotTok * 128;
+    static constexpr int kWideBytes = F8 ? kTileSlots * kVSlotBytes : 0;        // one V tile widened to f16
+    static constexpr size_t kFixedBytes = kWideStages * kWideBytes + kCtrlBytes;           // of shared memory, beside Q buffers and ring
 };
 
 // Scores of tokens that the row does not see become -inf, in TMEM: a pass of its own over a unit's last tiles, so that the
@@ -429,14 +453,62 @@ __device__ __noinline__ float2 move_offset(uint32_t s_addr, uint32_t o_addr, int
     return make_float2(next, alpha);
 }
 
-template <int D>
-__global__ void __launch_bounds__(kThreads, 1)
+// Q as e4m3 codes.  The code is that of the correctly rounded quotient x / q_scale: the product with the rounded reciprocal is
+// corrected twice by its exact remainder (Markstein 1990), without a branch.  That holds for scales in 2^[-60, 60] and
+// numerators clamped to where the code saturates anyway (448; NaN stays NaN); other scales divide.
+struct QScale {
+    float s, inv, lim;
+    bool usual;
+    __device__ explicit QScale(float scale) : s(scale), inv(1.f / scale), lim(1000.f * scale), usual(scale >= 0x1p-60f && scale <= 0x1p60f) {}
+    __device__ __forceinline__ float quotient(float x) const {
+        asm("min.NaN.f32 %0, %0, %1;\n\tmax.NaN.f32 %0, %0, %2;" : "+f"(x) : "f"(lim), "f"(-lim));
+        float t = x * inv;
+        t = fmaf(fmaf(-t, s, x), inv, t);
+        return fmaf(fmaf(-t, s, x), inv, t);
+    }
+};
+__device__ __noinline__ uint32_t unusual_codes(uint2 v, float s) {
+    return attn::pack_e4m3x4(__fdiv_rn(__uint_as_float(v.x << 16), s), __fdiv_rn(__uint_as_float(v.x & 0xffff0000u), s),
+                             __fdiv_rn(__uint_as_float(v.y << 16), s), __fdiv_rn(__uint_as_float(v.y & 0xffff0000u), s));
+}
+// One row, four elements per lane, into the K-major operand tile `q` ([row][128 B], 128-byte swizzle).
+__device__ __forceinline__ void store_q_row(uint8_t* q, int row, uint2 v, const QScale& qs) {
+    const int lane = threadIdx.x & 31;
+    uint32_t code;
+    if (qs.usual)
+        code = attn::pack_e4m3x4(qs.quotient(__uint_as_float(v.x << 16)), qs.quotient(__uint_as_float(v.x & 0xffff0000u)),
+                                 qs.quotient(__uint_as_float(v.y << 16)), qs.quotient(__uint_as_float(v.y & 0xffff0000u)));
+    else
+        code = unusual_codes(v, qs.s);
+    *reinterpret_cast<uint32_t*>(q + row * 128 + (((lane >> 2) ^ (row & 7)) << 4) + (lane & 3) * 4) = code;
+}
+__device__ __forceinline__ const __nv_bfloat16* row_of_lane(const __nv_bfloat16* qrow, int r) {
+    return (const __nv_bfloat16*)__shfl_sync(0xffffffffu, (unsigned long long)qrow, r);
+}
+// Four e4m3 codes as four f16 (exact).
+__device__ __forceinline__ uint2 widen4(uint32_t w) {
+    uint2 r;
+    asm("{\n\t.reg .b16 lo, hi;\n\t"
+        "mov.b32 {lo, hi}, %2;\n\t"
+        "cvt.rn.f16x2.e4m3x2 %0, lo;\n\t"
+        "cvt.rn.f16x2.e4m3x2 %1, hi;\n\t}"
+        : "=r"(r.x), "=r"(r.y) : "r"(w));
+    return r;
+}
+
+template <int D, bool F8>
+__global__ void __launch_bounds__(Cfg<D, F8>::kThreads, 1)
 attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ AttnTree tree, const __grid_constant__ AttnParams p,
                    const int n_stages) {
-    using C = Cfg<D>;
+    using C = Cfg<D, F8>;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t* sQ = smem;                                             // [2] Q buffers: per stream, or (split) of alternating units
-    uint8_t* ring = sQ + 2 * C::kQBytes;                            // [n_stages] K or V tiles
+    // Q buffers: per stream, or (split) of alternating units; e4m3: two per stream, or (split) two
+    uint8_t* sQ = smem;
+    const int q_bufs = F8 && p.mode != kSplit ? 4 : 2;
+    uint8_t* wide = sQ + q_bufs * C::kQBytes;                            // [2] V tiles widened to f16 (e4m3 cache)
+    uint8_t* ring = wide + kWideStages * C::kWideBytes;             // [n_stages] K or V tiles
+    // stages of a ring: one that K and V share, or (e4m3) two of half the stages
+    const int ring_n = F8 ? n_stages >> 1 : n_stages;
     Ctrl* ctrl = (Ctrl*)(ring + (size_t)n_stages * C::kStageBytes);
     float* xch = (float*)((uint8_t*)ctrl + kCtrlBytes);             // split: [128 rows][2 streams][offset, sum]
     int* cumT = (int*)(xch + (p.mode == kSplit ? kRows * 4 : 0));   // [B+1] tiles per unit, prefix-summed over the requests
@@ -451,23 +523,26 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
     // stream is still running; nothing of global memory is touched before it has completed)
     if (tid == 0) {
         const uint32_t readers = shared_kv ? 2 : 1;                 // issuing warps that read a K/V stage
-        for (int s = 0; s < n_stages; ++s) { ptx::mbar_init(&ctrl->full[s], 1); ptx::mbar_init(&ctrl->empty[s], readers); }
+        for (int s = 0; s < n_stages; ++s) { ptx::mbar_init(&ctrl->full[s], 1); ptx::mbar_init(&ctrl->empty[s], F8 && s >= ring_n ? kConvWarps : readers); }
+        if (F8)
+            for (int s = 0; s < kWideStages; ++s) { ptx::mbar_init(&ctrl->wide_full[s], kConvWarps); ptx::mbar_init(&ctrl->wide_empty[s], readers); }
         for (int g = 0; g < 2; ++g) {
-            ptx::mbar_init(&ctrl->q_full[g], 1); ptx::mbar_init(&ctrl->q_empty[g], split ? 2 : 1);
             ptx::mbar_init(&ctrl->s_full[g], 1); ptx::mbar_init(&ctrl->p_full[g][0], 4); ptx::mbar_init(&ctrl->p_full[g][1], 4);
             ptx::mbar_init(&ctrl->o_full[g], 1); ptx::mbar_init(&ctrl->turn[g], 1); ptx::mbar_init(&ctrl->pv_half[g], 1);
         }
+        for (int s = 0; s < q_bufs; ++s) { ptx::mbar_init(&ctrl->q_full[s], !F8 ? 1 : split ? 8 : 4); ptx::mbar_init(&ctrl->q_empty[s], split ? 2 : 1); }
         for (int s = 0; s < 4; ++s) ptx::mbar_init(&ctrl->pair[s], 2);
         ctrl->abort = 0;
         ctrl->status = p.status;
         ctrl->wait_limit = p.wait_limit;
         ptx::fence_mbar_init();
-        ptx::prefetch_tmap(&tm.k); ptx::prefetch_tmap(&tm.v); ptx::prefetch_tmap(&tm.kn); ptx::prefetch_tmap(&tm.vn); ptx::prefetch_tmap(&tm.q);
+        ptx::prefetch_tmap(&tm.k); ptx::prefetch_tmap(&tm.v); ptx::prefetch_tmap(&tm.kn); ptx::prefetch_tmap(&tm.vn);
+        if (!F8) ptx::prefetch_tmap(&tm.q);
     }
     // Rows that the Q copies do not fill are zeros: the tensor cores multiply 128 rows whatever the tile holds, and under the
     // power limit zeros are cheaper than whatever lies there.
     const int pad = kRows - p.gs * p.nodes_tile;
-    for (int i = tid; i < 2 * C::kHalves * pad * 8; i += kThreads) {
+    for (int i = tid; i < q_bufs * C::kHalves * pad * 8; i += C::kThreads) {
         const int half = i / (pad * 8), c = i - half * pad * 8;
         *reinterpret_cast<uint4*>(sQ + half * C::kQHalfBytes + p.gs * p.nodes_tile * 128 + c * 16) = make_uint4(0, 0, 0, 0);
     }
@@ -505,7 +580,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             // ======================================================================= K and V producers
             // Ring order (first use by the issuing warps): K of step 0, then per step V, next K -- of stream 0 and, when the
             // streams have K/V tiles of their own, of stream 1.  Both warps walk that order; each fills its own stages.
-            // (one copy of the code for both)
+            // (one copy of the code for both.  e4m3: V has a ring of its own, in front of the warps that widen it.)
             {
                 const bool V = warp == 3;
                 const CUtensorMap* const map = V ? &tm.v : &tm.k;
@@ -516,8 +591,12 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                 bool ok = true, stop = false;
                 auto skip = [&](int n) {
                     st += (uint32_t)n;
-                    if (st >= (uint32_t)n_stages) { st -= (uint32_t)n_stages; ph ^= 1; }
+                    if (st >= (uint32_t)ring_n) { st -= (uint32_t)ring_n; ph ^= 1; }
                 };
+                auto pass = [&](int n) {                           // stages that the other producer fills
+                    if (!F8) skip(n);
+                };
+                const int st0 = F8 && V ? ring_n : 0;              // the ring's first stage
                 // page ids of a tile, one per lane (0..7), fetched a tile ahead
                 int pg = 0, pg_t = -1, pg_next = 0;
                 auto fetch = [&](int tt) -> int {
@@ -531,9 +610,9 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                         pg_next = fetch(tt + 1);
                         pg_t = tt;
                     }
-                    if (!wait_bar(ctrl, &ctrl->empty[st], ph, 10)) { ok = false; return; }
-                    uint8_t* const dst = ring + (size_t)st * C::kStageBytes;
-                    uint64_t* const bar = &ctrl->full[st];
+                    if (!wait_bar(ctrl, &ctrl->empty[st0 + st], ph, 10)) { ok = false; return; }
+                    uint8_t* const dst = ring + (size_t)(st0 + st) * C::kStageBytes;
+                    uint64_t* const bar = &ctrl->full[st0 + st];
                     const int head = sg.g * p.heads_per_unit + stream_of(p, rb, g).head_off;
                     const int sl0 = tt * kTileSlots, n_sl = min(kTileSlots, sg.slots_all - sl0);
                     if (pg < 0 || pg >= p.num_pages) { dev_check(p, 400); pg = 0; }
@@ -614,7 +693,10 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     const uint8_t* src = (const uint8_t*)p.v_pool + ((size_t)(s.layer * p.layer_pages + page) * p.Hkv + s.g * p.heads_per_unit) * (size_t)(kSlotTok * C::kRowBytes);
                     for (int c = lane; c < p.heads_per_unit * kSlotTok * C::kRowBytes / 128; c += 32) ptx::prefetch_l2(src + c * 128);
                 };
-                if (V) { load_q(sg, 0); prefetch_ragged(sg); }
+                if (V) {
+                    if (!F8) load_q(sg, 0);
+                    prefetch_ragged(sg);
+                }
                 uint32_t n_seg = 0;
                 int prev = 0;                                      // K: stages of the step before (0, 1 or, with K/V of their own, 2)
                 // tiles of the step at t: 1, or (split) up to 2
@@ -629,16 +711,16 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                         Segment nx = sg;
                         if (seg_end && more) nx = next_segment(sg, left - w, p, s_len);
                         const bool next_two = more && !shared_kv && (!split || nx.t_last - (seg_end ? 0 : t + w) > 1);
-                        if (prev == 0) { skip(1 + (two ? 1 : 0)); prev = 1; }   // K of the first step
+                        if (prev == 0) { pass(1 + (two ? 1 : 0)); prev = 1; }   // K of the first step
 #pragma unroll 1
                         for (int g = 0; g < (two ? 2 : 1) && ok; ++g) {
                             emit(split ? t + g : t, g);
-                            if (g == 0) skip(more ? 1 : 0);
+                            if (g == 0) pass(more ? 1 : 0);
                         }
                         if (!ok) break;
-                        skip(next_two ? 1 : 0);
+                        pass(next_two ? 1 : 0);
                         if (seg_end && more) {
-                            load_q(nx, ++n_seg);
+                            if (!F8) load_q(nx, ++n_seg);
                             prefetch_ragged(nx);
                             sg = nx;
                             pg_t = -1;
@@ -649,7 +731,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     } else {
 #pragma unroll 1
                         for (int g = 0; g < 2 && ok; ++g) {
-                            skip(prev > g ? 1 : 0);                // V of the step before
+                            pass(prev > g ? 1 : 0);                // V of the step before
                             if (g == 0 || two) emit(split ? t + g : t, g);
                         }
                         if (!ok) break;
@@ -665,7 +747,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                 }
                 if (!ok && !stop) {
                     // let copies already in flight land before the CTA's shared memory goes away (every stage's last fill)
-                    for (int s = 0; s < n_stages; ++s) ptx::mbar_wait(&ctrl->full[s], (s < (int)st ? ph : ph ^ 1) ^ 1, 20000000ll);
+                    for (int s = 0; s < ring_n; ++s) ptx::mbar_wait(&ctrl->full[st0 + s], (s < (int)st ? ph : ph ^ 1) ^ 1, 20000000ll);
                 }
             }
         } else if (n_tiles > 0) {
@@ -674,26 +756,41 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             // tensor cores' queue covers, so one warp for both left them idle a third of the time.  They take turns issuing:
             // left to themselves the two streams fall into step, both in their softmax and then both waiting.  The whole
             // warp walks the schedule and one elected lane issues, which keeps descriptors in uniform registers.
-            const uint32_t hi_q = ptx::umma_desc_hi_sw128(1024), hi_kv = ptx::umma_desc_hi_sw128(C::kGroupStride);
+            const uint32_t hi_q = ptx::umma_desc_hi_sw128(1024), hi_k = ptx::umma_desc_hi_sw128(C::kGroupStride),
+                           hi_v = ptx::umma_desc_hi_sw128(C::kVHalves * 1024);
             const uint32_t q_lo = ptx::umma_desc_lo(ptx::smem_u32(sQ), 16);
             const uint32_t k_lo = ptx::umma_desc_lo(ptx::smem_u32(ring), 16);
-            const uint32_t v_lo = ptx::umma_desc_lo(ptx::smem_u32(ring), 1024);            // MN-major: LBO = next 64-column atom
-            const uint32_t idesc_pv = ptx::umma_idesc_bf16(kRows, D) | (1u << 16);         // B operand MN-major
+            const uint32_t v_lo = ptx::umma_desc_lo(ptx::smem_u32(F8 ? wide : ring), 1024);                    // MN-major: LBO = next 64-column atom
+            const uint32_t idesc_pv = (F8 ? attn::umma_idesc_plain(kRows, D) : ptx::umma_idesc_bf16(kRows, D)) | (1u << 16);      // B operand MN-major
             const uint32_t q_half = (uint32_t)(C::kQHalfBytes >> 4), q_buf = (uint32_t)(C::kQBytes >> 4);
             bool ok = true;
             uint32_t st = 0, ph = 0;                 // next ring stage
             uint32_t p_par = 0;                      // parity of the next P
-            auto skip = [&](int n) {                 // stages that only the other issuer reads
+            uint32_t wst = 0, wph = 0;               // e4m3: next widened V tile
+            auto skip_k = [&](int n) {               // stages that only the other issuer reads
                 st += (uint32_t)n;
-                if (st >= (uint32_t)n_stages) { st -= (uint32_t)n_stages; ph ^= 1; }
+                if (st >= (uint32_t)ring_n) { st -= (uint32_t)ring_n; ph ^= 1; }
+            };
+            auto skip_v = [&](int n) {
+                if (!F8) return skip_k(n);
+                wst += (uint32_t)n;
+                if (wst >= kWideStages) { wst -= kWideStages; wph ^= 1; }
             };
             auto wait = [&](uint64_t* bar, uint32_t parity, int where) { ok = ok && wait_bar(ctrl, bar, parity, where); };
-            auto take = [&]() -> uint32_t {          // wait for the next stage of the ring
+            auto take_k = [&]() -> uint32_t {        // wait for the next stage of the ring
                 const uint32_t s = st;
                 wait(&ctrl->full[s], ph, 21);
-                skip(1);
+                skip_k(1);
                 return s;
             };
+            auto take_v = [&]() -> uint32_t {
+                if (!F8) return take_k();
+                const uint32_t s = wst;
+                wait(&ctrl->wide_full[s], wph, 25);
+                skip_v(1);
+                return s;
+            };
+            uint64_t* const v_empty = F8 ? ctrl->wide_empty : ctrl->empty;
             // A cursor over the steps of a segment: tiles and slots from the step's first tile to the segment's (unit's) end.
             struct Cursor {
                 int tiles, slots;
@@ -710,22 +807,22 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
 #pragma unroll 1
             while (ok) {
                 // (tiles of its own: the ring holds, per step, V of stream 0, the next K of stream 0, V and next K of stream 1)
-                if (!shared_kv && g == 1) skip((cur.tiles > 0) + (nx.tiles > 0));
+                if (!shared_kv && g == 1) { skip_v(cur.tiles > 0); skip_k(nx.tiles > 0); }
                 const bool do_pv = cur.tiles > own, do_qk = nx.tiles > own;
-                const int buf = split ? (int)(seg & 1) : g;
+                const int buf = split ? (int)(seg & 1) : F8 ? g * 2 + (int)(seg & 1) : g;
                 uint32_t vst = 0, kst = 0;
-                if (do_pv) vst = take();
+                if (do_pv) vst = take_v();
                 if (do_qk) {
-                    kst = take();
-                    if (nx.first) wait(&ctrl->q_full[buf], (split ? seg >> 1 : seg) & 1, 20);
+                    kst = take_k();
+                    if (nx.first) wait(&ctrl->q_full[buf], (split || F8 ? seg >> 1 : seg) & 1, 20);
                 }
                 const int pv_sl = do_pv ? slots_of(cur) : 0;
-                const uint32_t vb = v_lo + vst * (uint32_t)(C::kStageBytes >> 4);
+                const uint32_t vb = v_lo + vst * (uint32_t)((F8 ? C::kWideBytes : C::kStageBytes) >> 4);
                 // O_g (+)= P V: one 16-token step per slot, 8 columns of P
                 auto pv = [&](int k0, int k1) {
 #pragma unroll 1
                     for (int k = k0; k < k1; ++k)
-                        ptx::umma_f16_tmem_a(o_d, s_d + (uint32_t)(k * 8), vb + (uint32_t)(k * (C::kSlotBytes / 16)), hi_kv, idesc_pv, k > 0 || !cur.first);
+                        ptx::umma_f16_tmem_a(o_d, s_d + (uint32_t)(k * 8), vb + (uint32_t)(k * (C::kVSlotBytes / 16)), hi_v, idesc_pv, k > 0 || !cur.first);
                 };
                 if (do_pv) {
                     // the first half of P is multiplied while the softmax is at the second
@@ -744,21 +841,23 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                 turn_par ^= 1;
                 if (!ok) break;
                 ptx::tc_fence_after();
-                const uint32_t idesc_qk = ptx::umma_idesc_bf16(kRows, slots_of(nx) * kSlotTok);
+                const uint32_t n_qk = slots_of(nx) * kSlotTok, idesc_qk = F8 ? attn::umma_idesc_plain(kRows, n_qk) : ptx::umma_idesc_bf16(kRows, n_qk);
                 const uint32_t kb = k_lo + kst * (uint32_t)(C::kStageBytes >> 4);
                 const uint32_t qa = q_lo + (uint32_t)buf * q_buf;
                 if (elect_one()) {
                     if (do_pv) {
                         pv(kTileSlots / 2, pv_sl);
-                        ptx::umma_commit(&ctrl->empty[vst]);
+                        ptx::umma_commit(&v_empty[vst]);
                         if (cur.tiles <= step + own) ptx::umma_commit(&ctrl->o_full[g]);      // the accumulator of this segment is complete
                     }
                     if (do_qk) {
                         // S_g = Q K^T: 32 bytes of every row per instruction
 #pragma unroll 1
-                        for (int kk = 0; kk < C::kRowBytes / 32; ++kk)
-                            ptx::umma_f16_lohi(s_d, qa + (kk >> 2) * q_half + (uint32_t)((kk & 3) * 2), hi_q,
-                                               kb + (uint32_t)((kk >> 2) * 64 + (kk & 3) * 2), hi_kv, idesc_qk, kk != 0);
+                        for (int kk = 0; kk < C::kRowBytes / 32; ++kk) {
+                            const uint32_t a = qa + (kk >> 2) * q_half + (uint32_t)((kk & 3) * 2), b = kb + (uint32_t)((kk >> 2) * 64 + (kk & 3) * 2);
+                            if (F8) attn::umma_e4m3_lohi(s_d, a, hi_q, b, hi_k, idesc_qk, kk != 0);
+                            else ptx::umma_f16_lohi(s_d, a, hi_q, b, hi_k, idesc_qk, kk != 0);
+                        }
                         ptx::umma_commit(&ctrl->s_full[g]);
                         ptx::umma_commit(&ctrl->empty[kst]);
                     }
@@ -767,7 +866,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     if (nx.tiles > 0 && nx.tiles <= step + own && (do_qk || nx.first)) ptx::umma_commit(&ctrl->q_empty[buf]);
                 }
                 __syncwarp();
-                if (!shared_kv && g == 0) skip((cur.tiles > sp) + (nx.tiles > sp));
+                if (!shared_kv && g == 0) { skip_v(cur.tiles > sp); skip_k(nx.tiles > sp); }
                 if (nx.tiles <= 0) break;
                 cur = nx;
                 nx.tiles -= step;
@@ -783,6 +882,101 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                 }
             }
         }
+    } else if (F8 && warp >= 12) {
+        // =========================================================================== V from e4m3 to f16
+        // (Exact.  P stays f16: rounded to e4m3, as an 8-bit P V would need it, each weight is off by up to 6%.)
+        const int c_tid = tid - 32 * 12, cw = warp - 12;
+        // A thread has the same place in every slot.  Eight neighbouring lanes take four chunks of 16 codes of rows r and r ^ 5:
+        // with the swizzle neither their loads nor their stores meet in a bank.
+        const int tok = (c_tid >> 6) * 8 + (((c_tid >> 4) & 3) ^ (((c_tid >> 2) & 1) * 5)), chunk = ((c_tid >> 3) & 1) * 4 + (c_tid & 3);
+        const uint32_t src_off = attn::kv_slot_off<1>(tok, chunk), dst_off0 = attn::kv_slot_off<2>(tok, 2 * chunk), dst_off1 = attn::kv_slot_off<2>(tok, 2 * chunk + 1);
+        // These warps also stage the next unit's Q while they are at this one's V: eight rows per V tile, loaded a tile ahead (a
+        // load takes ~3000 cycles here).  split: all four share the one operand; else two per stream.
+        const int q_all = p.gs * p.nodes_tile, q_grp = split ? 0 : cw >> 1, q_share = ((split ? (q_all + 3) >> 2 : (q_all + 1) >> 1) + 7) & ~7;
+        const int q_row0 = (split ? cw : cw & 1) * q_share, q_rows = min(q_share, q_all - q_row0);
+        const StreamId id = stream_of(p, rb, q_grp);
+        const QScale qs(p.q_scale);
+        uint2 qv[8];
+        int left = n_tiles;
+        uint32_t n_seg = 0, st = 0, ph = 0, wst = 0, wph = 1;
+        bool ok = true;
+        Segment sg = ctrl->first, nx = sg;
+        // (the first segment's Q is converted out of the buffers that these warps are about to fill)
+        if (left > 0) ok = wait_bar(ctrl, &ctrl->q_full[0], 0, 28) && (split || wait_bar(ctrl, &ctrl->q_full[2], 0, 28));
+#pragma unroll 1
+        while (left > 0 && ok) {
+            const int seg_tiles = sg.t_last - sg.t_first;
+            left -= seg_tiles;
+            int q_at = 0, q_loaded = 0, q_end = 0;                 // next Q: rows stored, loaded, and in all
+            if (left > 0) {
+                nx = next_segment(sg, left, p, s_len);
+                q_end = max(q_rows, 0);
+            }
+            ++n_seg;
+            const int q_buf = split ? (int)(n_seg & 1) : q_grp * 2 + (int)(n_seg & 1);
+            auto q_step = [&]() {                                  // store the rows that were loaded, load the next ones
+                if (q_at < q_loaded) {
+                    if (q_at == 0 && !wait_bar(ctrl, &ctrl->q_empty[q_buf], ((n_seg >> 1) & 1) ^ 1, 11)) { ok = false; return; }
+#pragma unroll 1
+                    for (; q_at < q_loaded; ++q_at) {
+                        store_q_row(sQ + q_buf * C::kQBytes, q_row0 + q_at, qv[0], qs);
+#pragma unroll
+                        for (int k = 0; k < 7; ++k) qv[k] = qv[k + 1];         // (rotated: registers take no index)
+                    }
+                }
+                if (q_loaded < q_end) {
+                    const int r = q_row0 + q_loaded + lane;        // (eight of the lanes count)
+                    const int hl = (id.rt / p.node_tiles) * p.gs + r % p.gs, node = (id.rt % p.node_tiles) * p.nodes_tile + r / p.gs;
+                    const uint32_t real = __ballot_sync(0xffffffffu, id.exists && r < p.gs * p.nodes_tile && hl < p.G && node < p.n);
+                    const __nv_bfloat16* row = p.q + (((size_t)(nx.layer * p.B + nx.b) * p.n + node) * (size_t)p.Hq + (nx.g * p.heads_per_unit + id.head_off) * p.G + hl) * D;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const __nv_bfloat16* src = row_of_lane(row, k);
+                        qv[k] = make_uint2(0, 0);
+                        if (real >> k & 1u) qv[k] = *reinterpret_cast<const uint2*>(src + lane * 4);
+                    }
+                    q_loaded += 8;
+                }
+            };
+            const int n_v = seg_tiles * (split || shared_kv ? 1 : 2);          // V tiles of this segment
+#pragma unroll 1
+            for (int i = 0; i < n_v || q_at < q_end; ++i) {
+            if (i >= n_v) {                                        // (a short segment: the rest of Q by itself)
+                q_step();
+                if (!ok) break;
+                continue;
+            }
+            if (!wait_bar(ctrl, &ctrl->full[ring_n + st], ph, 26) || !wait_bar(ctrl, &ctrl->wide_empty[wst], wph, 27)) { ok = false; break; }
+            const uint8_t* const src = ring + (size_t)(ring_n + st) * C::kStageBytes + src_off;
+            uint8_t* const dst = wide + (size_t)wst * C::kWideBytes;
+#pragma unroll 1
+            for (int k = 0; k < kTileSlots; k += 4) {
+                uint4 v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = *reinterpret_cast<const uint4*>(src + (k + j) * C::kSlotBytes);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint2 a = widen4(v[j].x), b = widen4(v[j].y), c = widen4(v[j].z), e = widen4(v[j].w);
+                    *reinterpret_cast<uint4*>(dst + (k + j) * C::kVSlotBytes + dst_off0) = make_uint4(a.x, a.y, b.x, b.y);
+                    *reinterpret_cast<uint4*>(dst + (k + j) * C::kVSlotBytes + dst_off1) = make_uint4(c.x, c.y, e.x, e.y);
+                }
+            }
+            ptx::fence_proxy_async();                              // (read by the tensor cores)
+            __syncwarp();
+            if (lane == 0) { ptx::mbar_arrive(&ctrl->wide_full[wst]); ptx::mbar_arrive(&ctrl->empty[ring_n + st]); }
+            if (++st == (uint32_t)ring_n) { st = 0; ph ^= 1; }
+            if (++wst == kWideStages) { wst = 0; wph ^= 1; }
+            q_step();
+            if (!ok) break;
+            }
+            if (left > 0 && ok && q_end == 0) ok = wait_bar(ctrl, &ctrl->q_empty[q_buf], ((n_seg >> 1) & 1) ^ 1, 11);      // (no arrival ahead of its phase)
+            if (left > 0 && ok) {
+                ptx::fence_proxy_async();
+                __syncwarp();
+                if (lane < 2) ptx::mbar_arrive(&ctrl->q_full[q_buf]);          // (twice: the first segment's Q comes from twice the warps)
+            }
+            sg = nx;
+        }
     } else {
         // =========================================================================== softmax / epilogue
         const int w4 = warp & 3;                                   // TMEM lane quarter of this warp
@@ -797,8 +991,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         const uint32_t lane_base = tmem_base + ((uint32_t)(w4 * 32) << 16);
         const uint32_t s_addr = lane_base + (uint32_t)(grp * kTileTok), o_addr = lane_base + kTmemO + (uint32_t)(grp * D);
         constexpr int kRowW = D + 4;                               // record: D accumulator columns, then (max, sum)
-        const float sc = p.scale_log2e;
-        const uint64_t sc2 = pack2(sc, sc);
+        float sc = p.scale_log2e;                                  // scores -> log2 units (e4m3: times the unit's Q and K scales)
         uint32_t xph = 0;                                          // parity of the split pair's exchange barrier
         auto pair_sync = [&]() -> bool {
             __syncwarp();
@@ -811,8 +1004,41 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         bool ok = true;
         int left = n_tiles;                                        // tiles from the segment's first to the range's end
         Segment sg = ctrl->first;
+        if (F8 && left > 0) {
+            // e4m3: the first segment's Q (the ones behind it are staged by the warps that widen V), each warp its rows, or (split)
+            // half of them
+            const int r0 = split ? grp * 16 : 0, r1 = split ? r0 + 16 : 32, buf = split ? 0 : grp * 2;
+            const QScale qs(p.q_scale);
+            const __nv_bfloat16* qrow = p.q + (((size_t)(sg.layer * p.B + sg.b) * p.n + node) * (size_t)p.Hq + (sg.g * p.heads_per_unit + id.head_off) * p.G + hl) * D;
+            const uint32_t real = __ballot_sync(0xffffffffu, row_ok);
+            // All rows are requested first, into the buffers of widened V, which are not in use yet.  (What this costs is mostly
+            // the fetch of code that runs once, at some 600 cycles per 128 bytes: the loops are as short as they can be.)
+            uint8_t* const raw = wide + (split ? 0 : grp * C::kWideBytes) + w4 * 32 * 256;
+            const int r_end = min(r1, 32 - __clz(real));
+#pragma unroll 1
+            for (int r = r0 + (lane >> 4); r < r1; r += 2) {
+                const __nv_bfloat16* src = row_of_lane(qrow, r);
+                if (real >> r & 1u)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ptx::smem_u32(raw + r * 256 + (lane & 15) * 16)), "l"(src + (lane & 15) * 8) : "memory");
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncwarp();
+#pragma unroll 1
+            for (int r = r0; r < r_end; ++r)
+                store_q_row(sQ + buf * C::kQBytes, w4 * 32 + r, real >> r & 1u ? *reinterpret_cast<const uint2*>(raw + r * 256 + lane * 8) : make_uint2(0, 0), qs);
+            ptx::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&ctrl->q_full[buf]);
+        }
 #pragma unroll 1
         while (left > 0 && ok) {
+            float vsc = 1.f;                                       // e4m3: the V scale
+            if (F8) {
+                const int h = sg.layer * p.Hkv + sg.g * p.heads_per_unit + id.head_off;
+                sc = p.scale_log2e * p.q_scale * __ldg(p.k_scale + h);
+                vsc = __ldg(p.v_scale + h);
+            }
+            const uint64_t sc2 = pack2(sc, sc);
             float off = -INFINITY, l_run = 0.f;                    // this row's offset (log2 units) and running sum
             bool redone = false;
             const int mine = split ? (sg.t_last - sg.t_first + 1 - grp) >> 1 : sg.t_last - sg.t_first;     // tiles of this stream
@@ -840,17 +1066,17 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                         uint64_t s0 = 0, s1 = 0;                   // (two zeros each)
                         tmem_ld_wait32(ra);
                         ptx::tmem_ld_32x32b_x32(s_addr + (uint32_t)(h * 64 + 32), rb_);
-                        exp_chunk(ra, sc2, no2, pk, s0, s1);
+                        exp_chunk<F8>(ra, sc2, no2, pk, s0, s1);
                         tmem_ld_wait32(rb_);
                         ptx::tmem_ld_32x32b_x32(s_addr + 64, ra);  // (of no use to the second half)
-                        exp_chunk(rb_, sc2, no2, pk + 16, s0, s1);
+                        exp_chunk<F8>(rb_, sc2, no2, pk + 16, s0, s1);
                         float a, b;
                         unpack2(add2(s0, s1), a, b);
                         const float half_sum = a + b;
                         // The offset moves when the sum outgrows the limit (an overflow makes it infinite, which counts): rare, and
                         // then this half is redone.  (The accumulator may be touched: the tile before was multiplied before this
                         // tile was scored, and for this tile's first half there is a barrier.)
-                        const bool grow = half_sum > kSumLimit && !redone;
+                        const bool grow = half_sum > kSumLimit<F8> && !redone;
                         if (__any_sync(0xffffffffu, grow)) {
                             tmem_ld_wait32(ra);
                             if (h == 1) {
@@ -918,13 +1144,14 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             }
             ptx::tc_fence_after();
             if (warp_has_rows) {
-                const float inv = 1.f / Lsum;
+                const float inv = 1.f / Lsum;                      // (e4m3: V codes times the unit's V scale)
                 // split: this warp combines its half of the columns of both accumulators; otherwise all columns of its own.
                 // (16 columns at a time: this runs once per unit, and what it costs is mostly the instruction fetch)
                 const int c_lo = split ? grp * (D / 2) : 0, c_hi = split ? c_lo + D / 2 : D;
                 const uint32_t o_first = split ? lane_base + kTmemO : o_addr;
                 if (!split) w0 = M != -INFINITY ? 1.f : 0.f;
                 if (whole) { w0 *= inv; w1 *= inv; }
+                if (F8) { w0 *= vsc; w1 *= vsc; }
 #pragma unroll 1
                 for (int c = c_lo; c < c_hi; c += 16) {
                     uint32_t r[16];
@@ -995,7 +1222,7 @@ __global__ void __launch_bounds__(attn::kMergeThreads) attn_merge_kernel(const _
 mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
                                  float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8, bool keep_rounding) {
-    if (f8 || keep_rounding) return mirror_attn_tile64_launch(ctx, kv, tree, ti, q, k_new, v_new, out, lse_out, partial_ws, stream, f8);
+    if (keep_rounding) return mirror_attn_tile64_launch(ctx, kv, tree, ti, q, k_new, v_new, out, lse_out, partial_ws, stream, f8);
     const int D = ctx->desc.head_dim, Hkv = ctx->desc.n_kv_heads, Hq = ctx->desc.n_q_heads;
     AttnParams p;
     p.L = kv->num_layers; p.B = tree->batch; p.n = ti.n; p.Hq = Hq; p.Hkv = Hkv; p.G = Hq / Hkv;
@@ -1036,6 +1263,10 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     p.tree_slots = (p.n + kSlotTok - 1) / kSlotTok;
     p.scale_log2e = ctx->scale * 1.4426950408889634f;
     p.page_table = kv->page_table; p.prefix_len = kv->prefix_len;
+    if (f8 && (!f8->k_scale || !f8->v_scale || !(f8->q_scale > 0.f))) return D != 128 ? MIRROR_ERR_UNSUPPORTED : MIRROR_ERR_ARG;
+    if (f8 && D != 128) return MIRROR_ERR_UNSUPPORTED;
+    p.q = (const __nv_bfloat16*)q;
+    p.k_scale = f8 ? f8->k_scale : nullptr; p.v_scale = f8 ? f8->v_scale : nullptr; p.q_scale = f8 ? f8->q_scale : 1.f;
     p.v_pool = (const __nv_bfloat16*)kv->v_pool;
     p.out = (__nv_bfloat16*)out; p.lse_out = lse_out;
     p.partial = partial_ws; p.begins = (attn::GroupBegin*)((uint8_t*)partial_ws - kWsNotesBytes); p.status = ctx->d_status;
@@ -1045,8 +1276,8 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     Maps tm;
     {
         // pool as (64 columns, 8 tokens, D/64 halves, 2 token groups, (layer*page)*head): one box is one page of one head,
-        // landing as [token / 8][half][token % 8][128 B]
-        const uint64_t total_pages = (uint64_t)(p.L - 1) * p.layer_pages + p.num_pages, row = (uint64_t)D * 2;
+        // landing as [token / 8][half][token % 8][128 B] (e4m3 pools through the same 16-bit map: 64 "columns" are a row's 128 bytes)
+        const uint64_t total_pages = (uint64_t)(p.L - 1) * p.layer_pages + p.num_pages, row = (uint64_t)D * (f8 ? 1 : 2);
         const uint64_t dims[5] = {64, 8, row / 128, 2, total_pages * (uint64_t)Hkv};
         const uint64_t strides[4] = {row, 128, 8 * row, kSlotTok * row};
         const uint32_t box[5] = {64, 8, (uint32_t)(row / 128), 2, 1};
@@ -1061,21 +1292,25 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         st = mirror_make_tmap(ctx, &tm.kn, k_new, 5, ndims, nstrides, nbox);
         if (st == MIRROR_OK) st = mirror_make_tmap(ctx, &tm.vn, v_new, 5, ndims, nstrides, nbox);
         if (st != MIRROR_OK) return st;
+        if (!f8) {
         // Q as (64 columns, heads, n nodes, D/64 halves, layer*request): one box is one half of a row tile
         const uint64_t qdims[5] = {64, (uint64_t)Hq, (uint64_t)p.n, row / 128, lb};
         const uint64_t qstrides[4] = {row, Hq * row, 128, (uint64_t)p.n * Hq * row};
         const uint32_t qbox[5] = {64, (uint32_t)p.gs, (uint32_t)p.nodes_tile, 1, 1};
         st = mirror_make_tmap(ctx, &tm.q, q, 5, qdims, qstrides, qbox);
         if (st != MIRROR_OK) return st;
+        }
     }
-    auto launch = [&](auto kern, auto merge, int stage_bytes) -> mirror_status {
-        const size_t fixed = 2 * (size_t)kRows * D * 2 + kCtrlBytes + (p.mode == kSplit ? kRows * 16 : 0) + (2 * (size_t)p.B + 1) * 4;
-        int stages = (int)((kSmemLimit - fixed) / stage_bytes);
+    auto launch = [&](auto cfg, auto kern, auto merge) -> mirror_status {
+        using C = decltype(cfg);
+        const size_t fixed = (f8 && p.mode != kSplit ? 4 : 2) * (size_t)C::kQBytes + C::kFixedBytes + (p.mode == kSplit ? kRows * 16 : 0) + (2 * (size_t)p.B + 1) * 4;
+        int stages = (int)((kSmemLimit - fixed) / C::kStageBytes);
         if (stages > kMaxStages) stages = kMaxStages;
+        if (f8) stages &= ~1;                               // (K and V have half each)
         if (stages < 4) return MIRROR_ERR_UNSUPPORTED;
-        const size_t smem = fixed + (size_t)stages * stage_bytes;
+        const size_t smem = fixed + (size_t)stages * C::kStageBytes;
         MIRROR_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
-        MIRROR_CUDA_OK(mirror_launch_pdl(kern, dim3(p.n_groups * p.n_cta), dim3(kThreads), smem, stream, tm, at, p, stages));
+        MIRROR_CUDA_OK(mirror_launch_pdl(kern, dim3(p.n_groups * p.n_cta), dim3(C::kThreads), smem, stream, tm, at, p, stages));
         ctx->launches += 1;
         MIRROR_CUDA_OK(cudaGetLastError());
         // One request: all units have the same length whatever it is, so the host can tell when the partition gives every
@@ -1091,6 +1326,7 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         }
         return MIRROR_OK;
     };
-    return D == 128 ? launch(attn_verify_kernel<128>, attn_merge_kernel<128>, Cfg<128>::kStageBytes)
-                    : launch(attn_verify_kernel<64>, attn_merge_kernel<64>, Cfg<64>::kStageBytes);
+    return f8         ? launch(Cfg<128, true>{}, attn_verify_kernel<128, true>, attn_merge_kernel<128>)
+           : D == 128 ? launch(Cfg<128, false>{}, attn_verify_kernel<128, false>, attn_merge_kernel<128>)
+                      : launch(Cfg<64, false>{}, attn_verify_kernel<64, false>, attn_merge_kernel<64>);
 }
