@@ -39,7 +39,8 @@
 // (128 rows and 64-token tiles per CTA, alternating two softmax groups, took 4360 cycles for the same work.)  What the
 // twelve warps execute per tile has to stay in the SM's instruction cache: loops are kept rolled and rare paths out of
 // line on purpose; unrolled, the same step took 4900 cycles, most of them in instruction fetch.  Tried and neutral: a
-// third of the exponentials as polynomials on the FMA pipe, and turns between the softmax warps of a scheduler.
+// third of the exponentials as polynomials on the FMA pipe, and Q K^T by halves of a tile behind the same half's P V (no
+// wait for scores, but 96 instead of 64 cycles of tensor core per 128 tokens: the same time at the power limit).
 // Measured (bf16, d = 128, tiles of 16-token pages): 80 layers x 16 requests x 520 rows 25.0 -> 20.5 ms at the same
 // power; 64 layers x 32768 tokens x 264 rows 4.0 -> 3.4 ms; e4m3 cache, 64 layers x 4 x 4096..16384 tokens x 136 rows (64-token
 // tiles with e4m3 P before): 2.25 -> 1.85 ms.
@@ -68,7 +69,7 @@ constexpr int kMaxStages = 10;
 template <bool F8> constexpr float kSumLimit = F8 ? 16384.f : 1.2089258196146292e24f;
 constexpr int kTmemCols = 512;
 constexpr int kTmemO = 2 * kTileTok;
-constexpr int kCtrlBytes = 512;
+constexpr int kCtrlBytes = 528;
 constexpr size_t kSmemLimit = 232448;               // 227 KB
 
 enum { kSplit = 0, kPaired = 1 };
@@ -185,6 +186,7 @@ struct Ctrl {
     uint64_t s_full[2], p_full[2][2], o_full[2];        // per stream (P: per half of the tile)
     uint64_t pv_half[2];                                // P V of a tile's first half is through
     uint64_t turn[2];                                   // the issuing warps take turns
+    uint64_t exp_turn[2][4];                            // the two softmax warps of a scheduler take turns
     uint64_t pair[4];                                   // split: the two softmax warps of a TMEM quarter meet
     Segment first;                                      // where this CTA's range begins
     int n_tiles;
@@ -531,7 +533,10 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             ptx::mbar_init(&ctrl->o_full[g], 1); ptx::mbar_init(&ctrl->turn[g], 1); ptx::mbar_init(&ctrl->pv_half[g], 1);
         }
         for (int s = 0; s < q_bufs; ++s) { ptx::mbar_init(&ctrl->q_full[s], !F8 ? 1 : split ? 8 : 4); ptx::mbar_init(&ctrl->q_empty[s], split ? 2 : 1); }
-        for (int s = 0; s < 4; ++s) ptx::mbar_init(&ctrl->pair[s], 2);
+        for (int s = 0; s < 4; ++s) {
+            ptx::mbar_init(&ctrl->pair[s], 2);
+            ptx::mbar_init(&ctrl->exp_turn[0][s], 1); ptx::mbar_init(&ctrl->exp_turn[1][s], 1);
+        }
         ctrl->abort = 0;
         ctrl->status = p.status;
         ctrl->wait_limit = p.wait_limit;
@@ -753,9 +758,11 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         } else if (n_tiles > 0) {
             // ======================================================================= tensor-core issuers
             // One warp per stream: what a warp executes between two chains (waits, ring bookkeeping, ~800 cycles) is more than the
-            // tensor cores' queue covers, so one warp for both left them idle a third of the time.  They take turns issuing:
-            // left to themselves the two streams fall into step, both in their softmax and then both waiting.  The whole
-            // warp walks the schedule and one elected lane issues, which keeps descriptors in uniform registers.
+            // tensor cores' queue covers, so one warp for both left them idle a third of the time.  They take turns issuing: left
+            // to themselves the two streams fall into step, both in their softmax and then both waiting.  (The turns also keep an
+            // issuer that has no tile in a step, or skips the other's stages, within one round of the ring: further ahead, a
+            // stage's parity would pass for that of the round before.)  The whole warp walks the schedule and one elected lane
+            // issues, which keeps descriptors in uniform registers.
             const uint32_t hi_q = ptx::umma_desc_hi_sw128(1024), hi_k = ptx::umma_desc_hi_sw128(C::kGroupStride),
                            hi_v = ptx::umma_desc_hi_sw128(C::kVHalves * 1024);
             const uint32_t q_lo = ptx::umma_desc_lo(ptx::smem_u32(sQ), 16);
@@ -1000,6 +1007,21 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             xph ^= 1;
             return r;
         };
+        // The two softmax warps of a scheduler, one of either stream, take turns at a tile's exponentials: left to themselves the
+        // streams fall into step, both at the special-function unit and then both waiting for their scores.  Not over an e4m3
+        // cache: its Q K^T is over so soon that the turns cost more than the step (2.16 -> 2.35 ms).
+        uint32_t t_par = grp == 0 ? 1 : 0;
+        auto take_turn = [&]() -> bool {
+            if (F8) return true;
+            const bool r = wait_bar(ctrl, &ctrl->exp_turn[grp][w4], t_par, 36);
+            t_par ^= 1;
+            return r;
+        };
+        auto pass_turn = [&]() {
+            if (F8) return;
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&ctrl->exp_turn[grp ^ 1][w4]);
+        };
         uint32_t s_par = 0, o_par = 0;
         bool ok = true;
         int left = n_tiles;                                        // tiles from the segment's first to the range's end
@@ -1039,7 +1061,8 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                 vsc = __ldg(p.v_scale + h);
             }
             const uint64_t sc2 = pack2(sc, sc);
-            float off = -INFINITY, l_run = 0.f;                    // this row's offset (log2 units) and running sum
+            // this row's offset (log2 units) and running sum (rows that do not exist: one that makes every P 0)
+            float off = row_ok ? -INFINITY : 1e30f, l_run = 0.f;
             bool redone = false;
             const int mine = split ? (sg.t_last - sg.t_first + 1 - grp) >> 1 : sg.t_last - sg.t_first;     // tiles of this stream
             for (int i = 0; i < mine; ++i) {
@@ -1058,6 +1081,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     float sum = 0.f;
                     uint32_t ra[32];
                     ptx::tmem_ld_32x32b_x32(s_addr, ra);
+                    if (!take_turn()) { ok = false; break; }
 #pragma unroll 1
                     for (int h = 0; h < 2;) {
                         uint32_t pk[32], rb_[32];
@@ -1076,6 +1100,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                         // The offset moves when the sum outgrows the limit (an overflow makes it infinite, which counts): rare, and
                         // then this half is redone.  (The accumulator may be touched: the tile before was multiplied before this
                         // tile was scored, and for this tile's first half there is a barrier.)
+                        if (h == 1 && !redone) pass_turn();
                         const bool grow = half_sum > kSumLimit<F8> && !redone;
                         if (__any_sync(0xffffffffu, grow)) {
                             tmem_ld_wait32(ra);
@@ -1103,10 +1128,15 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     if (!ok) break;
                     tmem_ld_wait32(ra);
                     l_run += sum;
-                } else if (lane == 0) {
-                    ptx::mbar_arrive(&ctrl->p_full[grp][0]);
-                    ptx::mbar_arrive(&ctrl->p_full[grp][1]);
+                } else {
+                    if (!take_turn()) { ok = false; break; }
+                    pass_turn();
+                    if (lane == 0) { ptx::mbar_arrive(&ctrl->p_full[grp][0]); ptx::mbar_arrive(&ctrl->p_full[grp][1]); }
                 }
+            }
+            if (ok && split && grp == 1 && ((sg.t_last - sg.t_first) & 1)) {       // (stream 0 has one tile more)
+                ok = take_turn();
+                pass_turn();
             }
             if (!ok) break;
             // ---- end of this CTA's part of the unit
