@@ -1252,7 +1252,7 @@ __global__ void __launch_bounds__(attn::kMergeThreads) attn_merge_kernel(const _
 mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
                                  float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8, bool keep_rounding) {
-    if (keep_rounding) return mirror_attn_tile64_launch(ctx, kv, tree, ti, q, k_new, v_new, out, lse_out, partial_ws, stream, f8);
+    if (keep_rounding && !f8) return mirror_attn_tile64_launch(ctx, kv, tree, ti, q, k_new, v_new, out, lse_out, partial_ws, stream);
     const int D = ctx->desc.head_dim, Hkv = ctx->desc.n_kv_heads, Hq = ctx->desc.n_q_heads;
     AttnParams p;
     p.L = kv->num_layers; p.B = tree->batch; p.n = ti.n; p.Hq = Hq; p.Hkv = Hkv; p.G = Hq / Hkv;

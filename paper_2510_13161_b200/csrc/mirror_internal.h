@@ -119,13 +119,13 @@ struct MirrorAttnFp8 {
 // serialization.
 mirror_status mirror_kv_quantize_launch(mirror_ctx* ctx, const void* x, int n_layers, int64_t layer_stride, int64_t layer_elems,
                                        int inner, const float* scale, void* out_fp8, cudaStream_t stream);
-// keep_rounding: the call has to give the same bits as earlier ones on the same inputs and sizes (mirror_target_forward).
+// keep_rounding: every sum keeps the order of the 64-token kernel (mirror_target_forward in deep stacks, see attn_tile64.cu).
 mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
                                  float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8 = nullptr, bool keep_rounding = false);
 mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                         const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
-                                        float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8);
+                                        float* partial_ws, cudaStream_t stream);
 
 // bf16 tensor map with 128-byte swizzle.  dims/box are innermost-first; strides_bytes[i] is the byte
 // stride of dimension i+1 (rank-1 entries).
