@@ -18,6 +18,7 @@
 namespace {
 
 constexpr int kGreedyThreads = 256;
+constexpr int kFoldThreads = 1024;                    // of a greedy block that folds the LM head's partials itself
 constexpr int kThreads = 512;                         // of a CTA of the clusters
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCluster = 16;                       // CTAs per request (above 8: opt-in)
@@ -120,16 +121,54 @@ __device__ __forceinline__ Choice choose(const AcceptTreeParams& tp, const int* 
     return c;
 }
 
-__global__ void __launch_bounds__(kGreedyThreads)
-accept_greedy_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs a) {
+// FOLD: the rows' argmax comes out of the LM head's row partials, in the block that needs it: a launch less (the merge kernel
+// in front and this one took 5.5 us of a toy model's step of 22).  Lanes are rows, warps share the partials.
+template <bool FOLD>
+__global__ void __launch_bounds__(FOLD ? kFoldThreads : kGreedyThreads)
+accept_greedy_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs a, const MirrorLmPartials parts, int32_t* argmax_out) {
+    constexpr int kBlockWarps = (FOLD ? kFoldThreads : kGreedyThreads) / 32;
     __shared__ int s_len[MIRROR_MAX_BRANCHES];
     __shared__ Choice s_choice;
+    __shared__ float s_max[FOLD ? kBlockWarps : 1][33];
+    __shared__ int s_idx[FOLD ? kBlockWarps : 1][33];
+    __shared__ int32_t s_argmax[FOLD ? MIRROR_MAX_NODES : 1];
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = tp.n;
     const int32_t* tok = a.tokens + (size_t)b * n;
-    const int32_t* am = a.target_argmax + (size_t)b * n;
+    const int32_t* am = FOLD ? s_argmax : a.target_argmax + (size_t)b * n;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    for (int br = warp; br < tp.n_branches; br += kGreedyThreads / 32) {
+    if (FOLD) {
+        const size_t M = (size_t)gridDim.x * n;
+        // the comparator (logit descending, id ascending) makes the result independent of the order
+        auto fold = [](float& m, int& i, float om, int oi) {
+            if (om > m || (om == m && om != -INFINITY && oi < i)) { m = om; i = oi; }
+        };
+#pragma unroll 1
+        for (int r0 = 0; r0 < n; r0 += 32) {
+            float m = -INFINITY;
+            int i = 0x7fffffff;
+            if (r0 + lane < n) {
+                const size_t at = (size_t)b * n + r0 + lane;
+#pragma unroll 4
+                for (int k = warp; k < parts.count; k += kBlockWarps) fold(m, i, parts.max[k * M + at], parts.idx[k * M + at]);
+            }
+            s_max[warp][lane] = m;
+            s_idx[warp][lane] = i;
+            __syncthreads();
+            if (r0 + warp < n) {                                   // (as many warps as lanes)
+                m = s_max[lane][warp];
+                i = s_idx[lane][warp];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) fold(m, i, __shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, i, o));
+                if (lane == 0) {
+                    s_argmax[r0 + warp] = i;
+                    argmax_out[(size_t)b * n + r0 + warp] = i;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    for (int br = warp; br < tp.n_branches; br += kBlockWarps) {
         const int len = tp.path_len[br];
         bool pass = true;
         if (lane < len) {
@@ -463,7 +502,7 @@ int cluster_size(const mirror_ctx* ctx, int batch) {
 
 mirror_status mirror_accept_launch(mirror_ctx* ctx, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                    const mirror_accept_in* in, const mirror_accept_out* out, cudaStream_t stream,
-                                   double* tree_scratch) {
+                                   double* tree_scratch, const MirrorLmPartials* partials, int32_t* argmax_out) {
     AcceptTreeParams tp;
     tp.n = ti.n;
     tp.n_branches = ti.n_branches;
@@ -489,7 +528,9 @@ mirror_status mirror_accept_launch(mirror_ctx* ctx, const mirror_tree* tree, con
     a.tree_scratch = tree_scratch;
     a.status = ctx->d_status;
     if (in->mode == MIRROR_ACCEPT_GREEDY) {
-        MIRROR_CUDA_OK(mirror_launch_pdl(accept_greedy_kernel, dim3(tree->batch), dim3(kGreedyThreads), 0, stream, tp, a));
+        const MirrorLmPartials none = {0, nullptr, nullptr};
+        if (partials) MIRROR_CUDA_OK(mirror_launch_pdl(accept_greedy_kernel<true>, dim3(tree->batch), dim3(kFoldThreads), 0, stream, tp, a, *partials, argmax_out));
+        else MIRROR_CUDA_OK(mirror_launch_pdl(accept_greedy_kernel<false>, dim3(tree->batch), dim3(kGreedyThreads), 0, stream, tp, a, none, argmax_out));
     } else {
         auto kern = in->mode == MIRROR_ACCEPT_SPEC_TREE ? accept_tree_kernel : accept_spec_kernel;
         const unsigned n_cta = (unsigned)cluster_size(ctx, tree->batch);

@@ -531,8 +531,12 @@ mirror_status lmhead_tail(mirror_ctx* ctx, const void* hidden, int M, const void
                           const int32_t* gather_tok, int n_gather, int32_t* argmax, float* maxlogit, float* lse, int32_t* topk_id,
                           float* topk_logprob, float* gather_logit, float* logits_out, float* lse_scratch, cudaStream_t stream,
                           void* topk_logprob_bf16, int P, float inv_T, float inv_T_log2e, const float* part_max, const int* part_idx,
-                          const float* part_sum, const float* cand_v = nullptr, const int* cand_i = nullptr) {
+                          const float* part_sum, const float* cand_v = nullptr, const int* cand_i = nullptr, MirrorLmPartials* defer = nullptr) {
     const int V = ctx->desc.vocab, H = ctx->desc.hidden;
+    if (defer) {
+        *defer = {P, part_max, part_idx};
+        return MIRROR_OK;
+    }
     float* lse_dst = lse ? lse : (topk > 0 ? lse_scratch : nullptr);
     if (topk > 0 && cand_v) {      // (four lists per partial: one per epilogue warp)
         if (4 * P > kListsPerThread * 1024) return MIRROR_ERR_UNSUPPORTED;
@@ -573,7 +577,7 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
                                    int32_t* argmax, float* maxlogit, float* lse, int32_t* topk_id,
                                    float* topk_logprob, float* gather_logit, float* logits_out,
                                    void* partial_ws, size_t partial_bytes, float* lse_scratch, cudaStream_t stream,
-                                   cudaEvent_t after_gemm, void* topk_logprob_bf16, void* topk_ws, size_t topk_ws_bytes) {
+                                   cudaEvent_t after_gemm, void* topk_logprob_bf16, void* topk_ws, size_t topk_ws_bytes, MirrorLmPartials* defer) {
     const int V = ctx->desc.vocab, H = ctx->desc.hidden;
     // Top-kappa inside the GEMM's epilogue whenever the caller's scratch holds the candidate lists; otherwise (or on the
     // single-CTA fallback kernel) the selection runs over spilled logits, which then have to be there.
@@ -595,7 +599,7 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
             return lmhead_tail(ctx, hidden, M, W, topk, gather_row, gather_tok, n_gather, argmax, maxlogit, lse, topk_id, topk_logprob,
                                gather_logit, logits_out, lse_scratch, stream, topk_logprob_bf16, P, inv_T, inv_T_log2e, part_max,
                                part_idx, part_sum, fused_topk ? (const float*)topk_ws : nullptr,
-                               fused_topk ? (const int*)((const float*)topk_ws + (size_t)4 * P * M * topk) : nullptr);
+                               fused_topk ? (const int*)((const float*)topk_ws + (size_t)4 * P * M * topk) : nullptr, defer);
         }
         if (st != MIRROR_ERR_WORKSPACE) return st;
     }
@@ -658,7 +662,7 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
 
     return lmhead_tail(ctx, hidden, M, W, topk, gather_row, gather_tok, n_gather, argmax, maxlogit, lse, topk_id, topk_logprob,
                        gather_logit, logits_out, lse_scratch, stream, topk_logprob_bf16, (int)P, p.inv_T, p.inv_T_log2e, p.part_max,
-                       p.part_idx, p.part_sum);
+                       p.part_idx, p.part_sum, nullptr, nullptr, defer);
 }
 
 extern "C" mirror_status mirror_lmhead_reduce(mirror_ctx* ctx, const void* hidden, int M, const void* W, int topk,

@@ -83,16 +83,24 @@ struct MirrorWsLayout {
 };
 void mirror_ws_layout(const mirror_ctx* ctx, size_t M, MirrorWsLayout* out, size_t B = 0);
 
+// Row partials (maximum, its id) that an LM-head GEMM left: `count` of [M] rows each.
+struct MirrorLmPartials {
+    int count;
+    const float* max;
+    const int* idx;
+};
+// partials: greedy only; the kernel folds them itself and leaves the rows' argmax in argmax_out.
 mirror_status mirror_accept_launch(mirror_ctx* ctx, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                    const mirror_accept_in* in, const mirror_accept_out* out, cudaStream_t stream,
-                                   double* tree_scratch = nullptr);
+                                   double* tree_scratch = nullptr, const MirrorLmPartials* partials = nullptr, int32_t* argmax_out = nullptr);
+// defer: the row partials are not merged, but described there (only the argmax was asked for).
 mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, int topk,
                                    const int32_t* gather_row, const int32_t* gather_tok, int n_gather,
                                    int32_t* argmax, float* maxlogit, float* lse, int32_t* topk_id,
                                    float* topk_logprob, float* gather_logit, float* logits_out,
                                    void* partial_ws, size_t partial_bytes, float* lse_scratch, cudaStream_t stream,
                                    cudaEvent_t after_gemm = nullptr, void* topk_logprob_bf16 = nullptr,
-                                   void* topk_ws = nullptr, size_t topk_ws_bytes = 0);
+                                   void* topk_ws = nullptr, size_t topk_ws_bytes = 0, MirrorLmPartials* defer = nullptr);
 // LM-head GEMM + per-unit row partials on CTA pairs (many hidden rows); *n_partials partials of [M] rows are left in
 // partial_ws for lmhead_merge_kernel.  mirror_lmhead_pair_partials(V) is that count.
 int mirror_lmhead_pair_partials(int V);

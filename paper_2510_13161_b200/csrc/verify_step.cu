@@ -191,9 +191,13 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     int32_t* d_argmax = argmax_out ? argmax_out : (int32_t*)(ws + L.argmax);
     float* d_lse = (float*)(ws + L.lse);
     float* d_logits = spec ? (float*)(ws + L.logits) : nullptr;
+    // greedy: the acceptance kernel folds the GEMM's row partials itself, a block per request.  (Up to 256 rows the GEMM leaves
+    // a partial per CTA, ~10 loads per lane; beyond, one per 128 vocabulary ids, and a block per row is worth its launch.)
+    MirrorLmPartials partials;
+    const bool defer = !spec && M <= 256;
     st = mirror_lmhead_launch(ctx, rows, (int)M, W, 0, nullptr, nullptr, 0, d_argmax, nullptr, spec ? d_lse : nullptr, nullptr,
                               nullptr, nullptr, d_logits, ws + L.lm_partial, L.lm_partial_bytes, d_lse, s,
-                              ev ? ctx->stage_ev[2] : nullptr);
+                              ev ? ctx->stage_ev[2] : nullptr, nullptr, nullptr, 0, defer ? &partials : nullptr);
     if (st != MIRROR_OK) return st;
 
     if (io) MIRROR_CUDA_OK(cudaStreamWaitEvent(s, ctx->copy_ev[kEvTokens], 0));
@@ -203,7 +207,7 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     in.lse = d_lse;
     // the tree rule keeps its running distribution in the workspace when the caller sized it for that
     double* tree_scratch = (acc->mode == MIRROR_ACCEPT_SPEC_TREE && ctx->ws_bytes >= L.end_accept) ? (double*)(ws + L.accept_scratch) : nullptr;
-    st = mirror_accept_launch(ctx, tree, ti, &in, out, s, tree_scratch);
+    st = mirror_accept_launch(ctx, tree, ti, &in, out, s, tree_scratch, defer ? &partials : nullptr, d_argmax);
     if (st != MIRROR_OK) return st;
     if (ev) MIRROR_CUDA_OK(cudaEventRecord(ctx->stage_ev[3], s));
     const mirror_accept_host_out* h = io ? io->h_out : nullptr;
