@@ -455,30 +455,17 @@ __device__ __noinline__ float2 move_offset(uint32_t s_addr, uint32_t o_addr, int
     return make_float2(next, alpha);
 }
 
-// Q as e4m3 codes.  The code is that of the correctly rounded quotient x / q_scale: the product with the rounded reciprocal is
-// corrected twice by its exact remainder (Markstein 1990), without a branch.  That holds for scales in 2^[-60, 60] and
-// numerators clamped to where the code saturates anyway (448; NaN stays NaN); other scales divide.
-struct QScale {
-    float s, inv, lim;
-    bool usual;
-    __device__ explicit QScale(float scale) : s(scale), inv(1.f / scale), lim(1000.f * scale), usual(scale >= 0x1p-60f && scale <= 0x1p60f) {}
-    __device__ __forceinline__ float quotient(float x) const {
-        asm("min.NaN.f32 %0, %0, %1;\n\tmax.NaN.f32 %0, %0, %2;" : "+f"(x) : "f"(lim), "f"(-lim));
-        float t = x * inv;
-        t = fmaf(fmaf(-t, s, x), inv, t);
-        return fmaf(fmaf(-t, s, x), inv, t);
-    }
-};
+// Q as e4m3 codes: those of the correctly rounded quotients x / q_scale.
 __device__ __noinline__ uint32_t unusual_codes(uint2 v, float s) {
-    return attn::pack_e4m3x4(__fdiv_rn(__uint_as_float(v.x << 16), s), __fdiv_rn(__uint_as_float(v.x & 0xffff0000u), s),
+    return pack_e4m3x4(__fdiv_rn(__uint_as_float(v.x << 16), s), __fdiv_rn(__uint_as_float(v.x & 0xffff0000u), s),
                              __fdiv_rn(__uint_as_float(v.y << 16), s), __fdiv_rn(__uint_as_float(v.y & 0xffff0000u), s));
 }
 // One row, four elements per lane, into the K-major operand tile `q` ([row][128 B], 128-byte swizzle).
-__device__ __forceinline__ void store_q_row(uint8_t* q, int row, uint2 v, const QScale& qs) {
+__device__ __forceinline__ void store_q_row(uint8_t* q, int row, uint2 v, const E4m3Scale& qs) {
     const int lane = threadIdx.x & 31;
     uint32_t code;
     if (qs.usual)
-        code = attn::pack_e4m3x4(qs.quotient(__uint_as_float(v.x << 16)), qs.quotient(__uint_as_float(v.x & 0xffff0000u)),
+        code = pack_e4m3x4(qs.quotient(__uint_as_float(v.x << 16)), qs.quotient(__uint_as_float(v.x & 0xffff0000u)),
                                  qs.quotient(__uint_as_float(v.y << 16)), qs.quotient(__uint_as_float(v.y & 0xffff0000u)));
     else
         code = unusual_codes(v, qs.s);
@@ -902,7 +889,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         const int q_all = p.gs * p.nodes_tile, q_grp = split ? 0 : cw >> 1, q_share = ((split ? (q_all + 3) >> 2 : (q_all + 1) >> 1) + 7) & ~7;
         const int q_row0 = (split ? cw : cw & 1) * q_share, q_rows = min(q_share, q_all - q_row0);
         const StreamId id = stream_of(p, rb, q_grp);
-        const QScale qs(p.q_scale);
+        const E4m3Scale qs(p.q_scale);
         uint2 qv[8];
         int left = n_tiles;
         uint32_t n_seg = 0, st = 0, ph = 0, wst = 0, wph = 1;
@@ -1030,7 +1017,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             // e4m3: the first segment's Q (the ones behind it are staged by the warps that widen V), each warp its rows, or (split)
             // half of them
             const int r0 = split ? grp * 16 : 0, r1 = split ? r0 + 16 : 32, buf = split ? 0 : grp * 2;
-            const QScale qs(p.q_scale);
+            const E4m3Scale qs(p.q_scale);
             const __nv_bfloat16* qrow = p.q + (((size_t)(sg.layer * p.B + sg.b) * p.n + node) * (size_t)p.Hq + (sg.g * p.heads_per_unit + id.head_off) * p.G + hl) * D;
             const uint32_t real = __ballot_sync(0xffffffffu, row_ok);
             // All rows are requested first, into the buffers of widened V, which are not in use yet.  (What this costs is mostly

@@ -682,7 +682,8 @@ bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk) {
 
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,
                                         void* partial_ws, size_t partial_bytes, cudaStream_t stream, int* n_partials,
-                                        const float* w_scale, const float* h_scale, int topk, void* topk_ws, size_t topk_ws_bytes) {
+                                        const float* w_scale, const float* h_scale, int topk, void* topk_ws, size_t topk_ws_bytes,
+                                        bool w_early) {
     const bool fp8 = w_scale != nullptr;
     if (fp8 && (!h_scale || ctx->desc.hidden % 128 != 0)) return MIRROR_ERR_SHAPE;
     // (e4m3 rows are staged exactly like bf16 rows of half as many elements: the same bytes, boxes and swizzle)
@@ -712,6 +713,7 @@ mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int
     const size_t P = p.n_chunks == 1 ? (size_t)2 * n_pairs : (size_t)2 * n_tiles;
     if (partial_bytes < P * M * 12) return MIRROR_ERR_WORKSPACE;
     p.w_keep = p.n_chunks > 1;
+    p.w_early = w_early;
     if (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_lm_left-- > 0) p.stall_after = ctx->tune.test_stall_after;
     p.inv_T = 1.0f / ctx->temperature;
     p.inv_T_log2e = p.inv_T * 1.4426950408889634f;

@@ -577,7 +577,8 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
                                    int32_t* argmax, float* maxlogit, float* lse, int32_t* topk_id,
                                    float* topk_logprob, float* gather_logit, float* logits_out,
                                    void* partial_ws, size_t partial_bytes, float* lse_scratch, cudaStream_t stream,
-                                   cudaEvent_t after_gemm, void* topk_logprob_bf16, void* topk_ws, size_t topk_ws_bytes, MirrorLmPartials* defer) {
+                                   cudaEvent_t after_gemm, void* topk_logprob_bf16, void* topk_ws, size_t topk_ws_bytes, MirrorLmPartials* defer,
+                                   bool w_early) {
     const int V = ctx->desc.vocab, H = ctx->desc.hidden;
     // Top-kappa inside the GEMM's epilogue whenever the caller's scratch holds the candidate lists; otherwise (or on the
     // single-CTA fallback kernel) the selection runs over spilled logits, which then have to be there.
@@ -589,7 +590,7 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
     if (M >= pair_min_rows && ctx->num_sms >= 2) {
         int P = 0;
         mirror_status st = mirror_lmhead_pair_launch(ctx, hidden, M, W, logits_out, partial_ws, partial_bytes, stream, &P, nullptr,
-                                                     nullptr, fused_topk ? topk : 0, topk_ws, topk_ws_bytes);
+                                                     nullptr, fused_topk ? topk : 0, topk_ws, topk_ws_bytes, w_early);
         if (st == MIRROR_OK) {
             if (after_gemm) MIRROR_CUDA_OK(cudaEventRecord(after_gemm, stream));
             const float inv_T = 1.0f / ctx->temperature, inv_T_log2e = inv_T * 1.4426950408889634f;
@@ -705,7 +706,10 @@ extern "C" mirror_status mirror_lmhead_reduce(mirror_ctx* ctx, const void* hidde
 // ---------------------------------------------------------------------------------------------------
 namespace {
 
-// one block per row: scale = max|x| / 448 (1 for an all-zero row), code = e4m3(x / scale), round to nearest even
+// one block per row: scale = max|x| / 448 (1 for an all-zero row), code = e4m3(x / scale), round to nearest even.
+// What bounds a few rows is latency: VEC (rows of whole 16-byte words) loads eight elements at a time, a row of up to 8192
+// all at once, and reads them once; 68 rows x 5120: 4.9 -> 1.9 us.
+template <bool VEC>
 __global__ void __launch_bounds__(256) quantize_rows_e4m3_kernel(const __nv_bfloat16* x, int cols, uint8_t* out, float* scale) {
     __shared__ float s_part[8];
     __shared__ float s_scale;
@@ -713,7 +717,25 @@ __global__ void __launch_bounds__(256) quantize_rows_e4m3_kernel(const __nv_bflo
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
     float amax = 0.f;
-    for (int c = threadIdx.x; c < cols; c += 256) amax = fmaxf(amax, fabsf(__bfloat162float(row[c])));
+    constexpr int kWords = VEC ? 4 : 1;
+    uint4 v[kWords];
+    const int words = cols / 8;
+    const bool kept = VEC && words <= 256 * kWords;
+    auto word_max = [&](const uint4& w) {
+        const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) amax = fmaxf(amax, fmaxf(fabsf(__uint_as_float(u[k] << 16)), fabsf(__uint_as_float(u[k] & 0xffff0000u))));
+    };
+    if (kept) {
+#pragma unroll
+        for (int k = 0; k < kWords; ++k) v[k] = threadIdx.x + 256 * k < words ? reinterpret_cast<const uint4*>(row)[threadIdx.x + 256 * k] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int k = 0; k < kWords; ++k) word_max(v[k]);
+    } else if (VEC) {
+        for (int c = threadIdx.x; c < words; c += 256) word_max(reinterpret_cast<const uint4*>(row)[c]);
+    } else {
+        for (int c = threadIdx.x; c < cols; c += 256) amax = fmaxf(amax, fabsf(__bfloat162float(row[c])));
+    }
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = amax;
     __syncthreads();
@@ -727,6 +749,21 @@ __global__ void __launch_bounds__(256) quantize_rows_e4m3_kernel(const __nv_bflo
     __syncthreads();
     const float sc = s_scale;
     uint8_t* dst = out + (size_t)blockIdx.x * cols;
+    const E4m3Scale es(sc);
+    if (VEC && es.usual) {
+#pragma unroll 1
+        for (int c = threadIdx.x; c < words; c += 256) {
+            const uint4 w = kept ? v[0] : reinterpret_cast<const uint4*>(row)[c];
+#pragma unroll
+            for (int k = 0; k + 1 < kWords; ++k) v[k] = v[k + 1];          // (rotated: registers take no index)
+            auto cv = [&](uint32_t a, uint32_t b) -> uint32_t {
+                return pack_e4m3x4(es.quotient(__uint_as_float(a << 16)), es.quotient(__uint_as_float(a & 0xffff0000u)),
+                                   es.quotient(__uint_as_float(b << 16)), es.quotient(__uint_as_float(b & 0xffff0000u)));
+            };
+            reinterpret_cast<uint2*>(dst)[c] = make_uint2(cv(w.x, w.y), cv(w.z, w.w));
+        }
+        return;
+    }
     for (int c = threadIdx.x; c < cols; c += 256)
         dst[c] = (uint8_t)__nv_cvt_float_to_fp8(__fdiv_rn(__bfloat162float(row[c]), sc), __NV_SATFINITE, __NV_E4M3);
 }
@@ -737,7 +774,8 @@ extern "C" mirror_status mirror_quantize_rows_fp8(mirror_ctx* ctx, const void* x
                                                   float* out_scale, void* stream) {
     if (!ctx || !x || !out_fp8 || !out_scale || rows <= 0 || cols <= 0) return MIRROR_ERR_ARG;
     MIRROR_CUDA_OK(cudaSetDevice(ctx->device));
-    MIRROR_CUDA_OK(mirror_launch_pdl(quantize_rows_e4m3_kernel, dim3((unsigned)rows), dim3(256), 0, (cudaStream_t)stream,
+    const bool vec = cols % 8 == 0 && !((uintptr_t)x & 15) && !((uintptr_t)out_fp8 & 7);
+    MIRROR_CUDA_OK(mirror_launch_pdl(vec ? quantize_rows_e4m3_kernel<true> : quantize_rows_e4m3_kernel<false>, dim3((unsigned)rows), dim3(256), 0, (cudaStream_t)stream,
                                      (const __nv_bfloat16*)x, cols, (uint8_t*)out_fp8, out_scale));
     ctx->launches += 1;
     MIRROR_CUDA_OK(cudaGetLastError());

@@ -93,14 +93,16 @@ struct MirrorLmPartials {
 mirror_status mirror_accept_launch(mirror_ctx* ctx, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                    const mirror_accept_in* in, const mirror_accept_out* out, cudaStream_t stream,
                                    double* tree_scratch = nullptr, const MirrorLmPartials* partials = nullptr, int32_t* argmax_out = nullptr);
-// defer: the row partials are not merged, but described there (only the argmax was asked for).
+// defer: the row partials are not merged, but described there (only the argmax was asked for).  w_early: no kernel that may
+// still be running when the one ahead of this launch begins writes W.
 mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, int topk,
                                    const int32_t* gather_row, const int32_t* gather_tok, int n_gather,
                                    int32_t* argmax, float* maxlogit, float* lse, int32_t* topk_id,
                                    float* topk_logprob, float* gather_logit, float* logits_out,
                                    void* partial_ws, size_t partial_bytes, float* lse_scratch, cudaStream_t stream,
                                    cudaEvent_t after_gemm = nullptr, void* topk_logprob_bf16 = nullptr,
-                                   void* topk_ws = nullptr, size_t topk_ws_bytes = 0, MirrorLmPartials* defer = nullptr);
+                                   void* topk_ws = nullptr, size_t topk_ws_bytes = 0, MirrorLmPartials* defer = nullptr,
+                                   bool w_early = false);
 // LM-head GEMM + per-unit row partials on CTA pairs (many hidden rows); *n_partials partials of [M] rows are left in
 // partial_ws for lmhead_merge_kernel.  mirror_lmhead_pair_partials(V) is that count.
 int mirror_lmhead_pair_partials(int V);
@@ -110,7 +112,7 @@ bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk);
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,
                                         void* partial_ws, size_t partial_bytes, cudaStream_t stream, int* n_partials,
                                         const float* w_scale = nullptr, const float* h_scale = nullptr,
-                                        int topk = 0, void* topk_ws = nullptr, size_t topk_ws_bytes = 0);
+                                        int topk = 0, void* topk_ws = nullptr, size_t topk_ws_bytes = 0, bool w_early = false);
 // Plain GEMM on CTA pairs: partial[s][M][N] (fp32) = x[M, K-slice s] * W[N, K-slice s]^T for the *k_slices slices that
 // mirror_linear_slices() picks (1 when the output tiles alone fill the GPU); the caller adds the slices in order.  w_early:
 // no kernel that may still be running when the one ahead of this launch begins writes W (see target_layer.cu).
@@ -377,6 +379,33 @@ __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.w
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 }  // namespace ptx
+
+// Four fp32 values as e4m3 codes in one word (element 0 in the lowest byte, as the tensor core reads an 8-bit operand);
+// values beyond +-448 saturate.
+__device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float d) {
+    uint32_t r;
+    asm("{\n\t.reg .b16 lo, hi;\n\t"
+        "cvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n\t"
+        "cvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n\t"
+        "mov.b32 %0, {lo, hi};\n\t}"
+        : "=r"(r) : "f"(a), "f"(b), "f"(c), "f"(d));
+    return r;
+}
+// Division by a scale on the way to e4m3: the correctly rounded quotient, which decides the code, without a branch.  The
+// product with the rounded reciprocal is corrected twice by its exact remainder (Markstein 1990).  That holds for `usual`
+// scales, 2^[-60, 60], and numerators clamped to where the code saturates anyway (448; NaN stays NaN); others divide.
+// (A division in the compiler's form is a branch each, and takes the slow one for zeros.)
+struct E4m3Scale {
+    float s, inv, lim;
+    bool usual;
+    __device__ explicit E4m3Scale(float scale) : s(scale), inv(1.f / scale), lim(1000.f * scale), usual(scale >= 0x1p-60f && scale <= 0x1p60f) {}
+    __device__ __forceinline__ float quotient(float x) const {
+        asm("min.NaN.f32 %0, %0, %1;\n\tmax.NaN.f32 %0, %0, %2;" : "+f"(x) : "f"(lim), "f"(-lim));
+        float t = x * inv;
+        t = fmaf(fmaf(-t, s, x), inv, t);
+        return copysignf(fmaf(fmaf(-t, s, x), inv, t), x);                 // (a zero keeps its sign)
+    }
+};
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t mirror_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
