@@ -182,6 +182,8 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     }
     if (ev) MIRROR_CUDA_OK(cudaEventRecord(ctx->stage_ev[1], s));
 
+    // (Its weights may be requested early: behind an attention launch, which waits for all before it, nothing of the caller's can
+    // still be writing them.)
     // LM-head rows: the given hidden states, else the last layer's attention output ([B*n, Hq*d] == [M, H])
     const void* rows = hidden;
     if (!rows) {
@@ -197,7 +199,7 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     const bool defer = !spec && M <= 256;
     st = mirror_lmhead_launch(ctx, rows, (int)M, W, 0, nullptr, nullptr, 0, d_argmax, nullptr, spec ? d_lse : nullptr, nullptr,
                               nullptr, nullptr, d_logits, ws + L.lm_partial, L.lm_partial_bytes, d_lse, s,
-                              ev ? ctx->stage_ev[2] : nullptr, nullptr, nullptr, 0, defer ? &partials : nullptr);
+                              ev ? ctx->stage_ev[2] : nullptr, nullptr, nullptr, 0, defer ? &partials : nullptr, !io);
     if (st != MIRROR_OK) return st;
 
     if (io) MIRROR_CUDA_OK(cudaStreamWaitEvent(s, ctx->copy_ev[kEvTokens], 0));
