@@ -8,29 +8,32 @@ namespace {
 
 struct CommitParams {
     int L, B, n, Hkv, d, gamma, max_pages, num_pages;
+    int advance;                          // 1: a block has all layers of its request, and moves the prefix itself
     long long layer_stride;               // elements between the layers' pools
     __nv_bfloat16* k_pool;
     __nv_bfloat16* v_pool;
     const __nv_bfloat16* k_new;           // [L, B, n, Hkv, d]
     const __nv_bfloat16* v_new;
     const int32_t* page_table;
-    const int32_t* prefix_len;
+    int32_t* prefix_len;
     const int32_t* accepted_nodes;        // [B, gamma]
     const int32_t* n_accepted;            // [B]
     int* status;
 };
 
-// grid (L, B): the block copies the (A + 1) x Hkv rows of d values of both tensors with 16-byte accesses
+// grid (L, B), or (1, B) when a request has so little to copy (16-byte accesses) that one block does it in a few steps: then the
+// prefix can be moved here as well, which saves the second launch (a third of the time for a toy model).
 __global__ void __launch_bounds__(256) kv_commit_kernel(const CommitParams p) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    const int layer = blockIdx.x, b = blockIdx.y;
+    const int b = blockIdx.y;
     int A = p.n_accepted[b];
     if (A < 0 || A > p.gamma) { if (threadIdx.x == 0 && atomicCAS(p.status, 0, MIRROR_DEV_CHECK) == 0) atomicExch(p.status + 1, 800); A = 0; }
     const int len = p.prefix_len[b];
     const int chunks_per_row = p.d / 8;                       // 16-byte chunks of one (token, head) row
-    const int total = (A + 1) * p.Hkv * chunks_per_row;
-    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+    const int per_layer = (A + 1) * p.Hkv * chunks_per_row, total = p.advance ? p.L * per_layer : per_layer;
+    for (int k = threadIdx.x; k < total; k += blockDim.x) {
+        const int layer = blockIdx.x + k / per_layer, i = k % per_layer;
         const int cc = i % chunks_per_row, h = (i / chunks_per_row) % p.Hkv, j = i / (chunks_per_row * p.Hkv);
         const int node = (j == 0) ? 0 : p.accepted_nodes[(size_t)b * p.gamma + j - 1];
         const int pos = len + j;
@@ -45,6 +48,10 @@ __global__ void __launch_bounds__(256) kv_commit_kernel(const CommitParams p) {
         const size_t dst = (size_t)layer * p.layer_stride + (((size_t)page * p.Hkv + h) * 16 + pos % 16) * p.d + cc * 8;
         *reinterpret_cast<uint4*>(p.k_pool + dst) = *reinterpret_cast<const uint4*>(p.k_new + src);
         *reinterpret_cast<uint4*>(p.v_pool + dst) = *reinterpret_cast<const uint4*>(p.v_new + src);
+    }
+    if (p.advance) {
+        __syncthreads();                                      // (every thread has read the old length)
+        if (threadIdx.x == 0) p.prefix_len[b] = len + A + 1;
     }
 }
 
@@ -84,9 +91,11 @@ static mirror_status kv_commit_impl(mirror_ctx* ctx, const mirror_kv* kv, const 
     p.accepted_nodes = accepted_nodes; p.n_accepted = n_accepted;
     p.status = ctx->d_status;
     cudaStream_t s = (cudaStream_t)stream;
-    MIRROR_CUDA_OK(mirror_launch_pdl(kv_commit_kernel, dim3((unsigned)p.L, (unsigned)p.B), dim3(256), 0, s, p));
-    MIRROR_CUDA_OK(mirror_launch_pdl(kv_advance_kernel, dim3((unsigned)((p.B + 127) / 128)), dim3(128), 0, s, p.B, p.gamma, n_accepted, prefix_len));
-    ctx->launches += 2;
+    p.advance = (long long)p.L * (p.gamma + 1) * p.Hkv * (p.d / 8) <= 4 * 256;
+    MIRROR_CUDA_OK(mirror_launch_pdl(kv_commit_kernel, dim3(p.advance ? 1u : (unsigned)p.L, (unsigned)p.B), dim3(256), 0, s, p));
+    ctx->launches += 1;
+    if (!p.advance) MIRROR_CUDA_OK(mirror_launch_pdl(kv_advance_kernel, dim3((unsigned)((p.B + 127) / 128)), dim3(128), 0, s, p.B, p.gamma, n_accepted, prefix_len));
+    if (!p.advance) ctx->launches += 1;
     MIRROR_CUDA_OK(cudaGetLastError());
     return MIRROR_OK;
 }
