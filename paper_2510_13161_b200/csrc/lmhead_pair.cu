@@ -173,10 +173,6 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
 // K maxima is at most the row's K-th best logit, since K different ids attain it.  A row whose maximum in a unit -- which
 // the reduction has anyway -- is below the bar is done with one comparison; after the first unit that is nearly every
 // row.  (What a list holds depends on timing, which candidates are best does not.)
-__device__ __forceinline__ uint32_t order_key(float x) {        // unsigned order = order of the floats; never 0
-    const uint32_t u = __float_as_uint(x);
-    return (u & 0x80000000u) ? ~u : u | 0x80000000u;
-}
 __device__ __forceinline__ size_t bar_word(int share, int row) { return ((size_t)share * kMaxChunkRows + row) * 8; }    // (a sector each)
 // Insertion by a whole warp: lane i has the list's i-th pair.
 __device__ __forceinline__ void topk_list_insert(float* lv, int* li, int K, float x, int xi) {
@@ -498,7 +494,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                     if (ok)
                         for (int w = 0; w < 4; ++w) {
                             const float m = all_max[w * kMaxChunkRows + c];
-                            if (m > -INFINITY) key = max(key, order_key(m));
+                            if (m > -INFINITY) key = max(key, mirror_order_key(m));
                         }
 #pragma unroll 4
                     for (int k = 0; k < K; ++k) {
@@ -513,7 +509,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                 const bool valid = q * 32 + lane < p.rows_cta && vid < p.V;
                 for (int cg = 0; ok && cg < n_cg; ++cg) {
                     const int c = cg * 32 + lane;
-                    unsigned cols = __ballot_sync(0xffffffffu, c < n_rows && unit_max[c] > -INFINITY && order_key(unit_max[c]) >= bars[c]);
+                    unsigned cols = __ballot_sync(0xffffffffu, c < n_rows && unit_max[c] > -INFINITY && mirror_order_key(unit_max[c]) >= bars[c]);
                     while (cols) {
                         const int j = __ffs(cols) - 1;
                         cols &= cols - 1;
@@ -522,7 +518,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                                      : "r"(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * p.acc_stride + cg * 32 + j)) : "memory");
                         asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(w) :: "memory");
                         const float x = valid ? __uint_as_float(w) : -INFINITY;
-                        unsigned hit = __ballot_sync(0xffffffffu, x > -INFINITY && order_key(x) >= bars[cg * 32 + j]);
+                        unsigned hit = __ballot_sync(0xffffffffu, x > -INFINITY && mirror_order_key(x) >= bars[cg * 32 + j]);
                         float* const lv = my_tv + (size_t)(cg * 32 + j) * K;
                         int* const li = my_ti + (size_t)(cg * 32 + j) * K;
                         if (__popc(hit) > 2) {

@@ -421,10 +421,13 @@ lmhead_topk_kernel(int V, int topk, float inv_T, const float* logits, const floa
 }
 
 // The same out of the candidate lists that the GEMM's epilogue left (n_lists = 4 P sorted lists of topk (logit, id) pairs per
-// row, laid out [list][row][topk], empty places hold -inf), behind the merge of the row's P partials.  One block per row;
-// a thread holds the heads of its lists, each round takes the best head and moves that list on, so a pair is read once
-// (rounds over all pairs took 41 us at 57 rows x 9472 candidates).  The row's bars are cleared for the next call.
+// row, laid out [list][row][topk], empty places hold -inf), behind the merge of the row's P partials.  One block per row.
+// The row's bar (the least of its words, see lmhead_pair.cu) is a lower bound of the topk-th best, so only what reaches it is
+// gathered, a few dozen pairs of the 9472, and each finds its own place by counting those before it.  Should more pass
+// than there is room for (many equal logits), rounds take the best head of all lists and move that list on, a barrier
+// each (8 rounds over 57 rows x 2368 lists take 4 us longer than counting).  The bars are cleared for the next call.
 constexpr int kListsPerThread = 2;
+constexpr int kMaxGathered = 1024;
 __global__ void __launch_bounds__(1024, 1)
 lmhead_topk_merge_kernel(int P, int topk, float inv_T, float inv_T_log2e, const float* part_max, const int* part_idx,
                          const float* part_sum, const float* list_v, const int* list_i, int32_t* argmax, float* maxlogit, float* lse,
@@ -435,7 +438,17 @@ lmhead_topk_merge_kernel(int P, int topk, float inv_T, float inv_T_log2e, const 
     const size_t stride = (size_t)M * topk, base = (size_t)row * topk;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (tid < topk) bars[((size_t)tid * kMaxChunkRows + row) * 8] = 0;         // (bar_word of lmhead_pair.cu)
+    __shared__ uint32_t s_bar;
+    __shared__ int s_n;
+    __shared__ float s_lse, s_cv[kMaxGathered];
+    __shared__ int s_ci[kMaxGathered];
+    if (warp == 0) {                               // (topk <= 32 words; bar_word and order_key of lmhead_pair.cu)
+        uint32_t* const word = bars + ((size_t)lane * kMaxChunkRows + row) * 8;
+        uint32_t key = lane < topk ? __ldcg(word) : 0xffffffffu;
+        if (lane < topk) *word = 0;
+        key = __reduce_min_sync(0xffffffffu, key);
+        if (lane == 0) { s_bar = key; s_n = 0; }
+    }
     const int n_lists = 4 * P;
     float row_lse = 0.f;                           // (thread 0's)
     float hv[kListsPerThread];
@@ -455,8 +468,46 @@ lmhead_topk_merge_kernel(int P, int topk, float inv_T, float inv_T_log2e, const 
         if (argmax) argmax[row] = r.idx;
         if (maxlogit) maxlogit[row] = r.m;
         if (lse) lse[row] = row_lse;
+        s_lse = row_lse;
     }
+    auto put = [&](int k, float v, int i) {
+        topk_id[base + k] = i;
+        const float lp = v * inv_T - s_lse;
+        if (topk_logprob) topk_logprob[base + k] = lp;
+        if (topk_logprob_bf16) topk_logprob_bf16[base + k] = __float2bfloat16_rn(lp);      // token-channel payload
+    };
     auto better = [](float v, int i, float w, int j) { return v > w || (v == w && i < j); };
+    // (the barrier inside fold_row lies between s_bar and here)
+#pragma unroll
+    for (int c = 0; c < kListsPerThread; ++c) {
+        float v = hv[c];
+        int i = hi[c];
+#pragma unroll 1
+        for (int at = 1; v > -INFINITY && mirror_order_key(v) >= s_bar; ++at) {
+            const int n = atomicAdd(&s_n, 1);
+            if (n >= kMaxGathered) break;
+            s_cv[n] = v;
+            s_ci[n] = i;
+            if (at == topk) break;
+            const size_t next = (size_t)(tid + c * 1024) * stride + base + at;
+            v = __ldcg(list_v + next);
+            i = __ldcg(list_i + next);
+        }
+    }
+    __syncthreads();
+    const int n = s_n;
+    if (n >= topk && n <= kMaxGathered) {
+        if (tid < n) {
+            const float v = s_cv[tid];
+            const int i = s_ci[tid];
+            int rank = 0;
+#pragma unroll 4
+            for (int k = 0; k < n; ++k) rank += better(s_cv[k], s_ci[k], v, i);
+            if (rank < topk) put(rank, v, i);
+        }
+        return;
+    }
+#pragma unroll 1
     for (int k = 0; k < topk; ++k) {
         float bv = hv[0];
         int bi = hi[0];
@@ -481,12 +532,7 @@ lmhead_topk_merge_kernel(int P, int topk, float inv_T, float inv_T_log2e, const 
 #pragma unroll
         for (int c = 0; c < kListsPerThread; ++c)
             if (hi[c] == bi && bi != 0x7fffffff) { ++pos[c]; load(c); }           // (ids are unique over all lists)
-        if (tid == 0) {
-            topk_id[base + k] = bi;
-            const float lp = bv * inv_T - row_lse;
-            if (topk_logprob) topk_logprob[base + k] = lp;
-            if (topk_logprob_bf16) topk_logprob_bf16[base + k] = __float2bfloat16_rn(lp);      // token-channel payload
-        }
+        if (tid == 0) put(k, bv, bi);
     }
 }
 

@@ -391,6 +391,11 @@ __device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float
         : "=r"(r) : "f"(a), "f"(b), "f"(c), "f"(d));
     return r;
 }
+__device__ __forceinline__ uint32_t mirror_order_key(float x) {        // unsigned order = order of the floats; never 0
+    const uint32_t u = __float_as_uint(x);
+    return (u & 0x80000000u) ? ~u : u | 0x80000000u;
+}
+
 // Division by a scale on the way to e4m3: the correctly rounded quotient, which decides the code, without a branch.  The
 // product with the rounded reciprocal is corrected twice by its exact remainder (Markstein 1990).  That holds for `usual`
 // scales, 2^[-60, 60], and numerators clamped to where the code saturates anyway (448; NaN stays NaN); others divide.
