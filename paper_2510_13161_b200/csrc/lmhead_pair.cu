@@ -227,7 +227,8 @@ __device__ __noinline__ void topk_list_merge(float* lv, int* li, int K, float x,
 // projections, split along K when there are fewer tiles than CTA pairs; the epilogue only stores fp32 partial sums.
 // kFp8 / kTopk: e4m3 operands with per-row scales / Top-kappa lists in the epilogue, as separate instantiations so that
 // the plain bf16 head carries none of their registers and branches.
-template <bool kReduce, bool kFp8, bool kTopk>
+// kEarly: a kernel of its own, since the few instructions that it adds in front of the wait cost the others 0.3-6% (code placement).
+template <bool kReduce, bool kFp8, bool kTopk, bool kEarly>
 __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CUtensorMap& tm_h, const PairParams& p) {
     extern __shared__ uint8_t smem_raw[];
     // (the dynamic shared window starts at the same offset in both CTAs, so the aligned layout is the same too)
@@ -272,7 +273,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
     const uint32_t tmem_base = ctrl->tmem_base;
     // The weights of the first stages, while the kernel ahead is still at work (their rows of x follow behind the wait).
     int n_early = 0;
-    if (p.w_early && warp == 0 && lane == 0 && pair < p.n_units) {
+    if (kEarly && p.w_early && warp == 0 && lane == 0 && pair < p.n_units) {
         int tile, slice, chunk;
         decode(pair, tile, slice, chunk);
         const int kb0 = slice * p.kb_per_slice;
@@ -294,20 +295,32 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
             int s = 0, n_issued = 0;
             uint32_t ph = 0;
             bool ok = true;
+            // the rows of x that belong to the weights requested early.  (A loop of its own: a test per K block in the main loop
+            // made 275 rows x 42306 x 2304 take 110 instead of 102 us.)
+            for (; kEarly && n_issued < n_early && ok; ++n_issued) {
+                if (p.stall_after >= 0 && n_issued >= p.stall_after) { ok = false; break; }           // (test aid, as below)
+                int tile, slice, chunk;
+                decode(pair, tile, slice, chunk);
+                tma_load_2d_pair(stage_base + s * p.stage_bytes + p.a_bytes, &tm_h, map_to_rank(&ctrl->full[s], 0), (slice * p.kb_per_slice + n_issued) * kBK,
+                                 chunk * p.chunk_rows + (int)rank * p.half_rows, pol_h);
+                if (++s == p.stages) { s = 0; ph ^= 1; }
+            }
+            int kb_skip = n_issued;
             for (int u = pair; u < p.n_units && ok; u += n_pairs) {
                 int tile, slice, chunk;
                 decode(u, tile, slice, chunk);
                 const int w_row = (tile * 2 + (int)rank) * p.rows_cta;
                 const int h_row = chunk * p.chunk_rows + (int)rank * p.half_rows;
                 const int kb_end = min(n_kb, (slice + 1) * p.kb_per_slice);
-                for (int kb = slice * p.kb_per_slice; kb < kb_end; ++kb) {
+                int kb = slice * p.kb_per_slice + kb_skip;
+                kb_skip = 0;
+                for (; kb < kb_end; ++kb) {
                     if (p.stall_after >= 0 && n_issued >= p.stall_after) { ok = false; break; }       // (test aid: neither arms nor copies)
                     if (ctrl->abort || !ptx::mbar_wait(&ctrl->empty[s], ph ^ 1, p.wait_limit)) { fail(p, ctrl, 11); ok = false; break; }
-                    const bool early = n_issued < n_early;
-                    if (rank == 0 && !early) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
+                    if (rank == 0) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
                     const uint32_t bar = map_to_rank(&ctrl->full[s], 0);
                     uint8_t* dst = stage_base + s * p.stage_bytes;
-                    if (!early) tma_load_2d_pair(dst, &tm_w, bar, kb * kBK, w_row, pol_w);
+                    tma_load_2d_pair(dst, &tm_w, bar, kb * kBK, w_row, pol_w);
                     tma_load_2d_pair(dst + p.a_bytes, &tm_h, bar, kb * kBK, h_row, pol_h);
                     ++n_issued;
                     if (++s == p.stages) { s = 0; ph ^= 1; }
@@ -481,6 +494,11 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                         }
                     }
                 }
+                if constexpr (!kTopk) {
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(map_to_rank(&ctrl->acc_empty[ab], 0));
+                }
             }
             if constexpr (kReduce && kTopk) {
                 // (all four warps meet here whatever happened to one of them)
@@ -534,7 +552,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                     }
                 }
             }
-            if (ok) {
+            if (kTopk && ok) {
                 ptx::tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(map_to_rank(&ctrl->acc_empty[ab], 0));
@@ -564,19 +582,23 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
 
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, false, false>(tm_w, tm_h, p);
+    pair_gemm_body<true, false, false, false>(tm_w, tm_h, p);
+}
+__global__ void __launch_bounds__(kThreads, 2)
+lmhead_pair_early_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
+    pair_gemm_body<true, false, false, true>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_topk_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, false, true>(tm_w, tm_h, p);
+    pair_gemm_body<true, false, true, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_fp8_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, true, false>(tm_w, tm_h, p);
+    pair_gemm_body<true, true, false, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 linear_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<false, false, false>(tm_w, tm_h, p);
+    pair_gemm_body<false, false, false, true>(tm_w, tm_h, p);
 }
 
 int next_pow2(int x) {
@@ -641,6 +663,7 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
     const size_t smem = (size_t)p.stages * p.stage_bytes + kCtrlBytes + (p.topk > 0 ? kTopkBytes : 0) + 1024;
     if (!ctx->lm_pair_attr_set) {
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+        MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_early_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_fp8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(linear_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
@@ -661,7 +684,7 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     if (p.fp8 && (p.topk > 0 || !reduce)) return MIRROR_ERR_UNSUPPORTED;
-    auto kern = !reduce ? linear_pair_kernel : p.fp8 ? lmhead_pair_fp8_kernel : p.topk > 0 ? lmhead_pair_topk_kernel : lmhead_pair_kernel;
+    auto kern = !reduce ? linear_pair_kernel : p.fp8 ? lmhead_pair_fp8_kernel : p.topk > 0 ? lmhead_pair_topk_kernel : p.w_early ? lmhead_pair_early_kernel : lmhead_pair_kernel;
     MIRROR_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, tm_w, tm_h, p));
     ctx->launches += 1;
     MIRROR_CUDA_OK(cudaGetLastError());
@@ -709,7 +732,7 @@ mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int
     const size_t P = p.n_chunks == 1 ? (size_t)2 * n_pairs : (size_t)2 * n_tiles;
     if (partial_bytes < P * M * 12) return MIRROR_ERR_WORKSPACE;
     p.w_keep = p.n_chunks > 1;
-    p.w_early = w_early;
+    p.w_early = w_early && ctas_per_sm_for(ctx->tune, M) == 2;       // (a weight stream; with more rows the tensor cores set the pace)
     if (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_lm_left-- > 0) p.stall_after = ctx->tune.test_stall_after;
     p.inv_T = 1.0f / ctx->temperature;
     p.inv_T_log2e = p.inv_T * 1.4426950408889634f;
