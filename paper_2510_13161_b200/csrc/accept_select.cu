@@ -407,7 +407,10 @@ accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
     int r = 0, A = 0, n_rej = 0, n_children = 0;
     double* const buf0 = a.tree_scratch ? a.tree_scratch + (size_t)b * 2 * V : nullptr;
     double* const buf1 = buf0 ? buf0 + V : nullptr;
-    int cur = 0;                                   // buffer that holds the current residual (when n_rej > 0)
+    // Buffer that holds the current residual (when n_rej > 0).  Residuals go to the two buffers in turn for the whole walk, never
+    // back to buf0 at a new row: a slower CTA may still be at the test that led there, which reads m[token] from `cur`.  What was
+    // last read from the other buffer lies behind the barrier of the pass that made `cur` the current one.
+    int cur = 0;
     double inv_Z = 1.0;                            // 1 / Z of the last effective rejection
     // m[v] at row r after the rejections recorded so far, from the logit or (kept) the unnormalised residual
     auto source = [&](const float* lr, int v) -> double { return buf0 && n_rej > 0 ? (cur ? buf1 : buf0)[v] : (double)lr[v]; };
@@ -443,7 +446,7 @@ accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
             }
             // rejected: normaliser of the residual (a residual without mass leaves m as it is)
             const float* qc = a.q_probs + ((size_t)b * (n - 1) + (c - 1)) * V;
-            double* const nxt = !buf0 ? nullptr : ((n_rej > 0 && cur == 0) ? buf1 : buf0);      // the buffer not in use
+            double* const nxt = !buf0 ? nullptr : (cur ? buf0 : buf1);
             draw.sums([&](int v) { return Loaded{source(lr, v), qc[v]}; },
                       [&](int v, const Loaded& in, double& x, double&) {
                           const double res = fmax(mass(in.m, lse_r, v) - (double)in.q, 0.0);

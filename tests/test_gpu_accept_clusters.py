@@ -35,3 +35,36 @@ def test_draws_at_the_edges_of_the_split(mode, V, B):
                 # (as in test_gpu_accept: fp64 sums in another order may differ on a knife edge only)
                 same = all(np.array_equal(got[f][b], ref[f][b]) for f in FIELDS if f != "reuse_slot")
                 assert same or ref["margin"][b] < 1e-9, (b, u, ref["margin"][b], {f: (got[f][b], ref[f][b]) for f in FIELDS})
+
+
+@pytest.mark.parametrize("V,B", [(70001, 1), (70001, 4), (40000, 9)])       # 16 and 8 CTAs per request
+def test_walk_that_rejects_accepts_and_rejects_again(V, B):
+    """A sibling is rejected (the residual goes to scratch memory), the next one passes the test against that residual, and its
+    child is rejected: the child's residual must not land where a slower CTA of the cluster still reads the sibling's test."""
+    kappa, gamma = 3, 3
+    m = make_mirror(cfg_for(V, kappa, gamma, B))
+    par = I.comb_parent(kappa, gamma)
+    logits, qp, tok, ua, ur = spec_case(B, kappa, gamma, V, 3 * V + B)
+    first = lambda k: 1 + k * gamma                             # noqa: E731  (root's k-th child)
+    for b in range(B):
+        for c, u in ((first(0), 1.0), (first(1), 0.0), (first(1) + 1, 1.0)):
+            ua[b, c] = u
+            if u == 1.0:                                        # q far above p at the token: rejected
+                qp[b, c - 1] *= 0.5
+                qp[b, c - 1, tok[b, c]] += 0.5
+    lse = torch.logsumexp(logits.double(), -1).float()
+    ref = O.accept_tree(tok.numpy(), logits.numpy(), lse.numpy(), qp.numpy(), ua.numpy(), ur.numpy(), par, gamma, True, 1.0)
+    assert (ref["n_accepted"] == 1).all() and (ref["accepted_nodes"][:, 0] == first(1)).all()
+    acc = m.accept_in(binding.ACCEPT_SPEC_TREE, True, logits=logits.cuda(), lse=lse.cuda(), q_probs=qp.cuda(), u_accept=ua.cuda(),
+                      u_resample=ur.cuda())
+    tree = m.tree(tok.cuda(), kappa, gamma)
+    first_run = None
+    for _ in range(100):
+        got = m.mirror_accept_select(tree, acc, tree_scratch=True).cpu()
+        first_run = first_run or got
+        for f in FIELDS:
+            assert np.array_equal(got[f], first_run[f]), f
+    assert m.device_status() == (0, 0)
+    for b in range(B):
+        same = all(np.array_equal(first_run[f][b], ref[f][b]) for f in FIELDS if f != "reuse_slot")
+        assert same or ref["margin"][b] < 1e-9, (b, ref["margin"][b])
