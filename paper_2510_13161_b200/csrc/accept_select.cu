@@ -68,14 +68,15 @@ __device__ __forceinline__ double warp_sum(double v) {
 struct NodeTest {
     double p, q, u;
 };
+__device__ __forceinline__ void bad_token(const AcceptArgs& a, int c) {      // (first error wins)
+    if (atomicCAS(a.status, 0, MIRROR_DEV_CHECK) == 0) atomicExch(a.status + 1, 100 + c);
+}
+// ok: the token is in the vocabulary (a node without one is rejected, and reported by whoever comes to it).
 __device__ __forceinline__ NodeTest node_test(const AcceptTreeParams& tp, const AcceptArgs& a, int b, int c, bool& ok) {
     NodeTest t = {0.0, 0.0, 0.0};
     const int x = a.tokens[(size_t)b * tp.n + c];
     ok = x >= 0 && x < a.V;
-    if (!ok) {
-        if (atomicCAS(a.status, 0, MIRROR_DEV_CHECK) == 0) atomicExch(a.status + 1, 100 + c);   // first error wins
-        return t;
-    }
+    if (!ok) return t;
     const size_t row = (size_t)b * tp.n + tp.parent[c];
     t.u = (double)a.u_accept[(size_t)b * tp.n + c];
     t.q = (double)a.q_probs[((size_t)b * (tp.n - 1) + (c - 1)) * a.V + x];
@@ -335,6 +336,7 @@ accept_spec_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
     if (tid > 0 && tid < n) {
         bool ok;
         const NodeTest t = node_test(tp, a, b, tid, ok);
+        if (!ok) bad_token(a, tid);
         s_pass[tid] = ok && t.u * t.q <= t.p;
     }
     __syncthreads();
@@ -443,6 +445,8 @@ accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
             if (s_ok[c]) {
                 const NodeTest t = s_test[c];
                 if (t.u * t.q <= (n_rej == 0 ? t.p : mass(source(lr, tok[c]), lse_r, tok[c]))) { next = c; break; }
+            } else if (tid == 0) {
+                bad_token(a, c);
             }
             // rejected: normaliser of the residual (a residual without mass leaves m as it is)
             const float* qc = a.q_probs + ((size_t)b * (n - 1) + (c - 1)) * V;

@@ -68,3 +68,29 @@ def test_walk_that_rejects_accepts_and_rejects_again(V, B):
     for b in range(B):
         same = all(np.array_equal(first_run[f][b], ref[f][b]) for f in FIELDS if f != "reuse_slot")
         assert same or ref["margin"][b] < 1e-9, (b, ref["margin"][b])
+
+
+@pytest.mark.parametrize("scratch", [False, True])
+def test_tree_rule_reports_tokens_outside_the_vocabulary_where_the_walk_meets_them(scratch):
+    """A node that the walk never comes to may hold anything (a padded tree); one that it comes to is rejected and reported."""
+    V, kappa, gamma, B = 9000, 3, 2, 2
+    m = make_mirror(cfg_for(V, kappa, gamma, B))
+    logits, qp, tok, ua, ur = spec_case(B, kappa, gamma, V, 17)
+    ua[:, 1] = ua[:, 2] = 0.0                                   # the first branch is accepted to its end
+    lse = torch.logsumexp(logits.double(), -1).float()
+    acc = m.accept_in(binding.ACCEPT_SPEC_TREE, True, logits=logits.cuda(), lse=lse.cuda(), q_probs=qp.cuda(), u_accept=ua.cuda(),
+                      u_resample=ur.cuda())
+    run = lambda t: m.mirror_accept_select(m.tree(t.cuda(), kappa, gamma), acc, tree_scratch=scratch).cpu()      # noqa: E731
+    ref = run(tok)
+    assert m.device_status() == (0, 0) and (ref["n_accepted"] == gamma).all()
+    padded = tok.clone()
+    padded[:, 1 + gamma:] = -1                                  # the other branches
+    got = run(padded)
+    assert m.device_status() == (0, 0)
+    for f in FIELDS:
+        assert np.array_equal(got[f], ref[f]), f
+    met = tok.clone()
+    met[1, 1] = V                                               # the first test of the second request
+    got = run(met)
+    assert m.device_status() == (6, 101)
+    assert got["n_accepted"][0] == gamma and 1 not in got["accepted_nodes"][1]
