@@ -1257,7 +1257,8 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         }
     }
     p.mode = p.n_rt == 1 ? kSplit : kPaired;
-    p.heads_per_unit = (p.n_rt > 1 && p.n_rt % 2 == 1 && Hkv % 2 == 0) ? 2 : 1;
+    // (a group of two heads needs a CTA per row tile: not with more row tiles than SMs, where a head alone still fits)
+    p.heads_per_unit = (p.n_rt > 1 && p.n_rt % 2 == 1 && Hkv % 2 == 0 && p.n_rt <= ctx->num_sms) ? 2 : 1;
     p.n_cta = p.heads_per_unit == 2 ? p.n_rt : (p.n_rt + 1) / 2;
     p.n_groups = ctx->num_sms / p.n_cta;
     if (ctx->tune.attn_groups >= 1 && ctx->tune.attn_groups <= p.n_groups) p.n_groups = ctx->tune.attn_groups;
