@@ -1268,7 +1268,7 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     // kernel behind a cut would: a launch and a pass over the records, ~6 us.
     const bool whole = ctx->tune.attn_whole_units != 0;
     const int64_t units = (int64_t)p.L * p.B * (Hkv / p.heads_per_unit);
-    if (units >= (1 << 24)) return MIRROR_ERR_SHAPE;
+    if (units > 0x7fffffff) return MIRROR_ERR_SHAPE;        // (a unit has a tile at least: the tiles are counted in 31 bits)
     p.units = (int)units;
     p.whole_groups = whole && units >= p.n_groups ? attn::whole_unit_groups(p.n_groups, units) : 0;
     p.never_cut = whole && (kv->max_pages_per_req + (p.n + kSlotTok - 1) / kSlotTok + kTileSlots - 1) / kTileSlots <= 6;

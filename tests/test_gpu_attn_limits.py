@@ -16,3 +16,18 @@ def test_more_row_tiles_than_sms(hq, kappa, gamma):
     x = I.gen_verify_inputs(cfg, 3, "cuda", with_lm_head=False)
     out, lse = run_gpu(make_mirror(cfg), x)
     compare(out, lse, oracle_attention(x), range(cfg.layers))
+
+
+def test_very_many_units():
+    """2^24 units of one token each: a token that sees only itself gets its own value back."""
+    L, B, H, d = 128, 1024, 128, 64
+    cfg = I.VerifyConfig("t", 1024, H, H, d, L, B, 0, 0, 1, 1, 64, "greedy", 0.02, 1.0)
+    m = make_mirror(cfg)
+    new = lambda: torch.zeros((L, B, 1, H, d), dtype=torch.bfloat16, device="cuda")       # noqa: E731
+    pool = torch.zeros((L, 1, H, 16, d), dtype=torch.bfloat16, device="cuda")
+    q, k, v, out = new(), new(), new().normal_(0, 1), new()
+    kv = m.kv(pool, pool, torch.zeros((B, 1), dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda"))
+    tree = m.tree(torch.zeros((B, 1), dtype=torch.int32, device="cuda"), 1, 1, parent=[-1])
+    m.mirror_attn_verify(kv, tree, q, k, v, out=out)
+    assert m.device_status() == (0, 0)
+    assert torch.equal(out, v)
