@@ -24,7 +24,7 @@
 //               of it reads without waiting for its completion.  Warp 1 owns TMEM
 //   warps 4..7, 8..11  softmax of stream 0 and of stream 1, one thread per row (TMEM lane): P = exp2(s * c - offset)
 //               over the first half of S's columns as bf16.  The row's offset is the maximum of the first tile in which
-//               it sees anything; it moves only when a half tile's sum of P passes 2^80 (that half is then redone from
+//               it sees anything; it moves only when a half tile's sum of P passes 2^14 (that half is then redone from
 //               S, which is still there), and is carried exactly through the sum and the division.
 // e4m3 cache (d = 128; F8): Q K^T multiplies codes (kind::f8f6f4, Q divided by its scale and rounded when it is staged), but P V
 // does not: four more warps (12..15) widen each V tile to f16, exactly, and P is f16.  In an 8-bit P V, P as e4m3 costs 2.6% of
@@ -64,9 +64,9 @@ constexpr int kTileSlots = 8;
 constexpr int kTileTok = kSlotTok * kTileSlots;     // 128
 constexpr int kRows = 128;                          // UMMA M: rows of a stream
 constexpr int kMaxStages = 10;
-// A half tile whose sum of P stays below this is as it should be: no P of it overflows its 16-bit format (bf16: 2^80, so that
-// no sum of them overflows fp32 either; f16, of the e4m3 cache: 2^14).
-template <bool F8> constexpr float kSumLimit = F8 ? 16384.f : 1.2089258196146292e24f;
+// A half tile whose sum of P stays below this is as it should be: no P of it overflows f16 (e4m3 cache), and sums of P V stay in
+// fp32's range for values up to 2^113 (bf16 P would allow more, but values of 1e25 under P of 2^43 already overflow).
+constexpr float kSumLimit = 16384.f;
 constexpr int kTmemCols = 512;
 constexpr int kTmemO = 2 * kTileTok;
 constexpr int kCtrlBytes = 528;
@@ -1088,7 +1088,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                         // then this half is redone.  (The accumulator may be touched: the tile before was multiplied before this
                         // tile was scored, and for this tile's first half there is a barrier.)
                         if (h == 1 && !redone) pass_turn();
-                        const bool grow = half_sum > kSumLimit<F8> && !redone;
+                        const bool grow = half_sum > kSumLimit && !redone;
                         if (__any_sync(0xffffffffu, grow)) {
                             tmem_ld_wait32(ra);
                             if (h == 1) {

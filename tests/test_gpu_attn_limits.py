@@ -1,4 +1,5 @@
 """Attention at the ends of what it accepts."""
+import numpy as np
 import pytest
 import torch
 
@@ -31,3 +32,22 @@ def test_very_many_units():
     m.mirror_attn_verify(kv, tree, q, k, v, out=out)
     assert m.device_status() == (0, 0)
     assert torch.equal(out, v)
+
+
+@pytest.mark.parametrize("hq", [4, 32])                     # one row tile per head, and two
+@pytest.mark.parametrize("grow", [13.0, 30.0, 50.0])        # nats by which the last page's scores exceed those of the first tile
+def test_large_values_behind_scores_that_grow(hq, grow):
+    """Values of 1e25 under weights that grow along the keys: sums of weights times values stay in fp32's range."""
+    cfg = config(hq, 2, 128, 2, 4, 600, 600, batch=1)
+    x = I.gen_verify_inputs(cfg, 9, "cuda", with_lm_head=False, shuffle_pages=False)
+    x.q.fill_(1.0)
+    x.k_pool.zero_(); x.k_new.zero_()
+    page = int(x.page_table[0, 36])
+    x.k_pool[0, page] = grow / 128.0 * np.sqrt(128.0)
+    x.v_pool.mul_(1e25); x.v_new.mul_(1e25)
+    out, lse = run_gpu(make_mirror(cfg), x)
+    o_ref, lse_ref = oracle_attention(x)[0]
+    assert torch.isfinite(out.float()).all()
+    # bf16 weights (equal ones here: 2^-9 of their sum at most) and bf16 outputs
+    assert np.abs(out[0].float().cpu().numpy() - o_ref).max() <= 1e-2 * np.abs(o_ref).max()
+    assert np.abs(lse[0].cpu().numpy() - lse_ref).max() <= 2e-3
