@@ -116,6 +116,7 @@ __device__ __forceinline__ void merge_boundary(const GroupBegin* table, int n_gr
     // One load: n_ch chunks (c0, c0 + n_blocks, ...) of the parts [k0, k0 + nk), with the parts' (max, sum) unless n_ch < 0 (then
     // only those).  false: the copies did not arrive (reported).
     auto fetch = [&](int k0, int nk, int c0, int n_ch, bool ml) -> bool {
+        ptx::fence_proxy_async();          // (the weights that weigh() stored where the copies land)
         __syncthreads();
         if (tid == 0) ptx::mbar_arrive_expect_tx(&s_bar, (uint32_t)(nk * (n_ch * 4096 + (ml ? 1024 : 0))));
         __syncthreads();

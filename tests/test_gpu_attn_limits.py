@@ -6,6 +6,7 @@ import torch
 from paper_2510_13161_b200 import inputs as I
 from tests.helpers import make_mirror, oracle_attention
 from tests.test_gpu_attn import compare, run_gpu
+from tests.test_gpu_attn_fp8 import run_and_compare, small
 from tests.test_gpu_attn_tiles import config
 
 pytestmark = pytest.mark.gpu
@@ -51,3 +52,27 @@ def test_large_values_behind_scores_that_grow(hq, grow):
     # bf16 weights (equal ones here: 2^-9 of their sum at most) and bf16 outputs
     assert np.abs(out[0].float().cpu().numpy() - o_ref).max() <= 1e-2 * np.abs(o_ref).max()
     assert np.abs(lse[0].cpu().numpy() - lse_ref).max() <= 2e-3
+
+
+@pytest.mark.parametrize("hq,hkv,d,prefix", [
+    (8, 1, 128, 40000),       # 148 parts, one row tile
+    (8, 1, 64, 20000),        # 79 parts
+    (32, 1, 128, 40000),      # 74 parts, four row tiles
+    (20, 4, 128, 33000),      # four units of 37 parts
+    (4, 4, 128, 17000),       # four units of 37 parts, few rows
+])
+def test_units_that_many_groups_share(hq, hkv, d, prefix):
+    """More parts per unit than the merge has room for at a time: it takes them in batches."""
+    cfg = config(hq, hkv, d, 3, 4, prefix, prefix, batch=1)
+    x = I.gen_verify_inputs(cfg, 13, "cuda", with_lm_head=False)
+    m = make_mirror(cfg)
+    out, lse = run_gpu(m, x)
+    compare(out, lse, oracle_attention(x), range(cfg.layers))
+    for _ in range(20):
+        again, lse2 = run_gpu(m, x)
+        assert torch.equal(again, out) and torch.equal(lse2, lse)
+
+
+@pytest.mark.parametrize("hq,hkv", [(8, 1), (32, 1), (20, 4)])
+def test_units_that_many_groups_share_over_an_8_bit_cache(hq, hkv):
+    run_and_compare(small(n_q_heads=hq, n_kv_heads=hkv, prefix_lo=33000, prefix_hi=33000, batch=1, layers=1), 14)
