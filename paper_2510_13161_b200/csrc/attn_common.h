@@ -80,10 +80,11 @@ constexpr int kMergeSmem = kMergeSlots * 10 * 128 * 4;      // their columns, th
 // and the arithmetic runs out of shared memory (17 parts of 85 rows: 15 us with loads in the loop over the parts, 8 with
 // eight parts' loads in flight).
 // map(row, GroupBegin) -> false, or the row's node and query head; record(group, slot) -> its record in slot 0 (of the unit
-// that began before the group's range) or 1, [column][128 rows], D accumulator columns, then (max, sum).
+// that began before the group's range) or 1, [column][128 rows], D accumulator columns, then (max, sum).  wait_limit: SM cycles
+// after which a wait gives up; stall: test aid, 1 makes the first wait run out (it expects bytes that nobody copies).
 template <int D, class Map, class Record>
 __device__ __forceinline__ void merge_boundary(const GroupBegin* table, int n_groups, int n, int Hq, int B, __nv_bfloat16* out, float* lse_out,
-                                               int* status, Map map, Record record) {
+                                               int* status, long long wait_limit, int stall, Map map, Record record) {
     extern __shared__ __align__(128) float s_cols[];                            // [slot][8 columns][128 rows]
     float(*const s_ml)[2][128] = (float(*)[2][128])(s_cols + kMergeSlots * 8 * 128);     // [part][max, then weight | sum][128 rows]
     __shared__ GroupBegin s_begin[512];
@@ -118,7 +119,7 @@ __device__ __forceinline__ void merge_boundary(const GroupBegin* table, int n_gr
     auto fetch = [&](int k0, int nk, int c0, int n_ch, bool ml) -> bool {
         ptx::fence_proxy_async();          // (the weights that weigh() stored where the copies land)
         __syncthreads();
-        if (tid == 0) ptx::mbar_arrive_expect_tx(&s_bar, (uint32_t)(nk * (n_ch * 4096 + (ml ? 1024 : 0))));
+        if (tid == 0) ptx::mbar_arrive_expect_tx(&s_bar, (uint32_t)(nk * (n_ch * 4096 + (ml ? 1024 : 0)) + 16 * stall));
         __syncthreads();
         for (int i = warp; i < nk * (n_ch + 1); i += kMergeThreads / 32) {
             const int c = i / nk, k = i - c * nk;
@@ -130,9 +131,12 @@ __device__ __forceinline__ void merge_boundary(const GroupBegin* table, int n_gr
                 asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                              ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(c == n_ch ? 1024u : 4096u), "r"(ptx::smem_u32(&s_bar)) : "memory");
         }
-        const bool ok = ptx::mbar_wait(&s_bar, phase);
+        const bool ok = ptx::mbar_wait(&s_bar, phase, wait_limit);
+        if (!ok) {
+            if (atomicCAS(status, 0, MIRROR_DEV_TIMEOUT) == 0) atomicExch(status + 1, 38);
+            ptx::mbar_wait(&s_bar, phase, 20000000ll);       // (the block's shared memory is not given back under copies in flight)
+        }
         phase ^= 1;
-        if (!ok && atomicCAS(status, 0, MIRROR_DEV_TIMEOUT) == 0) atomicExch(status + 1, 38);
         return __syncthreads_and(ok);
     };
     auto weigh = [&](int nk, float M) {                                         // maxima -> weights

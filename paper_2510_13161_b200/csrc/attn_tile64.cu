@@ -86,6 +86,7 @@ struct AttnParams {
     int* status;
     long long wait_limit;                 // SM cycles after which a wait gives up
     int stall_after;                      // test aid: the K producer stops after this many stages (-1: never)
+    int stall_merge;                      // test aid: 1: the merge's first wait runs out
 };
 
 struct UnitPos {                          // where a global tile index falls (indexes fit 31 bits: checked in the prologue)
@@ -863,7 +864,7 @@ template <int D>
 __global__ void __launch_bounds__(attn::kMergeThreads) attn_tile64_merge_kernel(const __grid_constant__ AttnParams p) {
     const int rb = blockIdx.y;
     attn::merge_boundary<D>(
-        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out, p.status,
+        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out, p.status, p.wait_limit, p.stall_merge,
         [&](int row, const attn::GroupBegin& u, int& node, int& head) {
             const int r_abs = rb * p.rows_per_rb + row;
             node = r_abs / p.G;
@@ -891,6 +892,7 @@ mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, co
     p.whole_groups = ctx->tune.attn_whole_units ? attn::whole_unit_groups(p.n_groups, (long long)kv->num_layers * tree->batch * ctx->desc.n_kv_heads) : 0;
     p.wait_limit = ctx->tune.wait_limit_cycles;
     p.stall_after = (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_attn_left-- > 0) ? ctx->tune.test_stall_after : -1;
+    p.stall_merge = ctx->tune.test_stall_merges > 0 && ctx->tune.test_stall_merges-- > 0;
     p.max_pages = kv->max_pages_per_req; p.num_pages = kv->num_pages;
     const int64_t page_elems = (int64_t)Hkv * kSlotTok * D;
     if (kv->layer_stride % page_elems != 0) return MIRROR_ERR_UNSUPPORTED;

@@ -106,6 +106,7 @@ struct AttnParams {
     int* status;
     long long wait_limit;                 // SM cycles after which a wait gives up
     int stall_after;                      // test aid: the K producer stops after this many stages (-1: never)
+    int stall_merge;                      // test aid: 1: the merge's first wait runs out
 };
 
 struct Maps {
@@ -1224,7 +1225,7 @@ __global__ void __launch_bounds__(attn::kMergeThreads) attn_merge_kernel(const _
     const int rb = blockIdx.y / n_str, grp = blockIdx.y % n_str;
     const StreamId id = stream_of(p, rb, grp);
     attn::merge_boundary<D>(
-        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out, p.status,
+        p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out, p.status, p.wait_limit, p.stall_merge,
         [&](int row, const attn::GroupBegin& u, int& node, int& head) {
             const int hl = (id.rt / p.node_tiles) * p.gs + row % p.gs;
             node = (id.rt % p.node_tiles) * p.nodes_tile + row / p.gs;
@@ -1274,6 +1275,7 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     p.never_cut = whole && (kv->max_pages_per_req + (p.n + kSlotTok - 1) / kSlotTok + kTileSlots - 1) / kTileSlots <= 6;
     p.wait_limit = ctx->tune.wait_limit_cycles;
     p.stall_after = (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_attn_left-- > 0) ? ctx->tune.test_stall_after : -1;
+    p.stall_merge = ctx->tune.test_stall_merges > 0 && ctx->tune.test_stall_merges-- > 0;
     p.max_pages = kv->max_pages_per_req; p.num_pages = kv->num_pages;
     const int64_t page_elems = (int64_t)Hkv * kSlotTok * D;
     if (kv->layer_stride % page_elems != 0) return MIRROR_ERR_UNSUPPORTED;

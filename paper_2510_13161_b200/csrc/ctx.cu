@@ -78,6 +78,7 @@ void mirror_tuning_from_env(MirrorTuning* t) {
     geti("MIRROR_LM_PAIR_MIN_ROWS", &t->lm_pair_min_rows, 0, 1 << 30);
     geti("MIRROR_LM_KGROUP", &t->lm_kgroup, 1, 64);
     geti("MIRROR_TEST_STALL_AFTER_STAGES", &t->test_stall_after, 0, 1 << 30);
+    geti("MIRROR_TEST_STALL_MERGES", &t->test_stall_merges, 0, 1 << 30);
     if (const char* e = getenv("MIRROR_WAIT_LIMIT_CYCLES")) { const long long x = strtoll(e, nullptr, 10); if (x >= 1000) t->wait_limit_cycles = x; }
 }
 

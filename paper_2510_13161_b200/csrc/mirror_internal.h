@@ -21,7 +21,7 @@ struct MirrorTreeInfo {            // host-side digest of one token tree, rebuil
 };
 
 // Tuning values, read ONCE from the environment when a context is created (defaults measured on B200); a context made
-// on the stack by the no-allocation entry point keeps the defaults.  The last two exist for the tests of the bounded
+// on the stack by the no-allocation entry point keeps the defaults.  The last ones exist for the tests of the bounded
 // waits: a short limit, and a producer that stops issuing copies after a number of stages, so that a consumer's wait
 // runs out and the kernel has to unwind (nothing traps, nothing spins without limit, no memory fault is provoked).
 struct MirrorTuning {
@@ -38,6 +38,7 @@ struct MirrorTuning {
     int test_stall_after = -1;       // MIRROR_TEST_STALL_AFTER_STAGES: a producer issues this many stages, then stops (-1: off);
                                      // applies to the FIRST attention launch and the first LM-head launch of a context only
     int test_stall_attn_left = 1, test_stall_lm_left = 1;
+    int test_stall_merges = 0;       // MIRROR_TEST_STALL_MERGES: in this many attention launches the merge's first wait runs out
 };
 void mirror_tuning_from_env(MirrorTuning* t);
 

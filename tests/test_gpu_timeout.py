@@ -67,3 +67,21 @@ def test_lmhead_pair_wait_runs_out_and_the_context_stays_usable(M, monkeypatch):
     for r in np.nonzero(got != red["argmax"])[0]:
         assert logits[r, red["argmax"][r]] - logits[r, got[r]] < 2e-3
     assert np.abs(res["lse"].cpu().numpy() - red["lse"]).max() <= 2e-3
+
+
+@pytest.mark.parametrize("prefix", [3000, 40000])          # a unit's parts in one batch, and in several
+def test_attention_merge_wait_runs_out_and_the_context_stays_usable(prefix, monkeypatch):
+    cfg = I.VerifyConfig("t", 1024, 8, 1, 128, 1, 1, prefix, prefix, 3, 4, 64, "greedy", 0.02, 1.0)
+    x = I.gen_verify_inputs(cfg, 3, "cuda", with_lm_head=False)
+    monkeypatch.setenv("MIRROR_TEST_STALL_MERGES", "1")
+    monkeypatch.setenv("MIRROR_WAIT_LIMIT_CYCLES", LIMIT)
+    m = make_mirror(cfg)
+    kv = m.kv(x.k_pool, x.v_pool, x.page_table, x.prefix_len)
+    tree = m.tree(x.tokens, cfg.kappa, cfg.gamma)
+    out = torch.zeros_like(x.q)
+    m.mirror_attn_verify(kv, tree, x.q, x.k_new, x.v_new, out=out)
+    assert m.device_status() == (7, 38)
+    m.mirror_attn_verify(kv, tree, x.q, x.k_new, x.v_new, out=out)
+    assert m.device_status() == (0, 0)
+    r = oracle_attention(x)[0][0]
+    assert np.abs(out[0].float().cpu().numpy() - r).max() <= 1e-2 * np.abs(r).max() + 1e-5
