@@ -201,16 +201,10 @@ class AcceptResult:
         self.decide_row = torch.empty(batch, **i32)
         self.reuse_slot = torch.empty(batch, **i32)
 
-    def __setattr__(self, name, value):
-        object.__setattr__(self, name, value)
-        object.__setattr__(self, "_struct", None)          # (another tensor: the addresses are looked up again)
-
     def struct(self) -> AcceptOut:
-        s = self._struct
-        if s is None:
-            s = AcceptOut(*[getattr(self, f).data_ptr() for f, _ in AcceptOut._fields_])
-            object.__setattr__(self, "_struct", s)
-        return s
+        # (addresses are read on each call: a tensor that was resized or re-pointed in place has another one)
+        return AcceptOut(self.n_accepted.data_ptr(), self.best_branch.data_ptr(), self.n_emitted.data_ptr(), self.emitted.data_ptr(),
+                         self.accepted_nodes.data_ptr(), self.decide_row.data_ptr(), self.reuse_slot.data_ptr())
 
     def cpu(self) -> dict:
         return {f: getattr(self, f).cpu().numpy() for f, _ in AcceptOut._fields_}
