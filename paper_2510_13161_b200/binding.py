@@ -138,8 +138,12 @@ def _ptr(t: Optional[torch.Tensor], dtype=None, name: str = "tensor"):
 
 
 def _stream(stream) -> int:
-    # (the raw handle: building a torch.cuda.Stream object costs 2 us a call)
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    try:                                                   # the raw handle: building a torch.cuda.Stream object costs 2 us a call
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:                                 # (private names: another release of torch may not have them)
+        return torch.cuda.current_stream().cuda_stream
 
 
 def mirror_trie_build(branch_tokens, root_token: int):

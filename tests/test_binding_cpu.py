@@ -1,4 +1,7 @@
 """The Python binding's own host work, without a GPU."""
+import types
+
+import pytest
 import torch
 
 from paper_2510_13161_b200 import binding
@@ -18,3 +21,13 @@ def test_accept_result_follows_its_tensors():
     assert passed() == current()
     out.decide_row.data = torch.empty(5, dtype=torch.int32)
     assert passed() == current()
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_current_stream_without_torchs_private_names(missing, monkeypatch):
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 11 + device, raising=False)
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 3, raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=22))
+    assert binding._stream(None) == 14 and binding._stream(types.SimpleNamespace(cuda_stream=33)) == 33
+    monkeypatch.delattr(torch._C, missing)
+    assert binding._stream(None) == 22
