@@ -696,7 +696,7 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
 int mirror_lmhead_pair_partials(int V) { return 2 * ((V + kPairV - 1) / kPairV); }
 
 bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk) {
-    return topk > 0 && M <= kMaxChunkRows && M >= ctx->tune.lm_pair_min_rows;
+    return topk > 0 && M <= kMaxChunkRows && M >= ctx->tune.lm_pair_min_rows && 8 * ctx->num_sms <= kMirrorTopkMaxLists;      // (4 per CTA, 2 CTAs per SM)
 }
 
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,

@@ -425,8 +425,8 @@ lmhead_topk_kernel(int V, int topk, float inv_T, const float* logits, const floa
 // The row's bar (the least of its words, see lmhead_pair.cu) is a lower bound of the topk-th best, so only what reaches it is
 // gathered, a few dozen pairs of the 9472, and each finds its own place by counting those before it.  Should more pass
 // than there is room for (many equal logits), rounds take the best head of all lists and move that list on, a barrier
-// each (8 rounds over 57 rows x 2368 lists take 4 us longer than counting).  The bars are cleared for the next call.
-constexpr int kListsPerThread = 2;
+// each (8 rounds over 57 rows x 1184 lists take 4 us longer than counting).  The bars are cleared for the next call.
+constexpr int kListsPerThread = kMirrorTopkMaxLists / 1024;
 constexpr int kMaxGathered = 1024;
 __global__ void __launch_bounds__(1024, 1)
 lmhead_topk_merge_kernel(int P, int topk, float inv_T, float inv_T_log2e, const float* part_max, const int* part_idx,
@@ -585,7 +585,6 @@ mirror_status lmhead_tail(mirror_ctx* ctx, const void* hidden, int M, const void
     }
     float* lse_dst = lse ? lse : (topk > 0 ? lse_scratch : nullptr);
     if (topk > 0 && cand_v) {      // (four lists per partial: one per epilogue warp)
-        if (4 * P > kListsPerThread * 1024) return MIRROR_ERR_UNSUPPORTED;
         MIRROR_CUDA_OK(mirror_launch_pdl(lmhead_topk_merge_kernel, dim3(M), dim3(1024), 0, stream, P, topk, inv_T, inv_T_log2e, part_max, part_idx,
                                          part_sum, cand_v, cand_i, argmax, maxlogit, lse, topk_id, topk_logprob,
                                          (__nv_bfloat16*)topk_logprob_bf16, M, ctx->d_topk_bar));

@@ -107,7 +107,9 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
 // LM-head GEMM + per-unit row partials on CTA pairs (many hidden rows); *n_partials partials of [M] rows are left in
 // partial_ws for lmhead_merge_kernel.  mirror_lmhead_pair_partials(V) is that count.
 int mirror_lmhead_pair_partials(int V);
-// Can the Top-kappa of M rows be selected inside the GEMM's epilogue?  (One row chunk.)
+// Can the Top-kappa of M rows be selected inside the GEMM's epilogue?  (One row chunk, and no more lists per row than the merge
+// takes: once the GEMM has raised the rows' bars the merge has to run, since it clears them for the next call.)
+constexpr int kMirrorTopkMaxLists = 2048;
 bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk);
 // w_scale / h_scale non-null: W and hidden are e4m3 bytes with one scale per row (the GEMM runs on kind::f8f6f4).
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,

@@ -85,3 +85,20 @@ def test_attention_merge_wait_runs_out_and_the_context_stays_usable(prefix, monk
     assert m.device_status() == (0, 0)
     r = oracle_attention(x)[0][0]
     assert np.abs(out[0].float().cpu().numpy() - r).max() <= 1e-2 * np.abs(r).max() + 1e-5
+
+
+def test_topk_after_a_wait_that_ran_out(monkeypatch):
+    """The rows' bars, which lie in the context, are clear again after a Top-kappa call that was given up."""
+    V, H, M, K = 6000, 512, 17, 8
+    cfg = I.VerifyConfig("t", H, 4, 2, 64, 1, 1, 16, 16, 2, 4, V, "greedy")
+    g = torch.Generator().manual_seed(6)
+    W = torch.empty((V, H), dtype=torch.bfloat16).normal_(0, 0.05, generator=g).cuda()
+    hid = torch.empty((M, H), dtype=torch.bfloat16).normal_(0, 1.0, generator=g).cuda()
+    m = stalled_mirror(cfg, monkeypatch)
+    m.mirror_lmhead_reduce(hid, W, topk=K)
+    code, detail = m.device_status()
+    assert code == 7 and detail in (11, 12, 13, 16), (code, detail)
+    plain = make_mirror(cfg).mirror_lmhead_reduce(hid, W, topk=K)
+    res = m.mirror_lmhead_reduce(hid * 0.125, W, topk=K)          # smaller logits: a bar left behind would hold them back
+    assert m.device_status() == (0, 0)
+    assert torch.equal(res["topk_id"], plain["topk_id"])
