@@ -97,16 +97,16 @@ finish_qkv_kernel(const float* partial, int slices, int M, int Hq, int Hkv, int 
 }
 
 // Residual add + RMSNorm: r = residual + split-K sum, x_out = bf16(r); normed = bf16(x_out / sqrt(mean(x_out^2) + eps)
-// * gamma) (from the ROUNDED x_out: what a later reader of x_out would compute).  A cluster of four CTAs of 256 threads
-// per row: with few rows one block per row leaves the chip empty and pulls a row's partial sums through one SM (17 rows x
-// 7 slices: 5.8 us).  A thread keeps its columns (every 1024th) in registers between the two passes and issues the loads
-// of all slices of all its columns before adding them (in slice order); the 32 warps' sums of squares meet in every
-// CTA's shared memory and are added in warp order.  partial == nullptr: plain RMSNorm of `residual`;
-// gamma == nullptr: no norm.
-constexpr int kNormThreads = 1024;            // per row, four CTAs together
-constexpr int kNormCluster = 4;
+// * gamma) (from the ROUNDED x_out: what a later reader of x_out would compute).  With few rows a cluster of four CTAs of
+// 256 threads per row: one block per row leaves the chip empty and pulls a row's partial sums through one SM (17 rows x
+// 7 slices: 5.8 us).  With many rows, when the blocks fill the chip anyway, one block of 1024 threads per row: the cluster's
+// barriers and 256-thread waves then cost more than they hide (see launch_residual_norm).  A thread keeps its columns (every
+// 1024th) in registers between the two passes and issues the loads of all slices of all its columns before adding them (in
+// slice order); the 32 warps' sums of squares meet in every CTA's shared memory and are added in warp order: the same bits
+// either way.  partial == nullptr: plain RMSNorm of `residual`; gamma == nullptr: no norm.
+constexpr int kNormThreads = 1024;            // per row, all CTAs together
 constexpr int kNormMaxCols = 16;              // columns per thread: rows of up to 16384 elements
-template <int kNormCols, int kUnroll>         // kNormCols * 1024 >= H; kUnroll slices' loads in flight at a time
+template <int kNormCols, int kUnroll, int kNormCluster>         // kNormCols * 1024 >= H; kUnroll slices' loads in flight at a time
 __global__ void __launch_bounds__(kNormThreads / kNormCluster)
 finish_residual_norm_kernel(const float* partial, int slices, int M, int H, const __nv_bfloat16* residual,
                             const __nv_bfloat16* gamma, float eps, __nv_bfloat16* x_out, __nv_bfloat16* normed) {
@@ -115,21 +115,22 @@ finish_residual_norm_kernel(const float* partial, int slices, int M, int H, cons
     const int t = rank * (kNormThreads / kNormCluster) + threadIdx.x;
     const size_t MN = (size_t)M * H, base = (size_t)row * H;
     // (a CTA may be written to once it has started: arrive now, wait in front of the exchange)
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (kNormCluster > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     float r[kNormCols], gm[kNormCols];
     auto load_early = [&]() {
 #pragma unroll
         for (int c = 0; c < kNormCols; ++c) {
             const int col = t + c * kNormThreads;
             r[c] = col < H ? __bfloat162float(residual[base + col]) : 0.f;
-            gm[c] = col < H && gamma ? __bfloat162float(gamma[col]) : 0.f;
+            if (kNormCluster > 1) gm[c] = col < H && gamma ? __bfloat162float(gamma[col]) : 0.f;        // (else: no registers to spare yet)
         }
     };
-    // behind a projection, the residual stream and the weight are older than the kernel ahead: no need to wait for it
-    if (partial) load_early();
+    // behind a projection, the residual stream and the weight are older than the kernel ahead: no need to wait for it (with many
+    // rows that hides nothing)
+    if (kNormCluster > 1 && partial) load_early();
     ptx::grid_dep_launch();
     ptx::grid_dep_wait();
-    if (!partial) load_early();
+    if (kNormCluster == 1 || !partial) load_early();
     if (partial) {
         // several slices' loads in flight at a time; the additions stay in slice order
 #pragma unroll 1
@@ -148,6 +149,10 @@ finish_residual_norm_kernel(const float* partial, int slices, int M, int H, cons
                 for (int c = 0; c < kNormCols; ++c) r[c] += v[k][c];
         }
     }
+    if (kNormCluster == 1) {
+#pragma unroll
+        for (int c = 0; c < kNormCols; ++c) gm[c] = t + c * kNormThreads < H && gamma ? __bfloat162float(gamma[t + c * kNormThreads]) : 0.f;
+    }
     float ss = 0.f;
 #pragma unroll
     for (int c = 0; c < kNormCols; ++c) {
@@ -162,14 +167,19 @@ finish_residual_norm_kernel(const float* partial, int slices, int M, int H, cons
     const bool norm = gamma && normed;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if ((threadIdx.x & 31) < kNormCluster) {                                   // lane j: this warp's sum to CTA j
-        uint32_t dst;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(ptx::smem_u32(&s_red[t >> 5])), "r"(threadIdx.x & 31));
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(ss) : "memory");
+    if (kNormCluster > 1) {
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if ((threadIdx.x & 31) < kNormCluster) {                               // lane j: this warp's sum to CTA j
+            uint32_t dst;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(ptx::smem_u32(&s_red[t >> 5])), "r"(threadIdx.x & 31));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(ss) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
+        if ((threadIdx.x & 31) == 0) s_red[t >> 5] = ss;
+        __syncthreads();
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (!norm) return;
     float tot = 0.f;
 #pragma unroll
@@ -210,19 +220,30 @@ finish_store_kernel(const float* partial, int slices, size_t MN, const __nv_bflo
 
 cudaError_t launch_residual_norm(cudaStream_t s, const float* partial, int slices, int M, int H, const __nv_bfloat16* residual,
                                  const __nv_bfloat16* gamma, float eps, __nv_bfloat16* x_out, __nv_bfloat16* normed) {
+    // Rows x columns per thread beyond which the chip is full with a block per row (mirror_rmsnorm, cluster / block in us: 100 x 8192
+    // 8.1 / 8.0, 150 x 8192 11.4 / 6.8, 300 x 5120 15.4 / 6.9, 1040 x 5120 46 / 16, 2000 x 16384 299 / 61; two layers of the 14B shape at 520
+    // rows 1193 / 1111).  Short rows behind a projection keep the cluster (six layers of 256 columns at 1040 rows: 655 / 681), as it
+    // requests the residual stream before the wait.
+    const int cols = H <= 4 * kNormThreads ? 4 : H <= 8 * kNormThreads ? 8 : 16;
+    const unsigned n_cta = M * cols <= 1024 || (partial && cols == 4) ? 4 : 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)M * kNormCluster);
-    cfg.blockDim = dim3(kNormThreads / kNormCluster);
+    cfg.gridDim = dim3((unsigned)M * n_cta);
+    cfg.blockDim = dim3(kNormThreads / n_cta);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = kNormCluster;
+    attr[1].val.clusterDim.x = n_cta;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    auto kern = H <= 4 * kNormThreads ? finish_residual_norm_kernel<4, 8> : H <= 8 * kNormThreads ? finish_residual_norm_kernel<8, 7> : finish_residual_norm_kernel<16, 3>;
+    cfg.numAttrs = n_cta > 1 ? 2 : 1;
+    auto kern = n_cta > 1 ? (cols == 4   ? finish_residual_norm_kernel<4, 8, 4>
+                             : cols == 8 ? finish_residual_norm_kernel<8, 7, 4>
+                                         : finish_residual_norm_kernel<16, 3, 4>)
+                          : (cols == 4   ? finish_residual_norm_kernel<4, 6, 1>
+                             : cols == 8 ? finish_residual_norm_kernel<8, 4, 1>
+                                         : finish_residual_norm_kernel<16, 2, 1>);
     return cudaLaunchKernelEx(&cfg, kern, partial, slices, M, H, residual, gamma, eps, x_out, normed);
 }
 

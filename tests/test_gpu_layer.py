@@ -226,3 +226,37 @@ def test_target_forward_repeated_runs_are_bitwise_equal():
         for k, v in first.items():
             assert torch.equal(out[k], v), k
     assert m.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("M,H", [(256, 4096), (257, 4096), (128, 8192), (129, 4160), (64, 16384), (65, 8256)])
+def test_rmsnorm_on_both_sides_of_the_block_rule(M, H):
+    """Few rows take a cluster of four CTAs each, many a block each: the sums are added in the same order, so a row has the same
+    bits alone and among many."""
+    x, g = rand_bf16((M, H), 2.0, 4), (1.0 + 0.1 * torch.randn(H, generator=torch.Generator().manual_seed(5))).to(torch.bfloat16)
+    m = make_mirror(I.VerifyConfig("t", 256, 4, 2, 64, 1, 1, 16, 16, 2, 4, 1024, "greedy"))
+    out = m.mirror_rmsnorm(x.cuda(), g.cuda(), 1e-6)
+    alone = m.mirror_rmsnorm(x[-2:].cuda(), g.cuda(), 1e-6)
+    assert m.device_status() == (0, 0)
+    assert torch.equal(out[-2:], alone)
+    ref = T.rmsnorm(f64(x), f64(g), 1e-6)
+    assert np.all(np.abs(f64(out) - ref) <= BF16_HALF_ULP * np.abs(ref) * 1.01 + 1e-6)
+
+
+@pytest.mark.parametrize("H,B", [(8256, 1), (8256, 6), (5120, 3), (5120, 12), (2048, 24)])        # 13 to 312 rows
+def test_norms_behind_projections_on_both_sides_of_the_block_rule(H, B):
+    case = dict(H=H, Hq=2, Hkv=1, d=64, inter=128, L=1, B=B, lo=5, hi=20, kappa=3, gamma=4, seed=8)
+    cfg, x, layers, norm_final, emb = layer_case(**case)
+    ref = run_oracle(cfg, x, layers, norm_final, emb, 1.0e4, 1e-6)
+    m = make_mirror(cfg)
+    dev = lambda t: t.cuda()
+    tgt = m.target([{k: dev(v) for k, v in w.items()} for w in layers], dev(norm_final), case["inter"], 1.0e4, 1e-6)
+    out = m.mirror_target_forward(tgt, m.kv(dev(x.k_pool), dev(x.v_pool), dev(x.page_table), dev(x.prefix_len)),
+                                  m.tree(dev(x.tokens), cfg.kappa, cfg.gamma), dev(emb))
+    assert m.device_status() == (0, 0)
+    # Wide rows over short sums (K = 128 behind sums of 8256): one step of an attention or gate value (2^-8 of it) moves an output by
+    # |w| 2^-8 |value|, ten and more of them add up, and 640 k outputs are looked at: the gate of later layers, 8 steps (seen: 3.2).
+    close(out["x_out"], ref[-1]["x"], "x_out", ulps=8.0, exact_frac=0.4)
+    # The norm itself is one rounding of fp32 work on the stored stream.
+    normed = T.rmsnorm(f64(out["x_out"]), f64(norm_final), 1e-6)
+    assert np.all(np.abs(f64(out["hidden"]) - normed) <= BF16_HALF_ULP * np.abs(normed) * 1.01 + 1e-6)
+    assert np.mean(I.bf16_bits(out["hidden"]) == T.bf16_round_bits(normed)) > 0.995
