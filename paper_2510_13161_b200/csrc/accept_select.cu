@@ -5,13 +5,15 @@
 // Thread 0 then picks the longest branch (lowest index on ties) and the deciding row R, and emits argmax[R].
 //
 // Speculative sampling and the rule over the tree draw a token by inverse CDF over the vocabulary, in fp64.  What bounds
-// them is the fp64 exponentials (150 k per pass: 30 us on one SM), so a CLUSTER of 8 or 16 CTAs per request shares the
-// vocabulary: 512-thread CTAs, each warp one contiguous chunk that it reads coalesced.  The chunks' sums go to every CTA
+// them is the fp64 exponentials (150 k per pass: 30 us on one SM), so a CLUSTER of up to 16 CTAs per request shares the
+// vocabulary (cluster_shape): each warp has one contiguous chunk that it reads coalesced.  The chunks' sums go to every CTA
 // through distributed shared memory; all of them scan the same numbers and take the same decisions, one cluster barrier
-// per pass, nothing spins.  The chunk that holds the crossing is then summed again in 16 parts and the part searched, so
+// per pass, nothing spins.  The chunk that holds the crossing is then summed again in a part per warp and the part searched, so
 // the search is three short steps.  (One block per request with a contiguous segment per thread: 97-117 us for 8 and 16
 // requests x 128-152 k ids.)
 #include <string.h>
+
+#include <algorithm>
 
 #include "mirror_internal.h"
 
@@ -19,11 +21,9 @@ namespace {
 
 constexpr int kGreedyThreads = 256;
 constexpr int kFoldThreads = 1024;                    // of a greedy block that folds the LM head's partials itself
-constexpr int kThreads = 512;                         // of a CTA of the clusters
-constexpr int kWarps = kThreads / 32;
-constexpr int kMaxCluster = 16;                       // CTAs per request (above 8: opt-in)
-constexpr int kMaxChunks = kMaxCluster * kWarps;
-constexpr int kAhead = 8;                             // ids a thread loads before it works on the first
+constexpr int kSpecThreads = 512;                     // of a CTA of the chain rule's clusters
+constexpr int kMaxWarps = 32;                         // of a CTA of the clusters: 16 or 32
+constexpr int kMaxChunks = 256;                       // warps of a cluster: up to 16 CTAs (above 8: opt-in) of 16 warps, or 8 of 32
 
 struct AcceptTreeParams {
     int n, n_branches, gamma;
@@ -200,14 +200,16 @@ __device__ __forceinline__ uint32_t remote(const void* smem, uint32_t rank) {   
 
 struct DrawShared {
     double sum[2][2][kMaxChunks];                         // [pass parity][which sum][chunk]: the same in every CTA after a pass
-    double sub[kWarps];
+    double sub[kMaxWarps];
     int token;                                            // CTA 0's: the drawn token (-1: none yet)
     int last;                                             // CTA 0's: last id with positive mass
 };
+template <int kWarps>
 struct Draw {
     DrawShared& s;
     int V, rank, n_cta, chunk_len, lo, hi;                // [lo, hi): this warp's chunk
     uint32_t pass = 0;
+    static constexpr int kAhead = kWarps == 32 ? 4 : 8;   // ids a thread loads before it works on the first (as registers allow)
     __device__ Draw(DrawShared& sh, int vocab) : s(sh), V(vocab) {
         uint32_t r, n;
         asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -221,8 +223,8 @@ struct Draw {
         cluster_barrier();                                // (every CTA of the cluster has started: its shared memory may be written to)
     }
     // One pass over the vocabulary: load(v) fetches what id v's masses need, add(v, loaded, x0, x1) adds them to x0 and x1;
-    // eight loads are in flight per thread.  Returns this warp's chunk sums to all CTAs.
-    template <class L, class F>
+    // kAhead loads are in flight per thread.  Returns this warp's chunk sums to all CTAs (kTwo: both, else the first).
+    template <bool kTwo, class L, class F>
     __device__ __forceinline__ void sums(L load, F add) {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         double x = 0.0, y = 0.0;
@@ -236,11 +238,11 @@ struct Draw {
             for (int k = 0; k < kAhead; ++k)
                 if (v0 + 32 * k < hi) add(v0 + 32 * k, in[k], x, y);
         }
-        const double sx = warp_sum(x), sy = warp_sum(y);
+        const double sx = warp_sum(x), sy = kTwo ? warp_sum(y) : 0.0;
         const uint32_t par = pass & 1;
         if (lane < n_cta) {
             asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote(&s.sum[par][0][rank * kWarps + warp], lane)), "d"(sx) : "memory");
-            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote(&s.sum[par][1][rank * kWarps + warp], lane)), "d"(sy) : "memory");
+            if (kTwo) asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote(&s.sum[par][1][rank * kWarps + warp], lane)), "d"(sy) : "memory");
         }
         cluster_barrier();        // (the words of this parity are written again two passes later, behind another barrier)
         ++pass;
@@ -322,13 +324,13 @@ struct Draw {
     }
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kSpecThreads, 1)
 accept_spec_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs a) {
     __shared__ DrawShared s_draw;
     __shared__ int s_len[MIRROR_MAX_BRANCHES];
     __shared__ unsigned char s_pass[MIRROR_MAX_NODES];
     __shared__ Choice s_choice;
-    Draw draw(s_draw, a.V);
+    Draw<kSpecThreads / 32> draw(s_draw, a.V);
     const int b = blockIdx.x / draw.n_cta, tid = threadIdx.x, n = tp.n, V = a.V;
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
@@ -340,7 +342,7 @@ accept_spec_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
         s_pass[tid] = ok && t.u * t.q <= t.p;
     }
     __syncthreads();
-    for (int br = tid; br < tp.n_branches; br += kThreads) {
+    for (int br = tid; br < tp.n_branches; br += kSpecThreads) {
         int k = 0;
         while (k < tp.path_len[br] && s_pass[tp.path[br][k]]) ++k;
         s_len[br] = k;
@@ -357,7 +359,7 @@ accept_spec_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
         const float* lr = a.logits + row * V;
         const double lse = (double)a.lse[row];
         const float* qc = c.rej_node >= 0 ? a.q_probs + ((size_t)b * (n - 1) + (c.rej_node - 1)) * V : nullptr;
-        draw.sums([&](int v) { return make_float2(lr[v], qc ? qc[v] : 0.f); },
+        draw.template sums<true>([&](int v) { return make_float2(lr[v], qc ? qc[v] : 0.f); },
                   [&](int, float2 in, double& sp, double& sr) {
                       const double p = exp((double)in.x * a.inv_T - lse);
                       sp += p;
@@ -390,6 +392,7 @@ struct Loaded {
     float q;
 };
 
+template <int kThreads>
 __global__ void __launch_bounds__(kThreads, 1)
 accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs a) {
     __shared__ DrawShared s_draw;
@@ -398,7 +401,7 @@ accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
     __shared__ double s_Z[kMaxRejected];
     __shared__ int s_rej[kMaxRejected];
     __shared__ unsigned char s_path[MIRROR_MAX_DEPTH];
-    Draw draw(s_draw, a.V);
+    Draw<kThreads / 32> draw(s_draw, a.V);
     const int b = blockIdx.x / draw.n_cta, tid = threadIdx.x, n = tp.n, V = a.V;
     const int32_t* tok = a.tokens + (size_t)b * n;
     ptx::grid_dep_wait();
@@ -451,7 +454,7 @@ accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
             // rejected: normaliser of the residual (a residual without mass leaves m as it is)
             const float* qc = a.q_probs + ((size_t)b * (n - 1) + (c - 1)) * V;
             double* const nxt = !buf0 ? nullptr : (cur ? buf0 : buf1);
-            draw.sums([&](int v) { return Loaded{source(lr, v), qc[v]}; },
+            draw.template sums<false>([&](int v) { return Loaded{source(lr, v), qc[v]}; },
                       [&](int v, const Loaded& in, double& x, double&) {
                           const double res = fmax(mass(in.m, lse_r, v) - (double)in.q, 0.0);
                           if (nxt) nxt[v] = res;
@@ -481,7 +484,7 @@ accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
         const float* lr = a.logits + row * V;
         const double lse_r = (double)a.lse[row];
         // (a rejection has just added the same masses up: the draw needs them only up to a factor)
-        if (!summed) draw.sums([&](int v) { return source(lr, v); }, [&](int v, double in, double& x, double&) { x += raw(in, lse_r, v); });
+        if (!summed) draw.template sums<false>([&](int v) { return source(lr, v); }, [&](int v, double in, double& x, double&) { x += raw(in, lse_r, v); });
         extra = draw.pick(0, (double)a.u_resample[row], [&](int v) { return raw(source(lr, v), lse_r, v); });
     }
     if (draw.rank == 0) {
@@ -497,12 +500,24 @@ accept_tree_kernel(const __grid_constant__ AcceptTreeParams tp, const AcceptArgs
     cluster_barrier();                                    // no CTA may leave while a peer can still write to its shared memory
 }
 
-// CTAs per request: enough that a warp's chunk is a few steps, no more (a pass ends with a barrier of the cluster); 16 only
-// for few requests: a cluster lives in one GPC, and eight of 16 CTAs do not all fit at once (B = 8: 20.7 us against 16.9 with 8 CTAs).
-int cluster_size(const mirror_ctx* ctx, int batch) {
+// CTAs and threads per request.
+//   - Chain rule: enough CTAs that a warp's chunk is a few steps, no more (a pass ends with a barrier of the cluster); 16 only
+//     for few requests: a cluster lives in one GPC, and eight of 16 CTAs do not all fit at once (B = 8: 20.7 us against 16.9 with
+//     8 CTAs).
+//   - Tree rule: without scratch memory a pass costs an exponential and a chain of up to `siblings` subtractions and divisions
+//     per id: from four siblings on as many threads as there are ids, up to 8192, in 1024-thread CTAs where 16 CTAs do not fit (8
+//     siblings, 16 requests: 32000 ids 150 -> 84 us, 8192 ids 181 -> 94; a walk without rejections takes 4 us longer in
+//     1024-thread CTAs).  Else as the chain rule, but the walk has many passes: 8 CTAs from 16 k ids while they all fit (8 siblings,
+//     8 requests x 32000 ids: 42 -> 32 us; 16 requests, one branch: 15 -> 21).
+struct ClusterShape {
+    int n_cta, threads;
+};
+ClusterShape cluster_shape(const mirror_ctx* ctx, int batch, bool tree, bool scratch, int siblings) {
     const int V = ctx->desc.vocab;
-    if (V > 65536 && batch * 32 <= ctx->num_sms) return 16;
-    return V > 32768 ? 8 : V > 8192 ? 4 : 2;
+    const bool chains = tree && !scratch && siblings >= 4, few = batch * 32 <= ctx->num_sms;
+    if (few && V > (chains ? 4096 : 65536)) return {16, 512};
+    if (chains) return V > 4096 ? ClusterShape{8, 1024} : ClusterShape{V > 2048 ? 8 : V > 1024 ? 4 : 2, 512};
+    return {V > (tree && batch * 16 <= ctx->num_sms ? 16384 : 32768) ? 8 : V > 8192 ? 4 : 2, 512};
 }
 
 }  // namespace
@@ -539,11 +554,15 @@ mirror_status mirror_accept_launch(mirror_ctx* ctx, const mirror_tree* tree, con
         if (partials) MIRROR_CUDA_OK(mirror_launch_pdl(accept_greedy_kernel<true>, dim3(tree->batch), dim3(kFoldThreads), 0, stream, tp, a, *partials, argmax_out));
         else MIRROR_CUDA_OK(mirror_launch_pdl(accept_greedy_kernel<false>, dim3(tree->batch), dim3(kGreedyThreads), 0, stream, tp, a, none, argmax_out));
     } else {
-        auto kern = in->mode == MIRROR_ACCEPT_SPEC_TREE ? accept_tree_kernel : accept_spec_kernel;
-        const unsigned n_cta = (unsigned)cluster_size(ctx, tree->batch);
+        const bool by_tree = in->mode == MIRROR_ACCEPT_SPEC_TREE;
+        int siblings = 0, children[MIRROR_MAX_NODES] = {};
+        for (int i = 1; i < ti.n; ++i) siblings = std::max(siblings, ++children[ti.parent[i]]);
+        const ClusterShape shape = cluster_shape(ctx, tree->batch, by_tree, tree_scratch != nullptr, siblings);
+        auto kern = !by_tree ? accept_spec_kernel : shape.threads == 1024 ? accept_tree_kernel<1024> : accept_tree_kernel<512>;
+        const unsigned n_cta = (unsigned)shape.n_cta;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)tree->batch * n_cta);
-        cfg.blockDim = dim3(kThreads);
+        cfg.blockDim = dim3(shape.threads);
         cfg.dynamicSmemBytes = 0;
         cfg.stream = stream;
         cudaLaunchAttribute attr[2];

@@ -94,3 +94,31 @@ def test_tree_rule_reports_tokens_outside_the_vocabulary_where_the_walk_meets_th
     got = run(met)
     assert m.device_status() == (6, 101)
     assert got["n_accepted"][0] == gamma and 1 not in got["accepted_nodes"][1]
+
+
+@pytest.mark.parametrize("V,B", [(1000, 2), (1025, 2), (2049, 1), (4096, 3), (4097, 1), (4097, 6), (20000, 4), (33000, 5)])
+@pytest.mark.parametrize("kappa", [3, 4, 9])                    # siblings under the root: few, and enough for a thread per id
+@pytest.mark.parametrize("reject", [False, True])               # every sibling rejected, or as it comes
+def test_walks_over_many_siblings(V, B, kappa, reject):
+    gamma = 2
+    m = make_mirror(cfg_for(V, kappa, gamma, B))
+    par = I.comb_parent(kappa, gamma)
+    logits, qp, tok, ua, ur = spec_case(B, kappa, gamma, V, V + kappa)
+    if reject:
+        for b in range(B):
+            for k in range(kappa):
+                c = 1 + k * gamma
+                ua[b, c] = 1.0
+                qp[b, c - 1] *= 0.5
+                qp[b, c - 1, tok[b, c]] += 0.5
+    lse = torch.logsumexp(logits.double(), -1).float()
+    ref = O.accept_tree(tok.numpy(), logits.numpy(), lse.numpy(), qp.numpy(), ua.numpy(), ur.numpy(), par, gamma, True, 1.0)
+    acc = m.accept_in(binding.ACCEPT_SPEC_TREE, True, logits=logits.cuda(), lse=lse.cuda(), q_probs=qp.cuda(), u_accept=ua.cuda(),
+                      u_resample=ur.cuda())
+    tree = m.tree(tok.cuda(), kappa, gamma)
+    for scratch in (False, True):
+        got = m.mirror_accept_select(tree, acc, tree_scratch=scratch).cpu()
+        assert m.device_status() == (0, 0)
+        for b in range(B):
+            same = all(np.array_equal(got[f][b], ref[f][b]) for f in FIELDS if f != "reuse_slot")
+            assert same or ref["margin"][b] < 1e-9, (b, scratch, ref["margin"][b])
