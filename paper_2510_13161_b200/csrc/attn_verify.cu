@@ -86,6 +86,8 @@ struct AttnParams {
     int snap_cap;                         // boundaries move to a unit boundary that is at most this many tiles away
     int units;                            // layers x requests x heads (or pairs of heads)
     int whole_groups;                     // group count that divides the units evenly (attn::whole_unit_groups), 0: none
+    int unit_cuts;                        // fewer units than groups: groups per unit, rounded down; 0 otherwise
+    int cut_tiles;                        // tiles that a group may take longer for it
     int never_cut;                        // 1: units are so short that they are dealt out whole whatever their lengths
     int max_pages, num_pages, layer_pages;
     int tree_slots;
@@ -230,6 +232,11 @@ struct Partition {
     int n_groups, snap_tol;
     int share, rest;                      // total_tiles = n_groups * share + rest
 };
+// Does a group take at most `more` tiles longer when each unit of `tiles` has `cuts` groups to itself than in an even split over
+// `groups`?
+__host__ __device__ inline bool cuts_pay(int tiles, int units, int groups, int cuts, int more) {
+    return (long long)tiles * groups - (long long)tiles * units * cuts <= (long long)more * cuts * groups;
+}
 __device__ __forceinline__ Partition make_partition(const AttnParams& p, const int* cumT) {
     Partition q;
     const long long per = (long long)(p.Hkv / p.heads_per_unit) * cumT[p.B], total = per * p.L;
@@ -242,9 +249,17 @@ __device__ __forceinline__ Partition make_partition(const AttnParams& p, const i
     for (int b = 1; b < p.B; ++b) equal_units &= (cumT[b + 1] - cumT[b]) == cumT[1];
     // Else every group gets at least one tile, or two where its streams take alternate tiles (one alone would leave a stream
     // without work and the merge with twice the records).
-    q.n_groups = p.never_cut                        ? min(p.n_groups, p.units)
-               : p.whole_groups > 0 && equal_units ? p.whole_groups
-                                                   : min(p.n_groups, max(1, p.mode == kSplit ? q.total_tiles >> 1 : q.total_tiles));
+    const int split = p.mode == kSplit ? 1 : 0, most = min(p.n_groups, max(1, q.total_tiles >> split));
+    q.n_groups = p.never_cut ? min(p.n_groups, p.units) : p.whole_groups > 0 && equal_units ? p.whole_groups : most;
+    // Fewer units than groups, all of one length: the same number of groups for every unit, where that costs a group few tiles.
+    // (An even split over all groups makes most of them work on two units: a second Q, which an e4m3 cache converts, a second
+    // epilogue and record; whole units also need no merge.  64 units of 9 tiles over 74 groups, bf16 / e4m3: 53 -> 30 / 68 -> 36 us;
+    // 16 units over 37 groups, two each: 39 -> 33 / 54 -> 40.  But 16 units of 157 tiles over 74 groups, four each, bf16, which is
+    // 5 tiles longer: 95 -> 104.)
+    if (p.unit_cuts > 0 && equal_units && !p.never_cut) {
+        const int cuts = min(p.unit_cuts, max(1, cumT[1] >> split));
+        if (cuts_pay(cumT[1], p.units, most, cuts, p.cut_tiles)) q.n_groups = p.units * cuts;
+    }
     q.share = (int)((uint32_t)q.total_tiles / (uint32_t)q.n_groups);
     q.rest = q.total_tiles - q.share * q.n_groups;
     // A boundary that falls within snap_tol tiles of a unit boundary moves there (a cut costs about as much as a tile).
@@ -1272,7 +1287,10 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     if (units > 0x7fffffff) return MIRROR_ERR_SHAPE;        // (a unit has a tile at least: the tiles are counted in 31 bits)
     p.units = (int)units;
     p.whole_groups = whole && units >= p.n_groups ? attn::whole_unit_groups(p.n_groups, units) : 0;
-    p.never_cut = whole && (kv->max_pages_per_req + (p.n + kSlotTok - 1) / kSlotTok + kTileSlots - 1) / kTileSlots <= 6;
+    p.unit_cuts = whole && units < p.n_groups ? p.n_groups / (int)units : 0;
+    p.cut_tiles = f8 || p.unit_cuts == 1 ? 8 : 2;
+    const int most_tiles = (kv->max_pages_per_req + (p.n + kSlotTok - 1) / kSlotTok + kTileSlots - 1) / kTileSlots;      // of a unit
+    p.never_cut = whole && most_tiles <= 6;
     p.wait_limit = ctx->tune.wait_limit_cycles;
     p.stall_after = (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_attn_left-- > 0) ? ctx->tune.test_stall_after : -1;
     p.stall_merge = ctx->tune.test_stall_merges > 0 && ctx->tune.test_stall_merges-- > 0;
@@ -1335,7 +1353,7 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         MIRROR_CUDA_OK(cudaGetLastError());
         // One request: all units have the same length whatever it is, so the host can tell when the partition gives every
         // group whole units (each unit holds at least one tile): nothing is cut and the merge kernel has nothing to do.
-        const bool no_cuts = p.never_cut || (p.B == 1 && p.whole_groups > 0);
+        const bool no_cuts = p.never_cut || (p.B == 1 && (p.whole_groups > 0 || (p.unit_cuts == 1 && cuts_pay(most_tiles, p.units, p.n_groups, 1, p.cut_tiles))));
         if (p.n_groups > 1 && !no_cuts) {
             // which units the partition cut is only known on the device (it depends on the prefix lengths)
             const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)(p.n_cta * (p.mode == kSplit ? 1 : 2)));

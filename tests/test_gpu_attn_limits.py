@@ -76,3 +76,29 @@ def test_units_that_many_groups_share(hq, hkv, d, prefix):
 @pytest.mark.parametrize("hq,hkv", [(8, 1), (32, 1), (20, 4)])
 def test_units_that_many_groups_share_over_an_8_bit_cache(hq, hkv):
     run_and_compare(small(n_q_heads=hq, n_kv_heads=hkv, prefix_lo=33000, prefix_hi=33000, batch=1, layers=1), 14)
+
+
+@pytest.mark.parametrize("hq,hkv,d,kappa,gamma,layers,batch,lo,hi", [
+    (64, 8, 128, 8, 7, 8, 1, 1000, 1000),        # 64 units for 74 groups: one each, nothing to merge
+    (64, 8, 128, 8, 7, 4, 2, 1000, 1000),        # the same, with the merge launched in vain
+    (64, 8, 128, 8, 15, 2, 1, 1000, 1000),       # 16 units for 37 groups: two each
+    (16, 2, 64, 4, 8, 1, 1, 900, 900),           # 2 units for 148 groups: as many as the units have tiles for
+    (64, 8, 128, 8, 7, 4, 2, 990, 1130),         # units of two lengths: an even split
+    (64, 8, 128, 8, 7, 2, 1, 9000, 9000),        # long units: an even split
+    (16, 1, 128, 3, 4, 1, 1, 0, 0),              # one unit
+])
+def test_fewer_units_than_groups(hq, hkv, d, kappa, gamma, layers, batch, lo, hi):
+    cfg = config(hq, hkv, d, kappa, gamma, lo, hi, batch=batch, layers=layers)
+    x = I.gen_verify_inputs(cfg, 15, "cuda", with_lm_head=False)
+    out, lse = run_gpu(make_mirror(cfg), x)
+    which = sorted({0, layers - 1})
+    ref = oracle_attention(x, which)
+    compare(out, lse, ref, which)
+    x.page_table = torch.cat([x.page_table, x.page_table.new_full((batch, 2000), -1)], 1).contiguous()      # room for longer contexts
+    out, lse = run_gpu(make_mirror(cfg), x)
+    compare(out, lse, ref, which)
+
+
+@pytest.mark.parametrize("kw", [dict(kappa=8, gamma=7, layers=4, batch=2), dict(kappa=8, gamma=15, layers=2, batch=1), dict(kappa=4, gamma=4, layers=1, batch=1)])
+def test_fewer_units_than_groups_over_an_8_bit_cache(kw):
+    run_and_compare(small(n_q_heads=64, n_kv_heads=8, hidden=8192, prefix_lo=1000, prefix_hi=1000, **kw), 16)
