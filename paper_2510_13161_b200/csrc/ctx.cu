@@ -247,9 +247,11 @@ extern "C" mirror_status mirror_workspace_bytes(const mirror_ctx* ctx, const mir
     size_t need = L.end_attn;
     if (what & (MIRROR_WS_LMHEAD | 4u)) need = L.end_lmhead;
     if (what & 32u) {
-        // room for the candidate lists; and for the logits where the largest kappa could not be selected in the epilogue
+        // room for the candidate lists; and for the logits where the largest kappa could not be selected in the epilogue, or
+        // some kappa is better selected from them
+        const int M = (int)((size_t)tree->batch * tree->n_nodes);
         if (L.lm_topk_bytes && L.end_topk > need) need = L.end_topk;
-        if (!mirror_lmhead_topk_fusable(ctx, (int)((size_t)tree->batch * tree->n_nodes), MIRROR_MAX_TOPK) && L.end_logits > need) need = L.end_logits;
+        if ((!mirror_lmhead_topk_fusable(ctx, M, MIRROR_MAX_TOPK) || mirror_lmhead_topk_spills(ctx, M, 1)) && L.end_logits > need) need = L.end_logits;
     }
     if (what & 8u) need = L.end_logits > need ? L.end_logits : need;
     if (what & 16u) need = L.end_accept;

@@ -39,7 +39,8 @@ extern "C" mirror_status mirror_early_exit_tap(mirror_ctx* ctx, const void* hidd
     MirrorWsLayout L;
     mirror_ws_layout(ctx, (size_t)M, &L);
     uint8_t* ws = (uint8_t*)ctx->ws;
-    if (L.lm_topk_bytes && ctx->ws_bytes >= L.end_topk && mirror_lmhead_topk_fusable(ctx, M, kappa)) {
+    const bool spill = mirror_lmhead_topk_spills(ctx, M, kappa) && ctx->ws_bytes >= L.end_logits;
+    if (!spill && L.lm_topk_bytes && ctx->ws_bytes >= L.end_topk && mirror_lmhead_topk_fusable(ctx, M, kappa)) {
         // the Top-kappa is selected inside the GEMM's epilogue: the proxy's logits never reach memory
         return mirror_lmhead_launch(ctx, hidden_le, M, W, kappa, nullptr, nullptr, 0, nullptr, nullptr, nullptr, msg_ids, nullptr,
                                     nullptr, nullptr, ws + L.lm_partial, L.lm_partial_bytes, (float*)(ws + L.lse),

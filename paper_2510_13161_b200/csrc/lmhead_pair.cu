@@ -699,6 +699,16 @@ bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk) {
     return topk > 0 && M <= kMaxChunkRows && M >= ctx->tune.lm_pair_min_rows && 8 * ctx->num_sms <= kMirrorTopkMaxLists;      // (4 per CTA, 2 CTAs per SM)
 }
 
+// In a CTA's first unit there is no bar yet, and every row costs its epilogue warps a sort (1.2 us a row in all), however small
+// the vocabulary; a selection from spilled logits costs kappa passes over a row's V logits, 148 rows at a time.  (us, fused /
+// spilled: 256 rows x 1024 ids, kappa 16: 354 / 48; 128 x 8192, 8: 167 / 47; 256 x 32000, 32: 403 / 371; 57 x 16000, 8: 88 / 45,
+// 57 x 50000, 8: 111 / 109; 17 x 16000, 8: 39 / 39; 57 x 152064, 8: 166 / 404.)  Large vocabularies stay fused: their logits are
+// tens of MB.
+bool mirror_lmhead_topk_spills(const mirror_ctx* ctx, int M, int topk) {
+    const long long V = ctx->desc.vocab;
+    return V <= 65536 && V * (topk + 4) <= 5200ll * (M - 16);
+}
+
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,
                                         void* partial_ws, size_t partial_bytes, cudaStream_t stream, int* n_partials,
                                         const float* w_scale, const float* h_scale, int topk, void* topk_ws, size_t topk_ws_bytes,

@@ -729,7 +729,8 @@ extern "C" mirror_status mirror_lmhead_reduce(mirror_ctx* ctx, const void* hidde
     float* lse_scratch = (float*)((uint8_t*)ctx->ws + L.lse);
     void* topk_ws = nullptr;
     if (topk > 0) {
-        if (L.lm_topk_bytes && ctx->ws_bytes >= L.end_topk && mirror_lmhead_topk_fusable(ctx, M, topk)) {
+        const bool spill = mirror_lmhead_topk_spills(ctx, M, topk) && (logits_out || ctx->ws_bytes >= L.end_logits);
+        if (!spill && L.lm_topk_bytes && ctx->ws_bytes >= L.end_topk && mirror_lmhead_topk_fusable(ctx, M, topk)) {
             topk_ws = (uint8_t*)ctx->ws + L.lm_topk;       // Top-kappa inside the GEMM's epilogue: no [M, V] buffer
             need = L.end_topk;
         } else if (!logits_out) {

@@ -111,6 +111,8 @@ int mirror_lmhead_pair_partials(int V);
 // takes: once the GEMM has raised the rows' bars the merge has to run, since it clears them for the next call.)
 constexpr int kMirrorTopkMaxLists = 2048;
 bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk);
+// ... and is it better selected from spilled logits, where the workspace has room for them?
+bool mirror_lmhead_topk_spills(const mirror_ctx* ctx, int M, int topk);
 // w_scale / h_scale non-null: W and hidden are e4m3 bytes with one scale per row (the GEMM runs on kind::f8f6f4).
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,
                                         void* partial_ws, size_t partial_bytes, cudaStream_t stream, int* n_partials,
