@@ -12,14 +12,19 @@ from tests.helpers import make_mirror
 
 pytestmark = pytest.mark.gpu
 
-# Tolerance against the oracle (8-bit Q, K and V, fp64 after the rounding).  The kernel also rounds the unnormalised softmax
-# weights to e4m3: each weight is off by at most 2^-4 of itself, so an output element is off by at most
-# 2^-4 * sum_j w_j |v_j| (checked element by element below: the derived bound).  The errors are independent from key to key
-# and mostly cancel: 1% .. 3% of the largest output on these shapes, depending on how the CTAs cut the units; FP8_REL is a
-# coarse gate on top of the derived bound.  The row sums are taken before that rounding: the log-sum-exp keeps the bf16
-# path's bound.
-FP8_REL = 5e-2
+# Tolerance against the oracle (8-bit Q, K and V, fp64 after the rounding).  K and Q enter as codes, V is widened exactly, and
+# the unnormalised softmax weights are f16: a weight is off by 2^-11 of itself, or by 2^-25 of the largest of its row's first
+# tile (at most 1 after the division) where it falls below f16's normal range.  The exponential, fp32 scores and fp32 sums
+# over up to 40 k keys add another 2^-11 of sum_j w_j |v_j|, the output's bf16 rounding 2^-8 of the result: element by element
+#     2^-10 sum_j w_j |v_j| + 2^-8 |ref| + 2^-25 keys max|v|
+# is checked below.  (Weights rounded to e4m3, as an 8-bit P V would need them, are off by 2^-4: 1% .. 3% of the largest output
+# on these shapes.)  FP8_REL is a gate relative to the largest output, as over a bf16 cache.
+FP8_REL = 1e-2
 LSE_ATOL = 2e-3
+
+
+def element_bound(ref, a_ref, keys, v_max):
+    return 2.0 ** -10 * a_ref + 2.0 ** -8 * np.abs(ref) + 2.0 ** -25 * keys * v_max
 
 
 def small(**kw):
@@ -66,12 +71,11 @@ def run_and_compare(cfg, seed, parent=None, q_std=1.0, layers=None, tweak=None):
         got = f32(out[l]).astype(np.float64)
         err, scale = np.abs(got - ref).max(), np.abs(ref).max()
         assert err <= FP8_REL * scale, (l, err, scale)
-        # the worst case, element by element: every weight off by 2^-4 of itself in the direction of its |v|
-        # (sum_j w_j |v_j|: the oracle again with the sign bits of the V codes cleared), plus the output's bf16 rounding
-        # and the weights that fall below the 8-bit format's range
+        # (sum_j w_j |v_j|: the oracle again with the sign bits of the V codes cleared)
         a_ref, _ = F.attention_layer_fp8(F.quantize_tensor(f32(x.q[l]), q_scale), q_scale, k8[l].cpu().numpy(), v8[l].cpu().numpy() & 0x7F,
                                          ks_h[l], vs_h[l], pt, pl, kn8[l].cpu().numpy(), vn8[l].cpu().numpy() & 0x7F, anc, 1.0 / np.sqrt(d))
-        assert (np.abs(got - ref) <= 2.0 ** -4 * a_ref + 2.0 ** -8 * np.abs(ref) + 2.0 ** -7 * scale).all(), l
+        bound = element_bound(ref, a_ref, int(pl.max()) + len(x.parent), 448.0 * float(vs_h[l].max()))
+        assert (np.abs(got - ref) <= bound).all(), (l, float((np.abs(got - ref) / bound).max()))
         np.testing.assert_allclose(lse[l].cpu().numpy(), lse_ref, atol=LSE_ATOL)
         worst = max(worst, err / scale)
     return worst

@@ -35,6 +35,18 @@ def test_row_quantisation_is_bit_exact(rows, cols):
     np.testing.assert_array_equal(codes.cpu().numpy(), rc)
 
 
+@pytest.mark.parametrize("rows,cols", [(5, 8192), (5, 8200), (3, 20000),       # kept in registers to the last word, and read twice
+                                       (4, 8), (4, 250), (3, 5121), (2, 1)])   # one word, and rows that are not whole words
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -80, 2.0 ** 80])                # scales that the reciprocal serves, and others
+def test_row_quantisation_of_any_row_is_bit_exact(rows, cols, scale):
+    x = (rand_bf16((rows, cols), 0.7, 3).float() * scale).to(torch.bfloat16)
+    m = make_mirror(lm_cfg(1024, 128))
+    codes, sc = m.mirror_quantize_rows_fp8(x.cuda())
+    rc, rs = F.quantize_rows(x.float().numpy())
+    np.testing.assert_array_equal(sc.cpu().numpy(), rs)
+    np.testing.assert_array_equal(codes.cpu().numpy(), rc)
+
+
 @pytest.mark.parametrize("M,V,H,T", [(17, 6000, 512, 1.0), (300, 4100, 256, 0.8), (128, 20000, 1024, 1.0)])
 def test_fp8_lmhead_matches_the_oracle_of_the_quantised_operands(M, V, H, T):
     W = rand_bf16((V, H), 0.05, 11); hid = rand_bf16((M, H), 1.0, 12)

@@ -194,3 +194,31 @@ def test_step_when_no_unit_is_cut_by_the_partition():
         ref = O.accept_greedy(tok, am.reshape(tok.shape), x.parent, cfg.gamma)
         for f in FIELDS:
             np.testing.assert_array_equal(got[f], ref[f], err_msg=f)
+
+
+@pytest.mark.parametrize("explicit_hidden", [False, True])
+@pytest.mark.parametrize("layers,batch", [(40, 1), (7, 3), (80, 2)])          # 54, 28 and 215 MB of inputs: pieces of 3 to 24 MB
+def test_host_buffer_step_in_many_pieces(layers, batch, explicit_hidden):
+    """Inputs far larger than what arrives while the (small) LM head runs: the layers are copied and attended to in several pieces
+    of growing size, the last layer first when the LM head needs it.  Short contexts: no unit is cut, whatever launch it is in."""
+    cfg = I.VerifyConfig("host", 8192, 64, 8, 128, layers, batch, 20, 300, 8, 8, 2000, "greedy", explicit_hidden=explicit_hidden)
+    m = make_mirror(cfg)
+    x = I.gen_verify_inputs(cfg, 1, "cuda")
+    assert (x.hidden is not None) == explicit_hidden
+    kv = m.kv(x.k_pool, x.v_pool, x.page_table, x.prefix_len)
+    names = ("q", "k_new", "v_new", "tokens")
+    h_in = {k: getattr(x, k).cpu().pin_memory() for k in names}
+    d_in = {k: torch.zeros_like(getattr(x, k)) for k in names}
+    acc = m.accept_in(binding.ACCEPT_GREEDY, True)
+    attn_h, attn_d = torch.zeros_like(x.q), torch.empty_like(x.q)
+    res_h, res_d = binding.AcceptResult(cfg.batch, cfg.gamma, "cuda"), binding.AcceptResult(cfg.batch, cfg.gamma, "cuda")
+    m.mirror_verify_step(kv, m.tree(x.tokens, cfg.kappa, cfg.gamma), x.q, x.k_new, x.v_new, x.hidden, x.W, acc, attn_d, out=res_d)
+    torch.cuda.synchronize()
+    m.mirror_verify_step_host(kv, m.tree(d_in["tokens"], cfg.kappa, cfg.gamma), h_in, d_in, x.hidden, x.W, acc, attn_h, res_h)
+    torch.cuda.synchronize()
+    assert m.device_status() == (0, 0)
+    assert torch.equal(attn_h, attn_d)
+    for f in FIELDS:
+        assert torch.equal(getattr(res_h, f), getattr(res_d, f)), f
+    for k in names:
+        assert torch.equal(d_in[k], getattr(x, k)), k
