@@ -20,6 +20,9 @@ namespace {
 
 constexpr int kFinThreads = 256;
 
+// Stacks up to this depth take the faster attention kernel.  Deeper ones keep the order of every sum (see attn_tile64.cu).
+constexpr int kKeepRoundingLayers = 4;
+
 struct TreeDepths {
     int depth[MIRROR_MAX_NODES];
 };
@@ -66,9 +69,6 @@ __device__ __forceinline__ void store4(__nv_bfloat16* dst, float a, float b, flo
 // [M, Hq, d] / [M, Hkv, d] tensors.  A thread does four rotation pairs (f, f + d/2) of one head; all slices of its columns
 // are loaded before they are added (the loads are independent, the order of the sum is fixed).  Few and small blocks: the
 // next kernel's blocks have to find room beside them (952 blocks of 64 threads took 4.7 us at 17 rows, these 2.5).
-// Stacks up to this depth take the faster attention kernel.  Deeper ones keep the order of every sum (see attn_tile64.cu): a
-// layer turns a difference of 0.25% of its attention output into 0.1..0.2% of its own, and 48 layers into 3.5%.
-constexpr int kKeepRoundingLayers = 4;
 constexpr int kQkvThreads = 128;
 __global__ void __launch_bounds__(kQkvThreads)
 finish_qkv_kernel(const float* partial, int slices, int M, int Hq, int Hkv, int d, const float2* cs,
