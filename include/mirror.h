@@ -130,7 +130,8 @@ typedef struct {
 #define MIRROR_WS_LMHEAD_LOGITS 10u /* mirror_lmhead_reduce with a workspace that can hold the fp32 logits [M, V] */
 #define MIRROR_WS_LMHEAD_TOPK 34u   /* mirror_lmhead_reduce with topk > 0, mirror_early_exit_tap.  Up to 256 rows the Top-kappa is
                                        selected inside the GEMM's epilogue: candidate lists instead of an [M, V] buffer; with more
-                                       rows this sizes like MIRROR_WS_LMHEAD_LOGITS (the selection reads spilled logits) */
+                                       rows, or a vocabulary of up to 65536 ids that is better selected from, this sizes like
+                                       MIRROR_WS_LMHEAD_LOGITS (the selection reads spilled logits) */
 #define MIRROR_WS_STEP_GREEDY 7u    /* mirror_verify_step, greedy */
 #define MIRROR_WS_STEP_SPEC 15u     /* mirror_verify_step, speculative sampling (holds the fp32 logits) */
 #define MIRROR_WS_ACCEPT_TREE 16u   /* adds the fp64 scratch of MIRROR_ACCEPT_SPEC_TREE (optional: without it the rule
@@ -198,7 +199,8 @@ mirror_status mirror_kv_quantize_fp8(mirror_ctx* ctx, const void* x, int n_layer
  *   logits_out fp32 [M, V], nullable: the full logits (needed by speculative sampling)
  * Needs a workspace sized for MIRROR_WS_LMHEAD; with topk > 0 one sized for MIRROR_WS_LMHEAD_TOPK: with up to 256 rows the
  * Top-kappa is then selected inside the GEMM's epilogue (sorted candidate lists, merged afterwards) and the logits never
- * reach memory; with more rows the selection runs over spilled fp32 logits. */
+ * reach memory; with more rows, and over small vocabularies where that is faster and the workspace has the room, the
+ * selection runs over spilled fp32 logits.  The result is the same. */
 mirror_status mirror_lmhead_reduce(mirror_ctx* ctx, const void* hidden, int M, const void* W, int topk,
                                    const int32_t* gather_row, const int32_t* gather_tok, int n_gather,
                                    int32_t* argmax, float* maxlogit, float* lse,
@@ -273,8 +275,8 @@ mirror_status mirror_accept_select(mirror_ctx* ctx, const mirror_tree* tree, con
  *   msg_ids          int32 [M, kappa]: candidate ids ordered by (logit descending, id ascending)
  *   msg_logprob_bf16 bf16 [M, kappa]: their log-probabilities logit/T - lse under the early-exit proxy (the token
  *                    channel's payload type)
- * kappa <= MIRROR_MAX_TOPK.  Needs a workspace sized for MIRROR_WS_LMHEAD_TOPK with M rows (up to 256 rows the selection
- * happens in the GEMM's epilogue and there is no [M, V] buffer).  msg_ids is what mirror_accept_select / mirror_verify_step take as cand_ids (n_cand =
+ * kappa <= MIRROR_MAX_TOPK.  Needs a workspace sized for MIRROR_WS_LMHEAD_TOPK with M rows (up to 256 rows and over a
+ * large vocabulary the selection happens in the GEMM's epilogue and there is no [M, V] buffer).  msg_ids is what mirror_accept_select / mirror_verify_step take as cand_ids (n_cand =
  * kappa) for the reuse decision of the same rows. */
 mirror_status mirror_early_exit_tap(mirror_ctx* ctx, const void* hidden_le, int M, const void* W, int kappa,
                                     int32_t* msg_ids, void* msg_logprob_bf16, void* stream);
