@@ -242,6 +242,9 @@ __device__ __forceinline__ Partition make_partition(const AttnParams& p, const i
     const long long per = (long long)(p.Hkv / p.heads_per_unit) * cumT[p.B], total = per * p.L;
     q.tiles_per_layer = (int)per;
     q.total_tiles = total < (1ll << 31) ? (int)total : -1;
+    q.n_groups = min(p.n_groups, p.units);
+    q.snap_tol = q.share = q.rest = 0;
+    if (p.never_cut) return q;                                        // (group_begin counts units; short launches fetch no more code)
     // Units of equal length (every request has the same number of tiles): a group count that divides the units, if one
     // exists within 15% of the CTA groups there are, gives every group the same number of WHOLE units: no unit is cut,
     // nothing is left to merge and all groups end together, which is worth more than the few SMs left idle.
@@ -250,13 +253,13 @@ __device__ __forceinline__ Partition make_partition(const AttnParams& p, const i
     // Else every group gets at least one tile, or two where its streams take alternate tiles (one alone would leave a stream
     // without work and the merge with twice the records).
     const int split = p.mode == kSplit ? 1 : 0, most = min(p.n_groups, max(1, q.total_tiles >> split));
-    q.n_groups = p.never_cut ? min(p.n_groups, p.units) : p.whole_groups > 0 && equal_units ? p.whole_groups : most;
+    q.n_groups = p.whole_groups > 0 && equal_units ? p.whole_groups : most;
     // Fewer units than groups, all of one length: the same number of groups for every unit, where that costs a group few tiles.
     // (An even split over all groups makes most of them work on two units: a second Q, which an e4m3 cache converts, a second
     // epilogue and record; whole units also need no merge.  64 units of 9 tiles over 74 groups, bf16 / e4m3: 53 -> 30 / 68 -> 36 us;
     // 16 units over 37 groups, two each: 39 -> 33 / 54 -> 40.  But 16 units of 157 tiles over 74 groups, four each, bf16, which is
     // 5 tiles longer: 95 -> 104.)
-    if (p.unit_cuts > 0 && equal_units && !p.never_cut) {
+    if (p.unit_cuts > 0 && equal_units) {
         const int cuts = min(p.unit_cuts, max(1, cumT[1] >> split));
         if (cuts_pay(cumT[1], p.units, most, cuts, p.cut_tiles)) q.n_groups = p.units * cuts;
     }
