@@ -219,11 +219,6 @@ __device__ __forceinline__ bool wait_bar(Ctrl* c, uint64_t* bar, uint32_t parity
     if (__all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity))) return true;
     return wait_slow(c, bar, parity, where);
 }
-__device__ __forceinline__ bool elect_one() {            // one lane of a converged warp
-    uint32_t r;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
-    return r != 0;
-}
 
 // How the tile sequence is cut into one range per CTA group.  (This runs in front of every launch's first copy, by one
 // warp and from a cold instruction cache: few divisions, and those of 32 bits.)
@@ -653,13 +648,13 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                         int row[kTileSlots];
 #pragma unroll
                         for (int k = 0; k < kTileSlots; ++k) row[k] = (row0 + __shfl_sync(0xffffffffu, pg, k)) * p.Hkv + head;
-                        if (elect_one()) {
+                        if (ptx::elect_one()) {
                             ptx::mbar_arrive_expect_tx(bar, (uint32_t)C::kStageBytes);
 #pragma unroll
                             for (int k = 0; k < kTileSlots; ++k) ptx::tma_load_5d(dst + k * C::kSlotBytes, map, bar, 0, 0, 0, 0, row[k]);
                         }
                     } else {
-                        const bool leader = elect_one();
+                        const bool leader = ptx::elect_one();
                         if (leader) ptx::mbar_arrive_expect_tx(bar, (uint32_t)((n_sl - (ragged >= 0)) * C::kSlotBytes));
 #pragma unroll 1
                         for (int k = 0; k < n_sl; ++k) {
@@ -842,7 +837,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     wait(&ctrl->p_full[g][0], p_par, 23);
                     if (!ok) break;
                     ptx::tc_fence_after();
-                    if (elect_one()) {
+                    if (ptx::elect_one()) {
                         pv(0, min(pv_sl, kTileSlots / 2));
                         ptx::umma_commit(&ctrl->pv_half[g]);
                     }
@@ -857,7 +852,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                 const uint32_t n_qk = slots_of(nx) * kSlotTok, idesc_qk = F8 ? attn::umma_idesc_plain(kRows, n_qk) : ptx::umma_idesc_bf16(kRows, n_qk);
                 const uint32_t kb = k_lo + kst * (uint32_t)(C::kStageBytes >> 4);
                 const uint32_t qa = q_lo + (uint32_t)buf * q_buf;
-                if (elect_one()) {
+                if (ptx::elect_one()) {
                     if (do_pv) {
                         pv(kTileSlots / 2, pv_sl);
                         ptx::umma_commit(&v_empty[vst]);

@@ -71,9 +71,12 @@ struct Ctrl {
     uint64_t empty[kMaxStages];             // UMMAs that read the stage have completed (multicast commit)
     uint64_t acc_full[kAcc];                // accumulator complete (multicast commit)
     uint64_t acc_empty[kAcc];               // leader only: 4 + 4 epilogue warps have drained the accumulator
+    int* status;
+    long long wait_limit;
     uint32_t tmem_base;
     volatile int abort;
 };
+static_assert(sizeof(Ctrl) <= 1024, "control block");
 
 __device__ __forceinline__ void fail(const PairParams& p, Ctrl* c, int where) {
     c->abort = 1;
@@ -98,22 +101,50 @@ __device__ __forceinline__ uint32_t map_to_rank(const void* smem_ptr, uint32_t r
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// bounded wait on a barrier that the other CTA of the pair arrives on
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, long long limit_cycles = 4000000000ll) {
-    const uint32_t a = ptx::smem_u32(bar);
+// Bounded waits by all lanes of a converged warp, which all get the same answer: one poll inline; parking, the abort flag and the
+// limit are out of line.  kCluster: the other CTA of the pair arrives on the barrier.
+template <bool kCluster>
+__device__ __forceinline__ bool try_wait(uint64_t* bar, uint32_t parity) {
+    if (!kCluster) return __all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity));
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(ptx::smem_u32(bar)), "r"(parity)
+        : "memory");
+    return __all_sync(0xffffffffu, ok != 0);
+}
+template <bool kCluster>
+__device__ __noinline__ bool wait_slow(Ctrl* c, uint64_t* bar, uint32_t parity, int where) {
     const long long t0 = clock64();
     for (;;) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(a), "r"(parity), "r"(MIRROR_PARK_NS)
-            : "memory");
-        if (ok) return true;
-        if (clock64() - t0 > limit_cycles) return false;
+        if (__all_sync(0xffffffffu, ptx::mbar_try_wait_park(bar, parity, MIRROR_PARK_NS)) && try_wait<kCluster>(bar, parity)) return true;
+        const bool late = clock64() - t0 > c->wait_limit;
+        if (__any_sync(0xffffffffu, c->abort || late)) {
+            c->abort = 1;
+            if (late && atomicCAS(c->status, 0, MIRROR_DEV_TIMEOUT) == 0) atomicExch(c->status + 1, where);
+            return false;
+        }
     }
+}
+template <bool kCluster = false>
+__device__ __forceinline__ bool wait_warp(Ctrl* c, uint64_t* bar, uint32_t parity, int where) {
+    return try_wait<kCluster>(bar, parity) || wait_slow<kCluster>(c, bar, parity, where);
+}
+// Has the phase completed?  (Does not block; try_wait may, for as long as the hardware likes: asked that way for the K block behind the
+// one at hand, the issuer held that one back until the other had arrived, and short launches took up to half as long again.)
+__device__ __forceinline__ bool poll(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(ptx::smem_u32(bar)), "r"(parity)
+        : "memory");
+    return __all_sync(0xffffffffu, ok != 0);
 }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* smem_result, uint32_t ncols) {    // one warp of EACH CTA
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(smem_result)), "r"(ncols)
@@ -134,24 +165,27 @@ __device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const void* map
         ::"r"(ptx::smem_u32(smem_dst)), "l"(map), "r"(bar_cluster_addr), "r"(x), "r"(y), "l"(policy)
         : "memory");
 }
-// D[tmem of both CTAs] (+)= A (128 rows from each CTA's shared memory) * B (N/2 rows from each CTA's shared memory)
-__device__ __forceinline__ void umma_pair_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                              uint32_t accumulate) {
+// D[tmem of both CTAs] (+)= A (128 rows from each CTA's shared memory) * B (N/2 rows from each CTA's shared memory); the low words of
+// the two descriptors, which share the high one
+__device__ __forceinline__ void umma_pair_f16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %3};\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 // the same for e4m3 operands (32 elements of K per instruction: the same 32 bytes of a 128-byte swizzled row)
-__device__ __forceinline__ void umma_pair_f8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                             uint32_t accumulate) {
+__device__ __forceinline__ void umma_pair_f8(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %3};\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], da, db, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 // instruction descriptor for e4m3 x e4m3 -> fp32, both operands K-major
@@ -258,6 +292,8 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
         }
         for (int a = 0; a < kAcc; ++a) { ptx::mbar_init(&ctrl->acc_full[a], 1); ptx::mbar_init(&ctrl->acc_empty[a], 8); }
         ctrl->abort = 0;
+        ctrl->status = p.status;
+        ctrl->wait_limit = p.wait_limit;
         ptx::fence_mbar_init();
         ptx::prefetch_tmap(&tm_w);
         ptx::prefetch_tmap(&tm_h);
@@ -273,13 +309,13 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
     const uint32_t tmem_base = ctrl->tmem_base;
     // The weights of the first stages, while the kernel ahead is still at work (their rows of x follow behind the wait).
     int n_early = 0;
-    if (kEarly && p.w_early && warp == 0 && lane == 0 && pair < p.n_units) {
+    if (kEarly && p.w_early && warp == 0 && pair < p.n_units) {
         int tile, slice, chunk;
         decode(pair, tile, slice, chunk);
         const int kb0 = slice * p.kb_per_slice;
         n_early = min(p.stages, min(n_kb, kb0 + p.kb_per_slice) - kb0);
         const uint64_t pol_w = p.w_keep ? ptx::policy_evict_normal() : ptx::policy_evict_first();
-        for (int s = 0; s < n_early; ++s) {
+        for (int s = 0; s < n_early && lane == 0; ++s) {
             if (rank == 0) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
             tma_load_2d_pair(stage_base + s * p.stage_bytes, &tm_w, map_to_rank(&ctrl->full[s], 0), (kb0 + s) * kBK, (tile * 2 + (int)rank) * p.rows_cta, pol_w);
         }
@@ -287,83 +323,92 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
 
+    // Producer and issuer: the whole warp walks the schedule and one elected lane issues, which keeps addresses and descriptors in
+    // uniform registers; the next K block's barrier is polled ahead of the instructions that hold the lane up.  What the issuer spends
+    // on a K block is the pace of a pair that its memory could feed faster, and of the tensor cores: with all of it in one lane 600 cycles
+    // (four UMMAs 280, a wait that need not wait 114, the commit 58), whatever the rows.  16 pairs alone, 2 x 64 rows each of 10 KB: 52 ->
+    // 108 GB/s per SM; LM head of 152064 x 5120 at 196 / 392 / 520 rows 334 / 594 / 849 -> 289 / 511 / 669 us.
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (both CTAs)
-        if (lane == 0) {
-            const uint64_t pol_w = p.w_keep ? ptx::policy_evict_normal() : ptx::policy_evict_first();
-            const uint64_t pol_h = ptx::policy_evict_last();
-            int s = 0, n_issued = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            // the rows of x that belong to the weights requested early.  (A loop of its own: a test per K block in the main loop
-            // made 275 rows x 42306 x 2304 take 110 instead of 102 us.)
-            for (; kEarly && n_issued < n_early && ok; ++n_issued) {
-                if (p.stall_after >= 0 && n_issued >= p.stall_after) { ok = false; break; }           // (test aid, as below)
-                int tile, slice, chunk;
-                decode(pair, tile, slice, chunk);
-                tma_load_2d_pair(stage_base + s * p.stage_bytes + p.a_bytes, &tm_h, map_to_rank(&ctrl->full[s], 0), (slice * p.kb_per_slice + n_issued) * kBK,
+        const uint64_t pol_w = p.w_keep ? ptx::policy_evict_normal() : ptx::policy_evict_first();
+        const uint64_t pol_h = ptx::policy_evict_last();
+        const uint32_t full0 = map_to_rank(&ctrl->full[0], 0);
+        int s = 0, n_issued = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        // the rows of x that belong to the weights requested early.  (A loop of its own: a test per K block in the main loop
+        // made 275 rows x 42306 x 2304 take 110 instead of 102 us.)
+        for (; kEarly && n_issued < n_early && ok; ++n_issued) {
+            if (p.stall_after >= 0 && n_issued >= p.stall_after) { ok = false; break; }           // (test aid, as below)
+            int tile, slice, chunk;
+            decode(pair, tile, slice, chunk);
+            if (ptx::elect_one())
+                tma_load_2d_pair(stage_base + s * p.stage_bytes + p.a_bytes, &tm_h, full0 + s * 8, (slice * p.kb_per_slice + n_issued) * kBK,
                                  chunk * p.chunk_rows + (int)rank * p.half_rows, pol_h);
+            if (++s == p.stages) { s = 0; ph ^= 1; }
+        }
+        int kb_skip = n_issued;
+        for (int u = pair; u < p.n_units && ok; u += n_pairs) {
+            int tile, slice, chunk;
+            decode(u, tile, slice, chunk);
+            const int w_row = (tile * 2 + (int)rank) * p.rows_cta;
+            const int h_row = chunk * p.chunk_rows + (int)rank * p.half_rows;
+            const int kb_end = min(n_kb, (slice + 1) * p.kb_per_slice);
+            int kb = slice * p.kb_per_slice + kb_skip;
+            kb_skip = 0;
+#pragma unroll 1
+            for (; kb < kb_end; ++kb) {
+                if (p.stall_after >= 0 && n_issued >= p.stall_after) { ok = false; break; }       // (test aid: neither arms nor copies)
+                if (!wait_warp(ctrl, &ctrl->empty[s], ph ^ 1, 11)) { ok = false; break; }
+                if (ptx::elect_one()) {
+                    if (rank == 0) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
+                    uint8_t* dst = stage_base + s * p.stage_bytes;
+                    tma_load_2d_pair(dst, &tm_w, full0 + s * 8, kb * kBK, w_row, pol_w);
+                    tma_load_2d_pair(dst + p.a_bytes, &tm_h, full0 + s * 8, kb * kBK, h_row, pol_h);
+                }
+                __syncwarp();
+                ++n_issued;
                 if (++s == p.stages) { s = 0; ph ^= 1; }
             }
-            int kb_skip = n_issued;
-            for (int u = pair; u < p.n_units && ok; u += n_pairs) {
-                int tile, slice, chunk;
-                decode(u, tile, slice, chunk);
-                const int w_row = (tile * 2 + (int)rank) * p.rows_cta;
-                const int h_row = chunk * p.chunk_rows + (int)rank * p.half_rows;
-                const int kb_end = min(n_kb, (slice + 1) * p.kb_per_slice);
-                int kb = slice * p.kb_per_slice + kb_skip;
-                kb_skip = 0;
-                for (; kb < kb_end; ++kb) {
-                    if (p.stall_after >= 0 && n_issued >= p.stall_after) { ok = false; break; }       // (test aid: neither arms nor copies)
-                    if (ctrl->abort || !ptx::mbar_wait(&ctrl->empty[s], ph ^ 1, p.wait_limit)) { fail(p, ctrl, 11); ok = false; break; }
-                    if (rank == 0) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
-                    const uint32_t bar = map_to_rank(&ctrl->full[s], 0);
-                    uint8_t* dst = stage_base + s * p.stage_bytes;
-                    tma_load_2d_pair(dst, &tm_w, bar, kb * kBK, w_row, pol_w);
-                    tma_load_2d_pair(dst + p.a_bytes, &tm_h, bar, kb * kBK, h_row, pol_h);
-                    ++n_issued;
-                    if (++s == p.stages) { s = 0; ph ^= 1; }
-                }
-            }
-            // (copies still in flight after a failure: the leader's issuer or its 2 s limit outlasts them, and both CTAs
-            // meet at the cluster barrier below before either one's shared memory goes away)
         }
+        // (copies still in flight after a failure: the leader's issuer or its 2 s limit outlasts them, and both CTAs
+        // meet at the cluster barrier below before either one's shared memory goes away)
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             // -------------------------------------------------------------- UMMA issuer (leader)
             const uint32_t idesc = kFp8 ? umma_idesc_e4m3(kPairV, p.chunk_rows) : ptx::umma_idesc_bf16(kPairV, p.chunk_rows);
-            const uint32_t stage_u32 = ptx::smem_u32(stage_base);
+            const uint32_t hi = ptx::umma_desc_hi_sw128(1024), lo0 = ptx::umma_desc_lo(ptx::smem_u32(stage_base), 16);
+            const uint32_t stage_lo = (uint32_t)p.stage_bytes >> 4, a_lo = (uint32_t)p.a_bytes >> 4;
             int s = 0, ab = 0;
-            uint32_t ph = 0, aph = 0;
+            uint32_t ph = 0, aph = 0, lo = lo0;
             bool ok = true;
             for (int u = pair; u < p.n_units && ok; u += n_pairs) {
-                if (ctrl->abort || !mbar_wait_cluster(&ctrl->acc_empty[ab], aph ^ 1, p.wait_limit)) { fail(p, ctrl, 12); ok = false; break; }
-                ptx::tc_fence_after();
+                if (!wait_warp<true>(ctrl, &ctrl->acc_empty[ab], aph ^ 1, 12)) { ok = false; break; }
                 const uint32_t d_tmem = tmem_base + (uint32_t)(ab * p.acc_stride);
                 int tile, slice, chunk;
                 decode(u, tile, slice, chunk);
                 const int nk = min(n_kb, (slice + 1) * p.kb_per_slice) - slice * p.kb_per_slice;
+                bool ready = poll(&ctrl->full[s], ph);
+#pragma unroll 1
                 for (int kb = 0; kb < nk; ++kb) {
-                    if (ctrl->abort || !ptx::mbar_wait(&ctrl->full[s], ph, p.wait_limit)) { fail(p, ctrl, 13); ok = false; break; }
+                    if (!ready && !wait_slow<false>(ctrl, &ctrl->full[s], ph, 13)) { ok = false; break; }
                     ptx::tc_fence_after();
-                    const uint32_t sa = stage_u32 + (uint32_t)(s * p.stage_bytes);
-                    const uint32_t sb = sa + (uint32_t)p.a_bytes;
-                    if constexpr (kFp8) {
+                    uint64_t* const done = &ctrl->empty[s];
+                    const uint32_t a = lo;
+                    lo += stage_lo;
+                    if (++s == p.stages) { s = 0; ph ^= 1; lo = lo0; }
+                    ready = poll(&ctrl->full[s], ph);              // (the next K block's; of no use behind the last one of all)
+                    if (ptx::elect_one()) {
 #pragma unroll
-                        for (int k4 = 0; k4 < kBK / 16; ++k4)
-                            umma_pair_f8(d_tmem, ptx::umma_desc_k_sw128(sa + k4 * 32), ptx::umma_desc_k_sw128(sb + k4 * 32), idesc,
-                                         (kb | k4) != 0);
-                    } else {
-#pragma unroll
-                        for (int k4 = 0; k4 < kBK / 16; ++k4)
-                            umma_pair_f16(d_tmem, ptx::umma_desc_k_sw128(sa + k4 * 32), ptx::umma_desc_k_sw128(sb + k4 * 32), idesc,
-                                          (kb | k4) != 0);
+                        for (int k4 = 0; k4 < kBK / 16; ++k4) {
+                            if (kFp8) umma_pair_f8(d_tmem, a + k4 * 2, a + a_lo + k4 * 2, hi, idesc, (kb | k4) != 0);
+                            else umma_pair_f16(d_tmem, a + k4 * 2, a + a_lo + k4 * 2, hi, idesc, (kb | k4) != 0);
+                        }
+                        umma_commit_pair(done);
+                        if (kb + 1 == nk) umma_commit_pair(&ctrl->acc_full[ab]);
                     }
-                    umma_commit_pair(&ctrl->empty[s]);
-                    if (++s == p.stages) { s = 0; ph ^= 1; }
+                    __syncwarp();
                 }
-                if (ok) umma_commit_pair(&ctrl->acc_full[ab]);
                 if (++ab == kAcc) { ab = 0; aph ^= 1; }
             }
         }
