@@ -79,6 +79,7 @@ constexpr int kMergeSmem = kMergeSlots * 10 * 128 * 4;      // their columns, th
 // code that runs once: a chunk of a record is 4 KB in one piece, so bulk copies bring everything a block needs at once,
 // and the arithmetic runs out of shared memory (17 parts of 85 rows: 15 us with loads in the loop over the parts, 8 with
 // eight parts' loads in flight).
+// The caller has waited for the records, and lets the kernel behind be launched.
 // map(row, GroupBegin) -> false, or the row's node and query head; record(group, slot) -> its record in slot 0 (of the unit
 // that began before the group's range) or 1, [column][128 rows], D accumulator columns, then (max, sum).  wait_limit: SM cycles
 // after which a wait gives up; stall: test aid, 1 makes the first wait run out (it expects bytes that nobody copies).
@@ -90,9 +91,7 @@ __device__ __forceinline__ void merge_boundary(const GroupBegin* table, int n_gr
     __shared__ GroupBegin s_begin[512];
     __shared__ uint64_t s_bar;
     const int tid = threadIdx.x, warp = tid >> 5, g = blockIdx.x + 1;
-    ptx::grid_dep_launch();                       // (the kernel behind only sets itself up before this one has completed)
     if (tid == 0) { ptx::mbar_init(&s_bar, 1); ptx::fence_mbar_init(); }
-    ptx::grid_dep_wait();
     for (int i = tid; i < n_groups; i += kMergeThreads) s_begin[i] = table[i];
     __syncthreads();
     const GroupBegin u = s_begin[g];

@@ -863,6 +863,8 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
 template <int D>
 __global__ void __launch_bounds__(attn::kMergeThreads) attn_tile64_merge_kernel(const __grid_constant__ AttnParams p) {
     const int rb = blockIdx.y;
+    ptx::grid_dep_launch();                       // (the kernel behind only sets itself up before this one has completed)
+    ptx::grid_dep_wait();
     attn::merge_boundary<D>(
         p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out, p.status, p.wait_limit, p.stall_merge,
         [&](int row, const attn::GroupBegin& u, int& node, int& head) {

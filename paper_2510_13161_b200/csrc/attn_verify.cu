@@ -47,6 +47,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "attn_common.h"
@@ -89,6 +90,10 @@ struct AttnParams {
     int unit_cuts;                        // fewer units than groups: groups per unit, rounded down; 0 otherwise
     int cut_tiles;                        // tiles that a group may take longer for it
     int never_cut;                        // 1: units are so short that they are dealt out whole whatever their lengths
+    float lm_ns;                          // > 0: time of the weight stream that is launched behind and runs beside this (see share_choice)
+    int deal;                             // 1: where SMs are left to it, whole units are dealt out
+    int group_chunk;                      // groups that fill whole TPCs (pairs of SMs)
+    int late_merge;                       // 1: the merge runs behind a launch that waited for this one
     int max_pages, num_pages, layer_pages;
     int tree_slots;
     float scale_log2e;
@@ -193,6 +198,7 @@ struct Ctrl {
     uint64_t pair[4];                                   // split: the two softmax warps of a TMEM quarter meet
     Segment first;                                      // where this CTA's range begins
     int n_tiles;
+    int group;                                          // which group this CTA belongs to
     int* status;
     long long wait_limit;
     uint32_t tmem_base;
@@ -224,6 +230,7 @@ __device__ __forceinline__ bool wait_bar(Ctrl* c, uint64_t* bar, uint32_t parity
 // warp and from a cold instruction cache: few divisions, and those of 32 bits.)
 struct Partition {
     int tiles_per_layer, total_tiles;     // (total_tiles -1: the sequence does not fit 31 bits)
+    bool whole;                           // units are dealt out whole, by number
     int n_groups, snap_tol;
     int share, rest;                      // total_tiles = n_groups * share + rest
 };
@@ -232,13 +239,64 @@ struct Partition {
 __host__ __device__ inline bool cuts_pay(int tiles, int units, int groups, int cuts, int more) {
     return (long long)tiles * groups - (long long)tiles * units * cuts <= (long long)more * cuts * groups;
 }
-__device__ __forceinline__ Partition make_partition(const AttnParams& p, const int* cumT) {
+// How many groups to use when a weight stream that does not depend on this launch follows it (lmhead_pair_free_kernel): it takes
+// whatever SMs are left.  Attention is bound by its exponentials and uses a quarter to two thirds of HBM, the stream uses nothing
+// else, so side by side they take less than one after the other.  A choice (0: all groups, up to 31) is weighed by the time at
+// which both are through: attention at kStepNs per step and kUnitSteps more per unit, the stream at the rate of the SMs that it has
+// meanwhile (kFullSms keep HBM busy) and of the bandwidth that is left to it, then alone; it has to gain 3%.  (48 layers x 2048
+// tokens x 285 rows before 1.56 GB of weights: 28 of 49 groups, 469 -> 433 us; unshared 447.)
+constexpr float kStepNs = 2100.f, kUnitSteps = 4.5f, kFullSms = 85.f, kHbmBytesNs = 6500.f, kShareGain = 0.97f;
+struct Share {
+    int g;
+    float total;                          // ns
+};
+__host__ __device__ inline Share share_choice(const AttnParams& p, float total_tiles, int most, int sms, float step_bytes, int choice) {
+    const float steps = p.mode == kSplit ? 0.5f * (total_tiles + (float)p.units) : total_tiles;
+    const float work = steps + kUnitSteps * (float)p.units;
+    int g = most - most * choice / 40;
+    if (g < 1) g = 1;
+    float t;
+    if (p.deal) {
+        const int k = (p.units + g - 1) / g;
+        g = (p.units + k - 1) / k;
+        t = (float)k * work / (float)p.units;
+    } else {
+        t = (work + kUnitSteps * (float)g) / (float)g;
+    }
+    t *= kStepNs;
+    const float hbm = 1.f - (float)g * step_bytes * steps / (work * kStepNs * kHbmBytesNs);
+    const float rate = fminf((float)(sms - g * p.n_cta) / kFullSms, fmaxf(hbm, 0.1f));
+    return {g, t + fmaxf(0.f, p.lm_ns - t * rate)};
+}
+__device__ __noinline__ int share_groups(const AttnParams& p, int total_tiles, int most, int sms, float step_bytes) {
+    const int lane = threadIdx.x & 31;
+    const Share s = share_choice(p, (float)total_tiles, most, sms, step_bytes, lane);
+    // the least total time, and of equals the most groups
+    const uint32_t key = (__float_as_uint(s.total) & ~31u) | (uint32_t)lane;
+    const uint32_t best = __reduce_min_sync(0xffffffffu, key);
+    const bool gains = __uint_as_float(best) < kShareGain * __shfl_sync(0xffffffffu, s.total, 0);
+    const int g = __shfl_sync(0xffffffffu, s.g, best & 31u);
+    return gains ? g : most;
+}
+__device__ __forceinline__ Partition make_partition(const AttnParams& p, const int* cumT, float step_bytes) {
     Partition q;
     const long long per = (long long)(p.Hkv / p.heads_per_unit) * cumT[p.B], total = per * p.L;
     q.tiles_per_layer = (int)per;
     q.total_tiles = total < (1ll << 31) ? (int)total : -1;
     q.n_groups = min(p.n_groups, p.units);
     q.snap_tol = q.share = q.rest = 0;
+    q.whole = p.never_cut != 0;
+    if (p.lm_ns > 0.f && q.total_tiles > 0 && q.n_groups > 1) {
+        const int most = min(p.n_groups, p.never_cut ? p.units : q.total_tiles), g = share_groups(p, q.total_tiles, most, gridDim.x, step_bytes);
+        if (g < most) {
+            q.n_groups = g;
+            q.whole |= p.deal != 0;
+            q.share = (int)((uint32_t)q.total_tiles / (uint32_t)g);
+            q.rest = q.total_tiles - q.share * g;
+            q.snap_tol = min(p.snap_cap, q.share >> 2);
+            return q;
+        }
+    }
     if (p.never_cut) return q;                                        // (group_begin counts units; short launches fetch no more code)
     // Units of equal length (every request has the same number of tiles): a group count that divides the units, if one
     // exists within 15% of the CTA groups there are, gives every group the same number of WHOLE units: no unit is cut,
@@ -268,7 +326,7 @@ __device__ __forceinline__ Partition make_partition(const AttnParams& p, const i
 __device__ __noinline__ int group_begin(const Partition& q, int g, const AttnParams& p, const int* cumT) {
     if (g <= 0) return 0;
     if (g >= q.n_groups) return q.total_tiles;
-    if (p.never_cut) {                                                // first tile of unit number units * g / n_groups
+    if (q.whole) {                                                    // first tile of unit number units * g / n_groups
         const int hu = p.Hkv / p.heads_per_unit, per = p.B * hu;
         const int us = p.units / q.n_groups, unit = us * g + (p.units - us * q.n_groups) * g / q.n_groups;
         const int layer = unit / per, r = unit - layer * per, b = r / hu;
@@ -281,6 +339,15 @@ __device__ __noinline__ int group_begin(const Partition& q, int g, const AttnPar
     const int best = (e - lo <= hi - e) ? lo : hi;
     const int dist = best > e ? best - e : e - best;
     return dist <= q.snap_tol ? best : e;
+}
+
+// A launch that leaves SMs to another one leaves whole TPCs (the other's CTAs come in pairs), spread over the chip as blocks are
+// over its GPCs: of every `chunk` groups all work or none.  Which one group number `g` stands for, of `most`, `used` of them at work.
+__host__ __device__ inline int spread_group(int g, int most, int used, int chunk) {
+    const int chunks = most / chunk, n = (used + chunk - 1) / chunk, c = g / chunk;
+    if (used >= most || n >= chunks || c >= chunks) return g;
+    const int r0 = c * n / chunks, r1 = (c + 1) * n / chunks;
+    return (r1 > r0 ? r0 : n + c - r0) * chunk + (g - c * chunk);
 }
 
 // Prefix lengths (clamped to the page table) and the tile counts they give, by one warp.
@@ -518,7 +585,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
     int* s_len = cumT + (p.B + 1);                                  // [B] clamped prefix lengths
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int group = blockIdx.x / p.n_cta, rb = blockIdx.x % p.n_cta;
+    const int rb = blockIdx.x % p.n_cta;
     const bool split = p.mode == kSplit;
     const bool shared_kv = stream_of(p, rb, 0).shared_kv;
 
@@ -564,7 +631,8 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
     ptx::grid_dep_launch();                 // the kernel behind may be scheduled as soon as SMs free up
     if (warp == 0) {
         load_lengths(p, cumT, s_len, true);
-        const Partition part = make_partition(p, cumT);
+        const Partition part = make_partition(p, cumT, (float)(C::kStageBytes * (split ? 4 : 2)));
+        const int block_group = blockIdx.x / p.n_cta, group = p.lm_ns > 0.f ? spread_group(block_group, p.n_groups, part.n_groups, p.group_chunk) : block_group;
         const bool fits = part.total_tiles >= 0 && (ptx::smem_u32(smem) & 1023) == 0;
         if (!fits && lane == 0) dev_check(p, 600);
         int x = 0;
@@ -572,9 +640,10 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         const int x1 = __shfl_sync(0xffffffffu, x, 1);
         if (lane == 0) {
             ctrl->n_tiles = x1 - x;
+            ctrl->group = group;
             if (x < x1) ctrl->first = first_segment(x, x1, p, cumT, s_len, part.tiles_per_layer);
             const Segment& s = ctrl->first;
-            if (rb == 0) p.begins[group] = {x < x1 && s.t_first > 0 ? 1 : 0, s.layer, s.b, s.g};
+            if (rb == 0 && group < p.n_groups) p.begins[group] = {x < x1 && s.t_first > 0 ? 1 : 0, s.layer, s.b, s.g};
         }
     }
     __syncthreads();
@@ -1148,7 +1217,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             float* lse_ptr = p.lse_out ? p.lse_out + (lb * p.Hq + head) * p.n + node : nullptr;
             const int slot = (sg.t_first > 0) ? 0 : 1;             // a unit that began before this CTA's range uses slot 0
             // record layout [column][row]: a warp's store of one column is one contiguous 128-byte line
-            float* rec = p.partial + (((size_t)blockIdx.x * 2 + slot) * 2 + (split ? 0 : grp)) * kRowW * kRows + row;
+            float* rec = p.partial + (((size_t)(ctrl->group * p.n_cta + rb) * 2 + slot) * 2 + (split ? 0 : grp)) * kRowW * kRows + row;
             left -= sg.t_last - sg.t_first;
             Segment nx = sg;
             if (left > 0) nx = next_segment(sg, left, p, s_len);
@@ -1237,6 +1306,9 @@ __global__ void __launch_bounds__(attn::kMergeThreads) attn_merge_kernel(const _
     const int n_str = p.mode == kSplit ? 1 : 2;
     const int rb = blockIdx.y / n_str, grp = blockIdx.y % n_str;
     const StreamId id = stream_of(p, rb, grp);
+    // (behind a launch that itself has waited for the attention, its records are complete: only this launch's end has to wait)
+    ptx::grid_dep_launch();                       // (the kernel behind only sets itself up before this one has completed)
+    if (!p.late_merge) ptx::grid_dep_wait();
     attn::merge_boundary<D>(
         p.begins, p.n_groups, p.n, p.Hq, p.B, p.out, p.lse_out, p.status, p.wait_limit, p.stall_merge,
         [&](int row, const attn::GroupBegin& u, int& node, int& head) {
@@ -1246,13 +1318,25 @@ __global__ void __launch_bounds__(attn::kMergeThreads) attn_merge_kernel(const _
             return id.exists && row < p.gs * p.nodes_tile && hl < p.G && node < p.n;
         },
         [&](int group, int slot) { return p.partial + (((size_t)(group * p.n_cta + rb) * 2 + slot) * 2 + grp) * (D + 4) * kRows; });
+    if (p.late_merge) ptx::grid_dep_wait();
+}
+
+mirror_status merge_launch(mirror_ctx* ctx, const AttnParams& p, cudaStream_t stream) {
+    auto merge = ctx->desc.head_dim == 128 ? attn_merge_kernel<128> : attn_merge_kernel<64>;
+    const dim3 grid((unsigned)(p.n_groups - 1), (unsigned)(p.n_cta * (p.mode == kSplit ? 1 : 2)));
+    MIRROR_CUDA_OK(cudaFuncSetAttribute(merge, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::kMergeSmem));
+    MIRROR_CUDA_OK(mirror_launch_pdl(merge, grid, dim3(attn::kMergeThreads), attn::kMergeSmem, stream, p));
+    ctx->launches += 1;
+    MIRROR_CUDA_OK(cudaGetLastError());
+    return MIRROR_OK;
 }
 
 }  // namespace
 
 mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
-                                 float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8, bool keep_rounding) {
+                                 float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8, bool keep_rounding,
+                                 MirrorAttnBeside* beside) {
     if (keep_rounding && !f8) return mirror_attn_tile64_launch(ctx, kv, tree, ti, q, k_new, v_new, out, lse_out, partial_ws, stream);
     const int D = ctx->desc.head_dim, Hkv = ctx->desc.n_kv_heads, Hq = ctx->desc.n_q_heads;
     AttnParams p;
@@ -1289,6 +1373,32 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     p.cut_tiles = f8 || p.unit_cuts == 1 ? 8 : 2;
     const int most_tiles = (kv->max_pages_per_req + (p.n + kSlotTok - 1) / kSlotTok + kTileSlots - 1) / kTileSlots;      // of a unit
     p.never_cut = whole && most_tiles <= 6;
+    // Beside a weight stream: whole units, where one request's are short (a cut costs about as much as two tiles, a launch behind it not counted).
+    p.lm_ns = 0.f;
+    p.deal = p.never_cut || (whole && p.B == 1 && units >= 2 * p.n_groups && most_tiles <= 64);
+    p.group_chunk = p.n_cta % 2 ? 2 : 1;
+    // One request: all units have the same length whatever it is, so the host can tell when the partition gives every
+    // group whole units (each unit holds at least one tile): nothing is cut and the merge kernel has nothing to do.
+    bool no_cuts = p.n_groups == 1 || p.never_cut || (p.B == 1 && (p.whole_groups > 0 || (p.unit_cuts == 1 && cuts_pay(most_tiles, p.units, p.n_groups, 1, p.cut_tiles))));
+    p.late_merge = 0;
+    if (beside) {
+        // Is the launch behind to run beside this one?  Its merge then comes last (~10 us): yes where there is none, where a shared
+        // chip is the faster one if prefixes are as long as the page table allows (the device, which knows them, decides), and
+        // unless this one takes so much longer that nothing is gained; with many rows, where what it fills in, the time
+        // between the first CTA's end and the last one's, is longer than the merge.
+        const float tiles = (float)most_tiles * (float)p.units, step_bytes = (float)(kTileTok * 2 * D * (f8 ? 1 : 2) * (p.mode == kSplit ? 2 : 1));
+        const int most = std::min(p.n_groups, p.units), sms = ctx->num_sms;
+        p.lm_ns = beside->work_ns;
+        const Share all = share_choice(p, tiles, most, sms, step_bytes, 0);
+        bool share = false;
+        if (beside->stream && beside->work_ns > 2e4f && 3 * most * p.n_cta > sms && p.n_groups > 1)
+            for (int c = 1; c < 32; ++c) share |= share_choice(p, tiles, most, sms, step_bytes, c).total < kShareGain * all.total;
+        const float attn_ns = all.total - p.lm_ns;
+        beside->granted = no_cuts || share || (beside->stream ? attn_ns < 8.f * beside->work_ns : attn_ns > 3e5f && beside->work_ns > 0.25f * attn_ns);
+        if (!share) p.lm_ns = 0.f;
+        else no_cuts = no_cuts && p.deal;
+        p.late_merge = beside->granted;
+    }
     p.wait_limit = ctx->tune.wait_limit_cycles;
     p.stall_after = (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_attn_left-- > 0) ? ctx->tune.test_stall_after : -1;
     p.stall_merge = ctx->tune.test_stall_merges > 0 && ctx->tune.test_stall_merges-- > 0;
@@ -1337,7 +1447,7 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         if (st != MIRROR_OK) return st;
         }
     }
-    auto launch = [&](auto cfg, auto kern, auto merge) -> mirror_status {
+    auto launch = [&](auto cfg, auto kern) -> mirror_status {
         using C = decltype(cfg);
         const size_t fixed = (f8 && p.mode != kSplit ? 4 : 2) * (size_t)C::kQBytes + C::kFixedBytes + (p.mode == kSplit ? kRows * 16 : 0) + (2 * (size_t)p.B + 1) * 4;
         int stages = (int)((kSmemLimit - fixed) / C::kStageBytes);
@@ -1346,23 +1456,40 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         if (stages < 4) return MIRROR_ERR_UNSUPPORTED;
         const size_t smem = fixed + (size_t)stages * C::kStageBytes;
         MIRROR_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
-        MIRROR_CUDA_OK(mirror_launch_pdl(kern, dim3(p.n_groups * p.n_cta), dim3(C::kThreads), smem, stream, tm, at, p, stages));
+        cudaLaunchConfig_t cfg_l = {};
+        cfg_l.gridDim = dim3((unsigned)(p.lm_ns > 0.f ? align_up((size_t)p.n_groups * p.n_cta, 2) : (size_t)p.n_groups * p.n_cta));
+        cfg_l.blockDim = dim3(C::kThreads);
+        cfg_l.dynamicSmemBytes = smem;
+        cfg_l.stream = stream;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;       // (neighbouring blocks on the SMs of a TPC: see spread_group)
+        attr[1].val.clusterDim.x = 2;
+        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+        cfg_l.attrs = attr;
+        cfg_l.numAttrs = p.lm_ns > 0.f ? 2 : 1;
+        MIRROR_CUDA_OK(cudaLaunchKernelEx(&cfg_l, kern, tm, at, p, stages));
         ctx->launches += 1;
         MIRROR_CUDA_OK(cudaGetLastError());
-        // One request: all units have the same length whatever it is, so the host can tell when the partition gives every
-        // group whole units (each unit holds at least one tile): nothing is cut and the merge kernel has nothing to do.
-        const bool no_cuts = p.never_cut || (p.B == 1 && (p.whole_groups > 0 || (p.unit_cuts == 1 && cuts_pay(most_tiles, p.units, p.n_groups, 1, p.cut_tiles))));
-        if (p.n_groups > 1 && !no_cuts) {
-            // which units the partition cut is only known on the device (it depends on the prefix lengths)
-            const dim3 mgrid((unsigned)(p.n_groups - 1), (unsigned)(p.n_cta * (p.mode == kSplit ? 1 : 2)));
-            MIRROR_CUDA_OK(cudaFuncSetAttribute(merge, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::kMergeSmem));
-            MIRROR_CUDA_OK(mirror_launch_pdl(merge, mgrid, dim3(attn::kMergeThreads), attn::kMergeSmem, stream, p));
-            ctx->launches += 1;
-            MIRROR_CUDA_OK(cudaGetLastError());
+        if (no_cuts) return MIRROR_OK;
+        if (p.late_merge) {
+            static_assert(sizeof(AttnParams) <= sizeof beside->merge, "room for the launch's parameters");
+            beside->merge_needed = true;
+            memcpy(beside->merge, &p, sizeof p);
+            return MIRROR_OK;
         }
-        return MIRROR_OK;
+        // which units the partition cut is only known on the device (it depends on the prefix lengths)
+        return merge_launch(ctx, p, stream);
     };
-    return f8         ? launch(Cfg<128, true>{}, attn_verify_kernel<128, true>, attn_merge_kernel<128>)
-           : D == 128 ? launch(Cfg<128, false>{}, attn_verify_kernel<128, false>, attn_merge_kernel<128>)
-                      : launch(Cfg<64, false>{}, attn_verify_kernel<64, false>, attn_merge_kernel<64>);
+    return f8         ? launch(Cfg<128, true>{}, attn_verify_kernel<128, true>)
+           : D == 128 ? launch(Cfg<128, false>{}, attn_verify_kernel<128, false>)
+                      : launch(Cfg<64, false>{}, attn_verify_kernel<64, false>);
+}
+
+mirror_status mirror_attn_late_merge(mirror_ctx* ctx, const MirrorAttnBeside& beside, cudaStream_t stream) {
+    if (!beside.merge_needed) return MIRROR_OK;
+    AttnParams p;
+    memcpy(&p, beside.merge, sizeof p);
+    return merge_launch(ctx, p, stream);
 }

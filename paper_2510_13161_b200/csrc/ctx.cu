@@ -59,6 +59,7 @@ extern "C" mirror_status mirror_create(mirror_ctx** out, const mirror_model_desc
         delete ctx;
         return MIRROR_ERR_CUDA;
     }
+    ctx->d_unit_ctr = (uint32_t*)ctx->d_status + 16;
     ctx->d_topk_bar = (uint32_t*)((uint8_t*)ctx->d_status + kBarAt);
     *out = ctx;
     return MIRROR_OK;

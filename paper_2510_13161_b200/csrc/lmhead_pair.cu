@@ -35,6 +35,7 @@ constexpr int kMaxStages = 8;
 constexpr int kAcc = 2;
 constexpr int kMaxChunkRows = 256;
 constexpr int kSmemBudget = 232448;
+constexpr int kUnitRing = 16;               // units named ahead (kFree); the producer is at most stages + 3 units ahead of the epilogue
 constexpr int kCtrlBytes = 1024 + 4 * kMaxChunkRows * 12;
 constexpr int kTopkBytes = 5 * kMaxChunkRows * 4;      // Top-kappa: each epilogue warp's row maxima of one unit, and the rows' bars
 
@@ -64,6 +65,9 @@ struct PairParams {
     long long wait_limit;                   // SM cycles after which a wait gives up
     int stall_after;                        // test aid: the producers stop after this many stages (-1: never)
     int w_early;                            // 1: W is older than the kernel ahead: the first stages' weights are requested before the wait
+    int running;                            // 1: a CTA keeps its rows' state over its units and leaves one partial; 0: a partial per unit
+    uint32_t* unit_ctr;                     // kFree: {next unit, pairs that are through}; both zero between launches
+    int n_own;                              // kFree: the first units, one per pair, that are not handed out by the counter (0 or the pairs)
 };
 
 struct Ctrl {
@@ -71,6 +75,8 @@ struct Ctrl {
     uint64_t empty[kMaxStages];             // UMMAs that read the stage have completed (multicast commit)
     uint64_t acc_full[kAcc];                // accumulator complete (multicast commit)
     uint64_t acc_empty[kAcc];               // leader only: 4 + 4 epilogue warps have drained the accumulator
+    uint64_t unit_full[kUnitRing];          // kFree: the leader has named this CTA's unit
+    int unit[kUnitRing];
     int* status;
     long long wait_limit;
     uint32_t tmem_base;
@@ -100,6 +106,10 @@ __device__ __forceinline__ uint32_t map_to_rank(const void* smem_ptr, uint32_t r
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// a word into the shared memory of a CTA of the pair, counted on a barrier there
+__device__ __forceinline__ void st_async(uint32_t cluster_addr, int v, uint32_t bar_cluster_addr) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(cluster_addr), "r"(v), "r"(bar_cluster_addr) : "memory");
 }
 // Bounded waits by all lanes of a converged warp, which all get the same answer: one poll inline; parking, the abort flag and the
 // limit are out of line.  kCluster: the other CTA of the pair arrives on the barrier.
@@ -262,7 +272,11 @@ __device__ __noinline__ void topk_list_merge(float* lv, int* li, int K, float x,
 // kFp8 / kTopk: e4m3 operands with per-row scales / Top-kappa lists in the epilogue, as separate instantiations so that
 // the plain bf16 head carries none of their registers and branches.
 // kEarly: a kernel of its own, since the few instructions that it adds in front of the wait cost the others 0.3-6% (code placement).
-template <bool kReduce, bool kFp8, bool kTopk, bool kEarly>
+// kFree: nothing that this launch reads is written by the kernel ahead (an attention launch, which has waited for all before it), so
+// its CTAs begin as SMs come free, and only their end waits.  They begin at very different times, so the pairs take units from
+// a counter: the leader's producer names them to both CTAs.  Results do not depend on who takes what: argmax does not, and
+// where sums are asked for every unit leaves partials of its own.
+template <bool kReduce, bool kFp8, bool kTopk, bool kEarly, bool kFree>
 __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CUtensorMap& tm_h, const PairParams& p) {
     extern __shared__ uint8_t smem_raw[];
     // (the dynamic shared window starts at the same offset in both CTAs, so the aligned layout is the same too)
@@ -291,6 +305,8 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
             ptx::mbar_init(&ctrl->empty[s], 1);
         }
         for (int a = 0; a < kAcc; ++a) { ptx::mbar_init(&ctrl->acc_full[a], 1); ptx::mbar_init(&ctrl->acc_empty[a], 8); }
+        if (kFree)
+            for (int i = 0; i < kUnitRing; ++i) ptx::mbar_init(&ctrl->unit_full[i], 1);
         ctrl->abort = 0;
         ctrl->status = p.status;
         ctrl->wait_limit = p.wait_limit;
@@ -320,8 +336,14 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
             tma_load_2d_pair(stage_base + s * p.stage_bytes, &tm_w, map_to_rank(&ctrl->full[s], 0), (kb0 + s) * kBK, (tile * 2 + (int)rank) * p.rows_cta, pol_w);
         }
     }
-    ptx::grid_dep_wait();
+    if (!kFree) ptx::grid_dep_wait();
     ptx::grid_dep_launch();
+    // kFree: unit number j of this pair, or (no more, or a failure) one past the last; whole warps
+    auto named_unit = [&](uint32_t j) -> int {
+        const uint32_t e = j % kUnitRing;
+        if (!wait_warp<true>(ctrl, &ctrl->unit_full[e], (j / kUnitRing) & 1, 17)) return p.n_units;
+        return *(volatile int*)&ctrl->unit[e];
+    };
 
     // Producer and issuer: the whole warp walks the schedule and one elected lane issues, which keeps addresses and descriptors in
     // uniform registers; the next K block's barrier is polled ahead of the instructions that hold the lane up.  What the issuer spends
@@ -348,7 +370,23 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
             if (++s == p.stages) { s = 0; ph ^= 1; }
         }
         int kb_skip = n_issued;
-        for (int u = pair; u < p.n_units && ok; u += n_pairs) {
+        auto name_unit = [&](uint32_t j) {                         // (the leader's)
+            if (ptx::elect_one()) {
+                int u = p.n_units;                                 // (as many pairs as units: no need to ask)
+                if (j == 0 && p.n_own > 0) u = pair;
+                else if (p.n_own < p.n_units) u = (int)min(p.n_own + atomicAdd(p.unit_ctr, 1u), (uint32_t)p.n_units);
+                for (uint32_t r = 0; r < 2; ++r) st_async(map_to_rank(&ctrl->unit[j % kUnitRing], r), u, map_to_rank(&ctrl->unit_full[j % kUnitRing], r));
+            }
+            __syncwarp();
+        };
+        auto take_unit = [&](uint32_t j) {
+            if (ptx::elect_one()) ptx::mbar_arrive_expect_tx(&ctrl->unit_full[j % kUnitRing], 4);
+            __syncwarp();
+            return named_unit(j);
+        };
+        uint32_t j = 0;
+        if (kFree && rank == 0) name_unit(0);
+        for (int u = kFree ? take_unit(0) : pair; u < p.n_units && ok; u = kFree ? take_unit(++j) : u + n_pairs) {
             int tile, slice, chunk;
             decode(u, tile, slice, chunk);
             const int w_row = (tile * 2 + (int)rank) * p.rows_cta;
@@ -356,6 +394,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
             const int kb_end = min(n_kb, (slice + 1) * p.kb_per_slice);
             int kb = slice * p.kb_per_slice + kb_skip;
             kb_skip = 0;
+            const int kb_name = min(kb + p.stages, kb_end) - 1;    // (the counter's answer takes ~1 us: asked for with all stages in flight)
 #pragma unroll 1
             for (; kb < kb_end; ++kb) {
                 if (p.stall_after >= 0 && n_issued >= p.stall_after) { ok = false; break; }       // (test aid: neither arms nor copies)
@@ -369,6 +408,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                 __syncwarp();
                 ++n_issued;
                 if (++s == p.stages) { s = 0; ph ^= 1; }
+                if (kFree && rank == 0 && kb == kb_name) name_unit(j + 1);
             }
         }
         // (copies still in flight after a failure: the leader's issuer or its 2 s limit outlasts them, and both CTAs
@@ -382,7 +422,8 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
             int s = 0, ab = 0;
             uint32_t ph = 0, aph = 0, lo = lo0;
             bool ok = true;
-            for (int u = pair; u < p.n_units && ok; u += n_pairs) {
+            uint32_t j = 0;
+            for (int u = kFree ? named_unit(0) : pair; u < p.n_units && ok; u = kFree ? named_unit(++j) : u + n_pairs) {
                 if (!wait_warp<true>(ctrl, &ctrl->acc_empty[ab], aph ^ 1, 12)) { ok = false; break; }
                 const uint32_t d_tmem = tmem_base + (uint32_t)(ab * p.acc_stride);
                 int tile, slice, chunk;
@@ -452,7 +493,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
         bool ok = true;
         // One row chunk: a CTA meets the same hidden rows in every unit and keeps a running state per row, flushed once
         // (one partial per CTA).  Several chunks: every unit flushes its own partial (one per 128-row vocabulary tile).
-        const bool running = p.n_chunks == 1;
+        const bool running = kFree ? p.running != 0 : p.n_chunks == 1;
         if (kReduce && running) {
             for (int c = lane; c < kMaxChunkRows; c += 32) { my_max[c] = -INFINITY; my_idx[c] = 0x7fffffff; my_sum[c] = 0.f; }
             __syncwarp();
@@ -461,7 +502,17 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
             for (int i = lane; i < p.M * p.topk; i += 32) { __stcg(my_tv + i, -INFINITY); __stcg(my_ti + i, 0x7fffffff); }      // empty
             __syncwarp();
         }
-        for (int u = pair; u < p.n_units; u += n_pairs) {
+        uint32_t j = 0;
+        // (a partial per unit: the four warps meet at barriers, so all of them go on or none)
+        auto next_unit = [&](uint32_t i) -> int {
+            const int u = ctrl->abort ? p.n_units : named_unit(i);
+            if (running) return u;
+            uint32_t go;
+            asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                         : "=r"(go) : "r"((uint32_t)(u < p.n_units)) : "memory");
+            return go ? u : p.n_units;
+        };
+        for (int u = kFree ? next_unit(0) : pair; u < p.n_units; u = kFree ? next_unit(++j) : u + n_pairs) {
             int tile, slice, chunk;
             decode(u, tile, slice, chunk);
             const int rbase = chunk * p.chunk_rows;
@@ -623,27 +674,38 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
         ptx::tc_fence_after();
         tmem_dealloc_pair(tmem_base, (uint32_t)p.tmem_cols);
     }
+    if (kFree) {
+        if (p.n_own < p.n_units && rank == 0 && tid == 0) {        // the last pair leaves the counter as it found it
+            __threadfence();
+            if (atomicAdd(p.unit_ctr + 1, 1u) + 1 == (uint32_t)n_pairs) p.unit_ctr[0] = p.unit_ctr[1] = 0;
+        }
+        ptx::grid_dep_wait();               // (whatever waits for this launch waits for the one ahead, too)
+    }
 }
 
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, false, false, false>(tm_w, tm_h, p);
+    pair_gemm_body<true, false, false, false, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_early_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, false, false, true>(tm_w, tm_h, p);
+    pair_gemm_body<true, false, false, true, false>(tm_w, tm_h, p);
+}
+__global__ void __launch_bounds__(kThreads, 2)
+lmhead_pair_free_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
+    pair_gemm_body<true, false, false, false, true>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_topk_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, false, true, false>(tm_w, tm_h, p);
+    pair_gemm_body<true, false, true, false, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_fp8_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, true, false, false>(tm_w, tm_h, p);
+    pair_gemm_body<true, true, false, false, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 linear_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<false, false, false, true>(tm_w, tm_h, p);
+    pair_gemm_body<false, false, false, true, false>(tm_w, tm_h, p);
 }
 
 int next_pow2(int x) {
@@ -682,6 +744,9 @@ mirror_status pair_shape(const MirrorTuning& tune, int M, int V, int H, PairPara
     p->wait_limit = tune.wait_limit_cycles;
     p->stall_after = -1;
     p->w_early = 0;
+    p->running = p->n_chunks == 1;
+    p->unit_ctr = nullptr;
+    p->n_own = 0;
     if (p->stages < 2) return MIRROR_ERR_SHAPE;
     p->k_slices = 1;
     p->kb_per_slice = H / kBK;
@@ -709,6 +774,7 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
     if (!ctx->lm_pair_attr_set) {
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_early_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+        MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_free_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_fp8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(linear_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
@@ -729,7 +795,7 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     if (p.fp8 && (p.topk > 0 || !reduce)) return MIRROR_ERR_UNSUPPORTED;
-    auto kern = !reduce ? linear_pair_kernel : p.fp8 ? lmhead_pair_fp8_kernel : p.topk > 0 ? lmhead_pair_topk_kernel : p.w_early ? lmhead_pair_early_kernel : lmhead_pair_kernel;
+    auto kern = !reduce ? linear_pair_kernel : p.fp8 ? lmhead_pair_fp8_kernel : p.topk > 0 ? lmhead_pair_topk_kernel : p.unit_ctr ? lmhead_pair_free_kernel : p.w_early ? lmhead_pair_early_kernel : lmhead_pair_kernel;
     MIRROR_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, tm_w, tm_h, p));
     ctx->launches += 1;
     MIRROR_CUDA_OK(cudaGetLastError());
@@ -757,7 +823,7 @@ bool mirror_lmhead_topk_spills(const mirror_ctx* ctx, int M, int topk) {
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,
                                         void* partial_ws, size_t partial_bytes, cudaStream_t stream, int* n_partials,
                                         const float* w_scale, const float* h_scale, int topk, void* topk_ws, size_t topk_ws_bytes,
-                                        bool w_early) {
+                                        MirrorLmStart start, bool sums) {
     const bool fp8 = w_scale != nullptr;
     if (fp8 && (!h_scale || ctx->desc.hidden % 128 != 0)) return MIRROR_ERR_SHAPE;
     // (e4m3 rows are staged exactly like bf16 rows of half as many elements: the same bytes, boxes and swizzle)
@@ -766,14 +832,18 @@ mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int
     // the units come out in whole waves over the pairs (152064 rows over 148 pairs: five units of 2 x 104 rows each
     // instead of four or five of 2 x 128).
     int rows_cta = kTileV;
-    if (ctas_per_sm_for(ctx->tune, M) == 2) {
+    const bool free_start = start == MIRROR_LM_AT_ONCE && !fp8 && topk == 0 && ctx->d_unit_ctr;
+    const bool stream_mode = ctas_per_sm_for(ctx->tune, M) == 2;
+    if (stream_mode) {
+        // (a partial per unit: as many units as the workspace has room for)
+        const size_t most = free_start && sums ? partial_bytes / ((size_t)M * 24) : SIZE_MAX;
         const int pairs = ctx->num_sms;
         long long best = -1;
         for (int r = kTileV; r >= 64; r -= 8) {
             const long long units = (V + 2 * r - 1) / (2 * r), waves = (units + pairs - 1) / pairs;
-            if (best < 0 || waves * r < best) { best = waves * r; rows_cta = r; }
+            if ((best < 0 || waves * r < best) && (size_t)units <= most) { best = waves * r; rows_cta = r; }
         }
-        if (ctx->tune.lm_rows >= 8 && ctx->tune.lm_rows <= kTileV && ctx->tune.lm_rows % 8 == 0) rows_cta = ctx->tune.lm_rows;
+        if (most == SIZE_MAX && ctx->tune.lm_rows >= 8 && ctx->tune.lm_rows <= kTileV && ctx->tune.lm_rows % 8 == 0) rows_cta = ctx->tune.lm_rows;
     }
     const int n_tiles = (V + 2 * rows_cta - 1) / (2 * rows_cta);
     PairParams p;
@@ -784,10 +854,18 @@ mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int
     if (n_pairs > p.n_units) n_pairs = p.n_units;
     if (n_pairs < 1) return MIRROR_ERR_UNSUPPORTED;
     // partials: one per CTA (single row chunk: running state) or one per 128-row vocabulary tile
-    const size_t P = p.n_chunks == 1 ? (size_t)2 * n_pairs : (size_t)2 * n_tiles;
+    if (free_start) {
+        p.running = p.n_chunks == 1 && !sums;
+        p.unit_ctr = ctx->d_unit_ctr;
+        // Few units to a pair: one each, in the order in which the pairs begin, and only the rest as they come.  (A unit takes as long as
+        // its chain of K blocks, however few pairs are at work: a pair that began early and took a second one would end last.
+        // 24 layers x 2 x 4807..18176 tokens before 18841 ids of 7424: 170 us in one wave, 190 by the counter.)
+        p.n_own = p.n_units <= 2 * n_pairs ? n_pairs : 0;
+    }
+    const size_t P = p.running ? (size_t)2 * n_pairs : (size_t)2 * n_tiles;
     if (partial_bytes < P * M * 12) return MIRROR_ERR_WORKSPACE;
     p.w_keep = p.n_chunks > 1;
-    p.w_early = w_early && ctas_per_sm_for(ctx->tune, M) == 2;       // (a weight stream; with more rows the tensor cores set the pace)
+    p.w_early = start == MIRROR_LM_WEIGHTS_EARLY && stream_mode;       // (a weight stream; with more rows the tensor cores set the pace)
     if (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_lm_left-- > 0) p.stall_after = ctx->tune.test_stall_after;
     p.inv_T = 1.0f / ctx->temperature;
     p.inv_T_log2e = p.inv_T * 1.4426950408889634f;

@@ -334,8 +334,20 @@ __device__ __forceinline__ RowPartial fold_row(int row, int M, int P, float inv_
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     RowPartial r = {-INFINITY, 0.f, 0x7fffffff};
     if (tid < 256) {
-        for (int k = tid; k < P; k += 256)
-            r.fold(part_max[(size_t)k * M + row], part_idx[(size_t)k * M + row], part_sum[(size_t)k * M + row], inv_T_log2e);
+        // (four partials' loads in flight: 764 partials of 77 rows took 17 us one after the other)
+        for (int k0 = tid; k0 < P; k0 += 4 * 256) {
+            float m[4], s[4];
+            int i[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const size_t at = (size_t)min(k0 + j * 256, P - 1) * M + row;
+                m[j] = k0 + j * 256 < P ? part_max[at] : -INFINITY;
+                i[j] = part_idx[at];
+                s[j] = part_sum[at];
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) r.fold(m[j], i[j], s[j], inv_T_log2e);
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const float om = __shfl_xor_sync(0xffffffffu, r.m, o), os = __shfl_xor_sync(0xffffffffu, r.s, o);
@@ -623,7 +635,7 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
                                    float* topk_logprob, float* gather_logit, float* logits_out,
                                    void* partial_ws, size_t partial_bytes, float* lse_scratch, cudaStream_t stream,
                                    cudaEvent_t after_gemm, void* topk_logprob_bf16, void* topk_ws, size_t topk_ws_bytes, MirrorLmPartials* defer,
-                                   bool w_early) {
+                                   MirrorLmStart start) {
     const int V = ctx->desc.vocab, H = ctx->desc.hidden;
     // Top-kappa inside the GEMM's epilogue whenever the caller's scratch holds the candidate lists; otherwise (or on the
     // single-CTA fallback kernel) the selection runs over spilled logits, which then have to be there.
@@ -635,7 +647,7 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
     if (M >= pair_min_rows && ctx->num_sms >= 2) {
         int P = 0;
         mirror_status st = mirror_lmhead_pair_launch(ctx, hidden, M, W, logits_out, partial_ws, partial_bytes, stream, &P, nullptr,
-                                                     nullptr, fused_topk ? topk : 0, topk_ws, topk_ws_bytes, w_early);
+                                                     nullptr, fused_topk ? topk : 0, topk_ws, topk_ws_bytes, start, lse || topk > 0);
         if (st == MIRROR_OK) {
             if (after_gemm) MIRROR_CUDA_OK(cudaEventRecord(after_gemm, stream));
             const float inv_T = 1.0f / ctx->temperature, inv_T_log2e = inv_T * 1.4426950408889634f;

@@ -52,6 +52,7 @@ struct mirror_ctx {
     float scale = 0.f;
     float temperature = 1.f;
     int* d_status = nullptr;        // [2]: {code, detail}
+    uint32_t* d_unit_ctr = nullptr; // [2] in the status' sector: the LM head's unit counter, zero between launches (lmhead_pair.cu)
     uint32_t* d_topk_bar = nullptr; // [MIRROR_MAX_TOPK][256 rows] sectors behind the status: zero between calls (lmhead_pair.cu)
     void* ws = nullptr;
     size_t ws_bytes = 0;
@@ -94,8 +95,13 @@ struct MirrorLmPartials {
 mirror_status mirror_accept_launch(mirror_ctx* ctx, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                    const mirror_accept_in* in, const mirror_accept_out* out, cudaStream_t stream,
                                    double* tree_scratch = nullptr, const MirrorLmPartials* partials = nullptr, int32_t* argmax_out = nullptr);
-// defer: the row partials are not merged, but described there (only the argmax was asked for).  w_early: no kernel that may
-// still be running when the one ahead of this launch begins writes W.
+// When an LM-head launch may begin.
+enum MirrorLmStart {
+    MIRROR_LM_AFTER,              // once the kernel ahead has completed
+    MIRROR_LM_WEIGHTS_EARLY,      // no kernel that may still be running when the one ahead begins writes W: its first tiles are requested early
+    MIRROR_LM_AT_ONCE             // nor does any, the one ahead included, write W or the hidden rows: as SMs come free, beside the one ahead
+};
+// defer: the row partials are not merged, but described there (only the argmax was asked for).
 mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, int topk,
                                    const int32_t* gather_row, const int32_t* gather_tok, int n_gather,
                                    int32_t* argmax, float* maxlogit, float* lse, int32_t* topk_id,
@@ -103,7 +109,7 @@ mirror_status mirror_lmhead_launch(mirror_ctx* ctx, const void* hidden, int M, c
                                    void* partial_ws, size_t partial_bytes, float* lse_scratch, cudaStream_t stream,
                                    cudaEvent_t after_gemm = nullptr, void* topk_logprob_bf16 = nullptr,
                                    void* topk_ws = nullptr, size_t topk_ws_bytes = 0, MirrorLmPartials* defer = nullptr,
-                                   bool w_early = false);
+                                   MirrorLmStart start = MIRROR_LM_AFTER);
 // LM-head GEMM + per-unit row partials on CTA pairs (many hidden rows); *n_partials partials of [M] rows are left in
 // partial_ws for lmhead_merge_kernel.  mirror_lmhead_pair_partials(V) is that count.
 int mirror_lmhead_pair_partials(int V);
@@ -113,11 +119,12 @@ constexpr int kMirrorTopkMaxLists = 2048;
 bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk);
 // ... and is it better selected from spilled logits, where the workspace has room for them?
 bool mirror_lmhead_topk_spills(const mirror_ctx* ctx, int M, int topk);
-// w_scale / h_scale non-null: W and hidden are e4m3 bytes with one scale per row (the GEMM runs on kind::f8f6f4).
+// sums: the partials' sums will be read (not only the maxima).  w_scale / h_scale non-null: W and hidden are e4m3 bytes with one scale per row (the GEMM runs on kind::f8f6f4).
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,
                                         void* partial_ws, size_t partial_bytes, cudaStream_t stream, int* n_partials,
                                         const float* w_scale = nullptr, const float* h_scale = nullptr,
-                                        int topk = 0, void* topk_ws = nullptr, size_t topk_ws_bytes = 0, bool w_early = false);
+                                        int topk = 0, void* topk_ws = nullptr, size_t topk_ws_bytes = 0,
+                                        MirrorLmStart start = MIRROR_LM_AFTER, bool sums = true);
 // Plain GEMM on CTA pairs: partial[s][M][N] (fp32) = x[M, K-slice s] * W[N, K-slice s]^T for the *k_slices slices that
 // mirror_linear_slices() picks (1 when the output tiles alone fill the GPU); the caller adds the slices in order.  w_early:
 // no kernel that may still be running when the one ahead of this launch begins writes W (see target_layer.cu).
@@ -134,10 +141,22 @@ struct MirrorAttnFp8 {
 // serialization.
 mirror_status mirror_kv_quantize_launch(mirror_ctx* ctx, const void* x, int n_layers, int64_t layer_stride, int64_t layer_elems,
                                        int inner, const float* scale, void* out_fp8, cudaStream_t stream);
+// What could be launched behind an attention launch without waiting for it, and how that is to be done.
+struct MirrorAttnBeside {
+    float work_ns = 0.f;                  // how long it takes on its own
+    bool stream = false;                  // it streams weights, and needs SMs only for that
+    bool granted = false;                 // answer: launch it so
+    // answer: the units that the partition cut are still to be merged, by mirror_attn_late_merge() behind a kernel that lets its
+    // successor start only once a launch that itself has waited for the attention is through
+    bool merge_needed = false;
+    unsigned char merge[512];
+};
 // keep_rounding: every sum keeps the order of the 64-token kernel (mirror_target_forward in deep stacks, see attn_tile64.cu).
 mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
-                                 float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8 = nullptr, bool keep_rounding = false);
+                                 float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8 = nullptr, bool keep_rounding = false,
+                                 MirrorAttnBeside* beside = nullptr);
+mirror_status mirror_attn_late_merge(mirror_ctx* ctx, const MirrorAttnBeside& beside, cudaStream_t stream);
 mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                         const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
                                         float* partial_ws, cudaStream_t stream);

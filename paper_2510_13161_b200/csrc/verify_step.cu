@@ -17,6 +17,11 @@ mirror_status check_kv(const mirror_ctx* ctx, const mirror_kv* kv, const mirror_
     return MIRROR_OK;
 }
 
+// Do two ranges of device memory have no byte in common?
+bool apart(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+    return (uintptr_t)a + a_bytes <= (uintptr_t)b || (uintptr_t)b + b_bytes <= (uintptr_t)a;
+}
+
 }  // namespace
 
 extern "C" mirror_status mirror_attn_verify(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree,
@@ -155,7 +160,19 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     };
     const bool ev = ctx->stage_ev_on && !io;
     if (ev) MIRROR_CUDA_OK(cudaEventRecord(ctx->stage_ev[0], s));
-    if (!io) {
+    // Hidden rows of the caller's own do not depend on the attention: the LM head is launched beside it (see lmhead_pair.cu), on the
+    // SMs that the attention leaves or has done with, and the attention's merge behind the decision.
+    const size_t attn_bytes = (size_t)kv->num_layers * q_layer;
+    const bool at_once = hidden && !io && !ev && (int)M >= ctx->tune.lm_pair_min_rows && apart(hidden, M * (size_t)ctx->desc.hidden * 2, attn_out, attn_bytes) &&
+                         apart(W, (size_t)ctx->desc.vocab * ctx->desc.hidden * 2, attn_out, attn_bytes);
+    MirrorAttnBeside beside;
+    if (at_once) {
+        const double bytes_ns = 2.0 * ctx->desc.vocab * ctx->desc.hidden / 6400.0, flops_ns = bytes_ns * M * 6400.0 / 1.2e6;
+        beside.work_ns = (float)std::max(bytes_ns, flops_ns);
+        beside.stream = M <= 128;                            // (more rows: the tensor cores set the LM head's pace, too)
+        st = mirror_attn_launch(ctx, kv, tree, ti, q, k_new, v_new, attn_out, nullptr, (float*)(ws + L.attn_partial), s, f8, false, &beside);
+        if (st != MIRROR_OK) return st;
+    } else if (!io) {
         st = mirror_attn_launch(ctx, kv, tree, ti, q, k_new, v_new, attn_out, nullptr, (float*)(ws + L.attn_partial), s, f8);
         if (st != MIRROR_OK) return st;
     } else {
@@ -206,7 +223,13 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     const bool defer = !spec && M <= 256;
     st = mirror_lmhead_launch(ctx, rows, (int)M, W, 0, nullptr, nullptr, 0, d_argmax, nullptr, spec ? d_lse : nullptr, nullptr,
                               nullptr, nullptr, d_logits, ws + L.lm_partial, L.lm_partial_bytes, d_lse, s,
-                              ev ? ctx->stage_ev[2] : nullptr, nullptr, nullptr, 0, defer ? &partials : nullptr, !io);
+                              ev ? ctx->stage_ev[2] : nullptr, nullptr, nullptr, 0, defer ? &partials : nullptr,
+                              beside.granted ? MIRROR_LM_AT_ONCE : io ? MIRROR_LM_AFTER : MIRROR_LM_WEIGHTS_EARLY);
+    if (st != MIRROR_OK) return st;
+
+    // The attention's merge, beside the kernel that folds the row partials, or (below) beside the acceptance that folds them itself.
+    // (The draws of the other acceptance kernels leave it no registers: behind them it took 15 us more.)
+    if (!defer) st = mirror_attn_late_merge(ctx, beside, s);
     if (st != MIRROR_OK) return st;
 
     if (io) MIRROR_CUDA_OK(cudaStreamWaitEvent(s, ctx->copy_ev[kEvTokens], 0));
@@ -217,6 +240,8 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     // the tree rule keeps its running distribution in the workspace when the caller sized it for that
     double* tree_scratch = (acc->mode == MIRROR_ACCEPT_SPEC_TREE && ctx->ws_bytes >= L.end_accept) ? (double*)(ws + L.accept_scratch) : nullptr;
     st = mirror_accept_launch(ctx, tree, ti, &in, out, s, tree_scratch, defer ? &partials : nullptr, d_argmax);
+    if (st != MIRROR_OK) return st;
+    if (defer) st = mirror_attn_late_merge(ctx, beside, s);
     if (st != MIRROR_OK) return st;
     if (ev) MIRROR_CUDA_OK(cudaEventRecord(ctx->stage_ev[3], s));
     const mirror_accept_host_out* h = io ? io->h_out : nullptr;
