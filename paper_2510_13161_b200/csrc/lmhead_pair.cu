@@ -77,6 +77,7 @@ struct Ctrl {
     uint64_t acc_empty[kAcc];               // leader only: 4 + 4 epilogue warps have drained the accumulator
     uint64_t unit_full[kUnitRing];          // kFree: the leader has named this CTA's unit
     int unit[kUnitRing];
+    alignas(16) float bcast[4][32];         // per epilogue warp: a value per column, for all lanes
     int* status;
     long long wait_limit;
     uint32_t tmem_base;
@@ -265,6 +266,35 @@ __device__ __noinline__ void topk_list_merge(float* lv, int* li, int K, float x,
     }
     if (lane < K) { __stcg(lv + lane, x); __stcg(li + lane, xi); }
     __syncwarp();
+}
+
+// The reduction of column j over the 32 lanes, for all columns at once, into lane j: at every step a lane gives away the half of its
+// columns that its partner keeps.  The tree is that of a butterfly per column, with a fifth of its shuffles.
+template <class Op>
+__device__ __forceinline__ float reduce_columns(float (&v)[32], Op op) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const float keep = up ? v[k + o] : v[k], give = up ? v[k] : v[k + o];
+            v[k] = op(keep, __shfl_xor_sync(0xffffffffu, give, o));
+        }
+    }
+    return v[0];
+}
+// f(j, lane j's x) for all j
+template <class F>
+__device__ __forceinline__ void for_lanes(float* bcast, float x, F f) {
+    __syncwarp();                                             // (the words' last readers)
+    bcast[threadIdx.x & 31] = x;
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) {
+        const float4 b = *reinterpret_cast<const float4*>(bcast + j);
+        f(j, b.x); f(j + 1, b.y); f(j + 2, b.z); f(j + 3, b.w);
+    }
 }
 
 // kReduce: LM head (row reductions in the epilogue, optional spill).  !kReduce: plain GEMM C = W h^T for the layer
@@ -534,18 +564,16 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                     int upd_i = 0x7fffffff;
                     const int ncol = n_rows - cg * 32;       // columns of this group that are hidden rows (the rest hold zeros)
                     if (any_valid && ncol > 0) {
-                        // The 32 columns go through the reductions side by side (no branch inside, so the shuffle
-                        // chains of different columns overlap); lane j keeps the result of column j.
-                        float v[32], m[32];
+                        // The 32 columns go through the reductions side by side; lane j ends with the result of column j.  (A butterfly per
+                        // column set the pace of short rows: 320 shuffles per warp and 32 columns, now 62 and two passes through shared memory.)
+                        float v[32];
                         if constexpr (kFp8) {
                             // logit = (sum of e4m3 products) * weight-row scale * hidden-row scale; lane j fetches column j's scale
                             const int cr = rbase + cg * 32 + lane;
-                            const float sh = cr < p.M ? p.h_scale[cr] : 0.f;
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) * (sw * __shfl_sync(0xffffffffu, sh, j)));
+                            for_lanes(ctrl->bcast[q], cr < p.M ? p.h_scale[cr] : 0.f, [&](int j, float sh) { r[j] = __float_as_uint(__uint_as_float(r[j]) * (sw * sh)); });
                         }
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) m[j] = v[j] = valid ? __uint_as_float(r[j]) : -INFINITY;
+                        for (int j = 0; j < 32; ++j) v[j] = valid ? __uint_as_float(r[j]) : -INFINITY;
                         if (p.logits_out && valid) {
                             float* dst = p.logits_out + ((size_t)slice * p.M + rbase + cg * 32) * p.V + vid;
 #pragma unroll
@@ -553,25 +581,16 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                                 if (j < ncol) dst[(size_t)j * p.V] = v[j];
                         }
                         if (kReduce) {
+                            float t[32];
 #pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) m[j] = fmaxf(m[j], __shfl_xor_sync(0xffffffffu, m[j], o));
-                        }
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const unsigned eq = __ballot_sync(0xffffffffu, v[j] == m[j]);
-                            if (lane == j) { upd_m = m[j]; upd_i = vid - lane + (__ffs(eq) - 1); }
-                            v[j] = exp2f((v[j] - m[j]) * p.inv_T_log2e);
-                        }
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
-                        }
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (lane == j) upd_s = v[j];
+                            for (int j = 0; j < 32; ++j) t[j] = v[j];
+                            upd_m = reduce_columns(t, [](float a, float b) { return fmaxf(a, b); });
+                            for_lanes(ctrl->bcast[q], upd_m, [&](int j, float m) {
+                                const unsigned eq = __ballot_sync(0xffffffffu, v[j] == m);
+                                if (lane == j) upd_i = vid - lane + (__ffs(eq) - 1);
+                                v[j] = exp2f((v[j] - m) * p.inv_T_log2e);
+                            });
+                            upd_s = reduce_columns(v, [](float a, float b) { return a + b; });
                         }
                     }
                     const int c = cg * 32 + lane;          // lane j holds column cg*32+j of this unit
