@@ -65,6 +65,7 @@ struct PairParams {
     long long wait_limit;                   // SM cycles after which a wait gives up
     int stall_after;                        // test aid: the producers stop after this many stages (-1: never)
     int w_early;                            // 1: W is older than the kernel ahead: the first stages' weights are requested before the wait
+    int sums;                               // 0: the partials' sums are not read
     int running;                            // 1: a CTA keeps its rows' state over its units and leaves one partial; 0: a partial per unit
     uint32_t* unit_ctr;                     // kFree: {next unit, pairs that are through}; both zero between launches
     int n_own;                              // kFree: the first units, one per pair, that are not handed out by the counter (0 or the pairs)
@@ -585,12 +586,18 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
 #pragma unroll
                             for (int j = 0; j < 32; ++j) t[j] = v[j];
                             upd_m = reduce_columns(t, [](float a, float b) { return fmaxf(a, b); });
+                            unsigned at_max = 0;
                             for_lanes(ctrl->bcast[q], upd_m, [&](int j, float m) {
                                 const unsigned eq = __ballot_sync(0xffffffffu, v[j] == m);
-                                if (lane == j) upd_i = vid - lane + (__ffs(eq) - 1);
-                                v[j] = exp2f((v[j] - m) * p.inv_T_log2e);
+                                if (lane == j) at_max = eq;
+                                v[j] -= m;
                             });
-                            upd_s = reduce_columns(v, [](float a, float b) { return a + b; });
+                            upd_i = vid - lane + (__ffs(at_max) - 1);
+                            if (p.sums) {
+#pragma unroll
+                                for (int j = 0; j < 32; ++j) v[j] = exp2f(v[j] * p.inv_T_log2e);
+                                upd_s = reduce_columns(v, [](float a, float b) { return a + b; });
+                            }
                         }
                     }
                     const int c = cg * 32 + lane;          // lane j holds column cg*32+j of this unit
@@ -764,6 +771,7 @@ mirror_status pair_shape(const MirrorTuning& tune, int M, int V, int H, PairPara
     p->stall_after = -1;
     p->w_early = 0;
     p->running = p->n_chunks == 1;
+    p->sums = 1;
     p->unit_ctr = nullptr;
     p->n_own = 0;
     if (p->stages < 2) return MIRROR_ERR_SHAPE;
@@ -873,6 +881,7 @@ mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int
     if (n_pairs > p.n_units) n_pairs = p.n_units;
     if (n_pairs < 1) return MIRROR_ERR_UNSUPPORTED;
     // partials: one per CTA (single row chunk: running state) or one per 128-row vocabulary tile
+    p.sums = sums;
     if (free_start) {
         p.running = p.n_chunks == 1 && !sums;
         p.unit_ctr = ctx->d_unit_ctr;
