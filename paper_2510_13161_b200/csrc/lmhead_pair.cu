@@ -628,20 +628,27 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                 float* const all_max = (float*)((uint8_t*)ctrl + kCtrlBytes);
                 uint32_t* const bars = (uint32_t*)(all_max + 4 * kMaxChunkRows);
                 asm volatile("bar.sync 1, 128;" ::: "memory");
-                for (int c = (warp - 2) * 32 + lane; c < n_rows; c += 128) {
-                    const int share = (int)(blockIdx.x % (uint32_t)K);
-                    uint32_t key = 0, bar = 0xffffffffu;
-                    if (ok)
-                        for (int w = 0; w < 4; ++w) {
-                            const float m = all_max[w * kMaxChunkRows + c];
-                            if (m > -INFINITY) key = max(key, mirror_order_key(m));
-                        }
-#pragma unroll 4
-                    for (int k = 0; k < K; ++k) {
-                        const uint32_t word = __ldcg(p.topk_bar + bar_word(k, c));
-                        if (k == share && key > word) atomicMax(p.topk_bar + bar_word(k, c), key);
-                        bar = min(bar, k == share ? max(word, key) : word);
+                const int share = (int)(blockIdx.x % (uint32_t)K);
+                for (int c = (warp - 2) * 32 + lane; ok && c < n_rows; c += 128) {
+                    uint32_t key = 0;
+                    for (int w = 0; w < 4; ++w) {
+                        const float m = all_max[w * kMaxChunkRows + c];
+                        if (m > -INFINITY) key = max(key, mirror_order_key(m));
                     }
+                    if (key > __ldcg(p.topk_bar + bar_word(share, c))) atomicMax(p.topk_bar + bar_word(share, c), key);
+                }
+                // The first unit's logits would all pass a bar that does not exist yet, and cost their warps a sort per row (1.2 us a row in
+                // all).  The other CTAs are at their first unit too: until each share has a word it is worth waiting, for as long as
+                // those sorts would take at most (no one has to arrive: a share that stays empty lets everything pass).
+                const bool first = u == pair && gridDim.x >= (uint32_t)K;
+                const long long t0 = clock64(), limit = 2000ll * n_rows;
+                for (int c = (warp - 2) * 32 + lane; c < n_rows; c += 128) {
+                    uint32_t bar;
+                    do {
+                        bar = 0xffffffffu;
+#pragma unroll 4
+                        for (int k = 0; k < K; ++k) bar = min(bar, __ldcg(p.topk_bar + bar_word(k, c)));
+                    } while (bar == 0 && first && clock64() - t0 < limit);
                     bars[c] = bar;
                 }
                 asm volatile("bar.sync 1, 128;" ::: "memory");
