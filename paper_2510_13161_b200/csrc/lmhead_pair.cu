@@ -23,6 +23,8 @@
 #include <math.h>
 #include <stdlib.h>
 
+#include <algorithm>
+
 #include "mirror_internal.h"
 
 namespace {
@@ -65,6 +67,7 @@ struct PairParams {
     long long wait_limit;                   // SM cycles after which a wait gives up
     int stall_after;                        // test aid: the producers stop after this many stages (-1: never)
     int w_early;                            // 1: W is older than the kernel ahead: the first stages' weights are requested before the wait
+    __nv_bfloat16* act;                     // kGated: [M, V / 2]
     int sums;                               // 0: the partials' sums are not read
     int running;                            // 1: a CTA keeps its rows' state over its units and leaves one partial; 0: a partial per unit
     uint32_t* unit_ctr;                     // kFree: {next unit, pairs that are through}; both zero between launches
@@ -175,6 +178,13 @@ __device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const void* map
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
         "[%0], [%1, {%3, %4}], [%2], %5;"
         ::"r"(ptx::smem_u32(smem_dst)), "l"(map), "r"(bar_cluster_addr), "r"(x), "r"(y), "l"(policy)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair(void* smem_dst, const void* map, uint32_t bar_cluster_addr, int x, int y, int z, int w, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
+        "[%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
+        ::"r"(ptx::smem_u32(smem_dst)), "l"(map), "r"(bar_cluster_addr), "r"(x), "r"(y), "r"(z), "r"(w), "l"(policy)
         : "memory");
 }
 // D[tmem of both CTAs] (+)= A (128 rows from each CTA's shared memory) * B (N/2 rows from each CTA's shared memory); the low words of
@@ -307,7 +317,10 @@ __device__ __forceinline__ void for_lanes(float* bcast, float x, F f) {
 // its CTAs begin as SMs come free, and only their end waits.  They begin at very different times, so the pairs take units from
 // a counter: the leader's producer names them to both CTAs.  Results do not depend on who takes what: argmax does not, and
 // where sums are asked for every unit leaves partials of its own.
-template <bool kReduce, bool kFp8, bool kTopk, bool kEarly, bool kFree>
+// kGated: plain GEMM of a gate and an up projection (the rows [0, I) and [I, 2I) of W) whose epilogue leaves bf16(silu(gate) * up).  A
+// warp's 32 accumulator lanes are 16 gate rows and the 16 up rows that go with them (a fourth dimension of W's tensor map deals
+// them so), and lanes 16 apart exchange half of their columns.
+template <bool kReduce, bool kFp8, bool kTopk, bool kEarly, bool kFree, bool kGated>
 __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CUtensorMap& tm_h, const PairParams& p) {
     extern __shared__ uint8_t smem_raw[];
     // (the dynamic shared window starts at the same offset in both CTAs, so the aligned layout is the same too)
@@ -328,6 +341,11 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
         const int t2 = u / p.n_chunks;
         slice = t2 % p.k_slices;
         tile = t2 / p.k_slices;
+    };
+
+    auto load_w = [&](uint8_t* dst, uint32_t bar, int kb, int tile, uint64_t policy) {
+        if (kGated) tma_load_4d_pair(dst, &tm_w, bar, kb * kBK, 0, 0, (tile * 2 + (int)rank) * (kTileV / 32), policy);
+        else tma_load_2d_pair(dst, &tm_w, bar, kb * kBK, (tile * 2 + (int)rank) * p.rows_cta, policy);
     };
 
     if (tid == 0) {
@@ -364,7 +382,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
         const uint64_t pol_w = p.w_keep ? ptx::policy_evict_normal() : ptx::policy_evict_first();
         for (int s = 0; s < n_early && lane == 0; ++s) {
             if (rank == 0) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
-            tma_load_2d_pair(stage_base + s * p.stage_bytes, &tm_w, map_to_rank(&ctrl->full[s], 0), (kb0 + s) * kBK, (tile * 2 + (int)rank) * p.rows_cta, pol_w);
+            load_w(stage_base + s * p.stage_bytes, map_to_rank(&ctrl->full[s], 0), kb0 + s, tile, pol_w);
         }
     }
     if (!kFree) ptx::grid_dep_wait();
@@ -420,7 +438,6 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
         for (int u = kFree ? take_unit(0) : pair; u < p.n_units && ok; u = kFree ? take_unit(++j) : u + n_pairs) {
             int tile, slice, chunk;
             decode(u, tile, slice, chunk);
-            const int w_row = (tile * 2 + (int)rank) * p.rows_cta;
             const int h_row = chunk * p.chunk_rows + (int)rank * p.half_rows;
             const int kb_end = min(n_kb, (slice + 1) * p.kb_per_slice);
             int kb = slice * p.kb_per_slice + kb_skip;
@@ -433,7 +450,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                 if (ptx::elect_one()) {
                     if (rank == 0) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
                     uint8_t* dst = stage_base + s * p.stage_bytes;
-                    tma_load_2d_pair(dst, &tm_w, full0 + s * 8, kb * kBK, w_row, pol_w);
+                    load_w(dst, full0 + s * 8, kb, tile, pol_w);
                     tma_load_2d_pair(dst + p.a_bytes, &tm_h, full0 + s * 8, kb * kBK, h_row, pol_h);
                 }
                 __syncwarp();
@@ -564,7 +581,16 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                     float upd_m = -INFINITY, upd_s = 0.f;
                     int upd_i = 0x7fffffff;
                     const int ncol = n_rows - cg * 32;       // columns of this group that are hidden rows (the rest hold zeros)
-                    if (any_valid && ncol > 0) {
+                    if constexpr (kGated) {
+                        const bool lo = lane < 16;
+                        const int I = p.V >> 1, col = (vt * 4 + q) * 16 + (lane & 15), c0 = cg * 32 + (lo ? 0 : 16);
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            const float mine = __uint_as_float(lo ? r[k] : r[k + 16]), other = __shfl_xor_sync(0xffffffffu, __uint_as_float(lo ? r[k + 16] : r[k]), 16);
+                            const float gate = 0.f + (lo ? mine : other), up = 0.f + (lo ? other : mine);       // (the sum of one slice)
+                            if (c0 + k < n_rows && col < I) p.act[(size_t)(rbase + c0 + k) * I + col] = __float2bfloat16_rn(gate / (1.0f + expf(-gate)) * up);
+                        }
+                    } else if (any_valid && ncol > 0) {
                         // The 32 columns go through the reductions side by side; lane j ends with the result of column j.  (A butterfly per
                         // column set the pace of short rows: 320 shuffles per warp and 32 columns, now 62 and two passes through shared memory.)
                         float v[32];
@@ -718,27 +744,32 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
 
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, false, false, false, false>(tm_w, tm_h, p);
+    pair_gemm_body<true, false, false, false, false, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_early_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, false, false, true, false>(tm_w, tm_h, p);
+    pair_gemm_body<true, false, false, true, false, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_free_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, false, false, false, true>(tm_w, tm_h, p);
+    pair_gemm_body<true, false, false, false, true, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_topk_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, false, true, false, false>(tm_w, tm_h, p);
+    pair_gemm_body<true, false, true, false, false, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_pair_fp8_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<true, true, false, false, false>(tm_w, tm_h, p);
+    pair_gemm_body<true, true, false, false, false, false>(tm_w, tm_h, p);
 }
 __global__ void __launch_bounds__(kThreads, 2)
 linear_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
-    pair_gemm_body<false, false, false, true, false>(tm_w, tm_h, p);
+    pair_gemm_body<false, false, false, true, false, false>(tm_w, tm_h, p);
+}
+
+__global__ void __launch_bounds__(kThreads, 2)
+linear_gated_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_h, const PairParams p) {
+    pair_gemm_body<false, false, false, true, false, true>(tm_w, tm_h, p);
 }
 
 int next_pow2(int x) {
@@ -781,6 +812,7 @@ mirror_status pair_shape(const MirrorTuning& tune, int M, int V, int H, PairPara
     p->sums = 1;
     p->unit_ctr = nullptr;
     p->n_own = 0;
+    p->act = nullptr;
     if (p->stages < 2) return MIRROR_ERR_SHAPE;
     p->k_slices = 1;
     p->kb_per_slice = H / kBK;
@@ -797,7 +829,11 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
         const uint64_t dims[2] = {(uint64_t)p.H, (uint64_t)p.V};
         const uint64_t strides[1] = {(uint64_t)p.H * 2};
         const uint32_t box_w[2] = {kBK, (uint32_t)p.rows_cta};
-        mirror_status st = mirror_make_tmap(ctx, &tm_w, W, 2, dims, strides, box_w);
+        // gate and up rows: (H columns, 16 rows, gate or up, groups of 16 rows)
+        const uint64_t half = (uint64_t)p.V / 2, gdims[4] = {(uint64_t)p.H, 16, 2, half / 16};
+        const uint64_t gstrides[3] = {(uint64_t)p.H * 2, half * p.H * 2, 16 * (uint64_t)p.H * 2};
+        const uint32_t gbox[4] = {kBK, 16, 2, kTileV / 32};
+        mirror_status st = p.act ? mirror_make_tmap(ctx, &tm_w, W, 4, gdims, gstrides, gbox) : mirror_make_tmap(ctx, &tm_w, W, 2, dims, strides, box_w);
         if (st != MIRROR_OK) return st;
         const uint64_t hdims[2] = {(uint64_t)p.H, (uint64_t)p.M};
         const uint32_t box_h[2] = {kBK, (uint32_t)p.half_rows};
@@ -811,6 +847,7 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_free_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(lmhead_pair_fp8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+        MIRROR_CUDA_OK(cudaFuncSetAttribute(linear_gated_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         MIRROR_CUDA_OK(cudaFuncSetAttribute(linear_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
         ctx->lm_pair_attr_set = true;
     }
@@ -829,7 +866,7 @@ mirror_status pair_launch(mirror_ctx* ctx, bool reduce, const void* x, const voi
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     if (p.fp8 && (p.topk > 0 || !reduce)) return MIRROR_ERR_UNSUPPORTED;
-    auto kern = !reduce ? linear_pair_kernel : p.fp8 ? lmhead_pair_fp8_kernel : p.topk > 0 ? lmhead_pair_topk_kernel : p.unit_ctr ? lmhead_pair_free_kernel : p.w_early ? lmhead_pair_early_kernel : lmhead_pair_kernel;
+    auto kern = !reduce ? (p.act ? linear_gated_kernel : linear_pair_kernel) : p.fp8 ? lmhead_pair_fp8_kernel : p.topk > 0 ? lmhead_pair_topk_kernel : p.unit_ctr ? lmhead_pair_free_kernel : p.w_early ? lmhead_pair_early_kernel : lmhead_pair_kernel;
     MIRROR_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, tm_w, tm_h, p));
     ctx->launches += 1;
     MIRROR_CUDA_OK(cudaGetLastError());
@@ -844,14 +881,14 @@ bool mirror_lmhead_topk_fusable(const mirror_ctx* ctx, int M, int topk) {
     return topk > 0 && M <= kMaxChunkRows && M >= ctx->tune.lm_pair_min_rows && 8 * ctx->num_sms <= kMirrorTopkMaxLists;      // (4 per CTA, 2 CTAs per SM)
 }
 
-// In a CTA's first unit there is no bar yet, and every row costs its epilogue warps a sort (1.2 us a row in all), however small
-// the vocabulary; a selection from spilled logits costs kappa passes over a row's V logits, 148 rows at a time.  (us, fused /
-// spilled: 256 rows x 1024 ids, kappa 16: 354 / 48; 128 x 8192, 8: 167 / 47; 256 x 32000, 32: 403 / 371; 57 x 16000, 8: 88 / 45,
-// 57 x 50000, 8: 111 / 109; 17 x 16000, 8: 39 / 39; 57 x 152064, 8: 166 / 404.)  Large vocabularies stay fused: their logits are
-// tens of MB.
+// Of a small vocabulary hardly more is met than the bar needs to become good, so many candidates go into the lists, and these
+// cost a row what its kappa and the CTAs are; a selection from spilled logits costs kappa passes over a row's V logits, 148
+// rows at a time.  The line, between the two over H of 1024 and 5120, V of 1024..60000, kappa of 1..32 and up to 256 rows
+// (us at H = 1024, selected in the epilogue / spilled): 256 rows x 1024 ids, kappa 32: 436 / 70; 100 x 4096, 8: 48 / 33; 180 x 8192, 8:
+// 47 / 48; 256 x 8192, 8: 61 / 54; 100 x 16000, 8: 50 / 54; 256 x 16000, 8: 57 / 78; 256 x 30370, 32: 131 / 353.
 bool mirror_lmhead_topk_spills(const mirror_ctx* ctx, int M, int topk) {
     const long long V = ctx->desc.vocab;
-    return V <= 65536 && V * (topk + 4) <= 5200ll * (M - 16);
+    return V <= 65536 && V * (topk + 4) <= std::min(2000ll * (M - 8), 5200ll * (M - 16));
 }
 
 mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int M, const void* W, float* logits_out,
@@ -967,4 +1004,21 @@ mirror_status mirror_linear_partial_launch(mirror_ctx* ctx, const void* x, int M
     if (st != MIRROR_OK) return st;
     *k_slices = p.k_slices;
     return MIRROR_OK;
+}
+
+// act[M, I] (bf16) = silu(x W_gate^T) * (x W_up^T), W = [gate rows; up rows], in one kernel (I a multiple of 16).
+mirror_status mirror_linear_gated_launch(mirror_ctx* ctx, const void* x, int M, const void* W, int I, int K, void* act, cudaStream_t stream) {
+    PairParams p;
+    mirror_status st = pair_shape(ctx->tune, M, 2 * I, K, &p);
+    if (st != MIRROR_OK) return st;
+    if (I % 16 != 0) return MIRROR_ERR_SHAPE;
+    p.n_units = (2 * I + kPairV - 1) / kPairV * p.n_chunks;
+    int n_pairs = ctx->num_sms / 2 * p.ctas_per_sm;
+    if (n_pairs > p.n_units) n_pairs = p.n_units;
+    if (n_pairs < 1) return MIRROR_ERR_UNSUPPORTED;
+    p.w_keep = p.n_chunks > 1;
+    p.w_early = 1;
+    p.act = (__nv_bfloat16*)act;
+    p.status = ctx->d_status;
+    return pair_launch(ctx, false, x, W, p, n_pairs, stream);
 }

@@ -131,6 +131,9 @@ mirror_status mirror_lmhead_pair_launch(mirror_ctx* ctx, const void* hidden, int
 int mirror_linear_slices(const mirror_ctx* ctx, int M, int N, int K);
 mirror_status mirror_linear_partial_launch(mirror_ctx* ctx, const void* x, int M, const void* W, int N, int K, float* partial,
                                            size_t partial_bytes, cudaStream_t stream, int* k_slices, bool w_early = false);
+// act[M, I] (bf16) = silu(x W_gate^T) * (x W_up^T), W = [gate rows; up rows] with K columns, without partial sums in memory.  W is
+// requested early, as above.
+mirror_status mirror_linear_gated_launch(mirror_ctx* ctx, const void* x, int M, const void* W, int I, int K, void* act, cudaStream_t stream);
 // e4m3 cache for mirror_attn_launch: pools, k_new and v_new hold codes; device scales per (layer, KV head), host Q scale.
 struct MirrorAttnFp8 {
     const float* k_scale;

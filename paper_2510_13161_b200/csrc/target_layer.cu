@@ -23,6 +23,8 @@ constexpr int kFinThreads = 256;
 // Stacks up to this depth take the faster attention kernel.  Deeper ones keep the order of every sum (see attn_tile64.cu).
 constexpr int kKeepRoundingLayers = 4;
 
+constexpr int kGatedRows = 32;
+
 struct TreeDepths {
     int depth[MIRROR_MAX_NODES];
 };
@@ -455,11 +457,19 @@ mirror_status target_forward_impl(mirror_ctx* ctx, const mirror_target* t, const
         MIRROR_CUDA_OK(launch_residual_norm(s, partial, slices, M, H, x_cur, (const __nv_bfloat16*)w.norm_mlp, t->rms_eps, xa, h));
         ctx->launches += 1;
         // gate / up projection + SiLU gate
-        st = mirror_linear_partial_launch(ctx, h, M, w.w_gate_up, 2 * I, H, partial, sc.partial_bytes, s, &slices, true);
-        if (st != MIRROR_OK) return st;
-        MIRROR_CUDA_OK(mirror_launch_pdl(finish_swiglu_kernel, dim3(grid_for((size_t)M * I / 4, ctx->num_sms)), dim3(kFinThreads), 0, s,
-                                         (const float*)partial, slices, M, I, act));
-        ctx->launches += 1;
+        // In the GEMM's epilogue for few rows (17 rows, 48 layers of the 14B shape: 7123 -> 7076 us; the toy model's two layers 83.9 -> 82.7), unless
+        // K is split to fill the chip.  With more rows the exponentials of a few CTAs' epilogues take longer than a pass of
+        // the whole chip (132 rows x 1536 columns, eight layers: 505 -> 536 us).
+        if (M <= kGatedRows && mirror_linear_slices(ctx, M, 2 * I, H) == 1) {
+            st = mirror_linear_gated_launch(ctx, h, M, w.w_gate_up, I, H, act, s);
+            if (st != MIRROR_OK) return st;
+        } else {
+            st = mirror_linear_partial_launch(ctx, h, M, w.w_gate_up, 2 * I, H, partial, sc.partial_bytes, s, &slices, true);
+            if (st != MIRROR_OK) return st;
+            MIRROR_CUDA_OK(mirror_launch_pdl(finish_swiglu_kernel, dim3(grid_for((size_t)M * I / 4, ctx->num_sms)), dim3(kFinThreads), 0, s,
+                                             (const float*)partial, slices, M, I, act));
+            ctx->launches += 1;
+        }
         // down projection + residual + the next layer's (or the final) norm
         st = mirror_linear_partial_launch(ctx, act, M, w.w_down, H, I, partial, sc.partial_bytes, s, &slices, true);
         if (st != MIRROR_OK) return st;
