@@ -126,28 +126,6 @@ __device__ __forceinline__ void dev_check(const AttnParams& p, int detail) {
 
 // ---- the tile sequence ---------------------------------------------------------------------------------------
 // Units in the order (layer, request, head or pair of heads); cumT[b] = KV tiles of one unit of the requests before b.
-struct UnitPos {
-    int layer, b, g;
-    int tile_in_unit, tiles_in_unit;
-    int unit_first_tile;
-};
-__device__ __noinline__ UnitPos locate(int x, const AttnParams& p, const int* cumT, int tiles_per_layer) {
-    UnitPos u;
-    const int hu = p.Hkv / p.heads_per_unit;
-    u.layer = (int)((uint32_t)x / (uint32_t)tiles_per_layer);         // (the tile count fits 31 bits: checked in the prologue)
-    const int rem = x - u.layer * tiles_per_layer;
-    int b = 0;
-    while (b + 1 < p.B && hu * cumT[b + 1] <= rem) ++b;
-    const int Tb = cumT[b + 1] - cumT[b];
-    const int r2 = rem - hu * cumT[b];
-    u.b = b;
-    u.g = (int)((uint32_t)r2 / (uint32_t)Tb);
-    u.tile_in_unit = r2 - u.g * Tb;
-    u.tiles_in_unit = Tb;
-    u.unit_first_tile = x - u.tile_in_unit;
-    return u;
-}
-
 __device__ __forceinline__ int tiles_of(int len, int tree_slots) {
     return ((len + kSlotTok - 1) / kSlotTok + tree_slots + kTileSlots - 1) / kTileSlots;
 }
@@ -165,14 +143,6 @@ __device__ __forceinline__ void fill_segment(Segment& s, int left, const AttnPar
     s.slots_all = s.pages_all + p.tree_slots;
     s.tiles = tiles_of(s.len, p.tree_slots);
     s.t_last = min(s.tiles, s.t_first + left);
-}
-__device__ __noinline__ Segment first_segment(int x, int x_end, const AttnParams& p, const int* cumT, const int* s_len,
-                                              int tiles_per_layer) {
-    const UnitPos u = locate(x, p, cumT, tiles_per_layer);
-    Segment s;
-    s.layer = u.layer; s.b = u.b; s.g = u.g; s.t_first = u.tile_in_unit;
-    fill_segment(s, x_end - x, p, s_len);
-    return s;
 }
 // the unit behind s (a segment that is followed by another one ends with its unit)
 __device__ __noinline__ Segment next_segment(const Segment& s, int left, const AttnParams& p, const int* s_len) {
@@ -250,23 +220,28 @@ struct Share {
     int g;
     float total;                          // ns
 };
+__host__ __device__ inline float quick_quotient(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fdividef(a, b);
+#else
+    return a / b;
+#endif
+}
 __host__ __device__ inline Share share_choice(const AttnParams& p, float total_tiles, int most, int sms, float step_bytes, int choice) {
-    const float steps = p.mode == kSplit ? 0.5f * (total_tiles + (float)p.units) : total_tiles;
-    const float work = steps + kUnitSteps * (float)p.units;
-    int g = most - most * choice / 40;
-    if (g < 1) g = 1;
-    float t;
-    if (p.deal) {
-        const int k = (p.units + g - 1) / g;
-        g = (p.units + k - 1) / k;
-        t = (float)k * work / (float)p.units;
+    const float units = (float)p.units, steps = p.mode == kSplit ? 0.5f * (total_tiles + units) : total_tiles;
+    const float work = steps + kUnitSteps * units;
+    float g = fmaxf((float)(most - ((most * choice * 1639) >> 16)), 1.f), t;         // (a fortieth of the groups less from choice to choice)
+    if (p.deal) {                                                     // (whole units; a quotient's last bit does not matter)
+        const float k = ceilf(quick_quotient(units, g) - 1e-3f);
+        g = ceilf(quick_quotient(units, k) - 1e-3f);
+        t = k * quick_quotient(work, units);
     } else {
-        t = (work + kUnitSteps * (float)g) / (float)g;
+        t = quick_quotient(work, g) + kUnitSteps;
     }
     t *= kStepNs;
-    const float hbm = 1.f - (float)g * step_bytes * steps / (work * kStepNs * kHbmBytesNs);
-    const float rate = fminf((float)(sms - g * p.n_cta) / kFullSms, fmaxf(hbm, 0.1f));
-    return {g, t + fmaxf(0.f, p.lm_ns - t * rate)};
+    const float hbm = 1.f - quick_quotient(g * step_bytes * steps, work * (kStepNs * kHbmBytesNs));
+    const float rate = fminf(((float)sms - g * (float)p.n_cta) * (1.f / kFullSms), fmaxf(hbm, 0.1f));
+    return {(int)g, t + fmaxf(0.f, p.lm_ns - t * rate)};
 }
 __device__ __noinline__ int share_groups(const AttnParams& p, int total_tiles, int most, int sms, float step_bytes) {
     const int lane = threadIdx.x & 31;
@@ -323,22 +298,46 @@ __device__ __forceinline__ Partition make_partition(const AttnParams& p, const i
     q.snap_tol = min(p.snap_cap, q.share >> 2);
     return q;
 }
-__device__ __noinline__ int group_begin(const Partition& q, int g, const AttnParams& p, const int* cumT) {
-    if (g <= 0) return 0;
-    if (g >= q.n_groups) return q.total_tiles;
+// Where group g's range begins: tile x of the sequence, tile t of unit (layer, b, g).  (Position and unit in one go: found again
+// from the position, and with the divisions of a fully rounded quotient in share_choice, this took 3500 to 8500 cycles of a launch.)
+struct Begin {
+    int x, layer, b, g, t;
+};
+__device__ __noinline__ Begin group_begin(const Partition& q, int g, const AttnParams& p, const int* cumT) {
+    Begin u = {g <= 0 ? 0 : q.total_tiles, 0, 0, 0, 0};
+    if (g <= 0 || g >= q.n_groups) return u;
+    const int hu = p.Hkv / p.heads_per_unit;
     if (q.whole) {                                                    // first tile of unit number units * g / n_groups
-        const int hu = p.Hkv / p.heads_per_unit, per = p.B * hu;
-        const int us = p.units / q.n_groups, unit = us * g + (p.units - us * q.n_groups) * g / q.n_groups;
-        const int layer = unit / per, r = unit - layer * per, b = r / hu;
-        return layer * q.tiles_per_layer + hu * cumT[b] + (r - b * hu) * (cumT[b + 1] - cumT[b]);
+        const uint32_t n = (uint32_t)q.n_groups, us = (uint32_t)p.units / n, rest = (uint32_t)p.units - us * n;
+        const uint32_t unit = us * g + (rest ? rest * g / n : 0), per = (uint32_t)(p.B * hu);
+        u.layer = (int)(unit / per);
+        u.g = (int)(unit - u.layer * per);
+        if (p.B > 1) {
+            u.b = (int)((uint32_t)u.g / (uint32_t)hu);
+            u.g -= u.b * hu;
+        }
+        u.x = u.layer * q.tiles_per_layer + hu * cumT[u.b] + u.g * (cumT[u.b + 1] - cumT[u.b]);
+        return u;
     }
-    const int e = q.share * g + (int)((uint32_t)(q.rest * g) / (uint32_t)q.n_groups);       // total_tiles * g / n_groups
-    if (q.snap_tol == 0) return e;
-    const UnitPos u = locate(e, p, cumT, q.tiles_per_layer);
-    const int lo = u.unit_first_tile, hi = lo + u.tiles_in_unit;
-    const int best = (e - lo <= hi - e) ? lo : hi;
-    const int dist = best > e ? best - e : e - best;
-    return dist <= q.snap_tol ? best : e;
+    u.x = q.share * g + (q.rest ? (int)((uint32_t)(q.rest * g) / (uint32_t)q.n_groups) : 0);       // total_tiles * g / n_groups
+    u.layer = (int)((uint32_t)u.x / (uint32_t)q.tiles_per_layer);     // (the tile count fits 31 bits: checked in the prologue)
+    int rem = u.x - u.layer * q.tiles_per_layer;
+    while (u.b + 1 < p.B && hu * cumT[u.b + 1] <= rem) ++u.b;
+    rem -= hu * cumT[u.b];
+    const int Tb = cumT[u.b + 1] - cumT[u.b];
+    u.g = (int)((uint32_t)rem / (uint32_t)Tb);
+    u.t = rem - u.g * Tb;
+    if (u.t <= Tb - u.t) {                                            // to the unit boundary close by
+        if (u.t <= q.snap_tol) { u.x -= u.t; u.t = 0; }
+    } else if (Tb - u.t <= q.snap_tol) {
+        u.x += Tb - u.t;
+        u.t = 0;
+        if (++u.g == hu) {
+            u.g = 0;
+            if (++u.b == p.B) { u.b = 0; ++u.layer; }
+        }
+    }
+    return u;
 }
 
 // A launch that leaves SMs to another one leaves whole TPCs (the other's CTAs come in pairs), spread over the chip as blocks are
@@ -635,15 +634,16 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         const int block_group = blockIdx.x / p.n_cta, group = p.lm_ns > 0.f ? spread_group(block_group, p.n_groups, part.n_groups, p.group_chunk) : block_group;
         const bool fits = part.total_tiles >= 0 && (ptx::smem_u32(smem) & 1023) == 0;
         if (!fits && lane == 0) dev_check(p, 600);
-        int x = 0;
-        if (fits && group < part.n_groups && lane < 2) x = group_begin(part, group + lane, p, cumT);
-        const int x1 = __shfl_sync(0xffffffffu, x, 1);
+        Begin u = {};
+        if (fits && group < part.n_groups && lane < 2) u = group_begin(part, group + lane, p, cumT);
+        const int x1 = __shfl_sync(0xffffffffu, u.x, 1);
         if (lane == 0) {
-            ctrl->n_tiles = x1 - x;
+            ctrl->n_tiles = x1 - u.x;
             ctrl->group = group;
-            if (x < x1) ctrl->first = first_segment(x, x1, p, cumT, s_len, part.tiles_per_layer);
-            const Segment& s = ctrl->first;
-            if (rb == 0 && group < p.n_groups) p.begins[group] = {x < x1 && s.t_first > 0 ? 1 : 0, s.layer, s.b, s.g};
+            Segment& s = ctrl->first;
+            s.layer = u.layer; s.b = u.b; s.g = u.g; s.t_first = u.t;
+            if (u.x < x1) fill_segment(s, x1 - u.x, p, s_len);
+            if (rb == 0 && group < p.n_groups) p.begins[group] = {u.x < x1 && u.t > 0 ? 1 : 0, u.layer, u.b, u.g};
         }
     }
     __syncthreads();
