@@ -40,10 +40,10 @@ __device__ __forceinline__ float sum_slices(const float* partial, int slices, si
 // alone would be off by milliradians) and shared by all layers.
 __global__ void rope_table_kernel(const int32_t* prefix_len, const TreeDepths td, int B, int n, int half, double theta,
                                   float2* cs) {
-    ptx::grid_dep_wait();
+    // (beside the first layer's norm, launched ahead of it, which lets this one start only once all before it has completed)
     ptx::grid_dep_launch();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= B * n * half) return;
+    if (idx >= B * n * half) { ptx::grid_dep_wait(); return; }
     const int f = idx % half, row = idx / half;
     const int b = row / n, i = row % n;
     const double pos = (double)prefix_len[b] + (double)td.depth[i];
@@ -51,6 +51,7 @@ __global__ void rope_table_kernel(const int32_t* prefix_len, const TreeDepths td
     double s, c;
     sincos(pos * inv_freq, &s, &c);
     cs[idx] = make_float2((float)c, (float)s);
+    ptx::grid_dep_wait();                   // (whatever waits for this launch waits for the norm, too)
 }
 
 __device__ __forceinline__ float4 sum_slices4(const float* partial, int slices, size_t slice_elems, size_t idx) {
@@ -130,8 +131,10 @@ finish_residual_norm_kernel(const float* partial, int slices, int M, int H, cons
     // behind a projection, the residual stream and the weight are older than the kernel ahead: no need to wait for it (with many
     // rows that hides nothing)
     if (kNormCluster > 1 && partial) load_early();
-    ptx::grid_dep_launch();
+    // (the kernel behind a norm of its own may rely on everything ahead of it being complete)
+    if (partial) ptx::grid_dep_launch();
     ptx::grid_dep_wait();
+    if (!partial) ptx::grid_dep_launch();
     if (kNormCluster == 1 || !partial) load_early();
     if (partial) {
         // several slices' loads in flight at a time; the additions stay in slice order
@@ -404,12 +407,12 @@ mirror_status target_forward_impl(mirror_ctx* ctx, const mirror_target* t, const
     TreeDepths td;
     for (int i = 0; i < MIRROR_MAX_NODES; ++i) td.depth[i] = i < n ? ti.depth[i] : 0;
     const int half = d / 2;
-    MIRROR_CUDA_OK(mirror_launch_pdl(rope_table_kernel, dim3((M * half + 255) / 256), dim3(256), 0, s, kv->prefix_len, td, B, n, half,
-                                     (double)t->rope_theta, cs));
-    ctx->launches += 1;
     // the first layer's input norm; every later one comes out of the finish kernel of the layer before
     MIRROR_CUDA_OK(launch_residual_norm(s, nullptr, 0, M, H, (const __nv_bfloat16*)x, (const __nv_bfloat16*)t->layers[0].norm_attn, t->rms_eps,
                                         nullptr, h));
+    ctx->launches += 1;
+    MIRROR_CUDA_OK(mirror_launch_pdl(rope_table_kernel, dim3((M * half + 255) / 256), dim3(256), 0, s, kv->prefix_len, td, B, n, half,
+                                     (double)t->rope_theta, cs));
     ctx->launches += 1;
 
     const int Nqkv = (Hq + 2 * Hkv) * d;
