@@ -11,7 +11,8 @@
 // in the order (tile major, chunk minor), so that at any time the pairs work on a handful of neighbouring tiles and
 // the chunks of one tile run on different pairs at the same moment: every weight tile leaves HBM once and the other
 // chunks hit it in L2.  Each unit leaves one partial (max, argmax, sum-exp) per hidden row and 128-row half tile;
-// lmhead_merge_kernel folds them in a fixed order, so the result does not depend on which pair ran which unit.
+// lmhead_merge_kernel folds them in a fixed order, so the result does not depend on which pair ran which unit (and a launch that
+// runs beside an attention launch hands them out by a counter: kFree).
 //
 // Per CTA, 6 warps as in lmhead_kernel: warp 0 TMA producer (own W rows + own half of the hidden chunk), warp 1
 // TMEM owner; in the pair's leader (cluster rank 0) its elected lane issues the UMMAs for both CTAs; warps 2..5

@@ -7,7 +7,8 @@
 // pair streams its share.  The GEMM leaves fp32 partial sums [slices][M][N]; a small "finish" kernel per projection
 // adds the slices in a fixed order and applies what follows the projection in the layer, so no activation makes an
 // extra trip through HBM: rotary embedding and the split into Q / K / V, residual add + the next RMSNorm, or the
-// SiLU gate.  Activations are stored in bf16 (one rounding per stored tensor), sums are fp32.
+// SiLU gate (with few rows, in the epilogue of the projection itself).  Activations are stored in bf16 (one rounding per stored
+// tensor), sums are fp32.
 // Every kernel is launched with programmatic stream serialization and waits for the kernel ahead before it touches
 // what that kernel writes.  The finishing kernels (and the attention's merge) let the kernel behind them be launched at once,
 // so that its set-up and its first weights overlap theirs; the GEMMs and the attention do so only once they have waited
@@ -460,7 +461,7 @@ mirror_status target_forward_impl(mirror_ctx* ctx, const mirror_target* t, const
         MIRROR_CUDA_OK(launch_residual_norm(s, partial, slices, M, H, x_cur, (const __nv_bfloat16*)w.norm_mlp, t->rms_eps, xa, h));
         ctx->launches += 1;
         // gate / up projection + SiLU gate
-        // In the GEMM's epilogue for few rows (17 rows, 48 layers of the 14B shape: 7123 -> 7076 us; the toy model's two layers 83.9 -> 82.7), unless
+        // In the GEMM's epilogue for few rows (17 rows, 48 layers of the 14B shape: 7123 -> 7052 us; the toy model's two layers 82.4 -> 81.0), unless
         // K is split to fill the chip.  With more rows the exponentials of a few CTAs' epilogues take longer than a pass of
         // the whole chip (132 rows x 1536 columns, eight layers: 505 -> 536 us).
         if (M <= kGatedRows && mirror_linear_slices(ctx, M, 2 * I, H) == 1) {
