@@ -87,6 +87,7 @@ struct AttnParams {
     long long wait_limit;                 // SM cycles after which a wait gives up
     int stall_after;                      // test aid: the K producer stops after this many stages (-1: never)
     int stall_merge;                      // test aid: 1: the merge's first wait runs out
+    int early;                            // 1: only q and the tree's K/V come from the kernel ahead (see mirror_attn_launch)
 };
 
 struct UnitPos {                          // where a global tile index falls (indexes fit 31 bits: checked in the prologue)
@@ -320,8 +321,11 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();                 // the merge kernel behind may be scheduled as soon as SMs free up
+    // (early: the producers wait in front of the tree's rows, the softmax warps in front of Q)
+    if (!p.early) {
+        ptx::grid_dep_wait();
+        ptx::grid_dep_launch();             // the merge kernel behind may be scheduled as soon as SMs free up
+    }
     // one warp finds this CTA's range of tiles and the part of a unit that it begins with
     if (warp == 0) {
         int acc = 0;
@@ -411,6 +415,7 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
                 const int n_slots = max(0, min(kStageSlots, sg.slots_all - sl0));      // slots that exist in this stage
                 const int n_tma = max(0, min(kStageSlots, sg.pages_full - sl0));       // leading slots that are whole pages
                 if (n_tma < n_slots) {
+                    if (p.early) ptx::grid_dep_wait();
                     // ragged page and tree tokens by asynchronous 16-byte copies (rows beyond the valid count are
                     // zero-filled), all in flight together; the loops are kept rolled: this path runs once per unit, and
                     // what it costs is mostly the instruction fetch
@@ -588,6 +593,10 @@ attn_tile64_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
         const unsigned long long anc0 = tree.anc[node][0], anc1 = tree.anc[node][1];
         const uint32_t lane_base = tmem_base + ((uint32_t)(w4 * 32) << 16);
         const uint32_t o_mine = lane_base + kTmemO + (uint32_t)(grp * D);       // this group's accumulator
+        if (p.early) {
+            ptx::grid_dep_wait();
+            ptx::grid_dep_launch();
+        }
         constexpr int kDH = D / 2;                                 // output columns this warp finalises
         constexpr int kRowW = D + 4;                               // partial: D accumulator columns, then (max, sum) twice
         // both warps that share a TMEM quarter arrive (bounded wait, like every other wait in this kernel)
@@ -880,7 +889,7 @@ __global__ void __launch_bounds__(attn::kMergeThreads) attn_tile64_merge_kernel(
 
 mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
-                                 float* partial_ws, cudaStream_t stream) {
+                                 float* partial_ws, cudaStream_t stream, bool early) {
     const int D = ctx->desc.head_dim, Hkv = ctx->desc.n_kv_heads, Hq = ctx->desc.n_q_heads;
     AttnParams p;
     p.L = kv->num_layers; p.B = tree->batch; p.n = ti.n; p.Hq = Hq; p.Hkv = Hkv; p.G = Hq / Hkv;
@@ -892,6 +901,7 @@ mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, co
     if (p.n_groups < 1 || p.n_groups * sizeof(attn::GroupBegin) > kWsNotesBytes) return MIRROR_ERR_SHAPE;
     p.snap_cap = ctx->tune.attn_snap;
     p.whole_groups = ctx->tune.attn_whole_units ? attn::whole_unit_groups(p.n_groups, (long long)kv->num_layers * tree->batch * ctx->desc.n_kv_heads) : 0;
+    p.early = early;
     p.wait_limit = ctx->tune.wait_limit_cycles;
     p.stall_after = (ctx->tune.test_stall_after >= 0 && ctx->tune.test_stall_attn_left-- > 0) ? ctx->tune.test_stall_after : -1;
     p.stall_merge = ctx->tune.test_stall_merges > 0 && ctx->tune.test_stall_merges-- > 0;

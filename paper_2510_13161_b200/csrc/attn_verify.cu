@@ -114,6 +114,7 @@ struct AttnParams {
     long long wait_limit;                 // SM cycles after which a wait gives up
     int stall_after;                      // test aid: the K producer stops after this many stages (-1: never)
     int stall_merge;                      // test aid: 1: the merge's first wait runs out
+    int early;                            // 1: only q and the tree's K/V come from the kernel ahead (see mirror_attn_launch)
 };
 
 struct Maps {
@@ -626,8 +627,11 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();                 // the kernel behind may be scheduled as soon as SMs free up
+    // (early: the K producer waits in front of the tree's rows, the V producer in front of Q)
+    if (!p.early) {
+        ptx::grid_dep_wait();
+        ptx::grid_dep_launch();             // the kernel behind may be scheduled as soon as SMs free up
+    }
     if (warp == 0) {
         load_lengths(p, cumT, s_len, true);
         const Partition part = make_partition(p, cumT, (float)(C::kStageBytes * (split ? 4 : 2)));
@@ -723,6 +727,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                             for (int k = 0; k < kTileSlots; ++k) ptx::tma_load_5d(dst + k * C::kSlotBytes, map, bar, 0, 0, 0, 0, row[k]);
                         }
                     } else {
+                        if (p.early && sl0 + n_sl > sg.pages_all) ptx::grid_dep_wait();
                         const bool leader = ptx::elect_one();
                         if (leader) ptx::mbar_arrive_expect_tx(bar, (uint32_t)((n_sl - (ragged >= 0)) * C::kSlotBytes));
 #pragma unroll 1
@@ -769,6 +774,10 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     for (int c = lane; c < p.heads_per_unit * kSlotTok * C::kRowBytes / 128; c += 32) ptx::prefetch_l2(src + c * 128);
                 };
                 if (V) {
+                    if (p.early) {
+                        ptx::grid_dep_wait();
+                        ptx::grid_dep_launch();
+                    }
                     if (!F8) load_q(sg, 0);
                     prefetch_ragged(sg);
                 }
@@ -1336,8 +1345,8 @@ mirror_status merge_launch(mirror_ctx* ctx, const AttnParams& p, cudaStream_t st
 mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
                                  float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8, bool keep_rounding,
-                                 MirrorAttnBeside* beside) {
-    if (keep_rounding && !f8) return mirror_attn_tile64_launch(ctx, kv, tree, ti, q, k_new, v_new, out, lse_out, partial_ws, stream);
+                                 MirrorAttnBeside* beside, bool early) {
+    if (keep_rounding && !f8) return mirror_attn_tile64_launch(ctx, kv, tree, ti, q, k_new, v_new, out, lse_out, partial_ws, stream, early);
     const int D = ctx->desc.head_dim, Hkv = ctx->desc.n_kv_heads, Hq = ctx->desc.n_q_heads;
     AttnParams p;
     p.L = kv->num_layers; p.B = tree->batch; p.n = ti.n; p.Hq = Hq; p.Hkv = Hkv; p.G = Hq / Hkv;
@@ -1373,6 +1382,7 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     p.cut_tiles = f8 || p.unit_cuts == 1 ? 8 : 2;
     const int most_tiles = (kv->max_pages_per_req + (p.n + kSlotTok - 1) / kSlotTok + kTileSlots - 1) / kTileSlots;      // of a unit
     p.never_cut = whole && most_tiles <= 6;
+    p.early = early && !f8;                                  // (over an e4m3 cache the softmax warps read q themselves)
     // Beside a weight stream: whole units, where one request's are short (a cut costs about as much as two tiles, a launch behind it not counted).
     p.lm_ns = 0.f;
     p.deal = p.never_cut || (whole && p.B == 1 && units >= 2 * p.n_groups && most_tiles <= 64);

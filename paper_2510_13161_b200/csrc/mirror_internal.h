@@ -154,15 +154,17 @@ struct MirrorAttnBeside {
     bool merge_needed = false;
     unsigned char merge[512];
 };
+// early: of what the launch reads, only q, k_new and v_new are written by the kernel ahead, and whatever ran before that one has
+// completed when this launch begins: lengths, page table and the cache's pages are read without waiting for it.
 // keep_rounding: every sum keeps the order of the 64-token kernel (mirror_target_forward in deep stacks, see attn_tile64.cu).
 mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
                                  float* partial_ws, cudaStream_t stream, const MirrorAttnFp8* f8 = nullptr, bool keep_rounding = false,
-                                 MirrorAttnBeside* beside = nullptr);
+                                 MirrorAttnBeside* beside = nullptr, bool early = false);
 mirror_status mirror_attn_late_merge(mirror_ctx* ctx, const MirrorAttnBeside& beside, cudaStream_t stream);
 mirror_status mirror_attn_tile64_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                         const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
-                                        float* partial_ws, cudaStream_t stream);
+                                        float* partial_ws, cudaStream_t stream, bool early);
 
 // bf16 tensor map with 128-byte swizzle.  dims/box are innermost-first; strides_bytes[i] is the byte
 // stride of dimension i+1 (rank-1 entries).

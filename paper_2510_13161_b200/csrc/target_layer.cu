@@ -440,7 +440,7 @@ mirror_status target_forward_impl(mirror_ctx* ctx, const mirror_target* t, const
             kv_l.k_pool = (const __nv_bfloat16*)kv->k_pool + (size_t)l * kv->layer_stride;
             kv_l.v_pool = (const __nv_bfloat16*)kv->v_pool + (size_t)l * kv->layer_stride;
             st = mirror_attn_launch(ctx, &kv_l, tree, ti, q_l, k_l, v_l, a_l, nullptr, (float*)((uint8_t*)ctx->ws + L.attn_partial), s, nullptr,
-                                    t->n_layers > kKeepRoundingLayers);
+                                    t->n_layers > kKeepRoundingLayers, nullptr, true);        // (behind finish_qkv_kernel, which lets it begin at once)
         } else {
             // the layer's new K/V rows as codes under the cache's scales (the caller commits them), then the 8-bit attention
             uint8_t* k8_l = (uint8_t*)f8->k_new8_out + (size_t)l * kv_elems;
