@@ -622,7 +622,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                             upd_i = vid - lane + (__ffs(at_max) - 1);
                             if (p.sums) {
 #pragma unroll
-                                for (int j = 0; j < 32; ++j) v[j] = exp2f(v[j] * p.inv_T_log2e);
+                                for (int j = 0; j < 32; ++j) v[j] = ptx::ex2_approx(v[j] * p.inv_T_log2e);      // (below 2^-126: 0 beside the maximum's 1)
                                 upd_s = reduce_columns(v, [](float a, float b) { return a + b; });
                             }
                         }
