@@ -110,8 +110,10 @@ __device__ __forceinline__ uint32_t map_to_rank(const void* smem_ptr, uint32_t r
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(ptx::smem_u32(smem_ptr)), "r"(rank));
     return r;
 }
+// (What it hands over is tensor memory that tcgen05.ld has already been waited for, nothing that the arriving thread wrote: a release at
+// cluster scope would hold a unit's end up behind its spilled logits and state; 132 rows x 137273 x 768: 82.7 -> 80.1 us.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // a word into the shared memory of a CTA of the pair, counted on a barrier there
 __device__ __forceinline__ void st_async(uint32_t cluster_addr, int v, uint32_t bar_cluster_addr) {
