@@ -114,7 +114,6 @@ struct AttnParams {
     long long wait_limit;                 // SM cycles after which a wait gives up
     int stall_after;                      // test aid: the K producer stops after this many stages (-1: never)
     int stall_merge;                      // test aid: 1: the merge's first wait runs out
-    int early;                            // 1: only q and the tree's K/V come from the kernel ahead (see mirror_attn_launch)
 };
 
 struct Maps {
@@ -566,7 +565,9 @@ __device__ __forceinline__ uint2 widen4(uint32_t w) {
     return r;
 }
 
-template <int D, bool F8>
+// kEarly: only q and the tree's K/V come from the kernel ahead (see mirror_attn_launch).  An instance of its own: the same as
+// run-time branches cost long calls, which never take them, 0.8% (64 layers, 32768 tokens, 33 nodes: 3608 -> 3639 us).
+template <int D, bool F8, bool kEarly>
 __global__ void __launch_bounds__(Cfg<D, F8>::kThreads, 1)
 attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ AttnTree tree, const __grid_constant__ AttnParams p,
                    const int n_stages) {
@@ -627,8 +628,8 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    // (early: the K producer waits in front of the tree's rows, the V producer in front of Q)
-    if (!p.early) {
+    // (kEarly: the K producer waits in front of the tree's rows, the V producer in front of Q)
+    if (!kEarly) {
         ptx::grid_dep_wait();
         ptx::grid_dep_launch();             // the kernel behind may be scheduled as soon as SMs free up
     }
@@ -727,7 +728,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                             for (int k = 0; k < kTileSlots; ++k) ptx::tma_load_5d(dst + k * C::kSlotBytes, map, bar, 0, 0, 0, 0, row[k]);
                         }
                     } else {
-                        if (p.early && sl0 + n_sl > sg.pages_all) ptx::grid_dep_wait();
+                        if (kEarly && sl0 + n_sl > sg.pages_all) ptx::grid_dep_wait();
                         const bool leader = ptx::elect_one();
                         if (leader) ptx::mbar_arrive_expect_tx(bar, (uint32_t)((n_sl - (ragged >= 0)) * C::kSlotBytes));
 #pragma unroll 1
@@ -774,7 +775,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     for (int c = lane; c < p.heads_per_unit * kSlotTok * C::kRowBytes / 128; c += 32) ptx::prefetch_l2(src + c * 128);
                 };
                 if (V) {
-                    if (p.early) {
+                    if (kEarly) {
                         ptx::grid_dep_wait();
                         ptx::grid_dep_launch();
                     }
@@ -1382,7 +1383,6 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
     p.cut_tiles = f8 || p.unit_cuts == 1 ? 8 : 2;
     const int most_tiles = (kv->max_pages_per_req + (p.n + kSlotTok - 1) / kSlotTok + kTileSlots - 1) / kTileSlots;      // of a unit
     p.never_cut = whole && most_tiles <= 6;
-    p.early = early && !f8;                                  // (over an e4m3 cache the softmax warps read q themselves)
     // Beside a weight stream: whole units, where one request's are short (a cut costs about as much as two tiles, a launch behind it not counted).
     p.lm_ns = 0.f;
     p.deal = p.never_cut || (whole && p.B == 1 && units >= 2 * p.n_groups && most_tiles <= 64);
@@ -1492,9 +1492,9 @@ mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mir
         // which units the partition cut is only known on the device (it depends on the prefix lengths)
         return merge_launch(ctx, p, stream);
     };
-    return f8         ? launch(Cfg<128, true>{}, attn_verify_kernel<128, true>)
-           : D == 128 ? launch(Cfg<128, false>{}, attn_verify_kernel<128, false>)
-                      : launch(Cfg<64, false>{}, attn_verify_kernel<64, false>);
+    if (f8) return launch(Cfg<128, true>{}, attn_verify_kernel<128, true, false>);        // (its softmax warps read q themselves)
+    if (D == 128) return launch(Cfg<128, false>{}, early ? attn_verify_kernel<128, false, true> : attn_verify_kernel<128, false, false>);
+    return launch(Cfg<64, false>{}, early ? attn_verify_kernel<64, false, true> : attn_verify_kernel<64, false, false>);
 }
 
 mirror_status mirror_attn_late_merge(mirror_ctx* ctx, const MirrorAttnBeside& beside, cudaStream_t stream) {
