@@ -61,7 +61,7 @@ struct PairParams {
     int topk;                               // > 0: the epilogue collects candidates for each row's topk best (logit, id) pairs
     float* part_topv;                       // [4 * CTA + warp][M][topk]: sorted lists
     int* part_topi;
-    uint32_t* topk_bar;                     // largest logit seen in each of topk shares of the vocabulary (bar_word; order_key, 0: none)
+    uint32_t* topk_bar;                     // largest logit seen in each of topk shares of the vocabulary (bar_word; order_key, 0: none, 1: none finite)
     int fp8;                                // 1: W and the hidden rows are e4m3 bytes (K counted in 128-byte blocks all the same)
     const float* w_scale;                   // fp8: [V] scale of each weight row
     const float* h_scale;                   // fp8: [M] scale of each hidden row
@@ -657,9 +657,11 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                 float* const all_max = (float*)((uint8_t*)ctrl + kCtrlBytes);
                 uint32_t* const bars = (uint32_t*)(all_max + 4 * kMaxChunkRows);
                 asm volatile("bar.sync 1, 128;" ::: "memory");
+                // (a row without a finite logit, an input's NaN, counts as met at the lowest key; a CTA beyond the vocabulary has met nothing)
                 const int share = (int)(blockIdx.x % (uint32_t)K);
+                const uint32_t seen = vt * p.rows_cta < p.V ? 1u : 0u;
                 for (int c = (warp - 2) * 32 + lane; ok && c < n_rows; c += 128) {
-                    uint32_t key = 0;
+                    uint32_t key = seen;
                     for (int w = 0; w < 4; ++w) {
                         const float m = all_max[w * kMaxChunkRows + c];
                         if (m > -INFINITY) key = max(key, mirror_order_key(m));
@@ -668,8 +670,9 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                 }
                 // The first unit's logits would all pass a bar that does not exist yet, and cost their warps a sort per row (1.2 us a row in
                 // all).  The other CTAs are at their first unit too: until each share has a word it is worth waiting, for as long as
-                // those sorts would take at most (no one has to arrive: a share that stays empty lets everything pass).
-                const bool first = u == pair && gridDim.x >= (uint32_t)K;
+                // those sorts would take at most (no one has to arrive: a share that stays empty lets everything pass), if there is
+                // a CTA with vocabulary for each share.
+                const bool first = u == pair && min((int)gridDim.x, (p.V + p.rows_cta - 1) / p.rows_cta) >= K;
                 const long long t0 = clock64(), limit = 2000ll * n_rows;
                 for (int c = (warp - 2) * 32 + lane; c < n_rows; c += 128) {
                     uint32_t bar;

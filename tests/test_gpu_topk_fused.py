@@ -82,3 +82,44 @@ def test_early_exit_tap_needs_no_logits_buffer():
         if not np.array_equal(got[r], ref["topk_id"][r]):
             assert np.abs(np.sort(logits[r, got[r]]) - np.sort(logits[r, ref["topk_id"][r]])).max() < TOL
     np.testing.assert_allclose(lp.float().cpu().numpy(), ref["topk_logprob"], atol=0.05)      # bf16 payload
+
+
+def call_us(call, n=15):
+    """Median device time of a call, in us."""
+    for _ in range(3):
+        call()
+    ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(n)]
+    for a, b in ev:
+        a.record(); call(); b.record()
+    torch.cuda.synchronize()
+    return sorted(a.elapsed_time(b) * 1e3 for a, b in ev)[n // 2]
+
+
+def test_a_row_without_a_finite_logit_does_not_hold_the_others_up():
+    """A CTA's first unit waits for the rows' bars, for up to 2000 cycles a row (260 us here): a row that has none to offer is not waited for."""
+    V, H, M, k = 70000, 256, 256, 8
+    W = rand_bf16((V, H), 0.05, 15).cuda(); hid = rand_bf16((M, H), 1.0, 16).cuda()
+    m = make_mirror(lm_cfg(V, H))
+    clean = m.mirror_lmhead_reduce(hid, W, topk=k)
+    bad = hid.clone(); bad[100] = float("nan")
+    res = m.mirror_lmhead_reduce(bad, W, topk=k)
+    rest = torch.arange(M, device="cuda") != 100
+    assert torch.equal(res["topk_id"][rest], clean["topk_id"][rest])
+    assert torch.equal(res["topk_logprob"][rest], clean["topk_logprob"][rest])
+    t0, t1 = call_us(lambda: m.mirror_lmhead_reduce(hid, W, topk=k)), call_us(lambda: m.mirror_lmhead_reduce(bad, W, topk=k))
+    assert m.device_status() == (0, 0)
+    assert t1 < t0 + 80, (t0, t1)
+
+
+def test_a_share_whose_only_cta_lies_beyond_the_vocabulary_is_not_waited_for():
+    """CTAs of 64 ids for kappa = 32: V = 1984 takes 32 of them, of which the last has no id left, so that a share stays empty as with the
+    30 of V = 1920, which wait for nothing (a wait: 40 us)."""
+    H, M, k = 256, 40, 32
+    hid, t = rand_bf16((M, H), 1.0, 18), {}
+    for V in (1920, 1984):
+        W = rand_bf16((V, H), 0.05, 17)
+        m, dh, dw = make_mirror(lm_cfg(V, H)), hid.cuda(), W.cuda()
+        check_topk(m.mirror_lmhead_reduce(dh, dw, topk=k), O.lmhead_logits(I.bf16_bits(hid), I.bf16_bits(W)), 1.0, k)
+        t[V] = call_us(lambda: m.mirror_lmhead_reduce(dh, dw, topk=k))
+        assert m.device_status() == (0, 0)
+    assert t[1984] < t[1920] + 20, t
