@@ -322,7 +322,7 @@ mirror_status mirror_trie_build(const int32_t* branch_tokens, int kappa, int gam
 
 /* One whole verify step on one stream: attention over all layers -> LM head rows -> reductions -> acceptance.
  *   hidden   bf16 [B*n, H], or NULL to feed the last layer's attention output (requires Hq*d == H).  Rows of the caller's own are
- *            read while the attention is running; rows that lie in attn_out are taken from what the attention leaves there
+ *            read while the attention is running; rows (and weights) that lie in attn_out are taken from what the attention leaves there
  *   attn_out bf16 [L, B, n, Hq, d]  (required: it is also the chained LM-head input)
  *   acc      mode, emit_bonus, q_probs, u_accept, u_resample, cand_ids are read; target_argmax / logits / lse
  *            are produced internally (in the workspace)

@@ -98,7 +98,7 @@ mirror_status mirror_accept_launch(mirror_ctx* ctx, const mirror_tree* tree, con
 // When an LM-head launch may begin.
 enum MirrorLmStart {
     MIRROR_LM_AFTER,              // once the kernel ahead has completed
-    MIRROR_LM_WEIGHTS_EARLY,      // no kernel that may still be running when the one ahead begins writes W: its first tiles are requested early
+    MIRROR_LM_WEIGHTS_EARLY,      // neither the kernel ahead nor any that may still be running when that one begins writes W: its first tiles are requested early
     MIRROR_LM_AT_ONCE             // nor does any, the one ahead included, write W or the hidden rows: as SMs come free, beside the one ahead
 };
 // defer: the row partials are not merged, but described there (only the argmax was asked for).

@@ -163,8 +163,9 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     // Hidden rows of the caller's own do not depend on the attention: the LM head is launched beside it (see lmhead_pair.cu), on the
     // SMs that the attention leaves or has done with, and the attention's merge behind the decision.
     const size_t attn_bytes = (size_t)kv->num_layers * q_layer;
-    const bool at_once = hidden && !io && !ev && (int)M >= ctx->tune.lm_pair_min_rows && apart(hidden, M * (size_t)ctx->desc.hidden * 2, attn_out, attn_bytes) &&
-                         apart(W, (size_t)ctx->desc.vocab * ctx->desc.hidden * 2, attn_out, attn_bytes);
+    const bool w_apart = apart(W, (size_t)ctx->desc.vocab * ctx->desc.hidden * 2, attn_out, attn_bytes);
+    const bool at_once = hidden && !io && !ev && (int)M >= ctx->tune.lm_pair_min_rows && w_apart &&
+                         apart(hidden, M * (size_t)ctx->desc.hidden * 2, attn_out, attn_bytes);
     MirrorAttnBeside beside;
     if (at_once) {
         const double bytes_ns = 2.0 * ctx->desc.vocab * ctx->desc.hidden / 6400.0, flops_ns = bytes_ns * M * 6400.0 / 1.2e6;
@@ -207,7 +208,7 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     if (ev) MIRROR_CUDA_OK(cudaEventRecord(ctx->stage_ev[1], s));
 
     // (Its weights may be requested early: behind an attention launch, which waits for all before it, nothing of the caller's can
-    // still be writing them.)
+    // still be writing them; nor does the attention, unless they lie in its output.)
     // LM-head rows: the given hidden states, else the last layer's attention output ([B*n, Hq*d] == [M, H])
     const void* rows = hidden;
     if (!rows) {
@@ -224,7 +225,7 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     st = mirror_lmhead_launch(ctx, rows, (int)M, W, 0, nullptr, nullptr, 0, d_argmax, nullptr, spec ? d_lse : nullptr, nullptr,
                               nullptr, nullptr, d_logits, ws + L.lm_partial, L.lm_partial_bytes, d_lse, s,
                               ev ? ctx->stage_ev[2] : nullptr, nullptr, nullptr, 0, defer ? &partials : nullptr,
-                              beside.granted ? MIRROR_LM_AT_ONCE : io ? MIRROR_LM_AFTER : MIRROR_LM_WEIGHTS_EARLY);
+                              beside.granted ? MIRROR_LM_AT_ONCE : io || !w_apart ? MIRROR_LM_AFTER : MIRROR_LM_WEIGHTS_EARLY);
     if (st != MIRROR_OK) return st;
 
     // The attention's merge, beside the kernel that folds the row partials, or (below) beside the acceptance that folds them itself.

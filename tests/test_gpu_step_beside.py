@@ -66,3 +66,22 @@ def test_hidden_rows_that_are_the_attention_output_wait_for_it():
     m.mirror_verify_step(kv, tree, x.q, x.k_new, x.v_new, attn[-1].reshape(cfg.rows, cfg.hidden), x.W, acc, attn, argmax_out=argmax[1])
     torch.cuda.synchronize()
     assert torch.equal(argmax[0], argmax[1])
+
+
+@pytest.mark.parametrize("own_rows", [True, False])
+def test_weights_that_are_the_attention_output_wait_for_it(own_rows):
+    """... whether the hidden rows are the caller's (LM head beside the attention) or the attention's (its weights requested early)."""
+    V = 64
+    cfg = I.VerifyConfig("w", 2048, 16, 8, 128, 6, 1, 900, 900, 4, 4, V, "greedy", explicit_hidden=own_rows)
+    x = I.gen_verify_inputs(cfg, 3, "cuda", force_hidden=own_rows)
+    m = make_mirror(cfg)
+    kv, tree, acc = m.kv(x.k_pool, x.v_pool, x.page_table, x.prefix_len), m.tree(x.tokens, 4, 4), m.accept_in(binding.ACCEPT_GREEDY, True)
+    ref = m.mirror_attn_verify(kv, tree, x.q, x.k_new, x.v_new)
+    rows = x.hidden if own_rows else ref[-1].reshape(cfg.rows, cfg.hidden)
+    want = m.mirror_lmhead_reduce(rows, ref.reshape(-1, cfg.hidden)[:V])["argmax"]
+    attn, argmax = torch.empty_like(x.q), torch.empty(cfg.rows, dtype=torch.int32, device="cuda")
+    for seed in range(3):
+        attn.normal_()                                     # (weights read too early would be these)
+        m.mirror_verify_step(kv, tree, x.q, x.k_new, x.v_new, x.hidden if own_rows else None, attn.reshape(-1, cfg.hidden)[:V], acc, attn, argmax_out=argmax)
+        assert m.device_status() == (0, 0)
+        assert torch.equal(attn, ref) and torch.equal(argmax, want)
