@@ -287,3 +287,19 @@ def test_a_wait_that_runs_out_beside_the_attention(mode, B, monkeypatch):
         got, want = c.out.cpu(), ref.out.cpu()
         for f in FIELDS:
             np.testing.assert_array_equal(got[f], want[f], err_msg=f)
+
+
+@pytest.mark.parametrize("mode", ["greedy", "spec_sampling"])
+def test_rows_per_unit_can_be_set(mode, monkeypatch):
+    """MIRROR_LM_ROWS, as for an LM head of its own, where the workspace has room for that many units' partials."""
+    case = dict(L=2, B=1, lo=100, hi=100, kappa=4, gamma=4, hq=16, mode=mode, hidden=512, vocab=20000)
+    ref, blocks = Case(**case), {}
+    ref.step()
+    for rows in (0, 32, 96, 128):
+        if rows:
+            monkeypatch.setenv("MIRROR_LM_ROWS", str(rows))
+        c = Case(**case)
+        blocks[rows] = kernels(c.step)["lmhead_pair_free_kernel"][1]
+        assert c.m.device_status() == (0, 0) and torch.equal(c.argmax, ref.argmax)
+    # a CTA per `rows` ids; 32 would be 313 pairs of CTAs, more than there are, and more units than partials where each has its own
+    assert blocks[96] == 2 * 105 and blocks[128] == 2 * 79 and blocks[32] == (296 if mode == "greedy" else blocks[0]), blocks
