@@ -148,6 +148,7 @@ mirror_status mirror_kv_quantize_launch(mirror_ctx* ctx, const void* x, int n_la
 struct MirrorAttnBeside {
     float work_ns = 0.f;                  // how long it takes on its own
     bool stream = false;                  // it streams weights, and needs SMs only for that
+    bool in_parts = false;                // ... in more units than fit the chip at a time, so that a few SMs get it ahead
     bool granted = false;                 // answer: launch it so
     // answer: the units that the partition cut are still to be merged, by mirror_attn_late_merge() behind a kernel that lets its
     // successor start only once a launch that itself has waited for the attention is through

@@ -171,6 +171,7 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
         const double bytes_ns = 2.0 * ctx->desc.vocab * ctx->desc.hidden / 6400.0, flops_ns = bytes_ns * M * 6400.0 / 1.2e6;
         beside.work_ns = (float)std::max(bytes_ns, flops_ns);
         beside.stream = M <= 128;                            // (more rows: the tensor cores set the LM head's pace, too)
+        beside.in_parts = ctx->desc.vocab > ctx->num_sms * 256;      // (a CTA pair per SM, units of up to 2 x 128 ids)
         st = mirror_attn_launch(ctx, kv, tree, ti, q, k_new, v_new, attn_out, nullptr, (float*)(ws + L.attn_partial), s, f8, false, &beside);
         if (st != MIRROR_OK) return st;
     } else if (!io) {

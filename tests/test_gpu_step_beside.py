@@ -175,6 +175,7 @@ _NAMES = {"attn_verify_kernel": "A", "lmhead_pair_free_kernel": "F", "lmhead_mer
     ("A2FRMD", dict(L=12, B=1, lo=1000, hi=1000, kappa=8, gamma=7, hq=40, mode="spec_tree", fp8=True)),
     ("A2FD", dict(L=60, B=3, lo=17, hi=90, kappa=4, gamma=4, hq=40, mode="greedy", fp8=True)),                   # short units
     ("A1FD", dict(L=40, B=1, lo=700, hi=700, kappa=4, gamma=4, hq=40, mode="greedy", fp8=True)),                 # whole ones
+    ("A1FD", dict(L=42, B=1, lo=106, hi=106, kappa=8, gamma=6, hq=56, mode="greedy", vocab=12480, hidden=7680)), # an LM head of one wave: no SMs left to it
     ("A1FRMD", dict(L=16, B=8, lo=1000, hi=3000, kappa=8, gamma=6, hq=40, mode="spec_sampling", hidden=4096)),   # 392 rows: two row chunks, sums, spilled logits
     ("A1FRMD", dict(L=16, B=8, lo=1000, hi=3000, kappa=8, gamma=6, hq=40, mode="greedy", hidden=4096)),
     ("A2FDM", dict(L=12, B=1, lo=200, hi=200, kappa=8, gamma=7, hq=40, mode="greedy", headroom=6000)),           # a table much longer than the prefix:
