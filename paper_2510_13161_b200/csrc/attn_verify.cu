@@ -144,7 +144,7 @@ __device__ __forceinline__ void fill_segment(Segment& s, int left, const AttnPar
     s.tiles = tiles_of(s.len, p.tree_slots);
     s.t_last = min(s.tiles, s.t_first + left);
 }
-// (not inlined: in the kernel's prologue it cost e4m3 calls of many units 0.6%, 12 requests of 336..1185 tokens 828.6 -> 823.5 us)
+// (out of line: code that runs once)
 __device__ __noinline__ void first_segment(Segment& s, int left, const AttnParams& p, const int* s_len) { fill_segment(s, left, p, s_len); }
 // the unit behind s (a segment that is followed by another one ends with its unit)
 __device__ __noinline__ Segment next_segment(const Segment& s, int left, const AttnParams& p, const int* s_len) {
@@ -177,26 +177,6 @@ struct Ctrl {
     volatile int abort;
 };
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block");
-
-// Bounded waits by all lanes of a converged warp, which all get the same answer.  One poll inline; what follows when the
-// barrier is not complete yet (parking in the barrier unit, the CTA's abort flag, the limit) is out of line: the code that
-// the twelve warps of a CTA run per tile has to stay in the SM's instruction cache.
-__device__ __noinline__ bool wait_slow(Ctrl* c, uint64_t* bar, uint32_t parity, int where) {
-    const long long t0 = clock64();
-    for (;;) {
-        if (__all_sync(0xffffffffu, ptx::mbar_try_wait_park(bar, parity, MIRROR_PARK_NS))) return true;
-        const bool late = clock64() - t0 > c->wait_limit;
-        if (__any_sync(0xffffffffu, c->abort || late)) {
-            c->abort = 1;
-            if (late && atomicCAS(c->status, 0, MIRROR_DEV_TIMEOUT) == 0) atomicExch(c->status + 1, where);
-            return false;
-        }
-    }
-}
-__device__ __forceinline__ bool wait_bar(Ctrl* c, uint64_t* bar, uint32_t parity, int where) {
-    if (__all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity))) return true;
-    return wait_slow(c, bar, parity, where);
-}
 
 // How the tile sequence is cut into one range per CTA group.  (This runs in front of every launch's first copy, by one
 // warp and from a cold instruction cache: few divisions, and those of 32 bits.)
@@ -567,8 +547,8 @@ __device__ __forceinline__ uint2 widen4(uint32_t w) {
     return r;
 }
 
-// kEarly: only q and the tree's K/V come from the kernel ahead (see mirror_attn_launch).  An instance of its own: the same as
-// run-time branches cost long calls, which never take them, 0.8% (64 layers, 32768 tokens, 33 nodes: 3608 -> 3639 us).
+// kEarly: only q and the tree's K/V come from the kernel ahead (see mirror_attn_launch).  An instance of its own: long calls never
+// take these branches.
 template <int D, bool F8, bool kEarly>
 __global__ void __launch_bounds__(Cfg<D, F8>::kThreads, 1)
 attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ AttnTree tree, const __grid_constant__ AttnParams p,
@@ -692,7 +672,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                         pg_next = fetch(tt + 1);
                         pg_t = tt;
                     }
-                    if (!wait_bar(ctrl, &ctrl->empty[st0 + st], ph, 10)) { ok = false; return; }
+                    if (!ptx::warp_wait(ctrl, &ctrl->empty[st0 + st], ph, 10)) { ok = false; return; }
                     uint8_t* const dst = ring + (size_t)(st0 + st) * C::kStageBytes;
                     uint64_t* const bar = &ctrl->full[st0 + st];
                     const int head = sg.g * p.heads_per_unit + stream_of(p, rb, g).head_off;
@@ -757,7 +737,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                     for (int k = 0; k < (split ? 1 : 2); ++k) {
                         const int buf = split ? (int)(n_seg & 1) : k;
                         const uint32_t use = split ? n_seg >> 1 : n_seg;          // how often this buffer has been filled
-                        if (!wait_bar(ctrl, &ctrl->q_empty[buf], (use & 1) ^ 1, 11)) { ok = false; break; }
+                        if (!ptx::warp_wait(ctrl, &ctrl->q_empty[buf], (use & 1) ^ 1, 11)) { ok = false; break; }
                         if (lane == 0) {
                             const StreamId id = stream_of(p, rb, k);
                             const int head = (s.g * p.heads_per_unit + id.head_off) * p.G + (id.rt / p.node_tiles) * p.gs;
@@ -865,7 +845,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                 wst += (uint32_t)n;
                 if (wst >= kWideStages) { wst -= kWideStages; wph ^= 1; }
             };
-            auto wait = [&](uint64_t* bar, uint32_t parity, int where) { ok = ok && wait_bar(ctrl, bar, parity, where); };
+            auto wait = [&](uint64_t* bar, uint32_t parity, int where) { ok = ok && ptx::warp_wait(ctrl, bar, parity, where); };
             auto take_k = [&]() -> uint32_t {        // wait for the next stage of the ring
                 const uint32_t s = st;
                 wait(&ctrl->full[s], ph, 21);
@@ -991,7 +971,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         bool ok = true;
         Segment sg = ctrl->first, nx = sg;
         // (the first segment's Q is converted out of the buffers that these warps are about to fill)
-        if (left > 0) ok = wait_bar(ctrl, &ctrl->q_full[0], 0, 28) && (split || wait_bar(ctrl, &ctrl->q_full[2], 0, 28));
+        if (left > 0) ok = ptx::warp_wait(ctrl, &ctrl->q_full[0], 0, 28) && (split || ptx::warp_wait(ctrl, &ctrl->q_full[2], 0, 28));
 #pragma unroll 1
         while (left > 0 && ok) {
             const int seg_tiles = sg.t_last - sg.t_first;
@@ -1005,7 +985,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             const int q_buf = split ? (int)(n_seg & 1) : q_grp * 2 + (int)(n_seg & 1);
             auto q_step = [&]() {                                  // store the rows that were loaded, load the next ones
                 if (q_at < q_loaded) {
-                    if (q_at == 0 && !wait_bar(ctrl, &ctrl->q_empty[q_buf], ((n_seg >> 1) & 1) ^ 1, 11)) { ok = false; return; }
+                    if (q_at == 0 && !ptx::warp_wait(ctrl, &ctrl->q_empty[q_buf], ((n_seg >> 1) & 1) ^ 1, 11)) { ok = false; return; }
 #pragma unroll 1
                     for (; q_at < q_loaded; ++q_at) {
                         store_q_row(sQ + q_buf * C::kQBytes, q_row0 + q_at, qv[0], qs);
@@ -1035,7 +1015,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                 if (!ok) break;
                 continue;
             }
-            if (!wait_bar(ctrl, &ctrl->full[ring_n + st], ph, 26) || !wait_bar(ctrl, &ctrl->wide_empty[wst], wph, 27)) { ok = false; break; }
+            if (!ptx::warp_wait(ctrl, &ctrl->full[ring_n + st], ph, 26) || !ptx::warp_wait(ctrl, &ctrl->wide_empty[wst], wph, 27)) { ok = false; break; }
             const uint8_t* const src = ring + (size_t)(ring_n + st) * C::kStageBytes + src_off;
             uint8_t* const dst = wide + (size_t)wst * C::kWideBytes;
 #pragma unroll 1
@@ -1058,7 +1038,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             q_step();
             if (!ok) break;
             }
-            if (left > 0 && ok && q_end == 0) ok = wait_bar(ctrl, &ctrl->q_empty[q_buf], ((n_seg >> 1) & 1) ^ 1, 11);      // (no arrival ahead of its phase)
+            if (left > 0 && ok && q_end == 0) ok = ptx::warp_wait(ctrl, &ctrl->q_empty[q_buf], ((n_seg >> 1) & 1) ^ 1, 11);      // (no arrival ahead of its phase)
             if (left > 0 && ok) {
                 ptx::fence_proxy_async();
                 __syncwarp();
@@ -1085,7 +1065,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         auto pair_sync = [&]() -> bool {
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&ctrl->pair[w4]);
-            const bool r = wait_bar(ctrl, &ctrl->pair[w4], xph, 35);
+            const bool r = ptx::warp_wait(ctrl, &ctrl->pair[w4], xph, 35);
             xph ^= 1;
             return r;
         };
@@ -1095,7 +1075,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         uint32_t t_par = grp == 0 ? 1 : 0;
         auto take_turn = [&]() -> bool {
             if (F8) return true;
-            const bool r = wait_bar(ctrl, &ctrl->exp_turn[grp][w4], t_par, 36);
+            const bool r = ptx::warp_wait(ctrl, &ctrl->exp_turn[grp][w4], t_par, 36);
             t_par ^= 1;
             return r;
         };
@@ -1149,7 +1129,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             const int mine = split ? (sg.t_last - sg.t_first + 1 - grp) >> 1 : sg.t_last - sg.t_first;     // tiles of this stream
             for (int i = 0; i < mine; ++i) {
                 const int t = split ? sg.t_first + 2 * i + grp : sg.t_first + i;
-                if (!wait_bar(ctrl, &ctrl->s_full[grp], s_par, 30)) { ok = false; break; }
+                if (!ptx::warp_wait(ctrl, &ctrl->s_full[grp], s_par, 30)) { ok = false; break; }
                 s_par ^= 1;
                 ptx::tc_fence_after();
                 if (warp_has_rows) {
@@ -1187,7 +1167,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                         if (__any_sync(0xffffffffu, grow)) {
                             tmem_ld_wait32(ra);
                             if (h == 1) {
-                                if (!wait_bar(ctrl, &ctrl->pv_half[grp], s_par ^ 1, 33)) { ok = false; break; }
+                                if (!ptx::warp_wait(ctrl, &ctrl->pv_half[grp], s_par ^ 1, 33)) { ok = false; break; }
                                 ptx::tc_fence_after();
                             }
                             const float2 m = move_offset(s_addr + (uint32_t)(h * 64), o_addr, i + h > 0 ? D : 0, grow, off, sc);
@@ -1239,7 +1219,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
                 xc[grp * 2 + 1] = l_run;
             }
             if (mine > 0) {
-                if (!wait_bar(ctrl, &ctrl->o_full[grp], o_par, 32)) { ok = false; break; }
+                if (!ptx::warp_wait(ctrl, &ctrl->o_full[grp], o_par, 32)) { ok = false; break; }
                 o_par ^= 1;
             }
             float M = off, Lsum = l_run;

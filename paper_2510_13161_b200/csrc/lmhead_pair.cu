@@ -110,46 +110,16 @@ __device__ __forceinline__ uint32_t map_to_rank(const void* smem_ptr, uint32_t r
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(ptx::smem_u32(smem_ptr)), "r"(rank));
     return r;
 }
-// (What it hands over is tensor memory that tcgen05.ld has already been waited for, nothing that the arriving thread wrote: a release at
-// cluster scope would hold a unit's end up behind its spilled logits and state; 132 rows x 137273 x 768: 82.7 -> 80.1 us.)
+// (Without a scope, that is a release within the CTA, although the waiter acquires at cluster scope: what it hands over is tensor memory,
+// whose reads tcgen05.wait::ld and, towards the waiter's UMMAs, tcgen05.fence::before_thread_sync have ordered; no memory that the arriving
+// thread wrote goes with it.  A release at cluster scope would hold a unit's end up behind its spilled logits and state; 132 rows x
+// 137273 x 768: 82.7 us, without 80.1.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // a word into the shared memory of a CTA of the pair, counted on a barrier there
 __device__ __forceinline__ void st_async(uint32_t cluster_addr, int v, uint32_t bar_cluster_addr) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(cluster_addr), "r"(v), "r"(bar_cluster_addr) : "memory");
-}
-// Bounded waits by all lanes of a converged warp, which all get the same answer: one poll inline; parking, the abort flag and the
-// limit are out of line.  kCluster: the other CTA of the pair arrives on the barrier.
-template <bool kCluster>
-__device__ __forceinline__ bool try_wait(uint64_t* bar, uint32_t parity) {
-    if (!kCluster) return __all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity));
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(ptx::smem_u32(bar)), "r"(parity)
-        : "memory");
-    return __all_sync(0xffffffffu, ok != 0);
-}
-template <bool kCluster>
-__device__ __noinline__ bool wait_slow(Ctrl* c, uint64_t* bar, uint32_t parity, int where) {
-    const long long t0 = clock64();
-    for (;;) {
-        if (__all_sync(0xffffffffu, ptx::mbar_try_wait_park(bar, parity, MIRROR_PARK_NS)) && try_wait<kCluster>(bar, parity)) return true;
-        const bool late = clock64() - t0 > c->wait_limit;
-        if (__any_sync(0xffffffffu, c->abort || late)) {
-            c->abort = 1;
-            if (late && atomicCAS(c->status, 0, MIRROR_DEV_TIMEOUT) == 0) atomicExch(c->status + 1, where);
-            return false;
-        }
-    }
-}
-template <bool kCluster = false>
-__device__ __forceinline__ bool wait_warp(Ctrl* c, uint64_t* bar, uint32_t parity, int where) {
-    return try_wait<kCluster>(bar, parity) || wait_slow<kCluster>(c, bar, parity, where);
 }
 // Has the phase completed?  (Does not block; try_wait may, for as long as the hardware likes: asked that way for the K block behind the
 // one at hand, the issuer held that one back until the other had arrived, and short launches took up to half as long again.)
@@ -315,7 +285,7 @@ __device__ __forceinline__ void for_lanes(float* bcast, float x, F f) {
 // projections, split along K when there are fewer tiles than CTA pairs; the epilogue only stores fp32 partial sums.
 // kFp8 / kTopk: e4m3 operands with per-row scales / Top-kappa lists in the epilogue, as separate instantiations so that
 // the plain bf16 head carries none of their registers and branches.
-// kEarly: a kernel of its own, since the few instructions that it adds in front of the wait cost the others 0.3-6% (code placement).
+// kEarly: a kernel of its own, since the few instructions that it adds in front of the wait cost the others up to 6%.
 // kFree: nothing that this launch reads is written by the kernel ahead (an attention launch, which has waited for all before it), so
 // its CTAs begin as SMs come free, and only their end waits.  They begin at very different times, so the pairs take units from
 // a counter: the leader's producer names them to both CTAs.  Results do not depend on who takes what: argmax does not, and
@@ -393,7 +363,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
     // kFree: unit number j of this pair, or (no more, or a failure) one past the last; whole warps
     auto named_unit = [&](uint32_t j) -> int {
         const uint32_t e = j % kUnitRing;
-        if (!wait_warp<true>(ctrl, &ctrl->unit_full[e], (j / kUnitRing) & 1, 17)) return p.n_units;
+        if (!ptx::warp_wait<true>(ctrl, &ctrl->unit_full[e], (j / kUnitRing) & 1, 17)) return p.n_units;
         return *(volatile int*)&ctrl->unit[e];
     };
 
@@ -449,7 +419,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
 #pragma unroll 1
             for (; kb < kb_end; ++kb) {
                 if (p.stall_after >= 0 && n_issued >= p.stall_after) { ok = false; break; }       // (test aid: neither arms nor copies)
-                if (!wait_warp(ctrl, &ctrl->empty[s], ph ^ 1, 11)) { ok = false; break; }
+                if (!ptx::warp_wait(ctrl, &ctrl->empty[s], ph ^ 1, 11)) { ok = false; break; }
                 if (ptx::elect_one()) {
                     if (rank == 0) ptx::mbar_arrive_expect_tx(&ctrl->full[s], 2u * (uint32_t)p.stage_bytes);
                     uint8_t* dst = stage_base + s * p.stage_bytes;
@@ -475,7 +445,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
             bool ok = true;
             uint32_t j = 0;
             for (int u = kFree ? named_unit(0) : pair; u < p.n_units && ok; u = kFree ? named_unit(++j) : u + n_pairs) {
-                if (!wait_warp<true>(ctrl, &ctrl->acc_empty[ab], aph ^ 1, 12)) { ok = false; break; }
+                if (!ptx::warp_wait<true>(ctrl, &ctrl->acc_empty[ab], aph ^ 1, 12)) { ok = false; break; }
                 const uint32_t d_tmem = tmem_base + (uint32_t)(ab * p.acc_stride);
                 int tile, slice, chunk;
                 decode(u, tile, slice, chunk);
@@ -483,7 +453,7 @@ __device__ __forceinline__ void pair_gemm_body(const CUtensorMap& tm_w, const CU
                 bool ready = poll(&ctrl->full[s], ph);
 #pragma unroll 1
                 for (int kb = 0; kb < nk; ++kb) {
-                    if (!ready && !wait_slow<false>(ctrl, &ctrl->full[s], ph, 13)) { ok = false; break; }
+                    if (!ready && !ptx::warp_wait_slow<false>(ctrl, &ctrl->full[s], ph, 13)) { ok = false; break; }
                     ptx::tc_fence_after();
                     uint64_t* const done = &ctrl->empty[s];
                     const uint32_t a = lo;

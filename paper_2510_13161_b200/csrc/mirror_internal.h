@@ -155,8 +155,10 @@ struct MirrorAttnBeside {
     bool merge_needed = false;
     unsigned char merge[512];
 };
-// early: of what the launch reads, only q, k_new and v_new are written by the kernel ahead, and whatever ran before that one has
-// completed when this launch begins: lengths, page table and the cache's pages are read without waiting for it.
+// early: lengths, page table and the cache's pages are read, and the notes written, without waiting for the kernel ahead.  That one
+// (finish_qkv_kernel) writes q, k_new and v_new and lets this launch begin at once; it may still be running then, and so may the GEMM ahead
+// of it, which itself had waited before it let anything begin: all that is older has completed.  Neither of the two may write lengths, page
+// table or cache pages, nor read or write the attention's notes and records.
 // keep_rounding: every sum keeps the order of the 64-token kernel (mirror_target_forward in deep stacks, see attn_tile64.cu).
 mirror_status mirror_attn_launch(mirror_ctx* ctx, const mirror_kv* kv, const mirror_tree* tree, const MirrorTreeInfo& ti,
                                  const void* q, const void* k_new, const void* v_new, void* out, float* lse_out,
@@ -251,6 +253,41 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
         if (mbar_try_wait_park(bar, parity, MIRROR_PARK_NS)) return true;
         if (clock64() - t0 > limit_cycles) return false;
     }
+}
+
+// Bounded waits by all lanes of a converged warp, which all get the same answer.  One poll inline; what follows when the
+// barrier is not complete yet (parking in the barrier unit, the CTA's abort flag, the limit) is out of line: the code that
+// the warps of a CTA run per tile has to stay in the SM's instruction cache.  C: a control block in shared memory with the members
+// abort, status and wait_limit.  kCluster: the other CTA of a pair arrives on the barrier.
+template <bool kCluster>
+__device__ __forceinline__ bool warp_try_wait(uint64_t* bar, uint32_t parity) {
+    if (!kCluster) return __all_sync(0xffffffffu, mbar_try_wait(bar, parity));
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return __all_sync(0xffffffffu, ok != 0);
+}
+template <bool kCluster, class C>
+__device__ __noinline__ bool warp_wait_slow(C* c, uint64_t* bar, uint32_t parity, int where) {
+    const long long t0 = clock64();
+    for (;;) {
+        if (__all_sync(0xffffffffu, mbar_try_wait_park(bar, parity, MIRROR_PARK_NS)) && (!kCluster || warp_try_wait<kCluster>(bar, parity))) return true;
+        const bool late = clock64() - t0 > c->wait_limit;
+        if (__any_sync(0xffffffffu, c->abort || late)) {
+            c->abort = 1;
+            if (late && atomicCAS(c->status, 0, MIRROR_DEV_TIMEOUT) == 0) atomicExch(c->status + 1, where);
+            return false;
+        }
+    }
+}
+template <bool kCluster = false, class C>
+__device__ __forceinline__ bool warp_wait(C* c, uint64_t* bar, uint32_t parity, int where) {
+    return warp_try_wait<kCluster>(bar, parity) || warp_wait_slow<kCluster>(c, bar, parity, where);
 }
 
 // ---- TMA -------------------------------------------------------------------------------------

@@ -161,7 +161,8 @@ mirror_status verify_step_impl(mirror_ctx* ctx, const mirror_kv* kv, const mirro
     const bool ev = ctx->stage_ev_on && !io;
     if (ev) MIRROR_CUDA_OK(cudaEventRecord(ctx->stage_ev[0], s));
     // Hidden rows of the caller's own do not depend on the attention: the LM head is launched beside it (see lmhead_pair.cu), on the
-    // SMs that the attention leaves or has done with, and the attention's merge behind the decision.
+    // SMs that the attention leaves or has done with.  The attention's merge then comes behind the LM head's: behind the decision where that
+    // folds the row partials itself, else in front of the decision, which waits for it.
     const size_t attn_bytes = (size_t)kv->num_layers * q_layer;
     const bool w_apart = apart(W, (size_t)ctx->desc.vocab * ctx->desc.hidden * 2, attn_out, attn_bytes);
     const bool at_once = hidden && !io && !ev && (int)M >= ctx->tune.lm_pair_min_rows && w_apart &&
