@@ -170,7 +170,7 @@ struct Ctrl {
     uint64_t pair[4];                                   // split: the two softmax warps of a TMEM quarter meet
     Segment first;                                      // where this CTA's range begins
     int n_tiles;
-    int group;                                          // which group this CTA belongs to
+    int place;                                          // this CTA's among the records: by its group, not by its block
     int* status;
     long long wait_limit;
     uint32_t tmem_base;
@@ -626,7 +626,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
         const int x1 = __shfl_sync(0xffffffffu, u.x, 1);
         if (lane == 0) {
             ctrl->n_tiles = x1 - u.x;
-            ctrl->group = group;
+            ctrl->place = group * p.n_cta + rb;
             Segment& s = ctrl->first;
             s.layer = u.layer; s.b = u.b; s.g = u.g; s.t_first = u.t;
             if (u.x < x1) first_segment(s, x1 - u.x, p, s_len);
@@ -1209,7 +1209,7 @@ attn_verify_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Attn
             float* lse_ptr = p.lse_out ? p.lse_out + (lb * p.Hq + head) * p.n + node : nullptr;
             const int slot = (sg.t_first > 0) ? 0 : 1;             // a unit that began before this CTA's range uses slot 0
             // record layout [column][row]: a warp's store of one column is one contiguous 128-byte line
-            float* rec = p.partial + (((size_t)(ctrl->group * p.n_cta + rb) * 2 + slot) * 2 + (split ? 0 : grp)) * kRowW * kRows + row;
+            float* rec = p.partial + (((size_t)ctrl->place * 2 + slot) * 2 + (split ? 0 : grp)) * kRowW * kRows + row;
             left -= sg.t_last - sg.t_first;
             Segment nx = sg;
             if (left > 0) nx = next_segment(sg, left, p, s_len);
